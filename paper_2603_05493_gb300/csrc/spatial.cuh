@@ -83,7 +83,11 @@ __device__ __forceinline__ void joint_sincos(float th, float* s, float* c) {
 // variable th: T_fixed * J(th).  Revolute: R = R_f R_J(th) with Rodrigues'
 // rotation R_J = c I + s [a]^ + (1-c) a a^T.  Prismatic: p = p_f + R_f a th.
 // (jt, ident: the link's joint type and whether its fixed rotation is the
-// identity, from a packed table the caller holds)
+// identity, from a packed table the caller holds; UNIT: the sine and cosine
+// scaled to s^2 + c^2 = 1 within a rounding -- the fast pair misses it by up to
+// 7e-7 -- so that R's inverse is its transpose and products of many R stay
+// rotations)
+template <bool UNIT = false>
 __device__ __forceinline__ void local_xf_m(const DevRobot& r, int k, float th, int jt, bool ident,
                                            float* R, float* p) {
   const float4* T4 = reinterpret_cast<const float4*>(r.Tf + 12 * k);
@@ -96,6 +100,11 @@ __device__ __forceinline__ void local_xf_m(const DevRobot& r, int k, float th, i
     const float4 a = ldp(reinterpret_cast<const float4*>(r.axis) + k);
     float s, c;
     joint_sincos(th, &s, &c);
+    if (UNIT) {
+      const float u = 0.5f * fmaf(-s, s, fmaf(-c, c, 1.0f));
+      s = fmaf(s, u, s);
+      c = fmaf(c, u, c);
+    }
     const float t = 1.0f - c;
     const float tx = t * a.x, ty = t * a.y, tz = t * a.z;
     const float sx = s * a.x, sy = s * a.y, sz = s * a.z;

@@ -18,35 +18,47 @@
 // tau_j += m_k S_k^T F_k and adds X_k^T F_k to the parent.
 //
 // Backward (the VJP of Alg. 4 and of FK; Alg. 5 and Alg. 1 give the
-// structure): every pass of the adjoint fits the same sweep.
-//   pre-order:  Fbar_k = S_k m_k taubar_j + X_k Fbar_pa          (base -> tips)
-//               (with the pose, v_k and a_k of the forward)
-//   post-order: the link's own terms
-//                 f_k    = I a_k + v_k x* I v_k
-//                 abar_k = I Fbar_k,
-//                 vbar_k = -crf(Fbar_k) I v_k - I crm(v_k) Fbar_k
-//                 W_k    = link-frame gradient wrench of the kinematic outputs
-//               plus the children's sums complete F_k, abar_k, vbar_k, W_k
-//               vbar_k += crf(S qd_k) abar_k
-//               qdd_bar = S^T abar_k
-//               qd_bar  = S^T vbar_k - S^T crf(v_k) abar_k
-//               q_bar   = (X_k Fbar_pa)^T crf(S) F_k - abar^T crm(S) X_k a_pa
-//                         - vbar^T crm(S) X_k v_pa + S^T W_k
-//               parent += X_k^T (F, abar, vbar, W)
-// The root's a_pa is the base acceleration -g, so its q_bar terms follow the
-// general formula; the v-dependence of a_k through v_k x_m (S qd) enters as
-// the crf(S qd) abar term.  Both are derived from Alg. 4 by reverse-mode
-// differentiation.
+// structure): every pass of the adjoint fits the same sweep.  It is written in
+// world axes about each link's own origin, with the Newton-Euler form of Alg. 4
+// (angular velocity w, angular acceleration al, acceleration A of the origin;
+// the origin's velocity cancels).  With the torque adjoints as joint rates,
+// wb and ub are the links' angular and linear velocity of that virtual motion,
+// and sum_j taubar_j tau_j = sum_k wb_k . n_k + ub_k . f_k.  s: the joint's
+// world axis, r: the offset from the parent's origin.
+//   pre-order:  W, w, al, A, wb, ub of the link from its parent's
+//   post-order: the link's (n, f) and the gradients gw, gal, gA of wb . n +
+//               ub . f (link_adjoint), its gradient wrench (Wn, Wf) of the
+//               kinematic outputs, plus the children's sums; the joint's
+//               gradients; the sums moved to the parent's origin:
+//               qdd_bar = s . gal,  qd_bar = s . gw + (w x s) . gal
+//               q_bar   = s . [Wn - w x gw - al x gal - A x gA - wb x n - ub x f]
+//               gw_pa  += gw + qd s x gal + grad_w [gA . (w x (w x r))]
+//               gal_pa += gal + r x gA,  gA_pa += gA
+//               n_pa   += n + r x f,  f_pa += f,  Wn_pa += Wn + r x Wf
+//               (revolute; the prismatic forms stand at the close)
+// Derived from Alg. 4 by reverse-mode differentiation.  Against link axes with
+// 6-vectors (24 floats of sums, a rotation of every vector at every link, up
+// and down) the sums are 21 floats, a move between links is a few crosses, and
+// nothing spills at the 128-register cap: humanoid48 backward 0.165 -> 0.138
+// ms, with the cost and states from control points 0.131 -> 0.102 ms, the
+// uneven batch's 0.234 -> 0.200 ms.  The sine and cosine are scaled to the
+// unit circle (UNIT in local_xf_m): gradient error against 64 bits 3.5e-6 ->
+// 1.0e-6 (humanoid, 32768 configurations), where without it the world
+// rotations' drift from orthogonality gave 5.5e-6.  Storing the states of
+// branching links and reloading them at their children's closes instead:
+// 0.149 ms, 2.1e-6.  The forward keeps link axes: its torques feed the
+// torque-limit hinges, and there the world form was no faster (0.079 and
+// 0.077 ms).
 //
 // Segmented sweeps.  A tree with few links per level but many links in total
 // leaves one thread per configuration with a long serial chain and, at a few
 // tens of thousands of configurations, few warps per SM.  The DFS order can
 // instead be cut into G contiguous segments, one warp per segment over the
 // same 32 configurations.  The warp of segment g first replays the ancestors
-// of its first link (pre-order data only: poses, v, a, Fbar; its own force,
+// of its first link (pre-order data only; its own force,
 // adjoint and wrench contributions are zero), then sweeps its links.  Every
-// post-order quantity above is linear in the accumulated F, abar, vbar, W
-// given the pre-order data, so the outputs of a link that several segments
+// post-order quantity above is linear in the accumulated sums given the
+// pre-order data, so the outputs of a link that several segments
 // hold (an ancestor of a segment's first link) are the sums of the
 // segments' partial outputs.  Those partials go to shared-memory slots and
 // the kernel adds them in segment order (deterministic) after a barrier; all
@@ -133,132 +145,74 @@ __device__ __forceinline__ float* seg_part(const Seg& sg, int k, int o) {
   return sg.part + ((size_t)(o * sg.ns + s) * sg.G + sg.g) * 32 + sg.lane;
 }
 
-__device__ __forceinline__ void motion_S6t(int jt, const float* ax, float* S) {
-  S[0] = S[1] = S[2] = S[3] = S[4] = S[5] = 0.0f;
+// c += a x b
+__device__ __forceinline__ void cross3_acc(const float* a, const float* b, float* c) {
+  c[0] = fmaf(a[1], b[2], fmaf(-a[2], b[1], c[0]));
+  c[1] = fmaf(a[2], b[0], fmaf(-a[0], b[2], c[1]));
+  c[2] = fmaf(a[0], b[1], fmaf(-a[1], b[0], c[2]));
+}
+// c -= a x b
+__device__ __forceinline__ void cross3_sub(const float* a, const float* b, float* c) {
+  c[0] = fmaf(-a[1], b[2], fmaf(a[2], b[1], c[0]));
+  c[1] = fmaf(-a[2], b[0], fmaf(a[0], b[2], c[1]));
+  c[2] = fmaf(-a[0], b[1], fmaf(a[1], b[0], c[2]));
+}
+// c += f a x (a x b) = f (a (a . b) - b (a . a)), f = 1 or -1
+template <int SIGN>
+__device__ __forceinline__ void centripetal_acc(const float* a, const float* b, float* c) {
+  const float ab = SIGN * dot3(a, b), aa = SIGN * dot3(a, a);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) c[i] = fmaf(-b[i], aa, fmaf(a[i], ab, c[i]));
+}
+// c += the gradient of g . (w x (w x b)) with respect to w: b (w . g) +
+// g (w . b) - 2 w (b . g)
+__device__ __forceinline__ void centripetal_grad(const float* w, const float* b, const float* g,
+                                                 float* c) {
+  const float wg = dot3(w, g), wb = dot3(w, b), bg = -2.0f * dot3(b, g);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) c[i] = fmaf(w[i], bg, fmaf(g[i], wb, fmaf(b[i], wg, c[i])));
+}
+
+// Motion of a link from its parent's, all in world axes: angular velocity w,
+// angular acceleration al and acceleration A of the link's origin, which sits
+// r from the parent's; s: the joint's axis in the world, vq, aq its rate and
+// acceleration (jt 1 revolute, 2 prismatic, 0 fixed).
+__device__ __forceinline__ void joint_motion(int jt, const float* s, const float* r, float vq,
+                                             float aq, const float* wp, const float* alp,
+                                             const float* Ap, float* w, float* al, float* A) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    w[i] = wp[i];
+    al[i] = alp[i];
+    A[i] = Ap[i];
+  }
+  cross3_acc(alp, r, A);
+  centripetal_acc<1>(wp, r, A);
   if (jt == 1) {
-    S[0] = ax[0]; S[1] = ax[1]; S[2] = ax[2];
+    const float sq[3] = {s[0] * vq, s[1] * vq, s[2] * vq};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      w[i] += sq[i];
+      al[i] = fmaf(s[i], aq, al[i]);
+    }
+    cross3_acc(wp, sq, al);
   } else if (jt == 2) {
-    S[3] = ax[0]; S[4] = ax[1]; S[5] = ax[2];
+    const float sq[3] = {2.0f * vq * s[0], 2.0f * vq * s[1], 2.0f * vq * s[2]};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) A[i] = fmaf(s[i], aq, A[i]);
+    cross3_acc(wp, sq, A);
   }
 }
 
-// The close's terms with the joint's motion subspace S = [a; 0] (JT = 1,
-// revolute), [0; a] (JT = 2, prismatic) or 0 (JT = 0, fixed), written per
-// joint type so that S's zero half costs nothing (the joint type is
-// warp-uniform: every lane closes the same link).  The same operations, in
-// the same order, as the dense 6-vector forms on the nonzero half.
-//   parent terms: X_k v_pa = v - S qd, X_k a_pa = a - S qdd - v x_m (S qd),
-//                 X_k Fbar_pa = Fbar - S taubar;
-//   gradients:    gq = XF . crf(S) F - ab . crm(S) Xa - vb . crm(S) Xv + S . W,
-//                 vb += qd crf(S) ab (before gq and gqd), gqdd = S . ab,
-//                 gqd = S . vb - S . crf(v) ab.
-template <int JT>
-__device__ __forceinline__ void close_parent_terms(const float* a, float vq, float aq, float tb,
-                                                   const float* cv, const float* ca,
-                                                   const float* cFb, float* Xv, float* Xa,
-                                                   float* XF) {
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    Xv[i] = cv[i];
-    Xa[i] = ca[i];
-    XF[i] = cFb[i];
-  }
-  if (JT == 0) return;
-  const float s[3] = {a[0] * vq, a[1] * vq, a[2] * vq};
-  float c[3];
-  if (JT == 1) {  // v x_m [s; 0] = [w x s; u x s]
-    float cu[3];
-    cross3(cv, s, c);
-    cross3(cv + 3, s, cu);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      Xv[i] = cv[i] - s[i];
-      Xa[i] = ca[i] - fmaf(a[i], aq, c[i]);
-      Xa[3 + i] = ca[3 + i] - cu[i];
-      XF[i] = fmaf(-a[i], tb, cFb[i]);
-    }
-  } else {  // v x_m [0; s] = [0; w x s]
-    cross3(cv, s, c);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      Xv[3 + i] = cv[3 + i] - s[i];
-      Xa[3 + i] = ca[3 + i] - fmaf(a[i], aq, c[i]);
-      XF[3 + i] = fmaf(-a[i], tb, cFb[3 + i]);
-    }
-  }
+// y = Io x for the rotational part of the compact inertia
+__device__ __forceinline__ void rot_inertia(const float* I, const float* x, float* y) {
+  y[0] = fmaf(I[8], x[2], fmaf(I[7], x[1], I[4] * x[0]));
+  y[1] = fmaf(I[9], x[2], fmaf(I[5], x[1], I[7] * x[0]));
+  y[2] = fmaf(I[6], x[2], fmaf(I[9], x[1], I[8] * x[0]));
 }
 
-template <int JT>
-__device__ __forceinline__ void close_joint_grads(const float* a, float vq, const float* F,
-                                                  const float* ab, float* vb, const float* Wr,
-                                                  const float* cv, const float* Xv,
-                                                  const float* Xa, const float* XF, float& gq,
-                                                  float& gqd, float& gqdd) {
-  gq = gqd = gqdd = 0.0f;
-  if (JT == 0) return;
-  constexpr int w = JT == 1 ? 0 : 3;  // the half of a 6-vector S lives in
-  float t[3], t2[3];
-  if (JT == 1) {  // crf([a; 0]) f = [a x f_n; a x f_f]
-    cross3(a, F, t);
-    cross3(a, F + 3, t2);
-    gq = fmaf(XF[5], t2[2], fmaf(XF[4], t2[1], fmaf(XF[3], t2[0],
-         fmaf(XF[2], t[2], fmaf(XF[1], t[1], XF[0] * t[0])))));
-    cross3(a, ab, t);
-    cross3(a, ab + 3, t2);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      vb[i] = fmaf(vq, t[i], vb[i]);
-      vb[3 + i] = fmaf(vq, t2[i], vb[3 + i]);
-    }
-  } else {  // crf([0; a]) f = [a x f_f; 0]
-    cross3(a, F + 3, t);
-    gq = fmaf(XF[2], t[2], fmaf(XF[1], t[1], XF[0] * t[0]));
-    cross3(a, ab + 3, t);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) vb[i] = fmaf(vq, t[i], vb[i]);
-  }
-  gqdd = dot3(a, ab + w);
-  // the half of crf(v) ab that S picks: [w x ab_n + u x ab_f] or [w x ab_f]
-  float cr[3];
-  if (JT == 1) {
-    float c1[3], c2[3];
-    cross3(cv, ab, c1);
-    cross3(cv + 3, ab + 3, c2);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) cr[i] = c1[i] + c2[i];
-  } else {
-    cross3(cv, ab + 3, cr);
-  }
-  gqd = dot3(a, vb + w) - dot3(a, cr);
-  // crm([a; 0]) m = [a x m_w; a x m_u],  crm([0; a]) m = [0; a x m_w]
-  if (JT == 1) {
-    cross3(a, Xa, t);
-    cross3(a, Xa + 3, t2);
-    gq -= fmaf(ab[5], t2[2], fmaf(ab[4], t2[1], fmaf(ab[3], t2[0],
-          fmaf(ab[2], t[2], fmaf(ab[1], t[1], ab[0] * t[0])))));
-    cross3(a, Xv, t);
-    cross3(a, Xv + 3, t2);
-    gq -= fmaf(vb[5], t2[2], fmaf(vb[4], t2[1], fmaf(vb[3], t2[0],
-          fmaf(vb[2], t[2], fmaf(vb[1], t[1], vb[0] * t[0])))));
-  } else {
-    cross3(a, Xa, t);
-    gq -= fmaf(ab[5], t[2], fmaf(ab[4], t[1], ab[3] * t[0]));
-    cross3(a, Xv, t);
-    gq -= fmaf(vb[5], t[2], fmaf(vb[4], t[1], vb[3] * t[0]));
-  }
-  gq += dot3(a, Wr + w);
-}
-
-__device__ __forceinline__ float dot6t(const float* a, const float* b) {
-  float s = 0.0f;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) s = fmaf(a[i], b[i], s);
-  return s;
-}
-
-// world pose W = P o L (12 floats each)
-__device__ __forceinline__ void compose(const float* P, const float* L, float* W) {
-  float t[3];
+// world pose W = P o L (12 floats each); t: the offset of W's origin from P's
+__device__ __forceinline__ void compose(const float* P, const float* L, float* W, float* t) {
   matmul3(P, L, W);
   rot(P, L + 9, t);
   W[9] = P[9] + t[0];
@@ -411,7 +365,8 @@ __device__ __forceinline__ void tree_fwd_seg(const DevRobot& r, const FwdArgs& A
           ap[i] = P.a[i];
         }
       }
-      compose(PW, L, cW);
+      float t[3];
+      compose(PW, L, cW, t);
     } else {
 #pragma unroll
       for (int i = 0; i < 12; ++i) cW[i] = L[i];
@@ -537,33 +492,24 @@ __device__ __forceinline__ void tree_fwd_one(const DevRobot& r, const FwdArgs& A
 // ---------------------------------------------------------------------------
 // backward: the whole adjoint in one sweep
 // ---------------------------------------------------------------------------
-// The close of a link needs the link's pre-order state (world pose W, v, a,
-// Fbar) and the three parent terms of its q_bar formula, X_k v_pa, X_k a_pa
-// and X_k Fbar_pa.  Neither comes from a stack.  One state lives in
-// registers: a push carries it down one link (W_k = W_pa L_k, v_k = X_k v_pa
-// + S qd, ...) and a close carries it back up by undoing the same maps:
-//   X_k v_pa    = v_k - S qd
-//   X_k a_pa    = a_k - S qdd - v_k x_m (S qd)
-//   X_k Fbar_pa = Fbar_k - S taubar
-//   v_pa = X_k^-1 (X_k v_pa),  a_pa, Fbar_pa likewise,  W_pa = W_k L_k^-1
-// (X^-1 [w; u] = [R w; R u + p x R w]).  The first three are the parent
-// terms the close needs, so a close reads no parent data at all, and the
-// push of a later child finds its parent's state in the registers.  The
-// rounding of the repeated maps and inverses drifts by a few float ulps
-// per link visited (measured on the humanoid: 5e-6 relative on the
-// gradients against a sweep that stored each branching link's state and
-// reloaded it, which was 4 % slower).  Per-depth stack entry, only what a
-// later step reads:
-//   tb  -- the link's torque adjoint m taubar (for X_k Fbar_pa), for a link
-//          with children (a leaf's close follows its push and reads it from
-//          a register);
-//   acc -- the children's sums of F, abar, vbar, W, stored only when the
-//          push of a sibling subtree interrupts them.
-// The link's own F, abar and vbar are formed at its close from its state, and
-// its gradient wrench of the kinematic outputs too (its world pose is in the
+// The close of a link needs the link's pre-order state (world pose W, w, al,
+// A, wb, ub).  It does not come from a stack.  One state lives in registers:
+// a push carries it down one link and a close carries it back up by undoing
+// the same maps (w_pa = w - s qd, ...; W_pa = W L^-1), so a close reads no
+// parent data at all, and the push of a later child finds its parent's state
+// in the registers.  The rounding of the repeated maps and inverses drifts by
+// a few float ulps per link visited.
+// Per-depth stack entry, only what a later step reads:
+//   tb  -- the link's torque adjoint m taubar, for a link with children (a
+//          leaf's close follows its push and reads it from a register);
+//   acc -- the children's sums of n, f, gw, gal, gA and the wrench, stored
+//          only when the push of a sibling subtree interrupts them.
+// The link's own terms are formed at its close from its state, and its
+// gradient wrench of the kinematic outputs too (its world pose is in the
 // registers there): nothing of the link's own travels through the stack.
+constexpr int kSums = 21;   // n 3, f 3, gw 3, gal 3, gA 3, wrench 6
 struct BEnt {
-  float aF[6], aab[6], avb[6], aWr[6];
+  float acc[kSums];
   float tb;
 };
 
@@ -578,40 +524,83 @@ __device__ __forceinline__ void chain_pose(const DevRobot& r, int l, const St& s
 #pragma unroll
       for (int i = 0; i < 12; ++i) P[i] = L[i];
     } else {
-      float T[12];
-      compose(P, L, T);
+      float T[12], t[3];
+      compose(P, L, T, t);
 #pragma unroll
       for (int i = 0; i < 12; ++i) P[i] = T[i];
     }
   }
 }
 
-// parent pose from a link's world pose W and its local transform L: W L^-1
-__device__ __forceinline__ void uncompose(const float* W, const float* L, float* P) {
+// parent pose from a link's world pose W and its local transform L: W L^-1;
+// t: the offset of W's origin from the parent's
+__device__ __forceinline__ void uncompose(const float* W, const float* L, float* P, float* t) {
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j)
       P[3 * i + j] =
           fmaf(W[3 * i + 2], L[3 * j + 2], fmaf(W[3 * i + 1], L[3 * j + 1], W[3 * i] * L[3 * j]));
-  float t[3];
   rot(P, L + 9, t);
   P[9] = W[9] - t[0];
   P[10] = W[10] - t[1];
   P[11] = W[11] - t[2];
 }
 
-__device__ __forceinline__ void point_wrench(const float* R, float4 sp, const float* g, float* w) {
-  float f[3], nn[3];
-  rotT(R, g, f);
-  const float c[3] = {sp.x, sp.y, sp.z};
-  cross3(c, f, nn);
-  w[0] += nn[0];
-  w[1] += nn[1];
-  w[2] += nn[2];
-  w[3] += f[0];
-  w[4] += f[1];
-  w[5] += f[2];
+// a point of a link (link coordinates sp) with gradient g adds the outer
+// product g sp^T to the link's rotation gradient G (row-major) and g to that
+// of its origin, f
+__device__ __forceinline__ void point_grad(float4 sp, const float* g, float* G, float* f) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    G[3 * i] = fmaf(g[i], sp.x, G[3 * i]);
+    G[3 * i + 1] = fmaf(g[i], sp.y, G[3 * i + 1]);
+    G[3 * i + 2] = fmaf(g[i], sp.z, G[3 * i + 2]);
+    f[i] += g[i];
+  }
+}
+
+// A link's own terms in the adjoint, in world axes about its origin: its
+// Newton-Euler wrench (moment n, force f; h = R m c)
+//   f = m A + al x h + w x (w x h),  n = Io al + w x (Io w) + h x A
+// and the gradients of wb . n + ub . f with respect to w, al and A,
+//   gA = m ub + wb x h,  gal = Io wb + h x ub,
+//   gw = (Io w) x wb + Io (wb x w) + grad_w [ub . (w x (w x h))],
+// in o[15] = n, f, gw, gal, gA.  Four products with Io: it is rotated to the
+// world once (45 operations, against 54 to rotate their arguments in and
+// results out).
+__device__ __forceinline__ void link_adjoint(const float* R, const float* I, const float* w,
+                                             const float* al, const float* A, const float* wb,
+                                             const float* ub, float* o) {
+  float T[9], J[10], h[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) rot_inertia(I, R + 3 * i, T + 3 * i);  // rows of R Io
+  J[0] = I[0];
+  J[4] = dot3(T, R);
+  J[5] = dot3(T + 3, R + 3);
+  J[6] = dot3(T + 6, R + 6);
+  J[7] = dot3(T, R + 3);
+  J[8] = dot3(T, R + 6);
+  J[9] = dot3(T + 3, R + 6);
+  rot(R, I + 1, h);
+  float Iw[3], c[3];
+  rot_inertia(J, w, Iw);
+  rot_inertia(J, al, o);
+  cross3_acc(w, Iw, o);
+  cross3_acc(h, A, o);  // n
+#pragma unroll
+  for (int i = 0; i < 3; ++i) o[3 + i] = J[0] * A[i];
+  cross3_acc(al, h, o + 3);
+  centripetal_acc<1>(w, h, o + 3);  // f
+  cross3(wb, w, c);
+  rot_inertia(J, c, o + 6);
+  cross3_acc(Iw, wb, o + 6);
+  centripetal_grad(w, h, ub, o + 6);  // gw
+  rot_inertia(J, wb, o + 9);
+  cross3_acc(h, ub, o + 9);  // gal
+#pragma unroll
+  for (int i = 0; i < 3; ++i) o[12 + i] = J[0] * ub[i];
+  cross3_acc(wb, h, o + 12);  // gA
 }
 
 // A thread's slot in shared memory for the upstream gradient rows that the
@@ -709,15 +698,15 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
     }
   }
 
-  // The state in registers: the pre-order data (W, v, a, Fbar) of the last
-  // pushed link after a push, of the closed link's parent after a close; the
-  // just-pushed link's torque adjoint (ctb, valid while fresh); and the
-  // accumulated children's sums (F, abar, vbar, W) of the entry the
-  // post-order closes next (an unwinding chain passes them on in registers;
-  // they are stored when a push interrupts).
-  float cW[12], cv[6], ca[6], cFb[6], ctb = 0.0f;
+  // The state in registers: the pre-order data (W, w, al, A, wb, ub) of the
+  // last pushed link after a push, of the closed link's parent after a close;
+  // the just-pushed link's torque adjoint (ctb, valid while fresh); and the
+  // accumulated children's sums of the entry the post-order closes next (an
+  // unwinding chain passes them on in registers; they are stored when a push
+  // interrupts).
+  float cW[12], cw[3], cal[3], cA[3], cwb[3], cub[3], ctb = 0.0f;
   bool fresh = false;
-  float pF[6], pab[6], pvb[6], pWr[6];
+  float ps[kSums];
   int pdep = -1;
   // bit e: entry e is an ancestor replayed for this segment (no own terms),
   // its acc holds children's sums
@@ -752,11 +741,16 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
     pend = k;
   };
 
-  // link-frame gradient wrench of link k's kinematic outputs (pose, spheres,
-  // the worst pair's spheres), from its world pose in cW
+  // gradient wrench of link k's kinematic outputs (pose, spheres, the worst
+  // pair's spheres) in world axes about its origin: the points' gradients
+  // join the rotation gradient G, whose wrench is the sum of the crosses of
+  // R's columns with G's
   auto wrench = [&](int k, float* w) {
+    float G[9];
 #pragma unroll
-    for (int i = 0; i < 6; ++i) w[i] = 0.0f;
+    for (int i = 0; i < 9; ++i) G[i] = 0.0f;
+    float* f = w + 3;
+    f[0] = f[1] = f[2] = 0.0f;
     const bool slot = pend == k;
     if (slot) asm volatile("cp.async.wait_group 0;" ::: "memory");
     pend = -1;
@@ -764,18 +758,9 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
       const float4* g4 = reinterpret_cast<const float4*>(A.g_pose + (b * n + k) * 12);
       const float4 x0 = slot ? gs.p[0] : __ldg(g4), x1 = slot ? gs.p[gs.stride] : __ldg(g4 + 1),
                    x2 = slot ? gs.p[2 * gs.stride] : __ldg(g4 + 2);
-      const float gg[12] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w, x2.x, x2.y, x2.z, x2.w};
-      const float* R = cW;
-      float Gm[9];  // R^T Rbar
-#pragma unroll
-      for (int ii = 0; ii < 3; ++ii)
-#pragma unroll
-        for (int jj = 0; jj < 3; ++jj)
-          Gm[3 * ii + jj] = fmaf(R[6 + ii], gg[6 + jj], fmaf(R[3 + ii], gg[3 + jj], R[ii] * gg[jj]));
-      w[0] = Gm[7] - Gm[5];
-      w[1] = Gm[2] - Gm[6];
-      w[2] = Gm[3] - Gm[1];
-      rotT(R, gg + 9, w + 3);
+      G[0] = x0.x; G[1] = x0.y; G[2] = x0.z; G[3] = x0.w; G[4] = x1.x;
+      G[5] = x1.y; G[6] = x1.z; G[7] = x1.w; G[8] = x2.x;
+      f[0] = x2.y; f[1] = x2.z; f[2] = x2.w;
     }
     if (sph4) {  // runs of 4 spheres: three float4 loads a run
       const int e1 = __ldg(r.ls_start + k + 1);
@@ -789,7 +774,7 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
                      x2 = fs ? gs.p[5 * gs.stride] : __ldg(g4 + 2);
         const float gg[12] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w, x2.x, x2.y, x2.z, x2.w};
 #pragma unroll
-        for (int i = 0; i < 4; ++i) point_wrench(cW, __ldg(r.sph + s + i), gg + 3 * i, w);
+        for (int i = 0; i < 4; ++i) point_grad(__ldg(r.sph + s + i), gg + 3 * i, G, f);
       }
     } else if (A.g_sph) {
       const int e1 = __ldg(r.ls_start + k + 1);
@@ -797,13 +782,20 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
         const int s = __ldg(r.ls_sph + e);
         const float* g = A.g_sph + (b * r.S + s) * 3;
         const float gg[3] = {__ldg(g), __ldg(g + 1), __ldg(g + 2)};
-        point_wrench(cW, __ldg(r.sph + s), gg, w);
+        point_grad(__ldg(r.sph + s), gg, G, f);
       }
     }
-    if (k == pl1) point_wrench(cW, __ldg(r.sph + ps1), u, w);
+    if (k == pl1) point_grad(__ldg(r.sph + ps1), u, G, f);
     if (k == pl2) {
       const float mu[3] = {-u[0], -u[1], -u[2]};
-      point_wrench(cW, __ldg(r.sph + ps2), mu, w);
+      point_grad(__ldg(r.sph + ps2), mu, G, f);
+    }
+    const float* R = cW;
+    w[0] = w[1] = w[2] = 0.0f;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const float rc[3] = {R[j], R[3 + j], R[6 + j]}, gc[3] = {G[j], G[3 + j], G[6 + j]};
+      cross3_acc(rc, gc, w);
     }
   };
 
@@ -814,94 +806,106 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
     const int cm = __ldg(r.chain_m + lcs + e);
     const int k = cm & 0xFF;
     const bool own = !((replayed >> e) & 1u);
-    // own terms: f = I a + v x* I v - f_ext, abar = I Fbar,
-    // vbar = -crf(Fbar) I v - I crm(v) Fbar, and the gradient wrench
-    float F[6], ab[6], vb[6], Wr[6];
+    // own terms (link_adjoint, minus the external wrench) and the gradient
+    // wrench of the kinematic outputs
+    float o[kSums];
     if (own) {
       float I[10];
       load_inertia(r, k, I);
-      rnea_force(I, cv, ca, F);
+      link_adjoint(cW, I, cw, cal, cA, cwb, cub, o);
       if (A.fext) {
         const float* fe = A.fext + (b * n + k) * 6;
+        const float xn[3] = {__ldg(fe), __ldg(fe + 1), __ldg(fe + 2)};
+        const float xf[3] = {__ldg(fe + 3), __ldg(fe + 4), __ldg(fe + 5)};
+        float t[3];
+        rot(cW, xn, t);
 #pragma unroll
-        for (int i = 0; i < 6; ++i) F[i] -= __ldg(fe + i);
+        for (int i = 0; i < 3; ++i) o[i] -= t[i];
+        rot(cW, xf, t);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) o[3 + i] -= t[i];
       }
-      float Iv[6], t1[6], t2[6], t3[6];
-      inertia_mul(I, cFb, ab);
-      inertia_mul(I, cv, Iv);
-      crf(cFb, Iv, t1);
-      crm(cv, cFb, t2);
-      inertia_mul(I, t2, t3);
-#pragma unroll
-      for (int i = 0; i < 6; ++i) vb[i] = -t1[i] - t3[i];
       if (kin_grad || k == pl1 || k == pl2) {
-        wrench(k, Wr);
+        wrench(k, o + 15);
         // the next close's rows, while this one computes
         if (use_slot && e - 1 >= tgt && !((replayed >> (e - 1)) & 1u))
           issue(__ldg(r.chain_m + lcs + e - 1) & 0xFF);
       } else {
 #pragma unroll
-        for (int i = 0; i < 6; ++i) Wr[i] = 0.0f;
+        for (int i = 15; i < kSums; ++i) o[i] = 0.0f;
       }
     } else {
 #pragma unroll
-      for (int i = 0; i < 6; ++i) F[i] = ab[i] = vb[i] = Wr[i] = 0.0f;
+      for (int i = 0; i < kSums; ++i) o[i] = 0.0f;
     }
     // plus the children's sums
     if (pdep == e) {
 #pragma unroll
-      for (int i = 0; i < 6; ++i) {
-        F[i] += pF[i];
-        ab[i] += pab[i];
-        vb[i] += pvb[i];
-        Wr[i] += pWr[i];
-      }
+      for (int i = 0; i < kSums; ++i) o[i] += ps[i];
     } else if ((accv >> e) & 1u) {
       const BEnt& E = stk[e];
 #pragma unroll
-      for (int i = 0; i < 6; ++i) {
-        F[i] += E.aF[i];
-        ab[i] += E.aab[i];
-        vb[i] += E.avb[i];
-        Wr[i] += E.aWr[i];
-      }
+      for (int i = 0; i < kSums; ++i) o[i] += E.acc[i];
     }
     pdep = -1;
+    float *sn = o, *sf = o + 3, *gw = o + 6, *gal = o + 9, *gA = o + 12, *Wn = o + 15,
+          *Wf = o + 18;
     const int j = ((cm >> 8) & 0x1FF) - 1;
     const int jt = (cm >> 17) & 3;
     const float4 a4 = ldp(reinterpret_cast<const float4*>(r.axis) + k);
     const float ax[3] = {a4.x, a4.y, a4.z};
     const float mm = ldp(reinterpret_cast<const float2*>(r.mimic) + k).x;
     const float vq = j >= 0 ? mm * st.vel(j) : 0.0f;
-    float L[12];
-    {
-      const float th = j >= 0 ? joint_var(r, k, st.pos(j)) : 0.0f;
-      local_xf_m(r, k, th, jt, ((cm >> 19) & 1) != 0, L, L + 9);
-    }
-    // the parent terms X_k v_pa, X_k a_pa, X_k Fbar_pa from the link's state
-    float Xv[6], Xa[6], XF[6];
-    if (e > 0) {
-      const float aq = j >= 0 ? mm * st.acc(j) : 0.0f;
-      const float tb = fresh ? ctb : stk[e].tb;
-      if (jt == 1)
-        close_parent_terms<1>(ax, vq, aq, tb, cv, ca, cFb, Xv, Xa, XF);
-      else if (jt == 2)
-        close_parent_terms<2>(ax, vq, aq, tb, cv, ca, cFb, Xv, Xa, XF);
-      else
-        close_parent_terms<0>(ax, vq, aq, tb, cv, ca, cFb, Xv, Xa, XF);
-    } else {  // the root: v_pa = 0, a_pa = the base acceleration, Fbar_pa = 0
-      const float ap[6] = {0.0f, 0.0f, 0.0f, r.abase[0], r.abase[1], r.abase[2]};
-      xf_motion(L, L + 9, ap, Xa);
+    const float aq = j >= 0 ? mm * st.acc(j) : 0.0f;
+    const float tb = fresh ? ctb : (e > 0 ? stk[e].tb : 0.0f);
+    float s[3];
+    rot(cW, ax, s);
+    // The joint's gradients.  Turning a revolute joint turns everything the
+    // subtree holds; what enters it from the parent stays, so with the sums
+    // as the gradients of the link's own w, al, A, wb, ub
+    //   gq   = s . [Wn - w x gw - al x gal - A x gA - wb x n - ub x f],
+    //   gqd  = s . gw + (w x s) . gal,  gqdd = s . gal,
+    // and w_pa also moves al through w_pa x s qd: gw += qd s x gal.  Sliding
+    // a prismatic joint moves the subtree's origin along s (through r).
+    float gq = 0.0f, gqd = 0.0f, gqdd = 0.0f;
+    if (jt == 1) {
+      float t[3] = {Wn[0], Wn[1], Wn[2]}, c[3];
+      cross3_sub(cw, gw, t);
+      cross3_sub(cal, gal, t);
+      cross3_sub(cA, gA, t);
+      cross3_sub(cwb, sn, t);
+      cross3_sub(cub, sf, t);
+      gq = dot3(s, t);
+      cross3(cw, s, c);
+      gqd = dot3(s, gw) + dot3(c, gal);
+      gqdd = dot3(s, gal);
+      const float sq[3] = {s[0] * vq, s[1] * vq, s[2] * vq};
+      cross3_acc(sq, gal, gw);
+      // the parent's w, al, wb
 #pragma unroll
-      for (int i = 0; i < 6; ++i) Xv[i] = XF[i] = 0.0f;
+      for (int i = 0; i < 3; ++i) {
+        cw[i] -= sq[i];
+        cal[i] = fmaf(-s[i], aq, fmaf(-vq, c[i], cal[i]));
+        cwb[i] = fmaf(-s[i], tb, cwb[i]);
+      }
+    } else if (jt == 2) {
+      float t[3] = {Wf[0], Wf[1], Wf[2]}, c[3], c2[3];
+      // gA . (al x s + w x (w x s)) + f . (wb x s) + s . Wf
+      cross3_acc(gA, cal, t);
+      cross3_acc(sf, cwb, t);
+      cross3(cw, s, c);
+      cross3(cw, c, c2);
+      gq = dot3(s, t) + dot3(gA, c2);
+      gqd = 2.0f * dot3(c, gA);
+      gqdd = dot3(s, gA);
+      const float sq[3] = {2.0f * vq * s[0], 2.0f * vq * s[1], 2.0f * vq * s[2]};
+      cross3_acc(sq, gA, gw);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        cA[i] = fmaf(-s[i], aq, fmaf(-2.0f * vq, c[i], cA[i]));
+        cub[i] = fmaf(-s[i], tb, cub[i]);
+      }
     }
-    float gq, gqd, gqdd;
-    if (jt == 1)
-      close_joint_grads<1>(ax, vq, F, ab, vb, Wr, cv, Xv, Xa, XF, gq, gqd, gqdd);
-    else if (jt == 2)
-      close_joint_grads<2>(ax, vq, F, ab, vb, Wr, cv, Xv, Xa, XF, gq, gqd, gqdd);
-    else
-      close_joint_grads<0>(ax, vq, F, ab, vb, Wr, cv, Xv, Xa, XF, gq, gqd, gqdd);
     if (FC && j >= 0) {
       float dqd = 0.0f, dqdd = 0.0f;  // the cost's direct gradients, once per joint
       if (own) {
@@ -945,43 +949,34 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
     }
     fresh = false;
     if (e > 0) {
+      float rv[3];  // the offset from the parent's origin
+      float L[12], Wp[12];
+      const float th = j >= 0 ? joint_var(r, k, st.pos(j)) : 0.0f;
+      local_xf_m<true>(r, k, th, jt, ((cm >> 19) & 1) != 0, L, L + 9);
+      uncompose(cW, L, Wp, rv);
+#pragma unroll
+      for (int i = 0; i < 12; ++i) cW[i] = Wp[i];
+      cross3_sub(cal, rv, cA);
+      centripetal_acc<-1>(cw, rv, cA);
+      cross3_sub(cwb, rv, cub);
+      // the sums about the parent's origin
+      centripetal_grad(cw, rv, gA, gw);
+      cross3_acc(rv, gA, gal);
+      cross3_acc(rv, sf, sn);
+      cross3_acc(rv, Wf, Wn);
       const BEnt& P = stk[e - 1];
       const bool has = (accv >> (e - 1)) & 1u;
       accv &= ~(1u << (e - 1));  // taken over by the pending registers
-      float up[6];
-      xf_force_T(L, L + 9, F, up);
 #pragma unroll
-      for (int i = 0; i < 6; ++i) pF[i] = has ? P.aF[i] + up[i] : up[i];
-      xf_force_T(L, L + 9, ab, up);
-#pragma unroll
-      for (int i = 0; i < 6; ++i) pab[i] = has ? P.aab[i] + up[i] : up[i];
-      xf_force_T(L, L + 9, vb, up);
-#pragma unroll
-      for (int i = 0; i < 6; ++i) pvb[i] = has ? P.avb[i] + up[i] : up[i];
-      xf_force_T(L, L + 9, Wr, up);
-#pragma unroll
-      for (int i = 0; i < 6; ++i) pWr[i] = has ? P.aWr[i] + up[i] : up[i];
+      for (int i = 0; i < kSums; ++i) ps[i] = has ? P.acc[i] + o[i] : o[i];
       pdep = e - 1;
-      // the parent's state: this link's maps undone
-      float Wp[12];
-      uncompose(cW, L, Wp);
-#pragma unroll
-      for (int i = 0; i < 12; ++i) cW[i] = Wp[i];
-      xf_motion_inv(L, L + 9, Xv, cv);
-      xf_motion_inv(L, L + 9, Xa, ca);
-      xf_motion_inv(L, L + 9, XF, cFb);
     }
   };
   auto flush = [&]() {  // the pending children's sums go to their entry
     if (pdep >= 0) {
       BEnt& P = stk[pdep];
 #pragma unroll
-      for (int i = 0; i < 6; ++i) {
-        P.aF[i] = pF[i];
-        P.aab[i] = pab[i];
-        P.avb[i] = pvb[i];
-        P.aWr[i] = pWr[i];
-      }
+      for (int i = 0; i < kSums; ++i) P.acc[i] = ps[i];
       accv |= 1u << pdep;
       pdep = -1;
     }
@@ -995,7 +990,7 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
     float L[12];
     {
       const float th = j >= 0 ? joint_var(r, k, st.pos(j)) : 0.0f;
-      local_xf_m(r, k, th, jt, ((ky >> 26) & 1) != 0, L, L + 9);
+      local_xf_m<true>(r, k, th, jt, ((ky >> 26) & 1) != 0, L, L + 9);
     }
     const float4 a4 = ldp(reinterpret_cast<const float4*>(r.axis) + k);
     const float ax[3] = {a4.x, a4.y, a4.z};
@@ -1022,30 +1017,36 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
     } else if (!FC && j >= 0 && A.g_tau) {
       tb = mm * __ldg(A.g_tau + (int64_t)j * B + b);
     }
-    float S[6];
-    motion_S6t(jt, ax, S);
-    // pose, v, a (dynamics forward) and Fbar_k = S m taubar + X Fbar_pa
-    float Wn[12], vn[6], an[6], XF[6];
+    // the link's state: pose, motion, and the torques' virtual motion
+    // wb = wb_pa + s tb, ub = ub_pa + wb_pa x r (prismatic: ub + s tb)
+    float Wn[12], s[3], rv[3], wn[3], aln[3], An[3];
     if (dep > 0) {
-      compose(cW, L, Wn);
-      rnea_va(L, L + 9, cv, ca, jt, ax, vq, aq, vn, an);
-      xf_motion(L, L + 9, cFb, XF);
+      compose(cW, L, Wn, rv);
+      rot(Wn, ax, s);
+      joint_motion(jt, s, rv, vq, aq, cw, cal, cA, wn, aln, An);
+      cross3_acc(cwb, rv, cub);
     } else {
 #pragma unroll
       for (int i = 0; i < 12; ++i) Wn[i] = L[i];
-      const float vp[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-      const float ap[6] = {0.0f, 0.0f, 0.0f, r.abase[0], r.abase[1], r.abase[2]};
-      rnea_va(L, L + 9, vp, ap, jt, ax, vq, aq, vn, an);
+      rot(Wn, ax, s);
 #pragma unroll
-      for (int i = 0; i < 6; ++i) XF[i] = 0.0f;
+      for (int i = 0; i < 3; ++i) {
+        cw[i] = cal[i] = cwb[i] = cub[i] = rv[i] = 0.0f;
+        cA[i] = r.abase[i];
+      }
+      joint_motion(jt, s, rv, vq, aq, cw, cal, cA, wn, aln, An);
     }
 #pragma unroll
     for (int i = 0; i < 12; ++i) cW[i] = Wn[i];
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      cv[i] = vn[i];
-      ca[i] = an[i];
-      cFb[i] = fmaf(S[i], tb, XF[i]);
+    for (int i = 0; i < 3; ++i) {
+      cw[i] = wn[i];
+      cal[i] = aln[i];
+      cA[i] = An[i];
+      if (jt == 2)
+        cub[i] = fmaf(s[i], tb, cub[i]);
+      else
+        cwb[i] = fmaf(s[i], tb, cwb[i]);
     }
     ctb = tb;
     fresh = true;
@@ -1054,10 +1055,13 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
     accv &= ~bit;
     replayed = own ? (replayed & ~bit) : (replayed | bit);
     if (nch > 0) stk[dep].tb = tb;
-    if (own && A.g_fext) {  // dL/df_ext,k = -Fbar_k
+    if (own && A.g_fext) {  // dL/df_ext,k = -(wb, ub) in link coordinates
       float* o = A.g_fext + (b * n + k) * 6;
+      float t[6];
+      rotT(cW, cwb, t);
+      rotT(cW, cub, t + 3);
 #pragma unroll
-      for (int i = 0; i < 6; ++i) o[i] = -cFb[i];
+      for (int i = 0; i < 6; ++i) o[i] = -t[i];
     }
   };
 
