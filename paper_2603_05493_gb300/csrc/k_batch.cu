@@ -42,41 +42,64 @@ __device__ __forceinline__ void pair_bar(int id) {
 }
 
 // shared memory: one item slot per pair (32 words, up to 32 pairs), then per
-// pair the partials [nout][ns_max][2][32]
-__host__ __device__ inline size_t batch_tree_words(int nout, int ns_max, int pairs) {
-  return 32 + (size_t)pairs * nout * ns_max * 64;
+// pair its robot's link records and walk words (n_max links), staged when the
+// pair's robot changes, and the partials [nout][ns_max][2][32]
+__host__ __device__ inline size_t batch_pair_words(int nout, int ns_max, int n_max) {
+  return (size_t)kRecWords * n_max + ((n_max + 31) & ~31) + (size_t)nout * ns_max * 64;
+}
+__host__ __device__ inline size_t batch_tree_words(int nout, int ns_max, int n_max, int pairs) {
+  return 32 + (size_t)pairs * batch_pair_words(nout, ns_max, n_max);
 }
 
-// the configuration a lane sweeps in item w, and whether it sweeps one:
+// The configuration a lane sweeps in item w, and whether it sweeps one (act):
 // mode 0 -- lane of the 32; the second warp only with a segment plan;
-// mode 1 -- configuration 32 g + lane of the 64
-__device__ __forceinline__ bool batch_lane(const int4& w, bool seg, int g, int lane, int64_t* b) {
-  if (w.w == 1) {
-    *b = (int64_t)w.y + 32 * g + lane;
-    return 32 * g + lane < w.z;
-  }
-  *b = (int64_t)w.y + lane;
-  return (seg || g == 0) && lane < w.z;
+// mode 1 -- configuration 32 g + lane of the 64.  A lane past the item's end
+// sweeps its last configuration again; false: the warp has none.
+__device__ __forceinline__ bool batch_lane(const int4& w, bool seg, int g, int lane, int64_t* b,
+                                           bool* act) {
+  const int first = w.w == 1 ? 32 * g : 0;
+  *act = first + lane < w.z;
+  *b = (int64_t)w.y + min(first + lane, w.z - 1);
+  return w.w == 1 ? first < w.z : (seg || g == 0);
+}
+
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+
+// the pair's robot changed: its records (with plan 0's slots, read only by a
+// segmented sweep) and walk words
+__device__ __forceinline__ void stage_robot(const DevRobot& r, float4* rec, uint32_t* wk, int i0) {
+  stage_recs(r, 0, rec, i0, 64);
+  for (int i = i0; i < r.n; i += 64) wk[i] = __ldg(r.walk + i);
 }
 
 __global__ void __launch_bounds__(256) batch_tree_fwd_kernel(const DevRobot* robots,
                                                              const BatchProblemDev* probs,
                                                              const int4* items, int n_items,
                                                              int* counter, BatchIO io,
-                                                             int ns_max) {
-  extern __shared__ float sm[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+                                                             int ns_max, int n_max) {
+  extern __shared__ __align__(16) float sm[];
+  const int lane = threadIdx.x & 31, warp = uniform(threadIdx.x >> 5);
   const int pi = warp >> 1, g = warp & 1, bar = 1 + pi;
   int* slot = reinterpret_cast<int*>(sm) + pi;
-  float* part = sm + 32 + (size_t)pi * ns_max * 64;
+  float* base = sm + 32 + (size_t)pi * batch_pair_words(1, ns_max, n_max);
+  float4* rec = reinterpret_cast<float4*>(base);
+  uint32_t* wk = reinterpret_cast<uint32_t*>(base + (size_t)kRecWords * n_max);
+  float* part = base + (size_t)kRecWords * n_max + ((n_max + 31) & ~31);
+  int cur = -1;
   for (;;) {
     if (g == 0 && lane == 0) *slot = atomicAdd(counter, 1);
     pair_bar(bar);
-    const int it = *slot;
+    const int it = uniform(*slot);
     if (it >= n_items) return;
     const int4 w = items[it];
     const BatchProblemDev pb = probs[w.x];
     const DevRobot& r = robots[pb.robot];
+    const int robot = uniform(pb.robot);
+    if (robot != cur) {
+      stage_robot(r, rec, wk, 32 * g + lane);
+      cur = robot;
+      pair_bar(bar);
+    }
     FwdArgs A{pb.H,
               io.q + pb.jo,
               io.qd ? io.qd + pb.jo : nullptr,
@@ -87,15 +110,20 @@ __global__ void __launch_bounds__(256) batch_tree_fwd_kernel(const DevRobot* rob
               nullptr,
               io.tau ? io.tau + pb.jo : nullptr,
               nullptr};
-    const bool seg = w.w == 0 && (r.seg_ok & 1);
+    const bool seg = uniform(w.w == 0 && (r.seg_ok & 1)) != 0;
     int64_t b;
-    const bool act = batch_lane(w, seg, g, lane, &b);
+    bool act;
+    const bool some = uniform(batch_lane(w, seg, g, lane, &b, &act)) != 0;
     const int ns = seg ? r.seg_ns[0] : 0;
     // one call site for both cases (a second inlined sweep would cost registers)
-    const Seg sg = seg ? Seg{r.seg_pos[0][g], r.seg_pos[0][g + 1], g, 2, r.seg_slot, part, ns, lane}
-                       : whole_sweep(r);
+    Seg sg = seg ? Seg{r.seg_pos[0][g], r.seg_pos[0][g + 1], g, 2, part, ns, lane}
+                 : whole_sweep(r);
+    sg.p0 = uniform(sg.p0);
+    sg.p1 = uniform(sg.p1);
     for (int q = 0; q < ns; ++q) part[(q * 2 + g) * 32 + lane] = 0.0f;
-    if (act) tree_fwd_seg(r, A, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, sg);
+    if (some)
+      tree_fwd_seg<kFwdLocal>(r, rec, SharedWalk{wk}, A, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b,
+                          act, sg);
     pair_bar(bar);
     if (lane < w.z && A.tau)
       for (int q = g; q < ns; q += 2) {
@@ -111,22 +139,32 @@ __global__ void __launch_bounds__(256, 2) batch_tree_bwd_kernel(const DevRobot* 
                                                              const BatchProblemDev* probs,
                                                              const int4* items, int n_items,
                                                              int* counter, BatchIO io,
-                                                             int ns_max) {
-  extern __shared__ float sm[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+                                                             int ns_max, int n_max) {
+  extern __shared__ __align__(16) float sm[];
+  const int lane = threadIdx.x & 31, warp = uniform(threadIdx.x >> 5);
   const int pi = warp >> 1, g = warp & 1, bar = 1 + pi;
   int* slot = reinterpret_cast<int*>(sm) + pi;
-  float* part = sm + 32 + (size_t)pi * 3 * ns_max * 64;
+  float* base = sm + 32 + (size_t)pi * batch_pair_words(3, ns_max, n_max);
+  float4* rec = reinterpret_cast<float4*>(base);
+  uint32_t* wk = reinterpret_cast<uint32_t*>(base + (size_t)kRecWords * n_max);
+  float* part = base + (size_t)kRecWords * n_max + ((n_max + 31) & ~31);
   // the gradient-row slots behind every pair's partials
-  const GradSlot gs = grad_slot_of(sm + batch_tree_words(3, ns_max, blockDim.x / 64));
+  const GradSlot gs = grad_slot_of(sm + batch_tree_words(3, ns_max, n_max, blockDim.x / 64));
+  int cur = -1;
   for (;;) {
     if (g == 0 && lane == 0) *slot = atomicAdd(counter, 1);
     pair_bar(bar);
-    const int it = *slot;
+    const int it = uniform(*slot);
     if (it >= n_items) return;
     const int4 w = items[it];
     const BatchProblemDev pb = probs[w.x];
     const DevRobot& r = robots[pb.robot];
+    const int robot = uniform(pb.robot);
+    if (robot != cur) {
+      stage_robot(r, rec, wk, 32 * g + lane);
+      cur = robot;
+      pair_bar(bar);
+    }
     BwdArgs A{pb.H,
               io.q + pb.jo,
               io.qd + pb.jo,
@@ -139,16 +177,21 @@ __global__ void __launch_bounds__(256, 2) batch_tree_bwd_kernel(const DevRobot* 
               io.gq + pb.jo,
               io.gqd + pb.jo,
               io.gqdd + pb.jo};
-    const bool seg = w.w == 0 && (r.seg_ok & 1);
+    const bool seg = uniform(w.w == 0 && (r.seg_ok & 1)) != 0;
     int64_t b;
-    const bool act = batch_lane(w, seg, g, lane, &b);
+    bool act;
+    const bool some = uniform(batch_lane(w, seg, g, lane, &b, &act)) != 0;
     const int ns = seg ? r.seg_ns[0] : 0;
     const size_t o = (size_t)ns * 64;  // one output's partials
-    const Seg sg = seg ? Seg{r.seg_pos[0][g], r.seg_pos[0][g + 1], g, 2, r.seg_slot, part, ns, lane}
-                       : whole_sweep(r);
+    Seg sg = seg ? Seg{r.seg_pos[0][g], r.seg_pos[0][g + 1], g, 2, part, ns, lane}
+                 : whole_sweep(r);
+    sg.p0 = uniform(sg.p0);
+    sg.p1 = uniform(sg.p1);
     for (int q = 0; q < ns; ++q)
       for (int k = 0; k < 3; ++k) part[k * o + (q * 2 + g) * 32 + lane] = 0.0f;
-    if (act) tree_bwd_seg<false>(r, A, FusedCost{}, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, sg, gs);
+    if (some)
+      tree_bwd_seg<false>(r, rec, SharedWalk{wk}, A, FusedCost{},
+                          ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg, gs);
     pair_bar(bar);
     if (lane < w.z)
       for (int q = g; q < ns; q += 2) {
@@ -205,15 +248,15 @@ __global__ void __launch_bounds__(256, 3) batch_pair_kernel(const DevRobot* robo
 // launchers
 // ---------------------------------------------------------------------------
 // the backward adds each thread's gradient-row slot (GradSlot)
-size_t batch_tree_smem(bool fwd, int ns_max, int threads) {
-  return sizeof(float) * batch_tree_words(fwd ? 1 : 3, ns_max, threads / 64) +
+size_t batch_tree_smem(bool fwd, int ns_max, int n_max, int threads) {
+  return sizeof(float) * batch_tree_words(fwd ? 1 : 3, ns_max, n_max, threads / 64) +
          (fwd ? 0 : 16 + (size_t)kGradSlotBytes * threads);
 }
 
 cudaError_t launch_batch_tree_fwd(const DevRobot* robots, const BatchProblemDev* probs, const int4* items,
                                   int n_items, int* counter, const BatchIO& io, int grid,
-                                  int ns_max, int threads, cudaStream_t s) {
-  const size_t smem = batch_tree_smem(true, ns_max, threads);
+                                  int ns_max, int n_max, int threads, cudaStream_t s) {
+  const size_t smem = batch_tree_smem(true, ns_max, n_max, threads);
   cudaError_t e = cudaFuncSetAttribute(batch_tree_fwd_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -221,14 +264,14 @@ cudaError_t launch_batch_tree_fwd(const DevRobot* robots, const BatchProblemDev*
   e = cudaMemsetAsync(counter, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   batch_tree_fwd_kernel<<<grid, threads, smem, s>>>(robots, probs, items, n_items, counter, io,
-                                                    ns_max);
+                                                    ns_max, n_max);
   return cudaGetLastError();
 }
 
 cudaError_t launch_batch_tree_bwd(const DevRobot* robots, const BatchProblemDev* probs, const int4* items,
                                   int n_items, int* counter, const BatchIO& io, int grid,
-                                  int ns_max, int threads, cudaStream_t s) {
-  const size_t smem = batch_tree_smem(false, ns_max, threads);
+                                  int ns_max, int n_max, int threads, cudaStream_t s) {
+  const size_t smem = batch_tree_smem(false, ns_max, n_max, threads);
   cudaError_t e = cudaFuncSetAttribute(batch_tree_bwd_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -236,7 +279,7 @@ cudaError_t launch_batch_tree_bwd(const DevRobot* robots, const BatchProblemDev*
   e = cudaMemsetAsync(counter, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   batch_tree_bwd_kernel<<<grid, threads, smem, s>>>(robots, probs, items, n_items, counter, io,
-                                                    ns_max);
+                                                    ns_max, n_max);
   return cudaGetLastError();
 }
 
@@ -269,8 +312,12 @@ cudaError_t batch_pair_max_blocks_per_sm(int warps, int ws_words, int rad_words,
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, batch_pair_kernel, warps * 32, smem);
 }
 
-cudaError_t batch_tree_max_blocks_per_sm(bool fwd, int ns_max, int threads, int* out) {
-  const size_t smem = batch_tree_smem(fwd, ns_max, threads);
+cudaError_t batch_tree_max_blocks_per_sm(bool fwd, int ns_max, int n_max, int threads, int* out) {
+  const size_t smem = batch_tree_smem(fwd, ns_max, n_max, threads);
+  if (smem > 227 * 1024) {  // the records of a block's pairs do not fit
+    *out = 0;
+    return cudaSuccess;
+  }
   cudaError_t e = cudaFuncSetAttribute(fwd ? batch_tree_fwd_kernel : batch_tree_bwd_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

@@ -8,26 +8,15 @@
 
 namespace wbe {
 
-// The sweeps read a link's fixed transform, axis, mimic factors and inertia
-// at its push (and the backward again at its close).  Every sweep kernel
-// stages these once per block in shared memory (kParamWords floats a link,
-// behind the partials or basis rows it also keeps there), where they no
-// longer compete with the depth-first stacks for L1.
-constexpr int kParamWords = 28;  // Tf 12, axis 4, inertia 10, mimic 2
+// Every sweep kernel stages the robot's link records (kRecWords floats a
+// link: fixed transform, axis, mimic factors, inertia, output indices) once
+// per block at the start of its shared memory: one base and constant offsets
+// for everything a push or close reads of a link, in eight 16-byte loads, and
+// out of the way of the depth-first stacks in L1.
 constexpr size_t kSegSmemMax = 227 * 1024;  // dynamic shared memory of one block
-__device__ __forceinline__ DevRobot stage_params(const DevRobot& r, float* dst) {
-  const int n = r.n;
-  for (int i = threadIdx.x; i < 12 * n; i += blockDim.x) dst[i] = __ldg(r.Tf + i);
-  for (int i = threadIdx.x; i < 4 * n; i += blockDim.x) dst[12 * n + i] = __ldg(r.axis + i);
-  for (int i = threadIdx.x; i < 10 * n; i += blockDim.x) dst[16 * n + i] = __ldg(r.inert + i);
-  for (int i = threadIdx.x; i < 2 * n; i += blockDim.x) dst[26 * n + i] = __ldg(r.mimic + i);
-  DevRobot s = r;
-  s.Tf = dst;
-  s.axis = dst + 12 * n;
-  s.inert = dst + 16 * n;
-  s.mimic = dst + 26 * n;
-  return s;
-}
+
+// this thread's warp, known to be the same for its whole warp
+__device__ __forceinline__ int warp_of() { return __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0); }
 
 // the block's dynamic shared memory covers `words` floats
 __device__ __forceinline__ bool smem_holds(size_t words) {
@@ -36,23 +25,36 @@ __device__ __forceinline__ bool smem_holds(size_t words) {
   return sizeof(float) * words <= dyn;
 }
 
-// FS: the force stack in shared memory behind the link parameters, as in the
-// segmented forward below
-template <bool FS>
+// the configuration b of this lane in the warp whose first is b0 (act); a lane
+// past the end takes the last one and act = false; false: the warp has none
+__device__ __forceinline__ bool own_config(int64_t B, int64_t b0, int64_t* b, bool* act) {
+  if (b0 >= B) return false;
+  const int64_t own = b0 + (threadIdx.x & 31);
+  *act = own < B;
+  *b = *act ? own : B - 1;
+  return true;
+}
+
+// MODE kFwdShared: the force stack in shared memory behind the link records,
+// as in the segmented forward below
+template <int MODE>
 __global__ void __launch_bounds__(256) tree_fwd_kernel(const __grid_constant__ DevRobot r,
-                                                       FwdArgs A) {
-  extern __shared__ float prm[];
-  if (FS && !smem_holds(kParamWords * (size_t)r.n + 6 * (size_t)r.maxdepth * blockDim.x)) return;
-  const DevRobot rs = stage_params(r, prm);
+                                                       const __grid_constant__ WalkTab wt,
+                                                       const __grid_constant__ FwdArgs A) {
+  extern __shared__ float4 rec[];
+  float* sm = reinterpret_cast<float*>(rec) + kRecWords * (size_t)r.n;
+  if (MODE == kFwdShared && !smem_holds(kRecWords * (size_t)r.n + 6 * (size_t)r.maxdepth * blockDim.x)) return;
+  stage_recs(r, -1, rec, threadIdx.x, blockDim.x);
   __syncthreads();
-  const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (b >= A.B) return;
+  int64_t b;
+  bool act;
+  if (!own_config(A.B, blockIdx.x * (int64_t)blockDim.x + 32 * warp_of(), &b, &act)) return;
   Seg sg = whole_sweep(r);
-  if (FS) {
-    sg.fst = prm + kParamWords * (size_t)r.n + threadIdx.x;
+  if (MODE == kFwdShared) {
+    sg.fst = reinterpret_cast<float2*>(sm) + threadIdx.x;
     sg.fstr = blockDim.x;
   }
-  tree_fwd_seg<ArrayStates, FS>(rs, A, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, sg);
+  tree_fwd_seg<MODE>(r, rec, ConstWalk{wt}, A, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg);
 }
 
 // The backward sweeps are capped at 128 registers (two 256-thread blocks per
@@ -63,12 +65,16 @@ __global__ void __launch_bounds__(256) tree_fwd_kernel(const __grid_constant__ D
 // 512 threads, so that one block per SM holds the staged link parameters once
 // and the shared-memory carveout stays small.
 __global__ void __launch_bounds__(256, 2) tree_bwd_kernel(const __grid_constant__ DevRobot r,
-                                                          BwdArgs A) {
-  extern __shared__ float prm[];
-  const DevRobot rs = stage_params(r, prm);
+                                                          const __grid_constant__ WalkTab wt,
+                                                          const __grid_constant__ BwdArgs A) {
+  extern __shared__ float4 rec[];
+  stage_recs(r, -1, rec, threadIdx.x, blockDim.x);
   __syncthreads();
-  const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (b < A.B) tree_bwd_one(rs, A, b);
+  int64_t b;
+  bool act;
+  if (!own_config(A.B, blockIdx.x * (int64_t)blockDim.x + 32 * warp_of(), &b, &act)) return;
+  tree_bwd_seg<false>(r, rec, ConstWalk{wt}, A, FusedCost{},
+                      ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, whole_sweep(r));
 }
 
 // Segmented sweeps, plan t (G = 2 << t segments).  A block holds CG groups of
@@ -76,44 +82,46 @@ __global__ void __launch_bounds__(256, 2) tree_bwd_kernel(const __grid_constant_
 // w / G.  Shared memory per group: the partial outputs [nout][ns][G][32] of
 // the ns links that several segments hold, summed in segment order after the
 // barrier by the group's warps (slot s by warp s % G).
-__device__ __forceinline__ Seg seg_of(const DevRobot& r, int t, float* part) {
-  const int G = 2 << t;
-  const int w = threadIdx.x >> 5;
-  const int g = w % G;
-  return Seg{r.seg_pos[t][g], r.seg_pos[t][g + 1], g, G, r.seg_slot + t * r.n,
-             part, r.seg_ns[t], (int)(threadIdx.x & 31)};
+__device__ __forceinline__ Seg seg_of(const DevRobot& r, int t, int g, float* part) {
+  return Seg{r.seg_pos[t][g], r.seg_pos[t][g + 1], g, 2 << t, part, r.seg_ns[t],
+             (int)(threadIdx.x & 31)};
 }
 
-// FS: the force stack in shared memory, [maxdepth][6][threads] floats behind
-// the link parameters (a link's F is stored when its first child is pushed
+// MODE kFwdShared: the force stack in shared memory, [maxdepth][3][threads] float2 behind
+// the partials (a link's F is stored when its first child is pushed
 // and read back at that child's close; in local memory these round trips
 // missed L1 61 % of the time)
-template <bool FS>
+template <int MODE>
 __global__ void __launch_bounds__(512) tree_fwd_seg_kernel(const __grid_constant__ DevRobot r,
-                                                           FwdArgs A, int t) {
-  extern __shared__ float part[];
+                                                           const __grid_constant__ WalkTab wt,
+                                                           const __grid_constant__ FwdArgs A,
+                                                           int t) {
+  extern __shared__ float4 rec[];
+  float* part = reinterpret_cast<float*>(rec) + kRecWords * (size_t)r.n;
   const int G = 2 << t;
   const int CG = blockDim.x / (32 * G);
-  const int cg = (threadIdx.x >> 5) / G;
+  const int wid = warp_of(), cg = wid / G;
   const int ns = r.seg_ns[t];
   // the launch reserves the stack for this block's threads; a block that
   // finds less shared memory than that does nothing (its outputs stay
   // unwritten) instead of indexing past it
-  if (FS && !smem_holds((size_t)CG * ns * G * 32 + kParamWords * (size_t)r.n +
+  if (MODE == kFwdShared && !smem_holds((size_t)CG * ns * G * 32 + kRecWords * (size_t)r.n +
                         6 * (size_t)r.maxdepth * blockDim.x))
     return;
-  Seg sg = seg_of(r, t, part + (size_t)cg * ns * G * 32);
+  Seg sg = seg_of(r, t, wid % G, part + (size_t)cg * ns * G * 32);
   for (int s = 0; s < ns; ++s) sg.part[(s * G + sg.g) * 32 + sg.lane] = 0.0f;
-  const DevRobot rs = stage_params(r, part + (size_t)CG * ns * G * 32);
-  if (FS) {
-    sg.fst = part + (size_t)CG * ns * G * 32 + kParamWords * (size_t)r.n + threadIdx.x;
+  stage_recs(r, t, rec, threadIdx.x, blockDim.x);
+  if (MODE == kFwdShared) {
+    sg.fst = reinterpret_cast<float2*>(part + (size_t)CG * ns * G * 32) + threadIdx.x;
     sg.fstr = blockDim.x;
   }
   __syncthreads();
-  const int64_t b = ((int64_t)blockIdx.x * CG + cg) * 32 + sg.lane;
-  if (b < A.B) tree_fwd_seg<ArrayStates, FS>(rs, A, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, sg);
+  int64_t b;
+  bool act = false;
+  if (own_config(A.B, ((int64_t)blockIdx.x * CG + cg) * 32, &b, &act))
+    tree_fwd_seg<MODE>(r, rec, ConstWalk{wt}, A, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg);
   __syncthreads();
-  if (b < A.B && A.tau) {
+  if (act && A.tau) {
     for (int s = sg.g; s < ns; s += G) {
       float acc = 0.0f;
       for (int h = 0; h < G; ++h) acc += sg.part[(s * G + h) * 32 + sg.lane];
@@ -124,25 +132,31 @@ __global__ void __launch_bounds__(512) tree_fwd_seg_kernel(const __grid_constant
 }
 
 __global__ void __launch_bounds__(512, 1) tree_bwd_seg_kernel(const __grid_constant__ DevRobot r,
-                                                           BwdArgs A, int t) {
-  extern __shared__ float part[];
+                                                           const __grid_constant__ WalkTab wt,
+                                                           const __grid_constant__ BwdArgs A,
+                                                           int t) {
+  extern __shared__ float4 rec[];
+  float* part = reinterpret_cast<float*>(rec) + kRecWords * (size_t)r.n;
   const int G = 2 << t;
   const int CG = blockDim.x / (32 * G);
-  const int cg = (threadIdx.x >> 5) / G;
+  const int wid = warp_of(), cg = wid / G;
   const int ns = r.seg_ns[t];
   const size_t o = (size_t)ns * G * 32;  // one output's partials
-  Seg sg = seg_of(r, t, part + (size_t)cg * 3 * o);
+  Seg sg = seg_of(r, t, wid % G, part + (size_t)cg * 3 * o);
   for (int s = 0; s < ns; ++s)
     for (int q = 0; q < 3; ++q) sg.part[q * o + (s * G + sg.g) * 32 + sg.lane] = 0.0f;
-  const DevRobot rs = stage_params(r, part + (size_t)CG * 3 * o);
-  // the gradient-row slots behind the link parameters (reserved by the
-  // launch when there are upstream pose or sphere gradients)
-  const GradSlot gs = grad_slot_of(part + (size_t)CG * 3 * o + kParamWords * (size_t)r.n);
+  stage_recs(r, t, rec, threadIdx.x, blockDim.x);
+  // the gradient-row slots behind the partials (reserved by the launch when
+  // there are upstream pose or sphere gradients)
+  const GradSlot gs = grad_slot_of(part + (size_t)CG * 3 * o);
   __syncthreads();
-  const int64_t b = ((int64_t)blockIdx.x * CG + cg) * 32 + sg.lane;
-  if (b < A.B) tree_bwd_seg<false>(rs, A, FusedCost{}, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, sg, gs);
+  int64_t b;
+  bool act = false;
+  if (own_config(A.B, ((int64_t)blockIdx.x * CG + cg) * 32, &b, &act))
+    tree_bwd_seg<false>(r, rec, ConstWalk{wt}, A, FusedCost{},
+                        ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg, gs);
   __syncthreads();
-  if (b < A.B) {
+  if (act) {
     for (int s = sg.g; s < ns; s += G) {
       float acc[3] = {0.0f, 0.0f, 0.0f};
       for (int h = 0; h < G; ++h)
@@ -156,45 +170,61 @@ __global__ void __launch_bounds__(512, 1) tree_bwd_seg_kernel(const __grid_const
   }
 }
 
+// a configuration's cost: its joints' terms, then the collision term
+__device__ __forceinline__ float total_cost(const FusedCost& fc, int64_t b, float c) {
+  return fc.d_min ? fmaf(fc.w, fmaxf(0.0f, -__ldg(fc.d_min + b)), c) : c;
+}
+
 // The same sweeps with the trajectory cost in their prologue (FusedCost):
 // separate kernels, so that the plain ones keep their register allocation.
 // The segmented one adds each configuration's cost terms over the segments
 // in segment order (deterministic) after the barrier.
 __global__ void __launch_bounds__(256, 2) tree_bwd_cost_kernel(
-    const __grid_constant__ DevRobot r, BwdArgs A, FusedCost fc) {
-  extern __shared__ float prm[];
-  const DevRobot rs = stage_params(r, prm);
+    const __grid_constant__ DevRobot r, const __grid_constant__ WalkTab wt,
+    const __grid_constant__ BwdArgs A, const __grid_constant__ FusedCost fc) {
+  extern __shared__ float4 rec[];
+  stage_recs(r, -1, rec, threadIdx.x, blockDim.x);
   __syncthreads();
-  const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (b < A.B) tree_bwd_cost_one(rs, A, fc, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b);
+  int64_t b;
+  bool act;
+  if (!own_config(A.B, blockIdx.x * (int64_t)blockDim.x + 32 * warp_of(), &b, &act)) return;
+  const float c = tree_bwd_seg<true>(r, rec, ConstWalk{wt}, A, fc,
+                                     ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act,
+                                     whole_sweep(r));
+  if (fc.cost) fc.cost[b] = total_cost(fc, b, c);
 }
 
 __global__ void __launch_bounds__(512, 1) tree_bwd_cost_seg_kernel(
-    const __grid_constant__ DevRobot r, BwdArgs A, FusedCost fc, int t) {
-  extern __shared__ float part[];
+    const __grid_constant__ DevRobot r, const __grid_constant__ WalkTab wt,
+    const __grid_constant__ BwdArgs A, const __grid_constant__ FusedCost fc, int t) {
+  extern __shared__ float4 rec[];
+  float* part = reinterpret_cast<float*>(rec) + kRecWords * (size_t)r.n;
   const int G = 2 << t;
   const int CG = blockDim.x / (32 * G);
-  const int cg = (threadIdx.x >> 5) / G;
+  const int wid = warp_of(), cg = wid / G;
   const int ns = r.seg_ns[t];
   const size_t o = (size_t)ns * G * 32;  // one output's partials
-  Seg sg = seg_of(r, t, part + (size_t)cg * (3 * o + G * 32));
+  Seg sg = seg_of(r, t, wid % G, part + (size_t)cg * (3 * o + G * 32));
   float* cpart = sg.part + 3 * o;  // [G][32] the segments' cost terms
   for (int s = 0; s < ns; ++s)
     for (int q = 0; q < 3; ++q) sg.part[q * o + (s * G + sg.g) * 32 + sg.lane] = 0.0f;
-  const DevRobot rs = stage_params(r, part + (size_t)CG * (3 * o + G * 32));
-  const GradSlot gs = grad_slot_of(part + (size_t)CG * (3 * o + G * 32) + kParamWords * (size_t)r.n);
+  stage_recs(r, t, rec, threadIdx.x, blockDim.x);
+  const GradSlot gs = grad_slot_of(part + (size_t)CG * (3 * o + G * 32));
   __syncthreads();
-  const int64_t b = ((int64_t)blockIdx.x * CG + cg) * 32 + sg.lane;
+  int64_t b;
+  bool act = false;
   float c = 0.0f;
-  if (b < A.B) c = tree_bwd_seg<true>(rs, A, fc, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, sg, gs);
+  if (own_config(A.B, ((int64_t)blockIdx.x * CG + cg) * 32, &b, &act))
+    c = tree_bwd_seg<true>(r, rec, ConstWalk{wt}, A, fc,
+                           ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg, gs);
   cpart[sg.g * 32 + sg.lane] = c;
   __syncthreads();
-  if (b < A.B && sg.g == 0 && fc.cost) {
+  if (act && sg.g == 0 && fc.cost) {
     float acc = 0.0f;
     for (int h = 0; h < G; ++h) acc += cpart[h * 32 + sg.lane];
-    fc.cost[b] = fc.d_min ? fmaf(fc.w, fmaxf(0.0f, -__ldg(fc.d_min + b)), acc) : acc;
+    fc.cost[b] = total_cost(fc, b, acc);
   }
-  if (b < A.B) {
+  if (act) {
     for (int s = sg.g; s < ns; s += G) {
       float acc[3] = {0.0f, 0.0f, 0.0f};
       for (int h = 0; h < G; ++h)
@@ -227,43 +257,51 @@ __device__ __forceinline__ SplineStates spline_states(const DevRobot& r, const S
   return SplineStates{sp.U + (tr * r.d) * sp.K + k, sp.K, bs};
 }
 
-__global__ void __launch_bounds__(256) tree_fwd_spline_kernel(const __grid_constant__ DevRobot r,
-                                                              FwdArgs A, SplineArgs sp) {
-  extern __shared__ float sm[];
-  const DevRobot rs = stage_params(r, sm + 12 * blockDim.x);
+template <int MODE>
+__global__ void __launch_bounds__(256) tree_fwd_spline_kernel(
+    const __grid_constant__ DevRobot r, const __grid_constant__ WalkTab wt,
+    const __grid_constant__ FwdArgs A, const __grid_constant__ SplineArgs sp) {
+  extern __shared__ float4 rec[];
+  float* sm = reinterpret_cast<float*>(rec) + kRecWords * (size_t)r.n;
+  stage_recs(r, -1, rec, threadIdx.x, blockDim.x);
   __syncthreads();
-  const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (b >= A.B) return;
+  int64_t b;
+  bool act;
+  if (!own_config(A.B, blockIdx.x * (int64_t)blockDim.x + 32 * warp_of(), &b, &act)) return;
   const SplineStates st = spline_states(r, sp, b, sm + 12 * threadIdx.x);
-  tree_fwd_seg(rs, A, st, b, whole_sweep(r));
+  tree_fwd_seg<MODE>(r, rec, ConstWalk{wt}, A, st, b, act, whole_sweep(r));
 }
 
-// FS as for tree_fwd_seg_kernel; the force stack follows the link parameters
-template <bool FS>
+// MODE as for tree_fwd_seg_kernel; the force stack follows the partials
+template <int MODE>
 __global__ void __launch_bounds__(512) tree_fwd_spline_seg_kernel(
-    const __grid_constant__ DevRobot r, FwdArgs A, SplineArgs sp, int t) {
-  extern __shared__ float sm[];
+    const __grid_constant__ DevRobot r, const __grid_constant__ WalkTab wt,
+    const __grid_constant__ FwdArgs A, const __grid_constant__ SplineArgs sp, int t) {
+  extern __shared__ float4 rec[];
+  float* sm = reinterpret_cast<float*>(rec) + kRecWords * (size_t)r.n;
   float* part = sm + 12 * blockDim.x;
   const int G = 2 << t;
   const int CG = blockDim.x / (32 * G);
-  const int cg = (threadIdx.x >> 5) / G;
+  const int wid = warp_of(), cg = wid / G;
   const int ns = r.seg_ns[t];
-  if (FS && !smem_holds(12 * (size_t)blockDim.x + (size_t)CG * ns * G * 32 +
-                        kParamWords * (size_t)r.n + 6 * (size_t)r.maxdepth * blockDim.x))
+  if (MODE == kFwdShared && !smem_holds(12 * (size_t)blockDim.x + (size_t)CG * ns * G * 32 +
+                        kRecWords * (size_t)r.n + 6 * (size_t)r.maxdepth * blockDim.x))
     return;
-  Seg sg = seg_of(r, t, part + (size_t)cg * ns * G * 32);
+  Seg sg = seg_of(r, t, wid % G, part + (size_t)cg * ns * G * 32);
   for (int s = 0; s < ns; ++s) sg.part[(s * G + sg.g) * 32 + sg.lane] = 0.0f;
-  const DevRobot rs = stage_params(r, part + (size_t)CG * ns * G * 32);
-  if (FS) {
-    sg.fst = part + (size_t)CG * ns * G * 32 + kParamWords * (size_t)r.n + threadIdx.x;
+  stage_recs(r, t, rec, threadIdx.x, blockDim.x);
+  if (MODE == kFwdShared) {
+    sg.fst = reinterpret_cast<float2*>(part + (size_t)CG * ns * G * 32) + threadIdx.x;
     sg.fstr = blockDim.x;
   }
   __syncthreads();
-  const int64_t b = ((int64_t)blockIdx.x * CG + cg) * 32 + sg.lane;
-  if (b < A.B)
-    tree_fwd_seg<SplineStates, FS>(rs, A, spline_states(r, sp, b, sm + 12 * threadIdx.x), b, sg);
+  int64_t b;
+  bool act = false;
+  if (own_config(A.B, ((int64_t)blockIdx.x * CG + cg) * 32, &b, &act))
+    tree_fwd_seg<MODE>(r, rec, ConstWalk{wt}, A, spline_states(r, sp, b, sm + 12 * threadIdx.x), b,
+                     act, sg);
   __syncthreads();
-  if (b < A.B && A.tau) {
+  if (act && A.tau) {
     for (int s = sg.g; s < ns; s += G) {
       float acc = 0.0f;
       for (int h = 0; h < G; ++h) acc += sg.part[(s * G + h) * 32 + sg.lane];
@@ -274,42 +312,54 @@ __global__ void __launch_bounds__(512) tree_fwd_spline_seg_kernel(
 }
 
 __global__ void __launch_bounds__(256, 2) tree_bwd_spline_cost_kernel(
-    const __grid_constant__ DevRobot r, BwdArgs A, FusedCost fc, SplineArgs sp) {
-  extern __shared__ float sm[];
-  const DevRobot rs = stage_params(r, sm + 12 * blockDim.x);
+    const __grid_constant__ DevRobot r, const __grid_constant__ WalkTab wt,
+    const __grid_constant__ BwdArgs A, const __grid_constant__ FusedCost fc,
+    const __grid_constant__ SplineArgs sp) {
+  extern __shared__ float4 rec[];
+  float* sm = reinterpret_cast<float*>(rec) + kRecWords * (size_t)r.n;
+  stage_recs(r, -1, rec, threadIdx.x, blockDim.x);
   __syncthreads();
-  const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (b >= A.B) return;
-  tree_bwd_cost_one(rs, A, fc, spline_states(r, sp, b, sm + 12 * threadIdx.x), b);
+  int64_t b;
+  bool act;
+  if (!own_config(A.B, blockIdx.x * (int64_t)blockDim.x + 32 * warp_of(), &b, &act)) return;
+  const float c = tree_bwd_seg<true>(r, rec, ConstWalk{wt}, A, fc,
+                                     spline_states(r, sp, b, sm + 12 * threadIdx.x), b, act,
+                                     whole_sweep(r));
+  if (fc.cost) fc.cost[b] = total_cost(fc, b, c);
 }
 
 __global__ void __launch_bounds__(512, 1) tree_bwd_spline_cost_seg_kernel(
-    const __grid_constant__ DevRobot r, BwdArgs A, FusedCost fc, SplineArgs sp, int t) {
-  extern __shared__ float sm[];
+    const __grid_constant__ DevRobot r, const __grid_constant__ WalkTab wt,
+    const __grid_constant__ BwdArgs A, const __grid_constant__ FusedCost fc,
+    const __grid_constant__ SplineArgs sp, int t) {
+  extern __shared__ float4 rec[];
+  float* sm = reinterpret_cast<float*>(rec) + kRecWords * (size_t)r.n;
   float* base = sm + 12 * blockDim.x;
   const int G = 2 << t;
   const int CG = blockDim.x / (32 * G);
-  const int cg = (threadIdx.x >> 5) / G;
+  const int wid = warp_of(), cg = wid / G;
   const int ns = r.seg_ns[t];
   const size_t o = (size_t)ns * G * 32;  // one output's partials
-  Seg sg = seg_of(r, t, base + (size_t)cg * (3 * o + G * 32));
+  Seg sg = seg_of(r, t, wid % G, base + (size_t)cg * (3 * o + G * 32));
   float* cpart = sg.part + 3 * o;  // [G][32] the segments' cost terms
   for (int s = 0; s < ns; ++s)
     for (int q = 0; q < 3; ++q) sg.part[q * o + (s * G + sg.g) * 32 + sg.lane] = 0.0f;
-  const DevRobot rs = stage_params(r, base + (size_t)CG * (3 * o + G * 32));
+  stage_recs(r, t, rec, threadIdx.x, blockDim.x);
   __syncthreads();
-  const int64_t b = ((int64_t)blockIdx.x * CG + cg) * 32 + sg.lane;
+  int64_t b;
+  bool act = false;
   float c = 0.0f;
-  if (b < A.B)
-    c = tree_bwd_seg<true>(rs, A, fc, spline_states(r, sp, b, sm + 12 * threadIdx.x), b, sg);
+  if (own_config(A.B, ((int64_t)blockIdx.x * CG + cg) * 32, &b, &act))
+    c = tree_bwd_seg<true>(r, rec, ConstWalk{wt}, A, fc,
+                           spline_states(r, sp, b, sm + 12 * threadIdx.x), b, act, sg);
   cpart[sg.g * 32 + sg.lane] = c;
   __syncthreads();
-  if (b < A.B && sg.g == 0 && fc.cost) {
+  if (act && sg.g == 0 && fc.cost) {
     float acc = 0.0f;
     for (int h = 0; h < G; ++h) acc += cpart[h * 32 + sg.lane];
-    fc.cost[b] = fc.d_min ? fmaf(fc.w, fmaxf(0.0f, -__ldg(fc.d_min + b)), acc) : acc;
+    fc.cost[b] = total_cost(fc, b, acc);
   }
-  if (b < A.B) {
+  if (act) {
     for (int s = sg.g; s < ns; s += G) {
       float acc[3] = {0.0f, 0.0f, 0.0f};
       for (int h = 0; h < G; ++h)
@@ -381,19 +431,19 @@ void fit_carveout(const void* kern, int threads, size_t smem) {
   cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
 }
 
-static size_t param_smem(const DevRobot& r) { return sizeof(float) * kParamWords * (size_t)r.n; }
+static size_t rec_smem(const DevRobot& r) { return sizeof(float) * kRecWords * (size_t)r.n; }
 
 static int seg_plan(int segments) { return segments == 2 ? 0 : segments == 4 ? 1 : 2; }
 static int seg_groups(int segments, int threads) { return std::max(1, threads / (32 * segments)); }
 
 // per group of G warps: the shared-slot partials of each output (tau in the
 // forward; gq, gqd, gqdd in the backward), plus, for the cost variant, one
-// cost term per segment; per block, the staged link parameters
+// cost term per segment; per block, the staged link records
 size_t tree_seg_smem(const DevRobot& r, int segments, int threads, bool fwd, bool cost) {
   const int t = seg_plan(segments);
   const size_t per =
       (size_t)(fwd ? 1 : 3) * r.seg_ns[t] * segments * 32 + (cost ? segments * 32 : 0);
-  return (size_t)seg_groups(segments, threads) * per * sizeof(float) + param_smem(r);
+  return (size_t)seg_groups(segments, threads) * per * sizeof(float) + rec_smem(r);
 }
 
 // a backward block's gradient-row slots (GradSlot), when it has upstream pose
@@ -403,8 +453,8 @@ size_t grad_slot_smem(int segments, int threads) {
 }
 
 template <class Args>
-static cudaError_t launch_seg(void (*kern)(DevRobot, Args, int), const DevRobot& r, const Args& a,
-                              int threads, int segments, bool fwd, size_t extra,
+static cudaError_t launch_seg(void (*kern)(DevRobot, WalkTab, Args, int), const DevRobot& r,
+                              const WalkTab& wt, const Args& a, int threads, int segments, bool fwd, size_t extra,
                               cudaStream_t s) {
   const int t = seg_plan(segments);
   const int CG = seg_groups(segments, threads);
@@ -415,12 +465,12 @@ static cudaError_t launch_seg(void (*kern)(DevRobot, Args, int), const DevRobot&
   fit_carveout((const void*)kern, 32 * segments * CG, smem);
   const int64_t groups = (a.B + 31) / 32;
   const int64_t grid = (groups + CG - 1) / CG;
-  kern<<<(unsigned)grid, 32 * segments * CG, smem, s>>>(r, a, t);
+  kern<<<(unsigned)grid, 32 * segments * CG, smem, s>>>(r, wt, a, t);
   return cudaGetLastError();
 }
 
-static cudaError_t launch_cost_seg(const DevRobot& r, const BwdArgs& a, const FusedCost& fc,
-                                   int threads, int segments, cudaStream_t s) {
+static cudaError_t launch_cost_seg(const DevRobot& r, const WalkTab& wt, const BwdArgs& a,
+                                   const FusedCost& fc, int threads, int segments, cudaStream_t s) {
   const int t = seg_plan(segments);
   const int CG = seg_groups(segments, threads);
   const size_t smem = tree_seg_smem(r, segments, threads, false, true) +
@@ -431,11 +481,11 @@ static cudaError_t launch_cost_seg(const DevRobot& r, const BwdArgs& a, const Fu
   fit_carveout((const void*)tree_bwd_cost_seg_kernel, 32 * segments * CG, smem);
   const int64_t groups = (a.B + 31) / 32;
   const int64_t grid = (groups + CG - 1) / CG;
-  tree_bwd_cost_seg_kernel<<<(unsigned)grid, 32 * segments * CG, smem, s>>>(r, a, fc, t);
+  tree_bwd_cost_seg_kernel<<<(unsigned)grid, 32 * segments * CG, smem, s>>>(r, wt, a, fc, t);
   return cudaGetLastError();
 }
 
-cudaError_t launch_tree_fwd(const DevRobot& r, const FwdArgs& a, int threads, int segments,
+cudaError_t launch_tree_fwd(const DevRobot& r, const WalkTab& wt, const FwdArgs& a, int threads, int segments,
                             cudaStream_t s) {
   if (threads <= 0) threads = 128;
   if (segments > 1) {
@@ -445,41 +495,44 @@ cudaError_t launch_tree_fwd(const DevRobot& r, const FwdArgs& a, int threads, in
     const size_t bt = (size_t)32 * segments * seg_groups(segments, threads);
     const size_t fs = sizeof(float) * 6 * (size_t)r.maxdepth * bt;
     if (a.tau && tree_seg_smem(r, segments, threads, true, false) + fs <= kSegSmemMax)
-      return launch_seg(tree_fwd_seg_kernel<true>, r, a, threads, segments, true, fs, s);
-    return launch_seg(tree_fwd_seg_kernel<false>, r, a, threads, segments, true, 0, s);
+      return launch_seg(tree_fwd_seg_kernel<kFwdShared>, r, wt, a, threads, segments, true, fs, s);
+    return launch_seg(a.tau ? tree_fwd_seg_kernel<kFwdLocal> : tree_fwd_seg_kernel<kFwdPose>, r, wt,
+                      a, threads, segments, true, 0, s);
   }
   const size_t fs = sizeof(float) * 6 * (size_t)r.maxdepth * threads;  // the force stack
-  const bool use_fs = a.tau && param_smem(r) + fs <= kSegSmemMax;
-  const size_t smem = param_smem(r) + (use_fs ? fs : 0);
-  auto kern = use_fs ? tree_fwd_kernel<true> : tree_fwd_kernel<false>;
+  const bool use_fs = a.tau && rec_smem(r) + fs <= kSegSmemMax;
+  const size_t smem = rec_smem(r) + (use_fs ? fs : 0);
+  auto kern = use_fs ? tree_fwd_kernel<kFwdShared>
+              : a.tau ? tree_fwd_kernel<kFwdLocal>
+                      : tree_fwd_kernel<kFwdPose>;
   cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   fit_carveout((const void*)kern, threads, smem);
   const int64_t grid = (a.B + threads - 1) / threads;
-  kern<<<(unsigned)grid, threads, smem, s>>>(r, a);
+  kern<<<(unsigned)grid, threads, smem, s>>>(r, wt, a);
   return cudaGetLastError();
 }
 
-cudaError_t launch_tree_bwd(const DevRobot& r, const BwdArgs& a, int threads, int segments,
+cudaError_t launch_tree_bwd(const DevRobot& r, const WalkTab& wt, const BwdArgs& a, int threads, int segments,
                             cudaStream_t s, const FusedCost* fc) {
   if (threads <= 0) threads = 128;
   if (segments > 1)
-    return fc ? launch_cost_seg(r, a, *fc, threads, segments, s)
-              : launch_seg(tree_bwd_seg_kernel, r, a, threads, segments, false,
+    return fc ? launch_cost_seg(r, wt, a, *fc, threads, segments, s)
+              : launch_seg(tree_bwd_seg_kernel, r, wt, a, threads, segments, false,
                            a.g_pose || a.g_sph ? grad_slot_smem(segments, threads) : 0, s);
-  const size_t smem = param_smem(r);
+  const size_t smem = rec_smem(r);
   fit_carveout(fc ? (const void*)tree_bwd_cost_kernel : (const void*)tree_bwd_kernel, threads,
                smem);
   const int64_t grid = (a.B + threads - 1) / threads;
   if (fc)
-    tree_bwd_cost_kernel<<<(unsigned)grid, threads, smem, s>>>(r, a, *fc);
+    tree_bwd_cost_kernel<<<(unsigned)grid, threads, smem, s>>>(r, wt, a, *fc);
   else
-    tree_bwd_kernel<<<(unsigned)grid, threads, smem, s>>>(r, a);
+    tree_bwd_kernel<<<(unsigned)grid, threads, smem, s>>>(r, wt, a);
   return cudaGetLastError();
 }
 
-cudaError_t launch_tree_fwd_spline(const DevRobot& r, const FwdArgs& a, const SplineArgs& sp,
+cudaError_t launch_tree_fwd_spline(const DevRobot& r, const WalkTab& wt, const FwdArgs& a, const SplineArgs& sp,
                                    int threads, int segments, cudaStream_t s) {
   if (threads <= 0) threads = 128;
   if (segments > 1) {
@@ -490,23 +543,26 @@ cudaError_t launch_tree_fwd_spline(const DevRobot& r, const FwdArgs& a, const Sp
     const size_t fs = sizeof(float) * 6 * (size_t)r.maxdepth * block;  // the force stack
     const bool use_fs = a.tau && base + fs <= kSegSmemMax;
     const size_t smem = use_fs ? base + fs : base;
-    auto kern = use_fs ? tree_fwd_spline_seg_kernel<true> : tree_fwd_spline_seg_kernel<false>;
+    auto kern = use_fs ? tree_fwd_spline_seg_kernel<kFwdShared>
+                : a.tau ? tree_fwd_spline_seg_kernel<kFwdLocal>
+                        : tree_fwd_spline_seg_kernel<kFwdPose>;
     cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     fit_carveout((const void*)kern, block, smem);
     const int64_t grid = ((a.B + 31) / 32 + CG - 1) / CG;
-    kern<<<(unsigned)grid, block, smem, s>>>(r, a, sp, t);
+    kern<<<(unsigned)grid, block, smem, s>>>(r, wt, a, sp, t);
     return cudaGetLastError();
   }
-  const size_t smem = 12 * sizeof(float) * threads + param_smem(r);
-  fit_carveout((const void*)tree_fwd_spline_kernel, threads, smem);
+  const size_t smem = 12 * sizeof(float) * threads + rec_smem(r);
+  auto kern = a.tau ? tree_fwd_spline_kernel<kFwdLocal> : tree_fwd_spline_kernel<kFwdPose>;
+  fit_carveout((const void*)kern, threads, smem);
   const int64_t grid = (a.B + threads - 1) / threads;
-  tree_fwd_spline_kernel<<<(unsigned)grid, threads, smem, s>>>(r, a, sp);
+  kern<<<(unsigned)grid, threads, smem, s>>>(r, wt, a, sp);
   return cudaGetLastError();
 }
 
-cudaError_t launch_tree_bwd_spline_cost(const DevRobot& r, const BwdArgs& a, const FusedCost& fc,
+cudaError_t launch_tree_bwd_spline_cost(const DevRobot& r, const WalkTab& wt, const BwdArgs& a, const FusedCost& fc,
                                         const SplineArgs& sp, int threads, int segments,
                                         cudaStream_t s) {
   if (threads <= 0) threads = 128;
@@ -520,13 +576,13 @@ cudaError_t launch_tree_bwd_spline_cost(const DevRobot& r, const BwdArgs& a, con
     if (e != cudaSuccess) return e;
     fit_carveout((const void*)tree_bwd_spline_cost_seg_kernel, block, smem);
     const int64_t grid = ((a.B + 31) / 32 + CG - 1) / CG;
-    tree_bwd_spline_cost_seg_kernel<<<(unsigned)grid, block, smem, s>>>(r, a, fc, sp, t);
+    tree_bwd_spline_cost_seg_kernel<<<(unsigned)grid, block, smem, s>>>(r, wt, a, fc, sp, t);
     return cudaGetLastError();
   }
-  const size_t smem = 12 * sizeof(float) * threads + param_smem(r);
+  const size_t smem = 12 * sizeof(float) * threads + rec_smem(r);
   fit_carveout((const void*)tree_bwd_spline_cost_kernel, threads, smem);
   const int64_t grid = (a.B + threads - 1) / threads;
-  tree_bwd_spline_cost_kernel<<<(unsigned)grid, threads, smem, s>>>(r, a, fc, sp);
+  tree_bwd_spline_cost_kernel<<<(unsigned)grid, threads, smem, s>>>(r, wt, a, fc, sp);
   return cudaGetLastError();
 }
 

@@ -82,22 +82,19 @@ __device__ __forceinline__ void joint_sincos(float th, float* s, float* c) {
 // Local transform of link k (parent joint frame -> link frame) for joint
 // variable th: T_fixed * J(th).  Revolute: R = R_f R_J(th) with Rodrigues'
 // rotation R_J = c I + s [a]^ + (1-c) a a^T.  Prismatic: p = p_f + R_f a th.
-// (jt, ident: the link's joint type and whether its fixed rotation is the
-// identity, from a packed table the caller holds; UNIT: the sine and cosine
+// (T4: T_fixed as three float4, a: the axis, jt, ident: the joint type and
+// whether the fixed rotation is the identity; UNIT: the sine and cosine
 // scaled to s^2 + c^2 = 1 within a rounding -- the fast pair misses it by up to
 // 7e-7 -- so that R's inverse is its transpose and products of many R stay
 // rotations)
 template <bool UNIT = false>
-__device__ __forceinline__ void local_xf_m(const DevRobot& r, int k, float th, int jt, bool ident,
-                                           float* R, float* p) {
-  const float4* T4 = reinterpret_cast<const float4*>(r.Tf + 12 * k);
-  const float4 t0 = ldp(T4), t1 = ldp(T4 + 1), t2 = ldp(T4 + 2);
-  const float Rf[9] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w, t2.x};
+__device__ __forceinline__ void local_xf_q(const float4* T4, float4 a, float th, int jt,
+                                           bool ident, float* R, float* p) {
+  const float4 t2 = T4[2];
   p[0] = t2.y;
   p[1] = t2.z;
   p[2] = t2.w;
   if (jt == 1) {
-    const float4 a = ldp(reinterpret_cast<const float4*>(r.axis) + k);
     float s, c;
     joint_sincos(th, &s, &c);
     if (UNIT) {
@@ -122,13 +119,16 @@ __device__ __forceinline__ void local_xf_m(const DevRobot& r, int k, float th, i
 #pragma unroll
       for (int i = 0; i < 9; ++i) R[i] = Rj[i];
     } else {
+      const float4 t0 = T4[0], t1 = T4[1];
+      const float Rf[9] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w, t2.x};
       matmul3(Rf, Rj, R);
     }
   } else {
+    const float4 t0 = T4[0], t1 = T4[1];
+    const float Rf[9] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w, t2.x};
 #pragma unroll
     for (int i = 0; i < 9; ++i) R[i] = Rf[i];
     if (jt == 2) {
-      const float4 a = ldp(reinterpret_cast<const float4*>(r.axis) + k);
       const float s[3] = {a.x * th, a.y * th, a.z * th};
       float Rs[3];
       rot(Rf, s, Rs);
@@ -140,7 +140,9 @@ __device__ __forceinline__ void local_xf_m(const DevRobot& r, int k, float th, i
 }
 
 __device__ __forceinline__ void local_xf(const DevRobot& r, int k, float th, float* R, float* p) {
-  local_xf_m(r, k, th, __ldg(r.jtype + k), __ldg(r.rot_id + k) != 0, R, p);
+  local_xf_q(reinterpret_cast<const float4*>(r.Tf + 12 * k),
+             reinterpret_cast<const float4*>(r.axis)[k], th, __ldg(r.jtype + k),
+             __ldg(r.rot_id + k) != 0, R, p);
 }
 
 // motion vector m (parent coords) -> child coords

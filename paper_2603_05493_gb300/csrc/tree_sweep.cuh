@@ -42,7 +42,7 @@
 // nothing spills at the 128-register cap: humanoid48 backward 0.165 -> 0.138
 // ms, with the cost and states from control points 0.131 -> 0.102 ms, the
 // uneven batch's 0.234 -> 0.200 ms.  The sine and cosine are scaled to the
-// unit circle (UNIT in local_xf_m): gradient error against 64 bits 3.5e-6 ->
+// unit circle (UNIT in local_xf_q): gradient error against 64 bits 3.5e-6 ->
 // 1.0e-6 (humanoid, 32768 configurations), where without it the world
 // rotations' drift from orthogonality gave 5.5e-6.  Storing the states of
 // branching links and reloading them at their children's closes instead:
@@ -72,24 +72,82 @@ namespace wbe {
 
 constexpr int TMAXD = 32;  // deepest tree the sweep kernels accept
 
-// One segment of a segmented sweep (see above).  slot == nullptr: the whole
+// The walk: one word a DFS position with what steers the sweep at it --
+// depth, joint and its type, the parent's position.  The single-robot kernels
+// take the words as a kernel argument: read at a warp-uniform position they
+// come from the constant bank into uniform registers, so the sweep's branches
+// need no reconvergence (with the words in global memory a fifth of the
+// forward's instructions were branches, barriers and moves around them).
+struct ConstWalk {
+  const WalkTab& t;
+  __device__ __forceinline__ uint32_t operator()(int pos) const { return t.w[pos]; }
+};
+struct SharedWalk {  // the batch's: staged with the link records, made uniform by a shuffle
+  const uint32_t* w;
+  __device__ __forceinline__ uint32_t operator()(int pos) const {
+    return __shfl_sync(0xffffffffu, w[pos], 0);
+  }
+};
+__device__ __forceinline__ int wk_dep(uint32_t w) { return w & 31; }
+__device__ __forceinline__ bool wk_branch(uint32_t w) { return (w >> 5) & 1; }  // >= 2 children
+__device__ __forceinline__ int wk_jt(uint32_t w) { return (w >> 6) & 3; }
+__device__ __forceinline__ bool wk_ident(uint32_t w) { return (w >> 8) & 1; }
+__device__ __forceinline__ bool wk_leaf(uint32_t w) { return (w >> 9) & 1; }
+__device__ __forceinline__ int wk_j(uint32_t w) { return (w >> 10) & 255; }
+__device__ __forceinline__ int wk_par(uint32_t w) { return (w >> 18) & 255; }
+
+// One segment of a segmented sweep (see above).  part == nullptr: the whole
 // DFS order, outputs written directly.
 struct Seg {
-  int p0, p1;          // DFS positions this segment owns
-  int g, G;            // segment index, segments per configuration
-  const int16_t* slot; // [n] shared output slot of a link or -1; nullptr = none
-  float* part;         // partial outputs of this group: [nout][ns][G][32]
-  int ns;              // shared slots
+  int p0, p1;   // DFS positions this segment owns
+  int g, G;     // segment index, segments per configuration
+  float* part;  // partial outputs of this group: [nout][ns][G][32]
+  int ns;       // shared slots
   int lane;
   // forward sweep with its force stack in shared memory: this thread's
-  // entry 0, and the stride of the [depth][6][threads] layout (the block's
+  // entry 0, and the stride of the [depth][3][threads] layout (the block's
   // threads)
-  float* fst = nullptr;
+  float2* fst = nullptr;
   int fstr = 0;
 };
 
 __device__ __forceinline__ Seg whole_sweep(const DevRobot& r) {
-  return Seg{0, r.n, 0, 1, nullptr, nullptr, 0, 0};
+  return Seg{0, r.n, 0, 1, nullptr, 0, 0};
+}
+
+// the position of the ancestor at depth c of position pos
+template <class WK>
+__device__ __forceinline__ int ancestor_at(const WK& wk, int pos, int c) {
+  uint32_t w = wk(pos);
+  while (wk_dep(w) > c) {
+    pos = wk_par(w);
+    w = wk(pos);
+  }
+  return pos;
+}
+
+// Copies the robot's link records into shared memory (kRecWords floats a
+// link, in DFS order; see DevRobot::recs) with the inertias and the shared
+// output slots of segment plan t (t < 0: none); thread i of nt.
+__device__ __forceinline__ void stage_recs(const DevRobot& r, int t, float4* dst, int i0, int nt) {
+  for (int i = i0; i < 8 * r.n; i += nt) {
+    float4 v = __ldg(r.recs + i);
+    const int w = i & 7;
+    if (w >= 4) {
+      const int k = __ldg(r.dfs + (i >> 3)).x;
+      const float* in = r.inert + 10 * k;
+      if (w < 6) {
+        const float* x = in + 4 * (w - 4);
+        v = make_float4(__ldg(x), __ldg(x + 1), __ldg(x + 2), __ldg(x + 3));
+      } else if (w == 6) {
+        v.x = __ldg(in + 8);
+        v.y = __ldg(in + 9);
+      } else {
+        v.y = __int_as_float(t >= 0 ? (int)__ldg(r.seg_slot + t * r.n + k) : -1);
+      }
+    }
+    dst[i] = v;
+  }
 }
 
 // L2 prefetch hint for a global input of the next link, so that its DRAM
@@ -101,6 +159,7 @@ __device__ __forceinline__ void pf(const void* p) { asm volatile("prefetch.L2 [%
 // The joint states (q, qd, qdd of joint j) of the sweep's configuration b,
 // from [d][B] arrays ...
 struct ArrayStates {
+  static constexpr bool kAhead = true;  // load the next link's values a link ahead
   const float* q;
   const float* qd;
   const float* qdd;
@@ -124,6 +183,7 @@ struct ArrayStates {
 // (q, qd, qdd), computed once per configuration.  Same arithmetic as the
 // B-spline forward kernel, so the states are the same bits.
 struct SplineStates {
+  static constexpr bool kAhead = false;  // a trajectory's control points stay in L1
   const float* u;
   int K;
   const float* bs;
@@ -137,10 +197,11 @@ struct SplineStates {
   __device__ __forceinline__ void prefetch(int j, bool) const { pf(u + (int64_t)j * K); }
 };
 
-// where the partial output o of link k goes, or nullptr for a direct write
-__device__ __forceinline__ float* seg_part(const Seg& sg, int k, int o) {
-  if (!sg.slot) return nullptr;
-  const int s = __ldg(sg.slot + k);
+// where the partial output o of the link with record q goes, or nullptr for a
+// direct write
+__device__ __forceinline__ float* seg_part(const Seg& sg, const float4* q, int o) {
+  if (!sg.part) return nullptr;
+  const int s = __float_as_int(q[7].y);
   if (s < 0) return nullptr;
   return sg.part + ((size_t)(o * sg.ns + s) * sg.G + sg.g) * 32 + sg.lane;
 }
@@ -204,42 +265,46 @@ __device__ __forceinline__ void joint_motion(int jt, const float* s, const float
   }
 }
 
-// y = Io x for the rotational part of the compact inertia
+// y += Io x for the rotational part of the compact inertia
+__device__ __forceinline__ void rot_inertia_acc(const float* I, const float* x, float* y) {
+  y[0] = fmaf(I[8], x[2], fmaf(I[7], x[1], fmaf(I[4], x[0], y[0])));
+  y[1] = fmaf(I[9], x[2], fmaf(I[5], x[1], fmaf(I[7], x[0], y[1])));
+  y[2] = fmaf(I[6], x[2], fmaf(I[9], x[1], fmaf(I[8], x[0], y[2])));
+}
+// y = Io x
 __device__ __forceinline__ void rot_inertia(const float* I, const float* x, float* y) {
   y[0] = fmaf(I[8], x[2], fmaf(I[7], x[1], I[4] * x[0]));
   y[1] = fmaf(I[9], x[2], fmaf(I[5], x[1], I[7] * x[0]));
   y[2] = fmaf(I[6], x[2], fmaf(I[9], x[1], I[8] * x[0]));
 }
 
-// world pose W = P o L (12 floats each); t: the offset of W's origin from P's
-__device__ __forceinline__ void compose(const float* P, const float* L, float* W, float* t) {
-  matmul3(P, L, W);
-  rot(P, L + 9, t);
-  W[9] = P[9] + t[0];
-  W[10] = P[10] + t[1];
-  W[11] = P[11] + t[2];
+// world pose W <- W o L (12 floats each); t: the offset of the new origin
+// from the old one
+__device__ __forceinline__ void compose(float* W, const float* L, float* t) {
+  rot(W, L + 9, t);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const float a = W[3 * i], b = W[3 * i + 1], c = W[3 * i + 2];
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      W[3 * i + j] = fmaf(c, L[6 + j], fmaf(b, L[3 + j], a * L[j]));
+    W[9 + i] += t[i];
+  }
 }
 
-template <class St>
-__device__ __forceinline__ void link_local_m(const DevRobot& r, int k, int meta, const St& st,
-                                             float* L) {  // meta: lmeta[k]
-  const int j = (meta & 0xFFFF) - 1;
-  const float th = j >= 0 ? joint_var(r, k, st.pos(j)) : 0.0f;
-  local_xf_m(r, k, th, (meta >> 16) & 0xFF, ((meta >> 24) & 1) != 0, L, L + 9);
-}
-template <class St>
-__device__ __forceinline__ void link_local(const DevRobot& r, int k, const St& st, float* L) {
-  const int j = __ldg(r.jidx + k);
-  const float th = j >= 0 ? joint_var(r, k, st.pos(j)) : 0.0f;
-  local_xf(r, k, th, L, L + 9);
+// local transform of the link with record q for its joint's value qj
+template <bool UNIT = false>
+__device__ __forceinline__ void link_local(const float4* q, uint32_t w, float qj, float* L) {
+  const int jt = wk_jt(w);
+  const float th = jt ? fmaf(q[3].w, qj, q[6].z) : 0.0f;
+  local_xf_q<UNIT>(q, q[3], th, jt, wk_ident(w), L, L + 9);
 }
 
-// the dfs_kj word of link k, built from the per-link arrays (for the
-// replayed ancestors of a segment, which are not at its DFS positions)
-__device__ __forceinline__ int packed_link(const DevRobot& r, int k) {
-  const int nch = min(__ldg(r.child_start + k + 1) - __ldg(r.child_start + k), 255);
-  return (__ldg(r.lmeta + k) & 0xFFFF) | (nch << 16) | ((int)__ldg(r.jtype + k) << 24) |
-         ((int)__ldg(r.rot_id + k) << 26);
+__device__ __forceinline__ void rec_inertia(const float4* q, float* I) {
+  const float4 a = q[4], b = q[5], c = q[6];
+  I[0] = a.x; I[1] = a.y; I[2] = a.z; I[3] = a.w;
+  I[4] = b.x; I[5] = b.y; I[6] = b.z; I[7] = b.w;
+  I[8] = c.x; I[9] = c.y;
 }
 
 // ---------------------------------------------------------------------------
@@ -255,238 +320,218 @@ struct FEnt {
   float v[6], a[6], F[6];
 };
 
-// FS: the accumulated forces F of the stack live in shared memory (sg.fst)
-// instead of the thread's local stack
-template <class St, bool FS = false>
-__device__ __forceinline__ void tree_fwd_seg(const DevRobot& r, const FwdArgs& A, const St& st,
-                                             int64_t b, const Seg& sg) {
+// MODE kFwdPose: poses only (its own instantiation: without the dynamics'
+// registers the poses-only sweep of the humanoid takes half the registers);
+// kFwdLocal: torques too when A.tau is given; kFwdShared: with torques, the
+// accumulated forces F of the stack in shared memory (sg.fst) instead of the
+// thread's local stack.  All 32 lanes of the warp take part; a
+// lane past the end sweeps the last configuration again and writes the same
+// values (act = false keeps it out of read-modify-write outputs).
+enum FwdMode { kFwdPose, kFwdLocal, kFwdShared };
+template <int MODE, class WK, class St>
+__device__ __forceinline__ void tree_fwd_seg(const DevRobot& r, const float4* rec, const WK& wk,
+                                             const FwdArgs& A, const St& st, int64_t b, bool act,
+                                             const Seg& sg) {
+  constexpr bool FS = MODE == kFwdShared;
   const int64_t B = A.B;
-  const int n = r.n;
-  const bool dyn = A.tau != nullptr;
+  const bool dyn = FS || (MODE != kFwdPose && A.tau != nullptr);
   FEnt stk[TMAXD];
-  if (dyn && r.mimic_shared)
+  if (dyn && r.mimic_shared && act)
     for (int j = 0; j < r.d; ++j) A.tau[(int64_t)j * B + b] = 0.0f;
+  float* const pose_b = A.pose ? A.pose + b * r.n * 12 : nullptr;
   // Register copies that spare most stack loads: the pre-order data of the
   // last pushed entry (never changes while the entry is on the stack; a link
-  // pushed right after its parent reads it from here), and the accumulated
-  // force of the entry that the post-order closes next (an unwinding chain
-  // passes it on in registers; it is stored when a push interrupts).
-  float cW[12], cv[6], ca[6];
-  int cdep = -1;
-  float pF[6];
-  int pdep = -1;
-  int lastk = 0;  // last pushed link; the stack holds its ancestor chain
-  int ck = 0;     // the link the next close takes
-
-  auto close = [&](int e) {
-    FEnt& E = stk[e];
-    // the link at depth e: the last pushed one, then each closed link's
-    // parent (one load off the critical path instead of two dependent ones
-    // into the ancestor chains: humanoid48 forward 0.0934 -> 0.0892 ms; the
-    // backward, at its register cap, spills more with it and is not faster)
-    const int k = ck;
-    ck = __ldg(r.parent + k);
-    float F[6];
-    if (pdep == e) {
+  // pushed right after its parent finds it here), and the accumulated force
+  // of the entry that the post-order closes next (an unwinding chain passes
+  // it on in registers; it is stored when a push interrupts).
+  float cW[12], cv[6], ca[6], pF[6];
 #pragma unroll
-      for (int i = 0; i < 6; ++i) F[i] = pF[i];
+  for (int i = 0; i < 6; ++i) cv[i] = ca[i] = pF[i] = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 12; ++i) cW[i] = 0.0f;
+  int cdep = -1, pdep = -1;
+  int ckp = 0;  // the position the next close takes: the last pushed one, then parents
+
+  auto load_F = [&](int e, float* F) {
+    if (FS) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const float2 x = sg.fst[(3 * e + i) * sg.fstr];
+        F[2 * i] = x.x;
+        F[2 * i + 1] = x.y;
+      }
     } else {
 #pragma unroll
-      for (int i = 0; i < 6; ++i) F[i] = FS ? sg.fst[(6 * e + i) * sg.fstr] : E.F[i];
+      for (int i = 0; i < 6; ++i) F[i] = stk[e].F[i];
     }
+  };
+  auto close = [&](int e) {
+    const uint32_t w = wk(ckp);
+    const float4* q = rec + 8 * ckp;
+    ckp = wk_par(w);
+    const int j = wk_j(w), jt = wk_jt(w);
+    const float qj = jt ? st.pos(j) : 0.0f;
+    if (pdep != e) load_F(e, pF);
     pdep = -1;
-    const int meta = __ldg(r.lmeta + k);
-    const int j = (meta & 0xFFFF) - 1;
-    if (j >= 0) {
-      const float4 a4 = ldp(reinterpret_cast<const float4*>(r.axis) + k);
+    if (jt) {
+      const float4 a4 = q[3];
       const float ax[3] = {a4.x, a4.y, a4.z};
-      const float mm = ldp(reinterpret_cast<const float2*>(r.mimic) + k).x;
-      const float t = mm * St_dot((meta >> 16) & 0xFF, ax, F);
-      float* pt = seg_part(sg, k, 0);
+      const float t = a4.w * (jt == 1 ? dot3(ax, pF) : dot3(ax, pF + 3));
+      float* pt = seg_part(sg, q, 0);
       if (pt) {
         *pt = t;
       } else {
         float* dst = A.tau + (int64_t)j * B + b;
-        *dst = r.mimic_shared ? *dst + t : t;
+        if (!r.mimic_shared)
+          *dst = t;
+        else if (act)
+          *dst += t;
       }
     }
     if (e > 0) {
-      float L[12], up[6];
-      link_local_m(r, k, meta, st, L);
-      xf_force_T(L, L + 9, F, up);
+      float L[12], up[6], F[6];
+      load_F(e - 1, F);
+      link_local(q, w, qj, L);
+      xf_force_T(L, L + 9, pF, up);
 #pragma unroll
-      for (int i = 0; i < 6; ++i)
-        pF[i] = (FS ? sg.fst[(6 * (e - 1) + i) * sg.fstr] : stk[e - 1].F[i]) + up[i];
+      for (int i = 0; i < 6; ++i) pF[i] = F[i] + up[i];
       pdep = e - 1;
     }
   };
   auto flush = [&]() {  // the pending force goes back to its stack entry
     if (pdep >= 0) {
+      if (FS) {
 #pragma unroll
-      for (int i = 0; i < 6; ++i) {
-        if (FS)
-          sg.fst[(6 * pdep + i) * sg.fstr] = pF[i];
-        else
-          stk[pdep].F[i] = pF[i];
+        for (int i = 0; i < 3; ++i)
+          sg.fst[(3 * pdep + i) * sg.fstr] = make_float2(pF[2 * i], pF[2 * i + 1]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) stk[pdep].F[i] = pF[i];
       }
       pdep = -1;
     }
   };
 
-  // pre-order of link k at depth dep; own = false replays an ancestor of
-  // the segment (pose, v, a only; no output, no force of its own); pre: the
-  // joint states (pq, pqd, pqdd) were loaded ahead by the caller
-  auto push = [&](int k, int dep, bool own, bool pre, float pq, float pqd, float pqdd, int ky) {
-    const int jk = (ky & 0xFFFF) - 1, nch = (ky >> 16) & 0xFF, jtk = (ky >> 24) & 3;
-    if (dyn) flush();  // the parent's force, when it is still pending
+  // pre-order of the link at pos; own = false replays an ancestor of the
+  // segment (pose, v, a only; no output, no force of its own); pq, pqd, pqdd:
+  // its joint's state
+  auto push = [&](int pos, uint32_t w, bool own, float pq, float pqd, float pqdd) {
+    const float4* q = rec + 8 * pos;
+    const int dep = wk_dep(w), jt = wk_jt(w);
     FEnt& E = stk[dep];
     float L[12];
-    {
-      const float th = jk >= 0 ? joint_var(r, k, pre ? pq : st.pos(jk)) : 0.0f;
-      local_xf_m(r, k, th, jtk, ((ky >> 26) & 1) != 0, L, L + 9);
-    }
-    float PW[12], vp[6], ap[6];
+    link_local(q, w, pq, L);
     if (dep > 0) {
-      if (dep == cdep + 1) {
-#pragma unroll
-        for (int i = 0; i < 12; ++i) PW[i] = cW[i];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) {
-          vp[i] = cv[i];
-          ap[i] = ca[i];
-        }
-      } else {
+      if (dep != cdep + 1) {  // a later child: its parent's pre-order data from the stack
         const FEnt& P = stk[dep - 1];
 #pragma unroll
-        for (int i = 0; i < 12; ++i) PW[i] = P.W[i];
+        for (int i = 0; i < 12; ++i) cW[i] = P.W[i];
 #pragma unroll
         for (int i = 0; i < 6; ++i) {
-          vp[i] = P.v[i];
-          ap[i] = P.a[i];
+          cv[i] = P.v[i];
+          ca[i] = P.a[i];
         }
       }
       float t[3];
-      compose(PW, L, cW, t);
+      compose(cW, L, t);
     } else {
 #pragma unroll
       for (int i = 0; i < 12; ++i) cW[i] = L[i];
-      vp[0] = vp[1] = vp[2] = vp[3] = vp[4] = vp[5] = 0.0f;
-      ap[0] = ap[1] = ap[2] = 0.0f;
-      ap[3] = r.abase[0];
-      ap[4] = r.abase[1];
-      ap[5] = r.abase[2];
+#pragma unroll
+      for (int i = 0; i < 6; ++i) cv[i] = ca[i] = 0.0f;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) ca[3 + i] = r.abase[i];
     }
     cdep = dep;
-    lastk = k;
-    ck = k;
-    if (nch > 1) {
+    ckp = pos;
+    if (wk_branch(w)) {
 #pragma unroll
       for (int i = 0; i < 12; ++i) E.W[i] = cW[i];
     }
-    if (own && A.pose) {
-      float4* dst = reinterpret_cast<float4*>(A.pose + (b * n + k) * 12);
+    const int k = __float_as_int(q[7].x) & 0xFF;
+    if (own && pose_b) {
+      float4* dst = reinterpret_cast<float4*>(pose_b + 12 * k);
       dst[0] = make_float4(cW[0], cW[1], cW[2], cW[3]);
       dst[1] = make_float4(cW[4], cW[5], cW[6], cW[7]);
       dst[2] = make_float4(cW[8], cW[9], cW[10], cW[11]);
     }
     if (dyn) {
-      const int j = jk;
-      const float4 a4 = ldp(reinterpret_cast<const float4*>(r.axis) + k);
+      const float4 a4 = q[3];
       const float ax[3] = {a4.x, a4.y, a4.z};
-      const float mm = ldp(reinterpret_cast<const float2*>(r.mimic) + k).x;
-      const float vq = j >= 0 ? mm * (pre ? pqd : st.vel(j)) : 0.0f;
-      const float aq = j >= 0 ? mm * (pre ? pqdd : st.acc(j)) : 0.0f;
-      rnea_va(L, L + 9, vp, ap, jtk, ax, vq, aq, cv, ca);
-      float F[6];
+      const float vq = a4.w * pqd, aq = a4.w * pqdd;
+      float vn[6], an[6];
+      rnea_va(L, L + 9, cv, ca, jt, ax, vq, aq, vn, an);
+#pragma unroll
+      for (int i = 0; i < 6; ++i) {
+        cv[i] = vn[i];
+        ca[i] = an[i];
+      }
+      // the force waits in the pending registers; a child's push stores it
       if (own) {
         float I[10];
-        load_inertia(r, k, I);
-        rnea_force(I, cv, ca, F);
+        rec_inertia(q, I);
+        rnea_force(I, cv, ca, pF);
         if (A.fext) {  // f_k = I a + v x* I v - f_ext,k
-          const float* fe = A.fext + (b * n + k) * 6;
+          const float* fe = A.fext + (b * r.n + k) * 6;
 #pragma unroll
-          for (int i = 0; i < 6; ++i) F[i] -= __ldg(fe + i);
+          for (int i = 0; i < 6; ++i) pF[i] -= __ldg(fe + i);
         }
       } else {
 #pragma unroll
-        for (int i = 0; i < 6; ++i) F[i] = 0.0f;
+        for (int i = 0; i < 6; ++i) pF[i] = 0.0f;
       }
-      if (nch > 1) {
+      if (wk_branch(w)) {
 #pragma unroll
         for (int i = 0; i < 6; ++i) {
           E.v[i] = cv[i];
           E.a[i] = ca[i];
         }
       }
-      // the force waits in the pending registers; a child's push stores it
-#pragma unroll
-      for (int i = 0; i < 6; ++i) pF[i] = F[i];
       pdep = dep;
     }
   };
 
+  // One loop over the replayed proper ancestors of the first link and the
+  // segment's links, one call site each for push and close; past the last
+  // link everything closes.  The joint state of the link pushed next is
+  // loaded one link ahead into registers, so that its latency overlaps the
+  // current link's closes and push.
+  const int nrep = wk_dep(wk(sg.p0)), total = nrep + sg.p1 - sg.p0;
   int sp = 0;
-  if (sg.p0 > 0) {  // replay the proper ancestors of the first link
-    const int k0 = __ldg(r.dfs + sg.p0).x;
-    const int c0 = __ldg(r.chain_start + k0), c1 = __ldg(r.chain_start + k0 + 1);
-    for (int c = c0; c < c1 - 1; ++c) {
-      const int a = __ldg(r.chain + c);
-      push(a, c - c0, false, false, 0.0f, 0.0f, 0.0f, packed_link(r, a));
-    }
-    sp = c1 - 1 - c0;
-  }
-  // The joint states of the link pushed next, loaded one link ahead into
-  // registers, so that their latency overlaps the current link's closes and
-  // push (measured on the 48-DoF humanoid at 2 segments x 448 threads:
-  // 0.0985 -> 0.0970 ms against the L2 prefetch hint it replaces).
+  int npos = ancestor_at(wk, sg.p0, 0);
+  uint32_t nw = wk(npos);
   float nq = 0.0f, nqd = 0.0f, nqdd = 0.0f;
-  int2 nkd = sg.p0 < sg.p1 ? __ldg(r.dfs_kj + sg.p0) : make_int2(0, 0);
-  {
-    const int j0 = sg.p0 < sg.p1 ? (nkd.y & 0xFFFF) - 1 : -1;
-    if (j0 >= 0) {
-      nq = st.pos(j0);
+  auto ahead = [&]() {
+    nq = nqd = nqdd = 0.0f;
+    if (wk_jt(nw)) {
+      const int j = wk_j(nw);
+      nq = st.pos(j);
       if (dyn) {
-        nqd = st.vel(j0);
-        nqdd = st.acc(j0);
+        nqd = st.vel(j);
+        nqdd = st.acc(j);
       }
     }
-  }
-  for (int pos = sg.p0; pos < sg.p1; ++pos) {
-    // link | depth << 8, (joint + 1) | children << 16 of this position: one
-    // load for what the DFS order, the joint index and the child table gave
-    // in four (humanoid48 forward 0.0898 -> 0.0885 ms), kept from the
-    // previous step's look-ahead rather than loaded again (0.0844 -> 0.0835
-    // ms; the backward, at its register cap, spills more with it: 0.1664 ->
-    // 0.1684 ms)
-    const int2 kd = nkd;
-    const int k = kd.x & 0xFF, dep = (kd.x >> 8) & 0xFF;
+  };
+  ahead();
+  for (int i = 0; i <= total; ++i) {
+    const bool end = i == total;
+    const int pos = npos;
+    const uint32_t w = nw;
+    const int dep = end ? 0 : wk_dep(w);
     const float cq = nq, cqd = nqd, cqdd = nqdd;
-    if (pos + 1 < sg.p1) {  // the next link's joint inputs
-      nkd = __ldg(r.dfs_kj + pos + 1);
-      const int jn = (nkd.y & 0xFFFF) - 1;
-      if (jn >= 0) {
-        nq = st.pos(jn);
-        if (dyn) {
-          nqd = st.vel(jn);
-          nqdd = st.acc(jn);
-        }
-      }
+    if (i + 1 < total) {
+      npos = i + 1 < nrep ? ancestor_at(wk, sg.p0, i + 1) : sg.p0 + i + 1 - nrep;
+      nw = wk(npos);
+      ahead();
     }
     if (dyn) {
       while (sp > dep) close(--sp);
       flush();
     }
+    if (end) break;
     sp = dep + 1;
-    push(k, dep, true, true, cq, cqd, cqdd, kd.y);
+    push(pos, w, i >= nrep, cq, cqd, cqdd);
   }
-  if (dyn) {
-    while (sp > 0) close(--sp);
-    flush();
-  }
-}
-
-__device__ __forceinline__ void tree_fwd_one(const DevRobot& r, const FwdArgs& A, int64_t b) {
-  tree_fwd_seg(r, A, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, whole_sweep(r));
 }
 
 // ---------------------------------------------------------------------------
@@ -518,33 +563,31 @@ template <class St>
 __device__ __forceinline__ void chain_pose(const DevRobot& r, int l, const St& st, float* P) {
   const int c0 = __ldg(r.chain_start + l), c1 = __ldg(r.chain_start + l + 1);
   for (int c = c0; c < c1; ++c) {
-    float L[12];
-    link_local(r, __ldg(r.chain + c), st, L);
+    float L[12], t[3];
+    const int k = __ldg(r.chain + c), j = __ldg(r.jidx + k);
+    local_xf(r, k, j >= 0 ? joint_var(r, k, st.pos(j)) : 0.0f, L, L + 9);
     if (c == c0) {
 #pragma unroll
       for (int i = 0; i < 12; ++i) P[i] = L[i];
     } else {
-      float T[12], t[3];
-      compose(P, L, T, t);
-#pragma unroll
-      for (int i = 0; i < 12; ++i) P[i] = T[i];
+      compose(P, L, t);
     }
   }
 }
 
-// parent pose from a link's world pose W and its local transform L: W L^-1;
-// t: the offset of W's origin from the parent's
-__device__ __forceinline__ void uncompose(const float* W, const float* L, float* P, float* t) {
+// parent pose from a link's world pose and its local transform: W <- W L^-1;
+// t: the offset of the old origin from the new one
+__device__ __forceinline__ void uncompose(float* W, const float* L, float* t) {
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
+  for (int i = 0; i < 3; ++i) {
+    const float a = W[3 * i], b = W[3 * i + 1], c = W[3 * i + 2];
 #pragma unroll
     for (int j = 0; j < 3; ++j)
-      P[3 * i + j] =
-          fmaf(W[3 * i + 2], L[3 * j + 2], fmaf(W[3 * i + 1], L[3 * j + 1], W[3 * i] * L[3 * j]));
-  rot(P, L + 9, t);
-  P[9] = W[9] - t[0];
-  P[10] = W[10] - t[1];
-  P[11] = W[11] - t[2];
+      W[3 * i + j] = fmaf(c, L[3 * j + 2], fmaf(b, L[3 * j + 1], a * L[3 * j]));
+  }
+  rot(W, L + 9, t);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) W[9 + i] -= t[i];
 }
 
 // a point of a link (link coordinates sp) with gradient g adds the outer
@@ -566,7 +609,7 @@ __device__ __forceinline__ void point_grad(float4 sp, const float* g, float* G, 
 // and the gradients of wb . n + ub . f with respect to w, al and A,
 //   gA = m ub + wb x h,  gal = Io wb + h x ub,
 //   gw = (Io w) x wb + Io (wb x w) + grad_w [ub . (w x (w x h))],
-// in o[15] = n, f, gw, gal, gA.  Four products with Io: it is rotated to the
+// added to o[15] = n, f, gw, gal, gA.  Four products with Io: it is rotated to the
 // world once (45 operations, against 54 to rotate their arguments in and
 // results out).
 __device__ __forceinline__ void link_adjoint(const float* R, const float* I, const float* w,
@@ -575,7 +618,6 @@ __device__ __forceinline__ void link_adjoint(const float* R, const float* I, con
   float T[9], J[10], h[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) rot_inertia(I, R + 3 * i, T + 3 * i);  // rows of R Io
-  J[0] = I[0];
   J[4] = dot3(T, R);
   J[5] = dot3(T + 3, R + 3);
   J[6] = dot3(T + 6, R + 6);
@@ -583,23 +625,24 @@ __device__ __forceinline__ void link_adjoint(const float* R, const float* I, con
   J[8] = dot3(T, R + 6);
   J[9] = dot3(T + 3, R + 6);
   rot(R, I + 1, h);
+  const float m = I[0];
   float Iw[3], c[3];
   rot_inertia(J, w, Iw);
-  rot_inertia(J, al, o);
+  rot_inertia_acc(J, al, o);
   cross3_acc(w, Iw, o);
   cross3_acc(h, A, o);  // n
 #pragma unroll
-  for (int i = 0; i < 3; ++i) o[3 + i] = J[0] * A[i];
+  for (int i = 0; i < 3; ++i) o[3 + i] = fmaf(m, A[i], o[3 + i]);
   cross3_acc(al, h, o + 3);
   centripetal_acc<1>(w, h, o + 3);  // f
   cross3(wb, w, c);
-  rot_inertia(J, c, o + 6);
+  rot_inertia_acc(J, c, o + 6);
   cross3_acc(Iw, wb, o + 6);
   centripetal_grad(w, h, ub, o + 6);  // gw
-  rot_inertia(J, wb, o + 9);
+  rot_inertia_acc(J, wb, o + 9);
   cross3_acc(h, ub, o + 9);  // gal
 #pragma unroll
-  for (int i = 0; i < 3; ++i) o[12 + i] = J[0] * ub[i];
+  for (int i = 0; i < 3; ++i) o[12 + i] = fmaf(m, ub[i], o[12 + i]);
   cross3_acc(wb, h, o + 12);  // gA
 }
 
@@ -638,15 +681,17 @@ __device__ __forceinline__ void cp16(float4* dst, const void* src) {
 // FC: compiled with the fused cost (a separate instantiation, so that the
 // plain sweep keeps its register allocation).  gs: the thread's gradient-row
 // slot, or none (the rows are then read with plain loads at each close).
-template <bool FC, class St>
-__device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& A,
-                                              const FusedCost& fc, const St& st, int64_t b,
-                                              const Seg& sg, GradSlot gs = GradSlot{}) {
+// act: as for tree_fwd_seg.
+template <bool FC, class WK, class St>
+__device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const float4* rec, const WK& wk,
+                                              const BwdArgs& A, const FusedCost& fc,
+                                              const St& st, int64_t b, bool act, const Seg& sg,
+                                              GradSlot gs = GradSlot{}) {
   const int64_t B = A.B;
   float cost_part = 0.0f;
   const int n = r.n;
   BEnt stk[TMAXD];
-  if (r.mimic_shared)
+  if (r.mimic_shared && act)
     for (int j = 0; j < r.d; ++j) {
       A.gq[(int64_t)j * B + b] = 0.0f;
       A.gqd[(int64_t)j * B + b] = 0.0f;
@@ -655,7 +700,7 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
   // the worst pair's gradient: u = g_dmin (c_i - c_j) / |c_i - c_j|, needed
   // only by the segment that owns one of the pair's links
   auto owned = [&](int k) {
-    if (!sg.slot) return true;
+    if (!sg.part) return true;
     const int p = __ldg(r.dfs_pos + k);
     return p >= sg.p0 && p < sg.p1;
   };
@@ -707,68 +752,72 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
   float cW[12], cw[3], cal[3], cA[3], cwb[3], cub[3], ctb = 0.0f;
   bool fresh = false;
   float ps[kSums];
+#pragma unroll
+  for (int i = 0; i < 12; ++i) cW[i] = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) cw[i] = cal[i] = cA[i] = cwb[i] = cub[i] = 0.0f;
+#pragma unroll
+  for (int i = 0; i < kSums; ++i) ps[i] = 0.0f;
   int pdep = -1;
   // bit e: entry e is an ancestor replayed for this segment (no own terms),
   // its acc holds children's sums
   uint32_t replayed = 0u, accv = 0u;
-  int lcs = 0;  // where the last pushed link's ancestor chain starts (the stack holds it)
+  int ckp = 0;  // the position the next close takes: the last pushed one, then parents
   const bool kin_grad = A.g_pose != nullptr || A.g_sph != nullptr;
   // sphere gradients of a link as float4 triples: the robot's spheres come
   // in runs of 4 (then b S + s is a multiple of 4) and the array (a slice of
   // a packed batch, possibly) is 16-byte aligned
   const bool sph4 = A.g_sph != nullptr && r.sph_vec4 &&
                     (reinterpret_cast<uintptr_t>(A.g_sph) & 15u) == 0;
-  // the link whose gradient rows are on their way into the slot (-1: none)
-  int pend = -1;
   const bool use_slot = gs.p != nullptr && kin_grad;
-  auto issue = [&](int k) {
+  auto issue = [&](const float4* q) {  // q: the link's record
+    const float4 m = q[7];
+    const int kn = __float_as_int(m.x);
     if (A.g_pose) {
-      const float4* g4 = reinterpret_cast<const float4*>(A.g_pose + (b * n + k) * 12);
+      const float4* g4 = reinterpret_cast<const float4*>(A.g_pose + (b * n + (kn & 0xFF)) * 12);
       cp16(gs.p, g4);
       cp16(gs.p + gs.stride, g4 + 1);
       cp16(gs.p + 2 * gs.stride, g4 + 2);
     }
-    if (sph4) {
-      const int e0 = __ldg(r.ls_start + k);
-      if (__ldg(r.ls_start + k + 1) > e0) {
-        const float4* g4 = reinterpret_cast<const float4*>(A.g_sph + (b * r.S + __ldg(r.ls_sph + e0)) * 3);
-        cp16(gs.p + 3 * gs.stride, g4);
-        cp16(gs.p + 4 * gs.stride, g4 + 1);
-        cp16(gs.p + 5 * gs.stride, g4 + 2);
-      }
+    if (sph4 && kn >= 256) {
+      const float4* g4 =
+          reinterpret_cast<const float4*>(A.g_sph + (b * r.S + __float_as_int(m.z)) * 3);
+      cp16(gs.p + 3 * gs.stride, g4);
+      cp16(gs.p + 4 * gs.stride, g4 + 1);
+      cp16(gs.p + 5 * gs.stride, g4 + 2);
     }
     asm volatile("cp.async.commit_group;");
-    pend = k;
   };
 
   // gradient wrench of link k's kinematic outputs (pose, spheres, the worst
   // pair's spheres) in world axes about its origin: the points' gradients
   // join the rotation gradient G, whose wrench is the sum of the crosses of
   // R's columns with G's
-  auto wrench = [&](int k, float* w) {
+  auto wrench = [&](const float4* q, float* w) {  // added to w
+    const float4 m = q[7];
+    const int kn = __float_as_int(m.x), k = kn & 0xFF, ns = kn >> 8, e0 = __float_as_int(m.w);
     float G[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) G[i] = 0.0f;
     float* f = w + 3;
-    f[0] = f[1] = f[2] = 0.0f;
-    const bool slot = pend == k;
+    // every owned link's rows were sent to the slot, at its push (a link closed
+    // next) or at its last child's close
+    const bool slot = use_slot;
     if (slot) asm volatile("cp.async.wait_group 0;" ::: "memory");
-    pend = -1;
     if (A.g_pose) {
       const float4* g4 = reinterpret_cast<const float4*>(A.g_pose + (b * n + k) * 12);
       const float4 x0 = slot ? gs.p[0] : __ldg(g4), x1 = slot ? gs.p[gs.stride] : __ldg(g4 + 1),
                    x2 = slot ? gs.p[2 * gs.stride] : __ldg(g4 + 2);
       G[0] = x0.x; G[1] = x0.y; G[2] = x0.z; G[3] = x0.w; G[4] = x1.x;
       G[5] = x1.y; G[6] = x1.z; G[7] = x1.w; G[8] = x2.x;
-      f[0] = x2.y; f[1] = x2.z; f[2] = x2.w;
+      f[0] += x2.y; f[1] += x2.z; f[2] += x2.w;
     }
     if (sph4) {  // runs of 4 spheres: three float4 loads a run
-      const int e1 = __ldg(r.ls_start + k + 1);
-      const int ef = __ldg(r.ls_start + k);
-      for (int e = ef; e < e1; e += 4) {
-        const int s = __ldg(r.ls_sph + e);
+      int s = __float_as_int(m.z);
+      for (int e = 0; e < ns; e += 4) {
+        if (e > 0) s = __ldg(r.ls_sph + e0 + e);
         const float4* g4 = reinterpret_cast<const float4*>(A.g_sph + (b * r.S + s) * 3);
-        const bool fs = slot && e == ef;
+        const bool fs = slot && e == 0;
         const float4 x0 = fs ? gs.p[3 * gs.stride] : __ldg(g4),
                      x1 = fs ? gs.p[4 * gs.stride] : __ldg(g4 + 1),
                      x2 = fs ? gs.p[5 * gs.stride] : __ldg(g4 + 2);
@@ -777,9 +826,8 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
         for (int i = 0; i < 4; ++i) point_grad(__ldg(r.sph + s + i), gg + 3 * i, G, f);
       }
     } else if (A.g_sph) {
-      const int e1 = __ldg(r.ls_start + k + 1);
-      for (int e = __ldg(r.ls_start + k); e < e1; ++e) {
-        const int s = __ldg(r.ls_sph + e);
+      for (int e = 0; e < ns; ++e) {
+        const int s = __ldg(r.ls_sph + e0 + e);
         const float* g = A.g_sph + (b * r.S + s) * 3;
         const float gg[3] = {__ldg(g), __ldg(g + 1), __ldg(g + 2)};
         point_grad(__ldg(r.sph + s), gg, G, f);
@@ -791,7 +839,6 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
       point_grad(__ldg(r.sph + ps2), mu, G, f);
     }
     const float* R = cW;
-    w[0] = w[1] = w[2] = 0.0f;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       const float rc[3] = {R[j], R[3 + j], R[6 + j]}, gc[3] = {G[j], G[3 + j], G[6 + j]};
@@ -802,17 +849,32 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
   // post-order of the link at depth e; the registers hold its state; tgt:
   // the closes go on down to depth tgt
   auto close = [&](int e, int tgt) {
-    // the link at depth e with its joint, type and rotation flag, one load
-    const int cm = __ldg(r.chain_m + lcs + e);
-    const int k = cm & 0xFF;
+    const uint32_t w = wk(ckp);
+    const float4* q = rec + 8 * ckp;
+    ckp = wk_par(w);
+    const int j = wk_j(w), jt = wk_jt(w);
+    // the joint's state first: its loads' latency overlaps the own terms
+    const float qj = jt ? st.pos(j) : 0.0f, vj = jt ? st.vel(j) : 0.0f, aj = jt ? st.acc(j) : 0.0f;
+    const float tb = fresh ? ctb : stk[e].tb;
     const bool own = !((replayed >> e) & 1u);
-    // own terms (link_adjoint, minus the external wrench) and the gradient
-    // wrench of the kinematic outputs
-    float o[kSums];
+    // the children's sums
+    if (pdep != e) {
+      if ((accv >> e) & 1u) {
+#pragma unroll
+        for (int i = 0; i < kSums; ++i) ps[i] = stk[e].acc[i];
+      } else {
+#pragma unroll
+        for (int i = 0; i < kSums; ++i) ps[i] = 0.0f;
+      }
+    }
+    pdep = -1;
+    // plus the own terms (link_adjoint, minus the external wrench) and the
+    // gradient wrench of the kinematic outputs
     if (own) {
       float I[10];
-      load_inertia(r, k, I);
-      link_adjoint(cW, I, cw, cal, cA, cwb, cub, o);
+      rec_inertia(q, I);
+      link_adjoint(cW, I, cw, cal, cA, cwb, cub, ps);
+      const int k = __float_as_int(q[7].x) & 0xFF;
       if (A.fext) {
         const float* fe = A.fext + (b * n + k) * 6;
         const float xn[3] = {__ldg(fe), __ldg(fe + 1), __ldg(fe + 2)};
@@ -820,44 +882,23 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
         float t[3];
         rot(cW, xn, t);
 #pragma unroll
-        for (int i = 0; i < 3; ++i) o[i] -= t[i];
+        for (int i = 0; i < 3; ++i) ps[i] -= t[i];
         rot(cW, xf, t);
 #pragma unroll
-        for (int i = 0; i < 3; ++i) o[3 + i] -= t[i];
+        for (int i = 0; i < 3; ++i) ps[3 + i] -= t[i];
       }
       if (kin_grad || k == pl1 || k == pl2) {
-        wrench(k, o + 15);
+        wrench(q, ps + 15);
         // the next close's rows, while this one computes
-        if (use_slot && e - 1 >= tgt && !((replayed >> (e - 1)) & 1u))
-          issue(__ldg(r.chain_m + lcs + e - 1) & 0xFF);
-      } else {
-#pragma unroll
-        for (int i = 15; i < kSums; ++i) o[i] = 0.0f;
+        if (use_slot && e - 1 >= tgt && !((replayed >> (e - 1)) & 1u)) issue(rec + 8 * ckp);
       }
-    } else {
-#pragma unroll
-      for (int i = 0; i < kSums; ++i) o[i] = 0.0f;
     }
-    // plus the children's sums
-    if (pdep == e) {
-#pragma unroll
-      for (int i = 0; i < kSums; ++i) o[i] += ps[i];
-    } else if ((accv >> e) & 1u) {
-      const BEnt& E = stk[e];
-#pragma unroll
-      for (int i = 0; i < kSums; ++i) o[i] += E.acc[i];
-    }
-    pdep = -1;
-    float *sn = o, *sf = o + 3, *gw = o + 6, *gal = o + 9, *gA = o + 12, *Wn = o + 15,
-          *Wf = o + 18;
-    const int j = ((cm >> 8) & 0x1FF) - 1;
-    const int jt = (cm >> 17) & 3;
-    const float4 a4 = ldp(reinterpret_cast<const float4*>(r.axis) + k);
+    float *sn = ps, *sf = ps + 3, *gw = ps + 6, *gal = ps + 9, *gA = ps + 12, *Wn = ps + 15,
+          *Wf = ps + 18;
+    const float4 a4 = q[3];
     const float ax[3] = {a4.x, a4.y, a4.z};
-    const float mm = ldp(reinterpret_cast<const float2*>(r.mimic) + k).x;
-    const float vq = j >= 0 ? mm * st.vel(j) : 0.0f;
-    const float aq = j >= 0 ? mm * st.acc(j) : 0.0f;
-    const float tb = fresh ? ctb : (e > 0 ? stk[e].tb : 0.0f);
+    const float mm = a4.w;
+    const float vq = mm * vj, aq = mm * aj;
     float s[3];
     rot(cW, ax, s);
     // The joint's gradients.  Turning a revolute joint turns everything the
@@ -906,15 +947,15 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
         cub[i] = fmaf(-s[i], tb, cub[i]);
       }
     }
-    if (FC && j >= 0) {
+    if (FC && jt) {
       float dqd = 0.0f, dqdd = 0.0f;  // the cost's direct gradients, once per joint
       if (own) {
         const int64_t at = (int64_t)j * B + b;
-        const float tj = __ldg(fc.tau + at), vj = st.vel(j), aj = st.acc(j);
+        const float tj = __ldg(fc.tau + at);
         dqd = 2.0f * (fc.length * vj + fc.e * (vj * tj) * tj);
         dqdd = 2.0f * fc.smooth * aj;
       }
-      float* p0 = seg_part(sg, k, 0);
+      float* p0 = seg_part(sg, q, 0);
       if (p0) {
         const size_t o = (size_t)sg.ns * sg.G * 32;
         p0[0] = mm * gq;
@@ -925,8 +966,8 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
         A.gqd[(int64_t)j * B + b] = mm * gqd + dqd;
         A.gqdd[(int64_t)j * B + b] = mm * gqdd + dqdd;
       }
-    } else if (j >= 0) {
-      float* p0 = seg_part(sg, k, 0);
+    } else if (jt) {
+      float* p0 = seg_part(sg, q, 0);
       if (p0) {
         const size_t o = (size_t)sg.ns * sg.G * 32;
         p0[0] = mm * gq;
@@ -936,26 +977,22 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
         float* o0 = A.gq + (int64_t)j * B + b;
         float* o1 = A.gqd + (int64_t)j * B + b;
         float* o2 = A.gqdd + (int64_t)j * B + b;
-        if (r.mimic_shared) {
-          *o0 += mm * gq;
-          *o1 += mm * gqd;
-          *o2 += mm * gqdd;
-        } else {
+        if (!r.mimic_shared) {
           *o0 = mm * gq;
           *o1 = mm * gqd;
           *o2 = mm * gqdd;
+        } else if (act) {
+          *o0 += mm * gq;
+          *o1 += mm * gqd;
+          *o2 += mm * gqdd;
         }
       }
     }
     fresh = false;
     if (e > 0) {
-      float rv[3];  // the offset from the parent's origin
-      float L[12], Wp[12];
-      const float th = j >= 0 ? joint_var(r, k, st.pos(j)) : 0.0f;
-      local_xf_m<true>(r, k, th, jt, ((cm >> 19) & 1) != 0, L, L + 9);
-      uncompose(cW, L, Wp, rv);
-#pragma unroll
-      for (int i = 0; i < 12; ++i) cW[i] = Wp[i];
+      float L[12], rv[3];
+      link_local<true>(q, w, qj, L);
+      uncompose(cW, L, rv);
       cross3_sub(cal, rv, cA);
       centripetal_acc<-1>(cw, rv, cA);
       cross3_sub(cwb, rv, cub);
@@ -964,11 +1001,12 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
       cross3_acc(rv, gA, gal);
       cross3_acc(rv, sf, sn);
       cross3_acc(rv, Wf, Wn);
-      const BEnt& P = stk[e - 1];
-      const bool has = (accv >> (e - 1)) & 1u;
-      accv &= ~(1u << (e - 1));  // taken over by the pending registers
+      if ((accv >> (e - 1)) & 1u) {  // and the parent's from earlier children
+        const BEnt& P = stk[e - 1];
+        accv &= ~(1u << (e - 1));  // taken over by the pending registers
 #pragma unroll
-      for (int i = 0; i < kSums; ++i) ps[i] = has ? P.acc[i] + o[i] : o[i];
+        for (int i = 0; i < kSums; ++i) ps[i] += P.acc[i];
+      }
       pdep = e - 1;
     }
   };
@@ -982,81 +1020,79 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
     }
   };
 
-  // pre-order of link k at depth dep (the registers hold its parent's state);
-  // own = false replays an ancestor of the segment (its own contributions
-  // are zero)
-  auto push = [&](int k, int dep, bool own, int ky, int cs) {
-    const int j = (ky & 0xFFFF) - 1, nch = (ky >> 16) & 0xFF, jt = (ky >> 24) & 3;
+  // pre-order of the link at pos (the registers hold its parent's state);
+  // own = false replays an ancestor of the segment (its own contributions are
+  // zero); pq, pqd, pqdd, pgt: its joint's state and torque adjoint (FC: its
+  // torque)
+  auto push = [&](int pos, uint32_t w, bool own, float pq, float pqd, float pqdd, float pgt) {
+    const float4* q = rec + 8 * pos;
+    const int dep = wk_dep(w), jt = wk_jt(w), j = wk_j(w);
     float L[12];
-    {
-      const float th = j >= 0 ? joint_var(r, k, st.pos(j)) : 0.0f;
-      local_xf_m<true>(r, k, th, jt, ((ky >> 26) & 1) != 0, L, L + 9);
-    }
-    const float4 a4 = ldp(reinterpret_cast<const float4*>(r.axis) + k);
+    link_local<true>(q, w, pq, L);
+    const float4 a4 = q[3];
     const float ax[3] = {a4.x, a4.y, a4.z};
-    const float mm = ldp(reinterpret_cast<const float2*>(r.mimic) + k).x;
-    const float vq = j >= 0 ? mm * st.vel(j) : 0.0f;
-    const float aq = j >= 0 ? mm * st.acc(j) : 0.0f;
+    const float mm = a4.w;
+    const float vq = mm * pqd, aq = mm * pqdd;
     // the adjoint of the force sweep's torque term: taubar of the joint
     float tb = 0.0f;
-    if (FC && j >= 0) {  // the cost's torque gradient, as the cost kernel forms it
-      const float t = __ldg(fc.tau + (int64_t)j * B + b), l = __ldg(fc.lo + j),
-                  h = __ldg(fc.hi + j);
-      const float v = st.vel(j), a = st.acc(j);
-      const float vt = v * t;
-      float gt = 2.0f * fc.e * v * vt;
-      gt += (t > h ? 1.0f : 0.0f) - (t < l ? 1.0f : 0.0f);
-      tb = mm * gt;
-      if (own) {
-        float c = fmaf(fc.smooth * a, a, 0.0f);
-        c = fmaf(fc.length * v, v, c);
-        c = fmaf(fc.e * vt, vt, c);
-        c += fmaxf(0.0f, t - h) + fmaxf(0.0f, l - t);
-        cost_part += c;
+    if (FC) {
+      if (jt) {  // the cost's torque gradient, as the cost kernel forms it
+        const float t = pgt, l = __ldg(fc.lo + j), h = __ldg(fc.hi + j);
+        const float v = pqd, a = pqdd;
+        const float vt = v * t;
+        float gt = 2.0f * fc.e * v * vt;
+        gt += (t > h ? 1.0f : 0.0f) - (t < l ? 1.0f : 0.0f);
+        tb = mm * gt;
+        if (own) {
+          float c = fmaf(fc.smooth * a, a, 0.0f);
+          c = fmaf(fc.length * v, v, c);
+          c = fmaf(fc.e * vt, vt, c);
+          c += fmaxf(0.0f, t - h) + fmaxf(0.0f, l - t);
+          cost_part += c;
+        }
       }
-    } else if (!FC && j >= 0 && A.g_tau) {
-      tb = mm * __ldg(A.g_tau + (int64_t)j * B + b);
+    } else {
+      tb = mm * pgt;
     }
     // the link's state: pose, motion, and the torques' virtual motion
     // wb = wb_pa + s tb, ub = ub_pa + wb_pa x r (prismatic: ub + s tb)
-    float Wn[12], s[3], rv[3], wn[3], aln[3], An[3];
+    float s[3], rv[3], wp[3], alp[3], Ap[3];
     if (dep > 0) {
-      compose(cW, L, Wn, rv);
-      rot(Wn, ax, s);
-      joint_motion(jt, s, rv, vq, aq, cw, cal, cA, wn, aln, An);
+      compose(cW, L, rv);
       cross3_acc(cwb, rv, cub);
     } else {
 #pragma unroll
-      for (int i = 0; i < 12; ++i) Wn[i] = L[i];
-      rot(Wn, ax, s);
+      for (int i = 0; i < 12; ++i) cW[i] = L[i];
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
         cw[i] = cal[i] = cwb[i] = cub[i] = rv[i] = 0.0f;
         cA[i] = r.abase[i];
       }
-      joint_motion(jt, s, rv, vq, aq, cw, cal, cA, wn, aln, An);
     }
-#pragma unroll
-    for (int i = 0; i < 12; ++i) cW[i] = Wn[i];
+    rot(cW, ax, s);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      cw[i] = wn[i];
-      cal[i] = aln[i];
-      cA[i] = An[i];
-      if (jt == 2)
-        cub[i] = fmaf(s[i], tb, cub[i]);
-      else
-        cwb[i] = fmaf(s[i], tb, cwb[i]);
+      wp[i] = cw[i];
+      alp[i] = cal[i];
+      Ap[i] = cA[i];
+    }
+    joint_motion(jt, s, rv, vq, aq, wp, alp, Ap, cw, cal, cA);
+    if (jt == 2) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) cub[i] = fmaf(s[i], tb, cub[i]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) cwb[i] = fmaf(s[i], tb, cwb[i]);
     }
     ctb = tb;
     fresh = true;
-    lcs = cs;
+    ckp = pos;
     const uint32_t bit = 1u << dep;
     accv &= ~bit;
     replayed = own ? (replayed & ~bit) : (replayed | bit);
-    if (nch > 0) stk[dep].tb = tb;
+    if (!wk_leaf(w)) stk[dep].tb = tb;
     if (own && A.g_fext) {  // dL/df_ext,k = -(wb, ub) in link coordinates
-      float* o = A.g_fext + (b * n + k) * 6;
+      float* o = A.g_fext + (b * n + (__float_as_int(q[7].x) & 0xFF)) * 6;
       float t[6];
       rotT(cW, cwb, t);
       rotT(cW, cub, t + 3);
@@ -1065,57 +1101,53 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const BwdArgs& 
     }
   };
 
+  // one loop over the replayed ancestors and the segment's links, as in the
+  // forward, the joint inputs of the next link loaded (or prefetched) ahead
+  const int nrep = wk_dep(wk(sg.p0)), total = nrep + sg.p1 - sg.p0;
   int sp = 0;
-  if (sg.p0 > 0) {  // replay the proper ancestors of the first link
-    const int k0 = __ldg(r.dfs + sg.p0).x;
-    const int c0 = __ldg(r.chain_start + k0), c1 = __ldg(r.chain_start + k0 + 1);
-    for (int c = c0; c < c1 - 1; ++c) {
-      const int a = __ldg(r.chain + c);
-      push(a, c - c0, false, packed_link(r, a), __ldg(r.chain_start + a));
+  int npos = ancestor_at(wk, sg.p0, 0);
+  uint32_t nw = wk(npos);
+  const float* const gt = FC ? fc.tau : A.g_tau;
+  float nq = 0.0f, nqd = 0.0f, nqdd = 0.0f, ngt = 0.0f;
+  auto fetch = [&]() {
+    nq = nqd = nqdd = ngt = 0.0f;
+    if (wk_jt(nw)) {
+      const int j = wk_j(nw);
+      nq = st.pos(j);
+      nqd = st.vel(j);
+      nqdd = st.acc(j);
+      if (gt) ngt = __ldg(gt + (int64_t)j * B + b);
     }
-    sp = c1 - 1 - c0;
-  }
-  for (int pos = sg.p0; pos < sg.p1; ++pos) {
-    const int2 kd = __ldg(r.dfs_kj + pos);  // link | depth << 8 | chain start << 16, joint word
-    const int k = kd.x & 0xFF, dep = (kd.x >> 8) & 0xFF;
-    const int2 kn = pos + 1 < sg.p1 ? __ldg(r.dfs_kj + pos + 1) : make_int2(0, 0);
-    // L2 prefetch of the next link's joint inputs.  The gradient rows its
-    // close reads are not prefetched: measured slower (the humanoid's
-    // backward 0.218 -> 0.210 ms without)
-    if (pos + 1 < sg.p1) {
-      const int jn = (kn.y & 0xFFFF) - 1;
-      if (jn >= 0) {
-        st.prefetch(jn, true);
-        if (A.g_tau) pf(A.g_tau + (int64_t)jn * B + b);
-        if (FC) pf(fc.tau + (int64_t)jn * B + b);
+  };
+  if (St::kAhead) fetch();
+  for (int i = 0; i <= total; ++i) {
+    const bool end = i == total, own = i >= nrep;
+    const int pos = npos;
+    const uint32_t w = nw;
+    const int dep = end ? 0 : wk_dep(w);
+    if (!St::kAhead && !end) fetch();
+    const float cq = nq, cqd = nqd, cqdd = nqdd, cgt = ngt;
+    if (i + 1 < total) {
+      npos = i + 1 < nrep ? ancestor_at(wk, sg.p0, i + 1) : sg.p0 + i + 1 - nrep;
+      nw = wk(npos);
+      if (St::kAhead) {
+        fetch();
+      } else if (wk_jt(nw)) {
+        st.prefetch(wk_j(nw), true);
+        if (gt) pf(gt + (int64_t)wk_j(nw) * B + b);
       }
     }
     while (sp > dep) close(--sp, dep);
     flush();
+    if (end) break;
     sp = dep + 1;
     // a link closed right after its push (a leaf, or the segment's last
     // link): its rows start on their way now
-    if (use_slot && (pos + 1 >= sg.p1 || ((kn.x >> 8) & 0xFF) <= dep)) issue(k);
-    push(k, dep, true, kd.y, kd.x >> 16);
+    if (use_slot && own && (i + 1 >= total || wk_dep(nw) <= dep)) issue(rec + 8 * pos);
+    push(pos, w, own, cq, cqd, cqdd, cgt);
   }
-  while (sp > 0) close(--sp, 0);
-  flush();
-  if (pend >= 0) asm volatile("cp.async.wait_group 0;" ::: "memory");
+  if (use_slot) asm volatile("cp.async.wait_group 0;" ::: "memory");
   return cost_part;
-}
-
-// the whole sweep of one configuration; with a fused cost it also writes the
-// configuration's cost (joint terms, then the collision term)
-__device__ __forceinline__ void tree_bwd_one(const DevRobot& r, const BwdArgs& A, int64_t b) {
-  tree_bwd_seg<false>(r, A, FusedCost{}, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b,
-                      whole_sweep(r));
-}
-
-template <class St>
-__device__ __forceinline__ void tree_bwd_cost_one(const DevRobot& r, const BwdArgs& A,
-                                                  const FusedCost& fc, const St& st, int64_t b) {
-  const float c = tree_bwd_seg<true>(r, A, fc, st, b, whole_sweep(r));
-  if (fc.cost) fc.cost[b] = fc.d_min ? fmaf(fc.w, fmaxf(0.0f, -__ldg(fc.d_min + b)), c) : c;
 }
 
 }  // namespace wbe

@@ -64,6 +64,7 @@ struct wb_robot {
   int device = 0;
   int num_sms = 0;
   DevRobot dev{};
+  WalkTab walk{};             // the sweeps' walk words (a kernel argument)
   void* dmem = nullptr;
   size_t dbytes = 0;
   float* d_inert = nullptr;   // device inertia array (inside dmem)
@@ -216,8 +217,9 @@ struct HostPlan {
   std::vector<uint32_t> bx;
   std::vector<int32_t> blk_pidx;
   std::vector<int4> lvm;
-  std::vector<int2> dfs, dfs_kj;
-  std::vector<int> lmeta, chain_m;
+  std::vector<int2> dfs;
+  std::vector<uint32_t> walk;
+  std::vector<float4> recs;
   std::vector<int16_t> chain_start, chain;
   int maxdepth = 0;
   int mimic_shared = 0;
@@ -577,17 +579,25 @@ static int plan_robot(const wb_tree* tree, const wb_spheres* sph, const wb_pairs
   H.jidx.swap(jidx);
   H.dfs_pos.assign(n, 0);
   for (int p = 0; p < n; ++p) H.dfs_pos[H.dfs[p].x] = (int16_t)p;
-  H.dfs_kj.resize(n);
+  // walk words and link records by DFS position (WalkTab, DevRobot::recs)
+  static_assert(WB_MAX_LINKS <= kWalkMax, "positions and joints take 8 bits of a walk word");
+  H.walk.resize(n);
+  H.recs.assign(8 * (size_t)n, make_float4(0, 0, 0, 0));
   for (int p = 0; p < n; ++p) {
-    const int k = H.dfs[p].x;
-    const int nch = std::min(child_start[k + 1] - child_start[k], 255);
-    H.dfs_kj[p] = make_int2(k | (H.dfs[p].y << 8) | ((int)H.chain_start[k] << 16),
-                            (H.jidx[k] + 1) | (nch << 16) | ((int)jtype[k] << 24) |
-                                ((int)rot_id[k] << 26));
+    const int k = H.dfs[p].x, pa = H.parent[k], nch = child_start[k + 1] - child_start[k];
+    H.walk[p] = (uint32_t)(H.dfs[p].y & 31) | (nch > 1 ? 1u << 5 : 0u) | ((uint32_t)jtype[k] << 6) |
+                ((uint32_t)rot_id[k] << 8) | (nch == 0 ? 1u << 9 : 0u) |
+                ((uint32_t)std::max<int>(H.jidx[k], 0) << 10) |
+                ((uint32_t)(pa < 0 ? 0 : H.dfs_pos[pa]) << 18);
+    float4* q = &H.recs[8 * (size_t)p];
+    std::memcpy(q, &Tf[12 * (size_t)k], 12 * sizeof(float));
+    q[3] = make_float4(axis[4 * (size_t)k], axis[4 * (size_t)k + 1], axis[4 * (size_t)k + 2],
+                       mimic[2 * (size_t)k]);
+    q[6].z = mimic[2 * (size_t)k + 1];
+    const int e0 = ls_start[k], ns = ls_start[k + 1] - e0;
+    const int32_t m[4] = {k | (ns << 8), -1, ns > 0 ? ls_sph[e0] : 0, e0};
+    std::memcpy(q + 7, m, sizeof(m));
   }
-  H.lmeta.resize(n);
-  for (int k = 0; k < n; ++k)
-    H.lmeta[k] = (H.jidx[k] + 1) | ((int)jtype[k] << 16) | ((int)rot_id[k] << 24);
   // a subtree is the contiguous DFS range up to the next position at the
   // same or a smaller depth
   H.dfs_end.assign(n, (int16_t)n);
@@ -708,16 +718,11 @@ int wb_load_robot(const wb_tree* tree, const wb_spheres* sph, const wb_pairs* pa
   pk.add_vec(H.lev_links, &D.lev_links);
   pk.add_vec(H.lvm, &D.lvm);
   pk.add_vec(H.dfs, &D.dfs);
-  pk.add_vec(H.dfs_kj, &D.dfs_kj);
-  pk.add_vec(H.lmeta, &D.lmeta);
+  pk.add_vec(H.recs, &D.recs);
+  pk.add_vec(H.walk, &D.walk);
+  std::copy(H.walk.begin(), H.walk.end(), R->walk.w);
   pk.add_vec(H.chain_start, &D.chain_start);
   pk.add_vec(H.chain, &D.chain);
-  H.chain_m.resize(H.chain.size());
-  for (size_t c = 0; c < H.chain.size(); ++c) {
-    const int k = H.chain[c];
-    H.chain_m[c] = k | ((H.jidx[k] + 1) << 8) | ((int)H.jtype[k] << 17) | ((int)H.rot_id[k] << 19);
-  }
-  pk.add_vec(H.chain_m, &D.chain_m);
   D.maxdepth = H.maxdepth;
   pk.add_vec(H.dfs_pos, &D.dfs_pos);
   pk.add_vec(H.dfs_end, &D.dfs_end);
@@ -971,8 +976,11 @@ static int pair_warps(wb_robot* R, bool bits, const wb_tune* tune, bool cull = t
 // measured on the 48-DoF humanoid at 32768 configurations: both passes best
 // at 2 segments (the register copies of the stack top make each warp
 // faster, so fewer segments suffice), 8 slower than 1.
-static int tree_segments(const wb_robot* R, const wb_tune* tune, int64_t B, int threads,
+// *tpb: the block's threads, lowered where the link records no longer leave
+// room for the partials of all its groups.
+static int tree_segments(const wb_robot* R, const wb_tune* tune, int64_t B, int* tpb,
                          bool fwd, int* out) {
+  const int threads = *tpb;
   const int req = tune ? tune->lanes_per_config : 0;
   const int ok = R->dev.seg_ok;
   int G = 1;
@@ -991,10 +999,19 @@ static int tree_segments(const wb_robot* R, const wb_tune* tune, int64_t B, int 
   }
   if (G == 1 && threads > 256)
     return fail(WB_EINVAL, "one-segment sweeps take at most 256 threads per block");
-  if (G > 1 && tree_seg_smem(R->dev, G, threads, fwd, !fwd) +
-                       (fwd ? 0 : grad_slot_smem(G, threads)) >
-                   227 * 1024)
+  // what a block needs: refused from the limit up, counting 28 floats a link
+  // record; the records' padding to kRecWords is made room for
+  auto need = [&](int threads_) {
+    return tree_seg_smem(R->dev, G, threads_, fwd, !fwd) + (fwd ? 0 : grad_slot_smem(G, threads_));
+  };
+  if (G > 1 && need(threads) - sizeof(float) * (kRecWords - 28) * (size_t)R->dev.n > kMaxBlockSmem)
     return fail(WB_ETOOBIG, "segmented sweep needs too much shared memory");
+  while (G > 1 && need(*tpb) > kMaxBlockSmem) {
+    if (*tpb >= 64 * G)
+      *tpb -= 32 * G;
+    else
+      G = G == 8 && (ok & 2) ? 4 : G > 2 && (ok & 1) ? 2 : 1;
+  }
   *out = G;
   return WB_OK;
 }
@@ -1049,7 +1066,7 @@ int wb_eval_ext(wb_robot* robot, int64_t B, const float* q, const float* qd, con
     if (!tree_ok) return fail(WB_ETOOBIG, "tree deeper than %d levels", tree_max_depth());
     if (pairs_wanted && !link_pose)
       return fail(WB_EINVAL, "the tree kernel needs link_pose when spheres or pairs are wanted");
-    const int tpb = (tune && tune->configs_per_block) ? tune->configs_per_block : 128;
+    int tpb = (tune && tune->configs_per_block) ? tune->configs_per_block : 128;
     if (tpb < 32 || tpb > 512 || tpb % 32)
       return fail(WB_EINVAL, "tree threads per block must be a multiple of 32 in [32, 512]");
     const int warps = pair_warps(robot, pair_bits != nullptr, tune, cull);
@@ -1059,8 +1076,8 @@ int wb_eval_ext(wb_robot* robot, int64_t B, const float* q, const float* qd, con
     if (pairs_wanted && pair_block_smem(robot->dev, warps, pair_bits != nullptr) > kMaxBlockSmem)
       return fail(WB_ETOOBIG, "%d pair warps per block need too much shared memory", warps);
     int G = 1;
-    if ((rc = tree_segments(robot, tune, B, tpb, true, &G))) return rc;
-    e = launch_tree_fwd(robot->dev, a, tpb, G, s);
+    if ((rc = tree_segments(robot, tune, B, &tpb, true, &G))) return rc;
+    e = launch_tree_fwd(robot->dev, robot->walk, a, tpb, G, s);
     if (e == cudaSuccess && pairs_wanted) {
       int bps = 0;
       e = pair_max_blocks_per_sm(robot->dev, warps, pair_bits != nullptr, &bps);
@@ -1270,12 +1287,12 @@ int wb_eval_backward_dir(wb_robot* robot, int64_t B, const float* q, const float
     e = launch_plain_bwd(robot->dev, a, 128, s);
   } else if (kernel == WB_KERNEL_TREE) {
     if (!tree_ok) return fail(WB_ETOOBIG, "tree deeper than %d levels", tree_max_depth());
-    const int tpb = (tune && tune->configs_per_block) ? tune->configs_per_block : 128;
+    int tpb = (tune && tune->configs_per_block) ? tune->configs_per_block : 128;
     if (tpb < 32 || tpb > 512 || tpb % 32)
       return fail(WB_EINVAL, "tree threads per block must be a multiple of 32 in [32, 512]");
     int G = 1;
-    if ((rc = tree_segments(robot, tune, B, tpb, false, &G))) return rc;
-    e = launch_tree_bwd(robot->dev, a, tpb, G, s);
+    if ((rc = tree_segments(robot, tune, B, &tpb, false, &G))) return rc;
+    e = launch_tree_bwd(robot->dev, robot->walk, a, tpb, G, s);
   } else if (kernel == WB_KERNEL_FUSED) {
     if (a.fext || a.g_fext) return fail(WB_EINVAL, "the fused kernels take no external forces");
     FusedShape sh;
@@ -1335,12 +1352,12 @@ int wb_eval_spline(wb_robot* robot, const wb_spline* spline, float* link_pose, f
   DeviceGuard guard(robot->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   FwdArgs a{B, nullptr, nullptr, nullptr, link_pose, sphere, d_min, worst_pair, tau, nullptr};
-  const int tpb = (tune && tune->configs_per_block) ? tune->configs_per_block : 128;
+  int tpb = (tune && tune->configs_per_block) ? tune->configs_per_block : 128;
   if (tpb < 32 || tpb > 512 || tpb % 32)
     return fail(WB_EINVAL, "tree threads per block must be a multiple of 32 in [32, 512]");
   int G = 1;
-  if ((rc = tree_segments(robot, tune, B, tpb, true, &G))) return rc;
-  cudaError_t e = launch_tree_fwd_spline(robot->dev, a, sp, tpb, G, s);
+  if ((rc = tree_segments(robot, tune, B, &tpb, true, &G))) return rc;
+  cudaError_t e = launch_tree_fwd_spline(robot->dev, robot->walk, a, sp, tpb, G, s);
   if (e == cudaSuccess && pairs_wanted) {
     const int warps = pair_warps(robot, false, tune, kernel != WB_KERNEL_TREE_NOCULL);
     if (warps < 1 || warps > 8) return fail(WB_ETOOBIG, "pair kernel does not fit on an SM");
@@ -1423,12 +1440,12 @@ int wb_eval_backward_spline_cost_dir(wb_robot* robot, const wb_spline* spline,
   fc.length = W.length;
   fc.e = W.energy * W.dt * W.dt;
   fc.cost = cost;
-  const int tpb = (tune && tune->configs_per_block) ? tune->configs_per_block : 128;
+  int tpb = (tune && tune->configs_per_block) ? tune->configs_per_block : 128;
   if (tpb < 32 || tpb > 512 || tpb % 32)
     return fail(WB_EINVAL, "tree threads per block must be a multiple of 32 in [32, 512]");
   int G = 1;
-  if ((rc = tree_segments(robot, tune, B, tpb, false, &G))) return rc;
-  const cudaError_t e = launch_tree_bwd_spline_cost(robot->dev, a, fc, sp, tpb, G,
+  if ((rc = tree_segments(robot, tune, B, &tpb, false, &G))) return rc;
+  const cudaError_t e = launch_tree_bwd_spline_cost(robot->dev, robot->walk, a, fc, sp, tpb, G,
                                                     static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "wb_eval_backward_spline_cost launch");
   return WB_OK;
@@ -1500,13 +1517,13 @@ int wb_eval_backward_cost_dir(wb_robot* robot, int64_t B, const float* q, const 
   fc.length = W.length;
   fc.e = W.energy * W.dt * W.dt;
   fc.cost = cost;
-  const int tpb = (tune && tune->configs_per_block) ? tune->configs_per_block : 128;
+  int tpb = (tune && tune->configs_per_block) ? tune->configs_per_block : 128;
   if (tpb < 32 || tpb > 512 || tpb % 32)
     return fail(WB_EINVAL, "tree threads per block must be a multiple of 32 in [32, 512]");
   int G = 1;
-  if ((rc = tree_segments(robot, tune, B, tpb, false, &G))) return rc;
+  if ((rc = tree_segments(robot, tune, B, &tpb, false, &G))) return rc;
   const cudaError_t e =
-      launch_tree_bwd(robot->dev, a, tpb, G, static_cast<cudaStream_t>(stream), &fc);
+      launch_tree_bwd(robot->dev, robot->walk, a, tpb, G, static_cast<cudaStream_t>(stream), &fc);
   if (e != cudaSuccess) return cuda_fail(e, "wb_eval_backward_cost launch");
   return WB_OK;
 }
@@ -1533,6 +1550,7 @@ struct wb_batch {
   int n_pitems = 0;
   int ws_words = 0, rad_words = 0;
   int ns_max = 0;  // most shared slots among the used robots' 2-segment sweep plans
+  int n_max = 0;   // most links among them
   wb_batch_sizes sizes{};
   // launch choices (wb_batch_set_tune / wb_batch_autotune): threads per block
   // of the forward and backward sweep passes, warps per block of the pair
@@ -1633,6 +1651,7 @@ int wb_batch_create(wb_robot* const* robots, int32_t n_robots, const wb_problem*
     Bt->ws_words = std::max(Bt->ws_words, pair_plan_words(D));
     Bt->rad_words = std::max(Bt->rad_words, (4 * D.Sg + 31) & ~31);
     Bt->ns_max = std::max(Bt->ns_max, seg2_slots(D));
+    Bt->n_max = std::max(Bt->n_max, D.n);
   }
   Bt->sizes = wb_batch_sizes{jo, po, so, co, n_problems, n_robots};
   // longest work first
@@ -1710,16 +1729,29 @@ void wb_free_batch(wb_batch* batch) {
   delete batch;
 }
 
-static int batch_grid_tree(const wb_batch* Bt, bool fwd, int* grid) {
-  const int pass = fwd ? 0 : 1, threads = Bt->threads[pass];
+// grid and threads per block of a sweep pass: the batch's choice of threads, or
+// half of it until the records of the block's pairs fit its shared memory
+// (one pair always does)
+static int batch_sweep_shape(bool fwd, int ns_max, int n_max, int n_items, int num_sms,
+                             int* threads, int* grid) {
   int bps = 0;
-  cudaError_t e = batch_tree_max_blocks_per_sm(fwd, Bt->ns_max, threads, &bps);
-  if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
-  if (bps < 1) return fail(WB_ETOOBIG, "batch sweep block of %d threads does not fit", threads);
-  const int pairs = threads / 64;  // an item per pair of warps
-  const int need = (Bt->n_titems[pass] + pairs - 1) / pairs;
-  *grid = std::max(1, std::min(need, bps * Bt->num_sms));
+  for (;; *threads /= 2) {
+    cudaError_t e = batch_tree_max_blocks_per_sm(fwd, ns_max, n_max, *threads, &bps);
+    if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
+    if (bps >= 1 || *threads <= 64) break;
+  }
+  if (bps < 1) return fail(WB_ETOOBIG, "batch sweep block of %d threads does not fit", *threads);
+  const int pairs = *threads / 64;  // an item per pair of warps
+  const int need = (n_items + pairs - 1) / pairs;
+  *grid = std::max(1, std::min(need, bps * num_sms));
   return WB_OK;
+}
+
+static int batch_grid_tree(const wb_batch* Bt, bool fwd, int* threads, int* grid) {
+  const int pass = fwd ? 0 : 1;
+  *threads = Bt->threads[pass];
+  return batch_sweep_shape(fwd, Bt->ns_max, Bt->n_max, Bt->n_titems[pass], Bt->num_sms, threads,
+                           grid);
 }
 
 // the pair pass's warps per block: the batch's choice, or the most that fit
@@ -1753,11 +1785,11 @@ int wb_batch_eval(wb_batch* batch, const float* q, const float* qd, const float*
   int* counters = const_cast<int*>(batch->d_counters);
   cudaError_t e = cudaSuccess;
   if (link_pose || tau) {
-    int grid = 1;
-    if ((rc = batch_grid_tree(batch, true, &grid))) return rc;
+    int threads = 0, grid = 1;
+    if ((rc = batch_grid_tree(batch, true, &threads, &grid))) return rc;
     e = launch_batch_tree_fwd(batch->d_robots, batch->d_probs, batch->d_titems[0],
                               batch->n_titems[0], counters, io, grid, batch->ns_max,
-                              batch->threads[0], s);
+                              batch->n_max, threads, s);
     if (e != cudaSuccess) return cuda_fail(e, "wb_batch_eval launch");
   }
   if (pairs && batch->n_pitems > 0) {
@@ -1800,11 +1832,11 @@ int wb_batch_eval_backward(wb_batch* batch, const float* q, const float* qd, con
   DeviceGuard guard(batch->device);
   BatchIO io{q, qd, qdd, nullptr, nullptr, nullptr, const_cast<int32_t*>(worst_pair), nullptr,
              g_pose, g_sphere, g_dmin, g_tau, gq, gqd, gqdd};
-  int grid = 1;
-  if ((rc = batch_grid_tree(batch, false, &grid))) return rc;
+  int threads = 0, grid = 1;
+  if ((rc = batch_grid_tree(batch, false, &threads, &grid))) return rc;
   cudaError_t e = launch_batch_tree_bwd(batch->d_robots, batch->d_probs, batch->d_titems[1],
                                         batch->n_titems[1], const_cast<int*>(batch->d_counters) + 2,
-                                        io, grid, batch->ns_max, batch->threads[1],
+                                        io, grid, batch->ns_max, batch->n_max, threads,
                                         static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "wb_batch_eval_backward launch");
   return WB_OK;
@@ -2069,7 +2101,7 @@ int wb_batch_eval_noalloc(wb_robot* const* robots, int32_t n_robots, const wb_pr
   plan.n_robots = n_robots;
   plan.n_problems = n_problems;
   plan.n_configs = (int)configs;
-  int ws_words = 0, rad_words = 0, ns_max = 0;
+  int ws_words = 0, rad_words = 0, ns_max = 0, n_max = 0;
   for (int i = 0; i < n_robots; ++i) {
     plan.robots[i] = robots[i]->dev;
     plan.scheds[i] = robots[i]->sched32;
@@ -2082,6 +2114,7 @@ int wb_batch_eval_noalloc(wb_robot* const* robots, int32_t n_robots, const wb_pr
     ws_words = std::max(ws_words, pair_plan_words(D));
     rad_words = std::max(rad_words, (4 * D.Sg + 31) & ~31);
     ns_max = std::max(ns_max, seg2_slots(D));
+    n_max = std::max(n_max, D.n);
   }
   // longest work first: robots by cost (stable), problems in order within one
   int n_titems = 0, n_pitems = 0;
@@ -2118,12 +2151,11 @@ int wb_batch_eval_noalloc(wb_robot* const* robots, int32_t n_robots, const wb_pr
   BatchIO io{q, qd, qdd, link_pose, sphere, d_min, worst_pair, tau,
              nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   if (link_pose || tau) {
-    int bps = 0;
-    e = batch_tree_max_blocks_per_sm(true, ns_max, 128, &bps);
-    if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
-    const int grid = std::max(1, std::min((n_titems + 1) / 2, std::max(bps, 1) * R0->num_sms));
+    int threads = 128, grid = 1;
+    const int rc2 = batch_sweep_shape(true, ns_max, n_max, n_titems, R0->num_sms, &threads, &grid);
+    if (rc2) return rc2;
     e = launch_batch_tree_fwd(T.robots, T.probs, T.titems, n_titems, T.counters, io, grid, ns_max,
-                              128, s);
+                              n_max, threads, s);
     if (e != cudaSuccess) return cuda_fail(e, "wb_batch_eval_noalloc launch");
   }
   if (pairs) {
@@ -2527,16 +2559,16 @@ extern "C" int wb_batch_autotune(wb_batch* batch, wb_batch_tune* tune, int32_t* 
     int* counters = const_cast<int*>(batch->d_counters);
     BatchIO io{q, qd, qdd, pose, sph, dmin, worst, tau, gpose, gsph, gdmin, gtau, gq, gqd, gqdd};
     auto sweep = [&](int pass) -> int {
-      int grid = 1, rc;
-      if ((rc = batch_grid_tree(batch, pass == 0, &grid))) return rc;
+      int threads = 0, grid = 1, rc;
+      if ((rc = batch_grid_tree(batch, pass == 0, &threads, &grid))) return rc;
       cudaError_t e =
           pass == 0
               ? launch_batch_tree_fwd(batch->d_robots, batch->d_probs, batch->d_titems[0],
                                       batch->n_titems[0], counters, io, grid, batch->ns_max,
-                                      batch->threads[0], s)
+                                      batch->n_max, threads, s)
               : launch_batch_tree_bwd(batch->d_robots, batch->d_probs, batch->d_titems[1],
                                       batch->n_titems[1], counters + 2, io, grid, batch->ns_max,
-                                      batch->threads[1], s);
+                                      batch->n_max, threads, s);
       return e == cudaSuccess ? WB_OK : cuda_fail(e, "batch autotune launch");
     };
     // robots whose segments are a choice: a 2-segment plan and some problem

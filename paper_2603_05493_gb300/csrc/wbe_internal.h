@@ -42,16 +42,15 @@ struct DevRobot {
   const int16_t* lev_start;  // [nlev+1]
   const int16_t* lev_links;  // [n] links grouped by level
   const int2* dfs;           // [n] depth-first pre-order: link, depth
-  const int2* dfs_kj;        // [n] the same positions packed for the sweeps: link |
-                             //   depth << 8 | chain_start[link] << 16, (joint + 1) |
-                             //   min(children, 255) << 16 | joint type << 24 | rot_id << 26
-  const int* lmeta;          // [n] per link: (joint + 1) | joint type << 16 | rot_id << 24
+  const float4* recs;        // [n][8] link records by DFS position, as the sweeps stage them:
+                             //   T_fixed 12; axis 3, mimic multiplier; inertia 10 (filled in
+                             //   from inert when staged), mimic offset, pad; link | spheres << 8,
+                             //   shared output slot (filled in), first sphere, first of ls_sph
+  const uint32_t* walk;      // [n] walk words by DFS position (WalkTab)
   int maxdepth;              // deepest link depth + 1
   int mimic_shared;          // 1 if some joint drives more than one link
   const int16_t* chain_start;// [n+1] ancestor chains (Alg. 1 "linkChain")
   const int16_t* chain;      // root -> link, link included
-  const int* chain_m;        // the chain's entries packed: link | (joint + 1) << 8 |
-                             //   joint type << 17 | rot_id << 19
   const int16_t* dfs_pos;    // [n] DFS position of each link
   const int16_t* dfs_end;    // [n] one past the last DFS position of its subtree
   // segmented sweeps with G = 2 << t segments, t = 0, 1, 2 (tree_sweep.cuh)
@@ -78,6 +77,15 @@ struct DevRobot {
   const int16_t* grp_link;   // [Sg] that link, or -1 (spheres on several links)
   const int32_t* blk_pidx;   // [nblk][16] pair index of (4gi+a, 4gj+b) or -1
 };
+
+// What steers the sweeps at each DFS position: depth | several children << 5 |
+// joint type << 6 | identity fixed rotation << 8 | leaf << 9 | joint << 10 |
+// the parent's position << 18.  A kernel argument of the single-robot sweeps.
+constexpr int kWalkMax = 256;
+struct WalkTab {
+  uint32_t w[kWalkMax];
+};
+constexpr int kRecWords = 32;  // floats of a link record
 
 // A per-lane schedule of pair blocks for the fused kernel with G lanes per
 // configuration: entry [r][l] is the block lane l processes in round r.
@@ -196,10 +204,12 @@ struct BatchIO {
 // warps per block).
 cudaError_t launch_batch_tree_fwd(const DevRobot* robots, const BatchProblemDev* probs,
                                   const int4* items, int n_items, int* counter, const BatchIO& io,
-                                  int grid, int ns_max, int threads, cudaStream_t s);
+                                  int grid, int ns_max, int n_max, int threads,
+                                  cudaStream_t s);
 cudaError_t launch_batch_tree_bwd(const DevRobot* robots, const BatchProblemDev* probs,
                                   const int4* items, int n_items, int* counter, const BatchIO& io,
-                                  int grid, int ns_max, int threads, cudaStream_t s);
+                                  int grid, int ns_max, int n_max, int threads,
+                                  cudaStream_t s);
 cudaError_t launch_batch_pair(const DevRobot* robots, const PairSchedule32* scheds,
                               const BatchProblemDev* probs, const int2* items, int n_items,
                               int* counter, const BatchIO& io, int grid, int warps, int ws_words,
@@ -233,7 +243,7 @@ __host__ __device__ NoAllocTables noalloc_tables(unsigned char* base);
 cudaError_t noalloc_scratch(int device, unsigned char** out);
 cudaError_t launch_noalloc_setup(const NoAllocPlan& plan, unsigned char* base, int grid,
                                  cudaStream_t s);
-cudaError_t batch_tree_max_blocks_per_sm(bool fwd, int ns_max, int threads, int* out);
+cudaError_t batch_tree_max_blocks_per_sm(bool fwd, int ns_max, int n_max, int threads, int* out);
 int pair_plan_words(const DevRobot& r);
 
 // launchers (return cudaGetLastError())
@@ -286,14 +296,14 @@ cudaError_t launch_trajopt_cost(int64_t B, int d, const float* tau, const float*
 // threads: threads per block, a multiple of 32, at most 256 for one segment
 // and 512 for a segmented sweep (its launch bounds); every sweep block also
 // stages the robot's link parameters in shared memory
-cudaError_t launch_tree_fwd(const DevRobot& r, const FwdArgs& a, int threads, int segments,
+cudaError_t launch_tree_fwd(const DevRobot& r, const WalkTab& wt, const FwdArgs& a, int threads, int segments,
                             cudaStream_t s);
-cudaError_t launch_tree_bwd(const DevRobot& r, const BwdArgs& a, int threads, int segments,
+cudaError_t launch_tree_bwd(const DevRobot& r, const WalkTab& wt, const BwdArgs& a, int threads, int segments,
                             cudaStream_t s, const FusedCost* fc = nullptr);
 // the sweeps with the joint states evaluated from control points
-cudaError_t launch_tree_fwd_spline(const DevRobot& r, const FwdArgs& a, const SplineArgs& sp,
+cudaError_t launch_tree_fwd_spline(const DevRobot& r, const WalkTab& wt, const FwdArgs& a, const SplineArgs& sp,
                                    int threads, int segments, cudaStream_t s);
-cudaError_t launch_tree_bwd_spline_cost(const DevRobot& r, const BwdArgs& a, const FusedCost& fc,
+cudaError_t launch_tree_bwd_spline_cost(const DevRobot& r, const WalkTab& wt, const BwdArgs& a, const FusedCost& fc,
                                         const SplineArgs& sp, int threads, int segments,
                                         cudaStream_t s);
 size_t tree_seg_smem(const DevRobot& r, int segments, int threads, bool fwd, bool cost = false);
