@@ -15,6 +15,11 @@ namespace wbe {
 // out of the way of the depth-first stacks in L1.
 constexpr size_t kSegSmemMax = 227 * 1024;  // dynamic shared memory of one block
 
+// floats at the start of a backward block's shared memory: records, spheres
+__host__ __device__ __forceinline__ size_t bwd_words(const DevRobot& r) {
+  return kRecWords * (size_t)r.n + 4 * (size_t)r.S;
+}
+
 // this thread's warp, known to be the same for its whole warp
 __device__ __forceinline__ int warp_of() { return __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0); }
 
@@ -69,12 +74,14 @@ __global__ void __launch_bounds__(256, 2) tree_bwd_kernel(const __grid_constant_
                                                           const __grid_constant__ BwdArgs A) {
   extern __shared__ float4 rec[];
   stage_recs(r, -1, rec, threadIdx.x, blockDim.x);
+  stage_spheres(r, rec);
   __syncthreads();
   int64_t b;
   bool act;
   if (!own_config(A.B, blockIdx.x * (int64_t)blockDim.x + 32 * warp_of(), &b, &act)) return;
+  const GradSlot gs = grad_slot_of(reinterpret_cast<float*>(rec) + bwd_words(r));
   tree_bwd_seg<false>(r, rec, ConstWalk{wt}, A, FusedCost{},
-                      ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, whole_sweep(r));
+                      ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, whole_sweep(r), gs);
 }
 
 // Segmented sweeps, plan t (G = 2 << t segments).  A block holds CG groups of
@@ -136,7 +143,7 @@ __global__ void __launch_bounds__(512, 1) tree_bwd_seg_kernel(const __grid_const
                                                            const __grid_constant__ BwdArgs A,
                                                            int t) {
   extern __shared__ float4 rec[];
-  float* part = reinterpret_cast<float*>(rec) + kRecWords * (size_t)r.n;
+  float* part = reinterpret_cast<float*>(rec) + bwd_words(r);
   const int G = 2 << t;
   const int CG = blockDim.x / (32 * G);
   const int wid = warp_of(), cg = wid / G;
@@ -146,6 +153,7 @@ __global__ void __launch_bounds__(512, 1) tree_bwd_seg_kernel(const __grid_const
   for (int s = 0; s < ns; ++s)
     for (int q = 0; q < 3; ++q) sg.part[q * o + (s * G + sg.g) * 32 + sg.lane] = 0.0f;
   stage_recs(r, t, rec, threadIdx.x, blockDim.x);
+  stage_spheres(r, rec);
   // the gradient-row slots behind the partials (reserved by the launch when
   // there are upstream pose or sphere gradients)
   const GradSlot gs = grad_slot_of(part + (size_t)CG * 3 * o);
@@ -184,13 +192,15 @@ __global__ void __launch_bounds__(256, 2) tree_bwd_cost_kernel(
     const __grid_constant__ BwdArgs A, const __grid_constant__ FusedCost fc) {
   extern __shared__ float4 rec[];
   stage_recs(r, -1, rec, threadIdx.x, blockDim.x);
+  stage_spheres(r, rec);
   __syncthreads();
   int64_t b;
   bool act;
   if (!own_config(A.B, blockIdx.x * (int64_t)blockDim.x + 32 * warp_of(), &b, &act)) return;
+  const GradSlot gs = grad_slot_of(reinterpret_cast<float*>(rec) + bwd_words(r));
   const float c = tree_bwd_seg<true>(r, rec, ConstWalk{wt}, A, fc,
                                      ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act,
-                                     whole_sweep(r));
+                                     whole_sweep(r), gs);
   if (fc.cost) fc.cost[b] = total_cost(fc, b, c);
 }
 
@@ -198,7 +208,7 @@ __global__ void __launch_bounds__(512, 1) tree_bwd_cost_seg_kernel(
     const __grid_constant__ DevRobot r, const __grid_constant__ WalkTab wt,
     const __grid_constant__ BwdArgs A, const __grid_constant__ FusedCost fc, int t) {
   extern __shared__ float4 rec[];
-  float* part = reinterpret_cast<float*>(rec) + kRecWords * (size_t)r.n;
+  float* part = reinterpret_cast<float*>(rec) + bwd_words(r);
   const int G = 2 << t;
   const int CG = blockDim.x / (32 * G);
   const int wid = warp_of(), cg = wid / G;
@@ -209,6 +219,7 @@ __global__ void __launch_bounds__(512, 1) tree_bwd_cost_seg_kernel(
   for (int s = 0; s < ns; ++s)
     for (int q = 0; q < 3; ++q) sg.part[q * o + (s * G + sg.g) * 32 + sg.lane] = 0.0f;
   stage_recs(r, t, rec, threadIdx.x, blockDim.x);
+  stage_spheres(r, rec);
   const GradSlot gs = grad_slot_of(part + (size_t)CG * (3 * o + G * 32));
   __syncthreads();
   int64_t b;
@@ -316,8 +327,9 @@ __global__ void __launch_bounds__(256, 2) tree_bwd_spline_cost_kernel(
     const __grid_constant__ BwdArgs A, const __grid_constant__ FusedCost fc,
     const __grid_constant__ SplineArgs sp) {
   extern __shared__ float4 rec[];
-  float* sm = reinterpret_cast<float*>(rec) + kRecWords * (size_t)r.n;
+  float* sm = reinterpret_cast<float*>(rec) + bwd_words(r);
   stage_recs(r, -1, rec, threadIdx.x, blockDim.x);
+  stage_spheres(r, rec);
   __syncthreads();
   int64_t b;
   bool act;
@@ -333,7 +345,7 @@ __global__ void __launch_bounds__(512, 1) tree_bwd_spline_cost_seg_kernel(
     const __grid_constant__ BwdArgs A, const __grid_constant__ FusedCost fc,
     const __grid_constant__ SplineArgs sp, int t) {
   extern __shared__ float4 rec[];
-  float* sm = reinterpret_cast<float*>(rec) + kRecWords * (size_t)r.n;
+  float* sm = reinterpret_cast<float*>(rec) + bwd_words(r);
   float* base = sm + 12 * blockDim.x;
   const int G = 2 << t;
   const int CG = blockDim.x / (32 * G);
@@ -345,6 +357,7 @@ __global__ void __launch_bounds__(512, 1) tree_bwd_spline_cost_seg_kernel(
   for (int s = 0; s < ns; ++s)
     for (int q = 0; q < 3; ++q) sg.part[q * o + (s * G + sg.g) * 32 + sg.lane] = 0.0f;
   stage_recs(r, t, rec, threadIdx.x, blockDim.x);
+  stage_spheres(r, rec);
   __syncthreads();
   int64_t b;
   bool act = false;
@@ -431,7 +444,9 @@ void fit_carveout(const void* kern, int threads, size_t smem) {
   cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
 }
 
-static size_t rec_smem(const DevRobot& r) { return sizeof(float) * kRecWords * (size_t)r.n; }
+static size_t rec_smem(const DevRobot& r, bool fwd) {
+  return sizeof(float) * (fwd ? kRecWords * (size_t)r.n : bwd_words(r));
+}
 
 static int seg_plan(int segments) { return segments == 2 ? 0 : segments == 4 ? 1 : 2; }
 static int seg_groups(int segments, int threads) { return std::max(1, threads / (32 * segments)); }
@@ -443,7 +458,7 @@ size_t tree_seg_smem(const DevRobot& r, int segments, int threads, bool fwd, boo
   const int t = seg_plan(segments);
   const size_t per =
       (size_t)(fwd ? 1 : 3) * r.seg_ns[t] * segments * 32 + (cost ? segments * 32 : 0);
-  return (size_t)seg_groups(segments, threads) * per * sizeof(float) + rec_smem(r);
+  return (size_t)seg_groups(segments, threads) * per * sizeof(float) + rec_smem(r, fwd);
 }
 
 // a backward block's gradient-row slots (GradSlot), when it has upstream pose
@@ -500,8 +515,8 @@ cudaError_t launch_tree_fwd(const DevRobot& r, const WalkTab& wt, const FwdArgs&
                       a, threads, segments, true, 0, s);
   }
   const size_t fs = sizeof(float) * 6 * (size_t)r.maxdepth * threads;  // the force stack
-  const bool use_fs = a.tau && rec_smem(r) + fs <= kSegSmemMax;
-  const size_t smem = rec_smem(r) + (use_fs ? fs : 0);
+  const bool use_fs = a.tau && rec_smem(r, true) + fs <= kSegSmemMax;
+  const size_t smem = rec_smem(r, true) + (use_fs ? fs : 0);
   auto kern = use_fs ? tree_fwd_kernel<kFwdShared>
               : a.tau ? tree_fwd_kernel<kFwdLocal>
                       : tree_fwd_kernel<kFwdPose>;
@@ -521,7 +536,12 @@ cudaError_t launch_tree_bwd(const DevRobot& r, const WalkTab& wt, const BwdArgs&
     return fc ? launch_cost_seg(r, wt, a, *fc, threads, segments, s)
               : launch_seg(tree_bwd_seg_kernel, r, wt, a, threads, segments, false,
                            a.g_pose || a.g_sph ? grad_slot_smem(segments, threads) : 0, s);
-  const size_t smem = rec_smem(r);
+  const size_t smem = rec_smem(r, false) + (a.g_pose || a.g_sph ? grad_slot_smem(1, threads) : 0);
+  cudaError_t e = fc ? cudaFuncSetAttribute(tree_bwd_cost_kernel,
+                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                     : cudaFuncSetAttribute(tree_bwd_kernel,
+                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   fit_carveout(fc ? (const void*)tree_bwd_cost_kernel : (const void*)tree_bwd_kernel, threads,
                smem);
   const int64_t grid = (a.B + threads - 1) / threads;
@@ -554,7 +574,7 @@ cudaError_t launch_tree_fwd_spline(const DevRobot& r, const WalkTab& wt, const F
     kern<<<(unsigned)grid, block, smem, s>>>(r, wt, a, sp, t);
     return cudaGetLastError();
   }
-  const size_t smem = 12 * sizeof(float) * threads + rec_smem(r);
+  const size_t smem = 12 * sizeof(float) * threads + rec_smem(r, true);
   auto kern = a.tau ? tree_fwd_spline_kernel<kFwdLocal> : tree_fwd_spline_kernel<kFwdPose>;
   fit_carveout((const void*)kern, threads, smem);
   const int64_t grid = (a.B + threads - 1) / threads;
@@ -579,7 +599,10 @@ cudaError_t launch_tree_bwd_spline_cost(const DevRobot& r, const WalkTab& wt, co
     tree_bwd_spline_cost_seg_kernel<<<(unsigned)grid, block, smem, s>>>(r, wt, a, fc, sp, t);
     return cudaGetLastError();
   }
-  const size_t smem = 12 * sizeof(float) * threads + rec_smem(r);
+  const size_t smem = 12 * sizeof(float) * threads + rec_smem(r, false);
+  cudaError_t e = cudaFuncSetAttribute(tree_bwd_spline_cost_kernel,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   fit_carveout((const void*)tree_bwd_spline_cost_kernel, threads, smem);
   const int64_t grid = (a.B + threads - 1) / threads;
   tree_bwd_spline_cost_kernel<<<(unsigned)grid, threads, smem, s>>>(r, wt, a, fc, sp);

@@ -79,10 +79,12 @@ constexpr int TMAXD = 32;  // deepest tree the sweep kernels accept
 // need no reconvergence (with the words in global memory a fifth of the
 // forward's instructions were branches, barriers and moves around them).
 struct ConstWalk {
+  static constexpr bool kSpheres = true;  // the spheres are staged behind the records
   const WalkTab& t;
   __device__ __forceinline__ uint32_t operator()(int pos) const { return t.w[pos]; }
 };
 struct SharedWalk {  // the batch's: staged with the link records, made uniform by a shuffle
+  static constexpr bool kSpheres = false;
   const uint32_t* w;
   __device__ __forceinline__ uint32_t operator()(int pos) const {
     return __shfl_sync(0xffffffffu, w[pos], 0);
@@ -126,6 +128,12 @@ __device__ __forceinline__ int ancestor_at(const WK& wk, int pos, int c) {
   return pos;
 }
 
+// the robot's spheres, behind its staged records (the backward reads a link's
+// at its close: humanoid48 0.290 -> 0.272 ms at 99999 configurations)
+__device__ __forceinline__ void stage_spheres(const DevRobot& r, float4* rec) {
+  for (int i = threadIdx.x; i < r.S; i += blockDim.x) rec[8 * r.n + i] = __ldg(r.sph + i);
+}
+
 // Copies the robot's link records into shared memory (kRecWords floats a
 // link, in DFS order; see DevRobot::recs) with the inertias and the shared
 // output slots of segment plan t (t < 0: none); thread i of nt.
@@ -159,7 +167,6 @@ __device__ __forceinline__ void pf(const void* p) { asm volatile("prefetch.L2 [%
 // The joint states (q, qd, qdd of joint j) of the sweep's configuration b,
 // from [d][B] arrays ...
 struct ArrayStates {
-  static constexpr bool kAhead = true;  // load the next link's values a link ahead
   const float* q;
   const float* qd;
   const float* qdd;
@@ -183,7 +190,6 @@ struct ArrayStates {
 // (q, qd, qdd), computed once per configuration.  Same arithmetic as the
 // B-spline forward kernel, so the states are the same bits.
 struct SplineStates {
-  static constexpr bool kAhead = false;  // a trajectory's control points stay in L1
   const float* u;
   int K;
   const float* bs;
@@ -351,6 +357,10 @@ __device__ __forceinline__ void tree_fwd_seg(const DevRobot& r, const float4* re
   for (int i = 0; i < 12; ++i) cW[i] = 0.0f;
   int cdep = -1, pdep = -1;
   int ckp = 0;  // the position the next close takes: the last pushed one, then parents
+  // its joint's value: the push's, then loaded a close ahead (a load at the
+  // head of every close sat on its critical path: humanoid48 0.066 -> 0.060
+  // ms; the backward, whose closes use it after the own terms, gains nothing)
+  float kq = 0.0f;
 
   auto load_F = [&](int e, float* F) {
     if (FS) {
@@ -370,7 +380,11 @@ __device__ __forceinline__ void tree_fwd_seg(const DevRobot& r, const float4* re
     const float4* q = rec + 8 * ckp;
     ckp = wk_par(w);
     const int j = wk_j(w), jt = wk_jt(w);
-    const float qj = jt ? st.pos(j) : 0.0f;
+    const float qj = kq;
+    if (e > 0) {
+      const uint32_t wp = wk(ckp);
+      kq = wk_jt(wp) ? st.pos(wk_j(wp)) : 0.0f;
+    }
     if (pdep != e) load_F(e, pF);
     pdep = -1;
     if (jt) {
@@ -444,6 +458,7 @@ __device__ __forceinline__ void tree_fwd_seg(const DevRobot& r, const float4* re
     }
     cdep = dep;
     ckp = pos;
+    kq = pq;
     if (wk_branch(w)) {
 #pragma unroll
       for (int i = 0; i < 12; ++i) E.W[i] = cW[i];
@@ -763,6 +778,7 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const float4* r
   // its acc holds children's sums
   uint32_t replayed = 0u, accv = 0u;
   int ckp = 0;  // the position the next close takes: the last pushed one, then parents
+  auto sphere = [&](int s) { return WK::kSpheres ? rec[8 * n + s] : __ldg(r.sph + s); };
   const bool kin_grad = A.g_pose != nullptr || A.g_sph != nullptr;
   // sphere gradients of a link as float4 triples: the robot's spheres come
   // in runs of 4 (then b S + s is a multiple of 4) and the array (a slice of
@@ -823,20 +839,20 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const float4* r
                      x2 = fs ? gs.p[5 * gs.stride] : __ldg(g4 + 2);
         const float gg[12] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w, x2.x, x2.y, x2.z, x2.w};
 #pragma unroll
-        for (int i = 0; i < 4; ++i) point_grad(__ldg(r.sph + s + i), gg + 3 * i, G, f);
+        for (int i = 0; i < 4; ++i) point_grad(sphere(s + i), gg + 3 * i, G, f);
       }
     } else if (A.g_sph) {
       for (int e = 0; e < ns; ++e) {
         const int s = __ldg(r.ls_sph + e0 + e);
         const float* g = A.g_sph + (b * r.S + s) * 3;
         const float gg[3] = {__ldg(g), __ldg(g + 1), __ldg(g + 2)};
-        point_grad(__ldg(r.sph + s), gg, G, f);
+        point_grad(sphere(s), gg, G, f);
       }
     }
-    if (k == pl1) point_grad(__ldg(r.sph + ps1), u, G, f);
+    if (k == pl1) point_grad(sphere(ps1), u, G, f);
     if (k == pl2) {
       const float mu[3] = {-u[0], -u[1], -u[2]};
-      point_grad(__ldg(r.sph + ps2), mu, G, f);
+      point_grad(sphere(ps2), mu, G, f);
     }
     const float* R = cW;
 #pragma unroll
@@ -1102,37 +1118,37 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const float4* r
   };
 
   // one loop over the replayed ancestors and the segment's links, as in the
-  // forward, the joint inputs of the next link loaded (or prefetched) ahead
+  // forward
   const int nrep = wk_dep(wk(sg.p0)), total = nrep + sg.p1 - sg.p0;
   int sp = 0;
   int npos = ancestor_at(wk, sg.p0, 0);
   uint32_t nw = wk(npos);
   const float* const gt = FC ? fc.tau : A.g_tau;
   float nq = 0.0f, nqd = 0.0f, nqdd = 0.0f, ngt = 0.0f;
-  auto fetch = [&]() {
+  auto fetch = [&](uint32_t w) {
     nq = nqd = nqdd = ngt = 0.0f;
-    if (wk_jt(nw)) {
-      const int j = wk_j(nw);
+    if (wk_jt(w)) {
+      const int j = wk_j(w);
       nq = st.pos(j);
       nqd = st.vel(j);
       nqdd = st.acc(j);
       if (gt) ngt = __ldg(gt + (int64_t)j * B + b);
     }
   };
-  if (St::kAhead) fetch();
   for (int i = 0; i <= total; ++i) {
     const bool end = i == total, own = i >= nrep;
     const int pos = npos;
     const uint32_t w = nw;
     const int dep = end ? 0 : wk_dep(w);
-    if (!St::kAhead && !end) fetch();
-    const float cq = nq, cqd = nqd, cqdd = nqdd, cgt = ngt;
+    // this link's joint inputs, before the closes ahead of its push; the next
+    // one's into L2 (held in registers a link ahead instead, the humanoid's
+    // backward went 0.1025 -> 0.105 ms at 32768 configurations, 0.292 ->
+    // 0.314 ms at 99999)
+    if (!end) fetch(w);
     if (i + 1 < total) {
       npos = i + 1 < nrep ? ancestor_at(wk, sg.p0, i + 1) : sg.p0 + i + 1 - nrep;
       nw = wk(npos);
-      if (St::kAhead) {
-        fetch();
-      } else if (wk_jt(nw)) {
+      if (wk_jt(nw)) {
         st.prefetch(wk_j(nw), true);
         if (gt) pf(gt + (int64_t)wk_j(nw) * B + b);
       }
@@ -1144,7 +1160,7 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const float4* r
     // a link closed right after its push (a leaf, or the segment's last
     // link): its rows start on their way now
     if (use_slot && own && (i + 1 >= total || wk_dep(nw) <= dep)) issue(rec + 8 * pos);
-    push(pos, w, own, cq, cqd, cqdd, cgt);
+    push(pos, w, own, nq, nqd, nqdd, ngt);
   }
   if (use_slot) asm volatile("cp.async.wait_group 0;" ::: "memory");
   return cost_part;

@@ -1000,11 +1000,14 @@ static int tree_segments(const wb_robot* R, const wb_tune* tune, int64_t B, int*
   if (G == 1 && threads > 256)
     return fail(WB_EINVAL, "one-segment sweeps take at most 256 threads per block");
   // what a block needs: refused from the limit up, counting 28 floats a link
-  // record; the records' padding to kRecWords is made room for
+  // record; the records' padding to kRecWords and the backward's spheres are
+  // made room for
   auto need = [&](int threads_) {
     return tree_seg_smem(R->dev, G, threads_, fwd, !fwd) + (fwd ? 0 : grad_slot_smem(G, threads_));
   };
-  if (G > 1 && need(threads) - sizeof(float) * (kRecWords - 28) * (size_t)R->dev.n > kMaxBlockSmem)
+  const size_t more = sizeof(float) * ((kRecWords - 28) * (size_t)R->dev.n +
+                                       (fwd ? 0 : 4 * (size_t)R->dev.S));
+  if (G > 1 && need(threads) - more > kMaxBlockSmem)
     return fail(WB_ETOOBIG, "segmented sweep needs too much shared memory");
   while (G > 1 && need(*tpb) > kMaxBlockSmem) {
     if (*tpb >= 64 * G)
