@@ -134,7 +134,8 @@ __global__ void __launch_bounds__(256) batch_tree_fwd_kernel(const DevRobot* rob
   }
 }
 
-// capped at 128 registers, as the single-robot backward sweeps
+// capped at 128 registers, as the single-robot backward sweeps (OPT as there)
+template <int OPT>
 __global__ void __launch_bounds__(256, 2) batch_tree_bwd_kernel(const DevRobot* robots,
                                                              const BatchProblemDev* probs,
                                                              const int4* items, int n_items,
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(256, 2) batch_tree_bwd_kernel(const DevRobot* 
     for (int q = 0; q < ns; ++q)
       for (int k = 0; k < 3; ++k) part[k * o + (q * 2 + g) * 32 + lane] = 0.0f;
     if (some)
-      tree_bwd_seg<false>(r, rec, SharedWalk{wk}, A, FusedCost{},
+      tree_bwd_seg<OPT>(r, rec, SharedWalk{wk}, A, FusedCost{},
                           ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg, gs);
     pair_bar(bar);
     if (lane < w.z)
@@ -268,18 +269,22 @@ cudaError_t launch_batch_tree_fwd(const DevRobot* robots, const BatchProblemDev*
   return cudaGetLastError();
 }
 
+// rows: every robot of the batch allows kBwdRows (its packed sphere slices are
+// then multiples of 12 floats, so all of them are aligned if the array is)
 cudaError_t launch_batch_tree_bwd(const DevRobot* robots, const BatchProblemDev* probs, const int4* items,
                                   int n_items, int* counter, const BatchIO& io, int grid,
-                                  int ns_max, int n_max, int threads, cudaStream_t s) {
+                                  int ns_max, int n_max, int threads, bool rows, cudaStream_t s) {
   const size_t smem = batch_tree_smem(false, ns_max, n_max, threads);
-  cudaError_t e = cudaFuncSetAttribute(batch_tree_bwd_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto kern = rows && io.g_pose && io.g_sph && (reinterpret_cast<uintptr_t>(io.g_sph) & 15u) == 0
+                  ? batch_tree_bwd_kernel<kBwdRows>
+                  : batch_tree_bwd_kernel<kBwdGeneral>;
+  cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  fit_carveout((const void*)batch_tree_bwd_kernel, threads, smem);
+  fit_carveout((const void*)kern, threads, smem);
   e = cudaMemsetAsync(counter, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
-  batch_tree_bwd_kernel<<<grid, threads, smem, s>>>(robots, probs, items, n_items, counter, io,
-                                                    ns_max, n_max);
+  kern<<<grid, threads, smem, s>>>(robots, probs, items, n_items, counter, io, ns_max, n_max);
   return cudaGetLastError();
 }
 
@@ -318,13 +323,11 @@ cudaError_t batch_tree_max_blocks_per_sm(bool fwd, int ns_max, int n_max, int th
     *out = 0;
     return cudaSuccess;
   }
-  cudaError_t e = cudaFuncSetAttribute(fwd ? batch_tree_fwd_kernel : batch_tree_bwd_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto kern = fwd ? batch_tree_fwd_kernel : batch_tree_bwd_kernel<kBwdGeneral>;
+  cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return fwd ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, batch_tree_fwd_kernel, threads,
-                                                             smem)
-             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, batch_tree_bwd_kernel, threads,
-                                                             smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kern, threads, smem);
 }
 
 int pair_plan_words(const DevRobot& r) { return PairPlan(r.n, r.Sg, r.P, false).total; }

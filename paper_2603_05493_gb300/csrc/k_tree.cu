@@ -69,6 +69,7 @@ __global__ void __launch_bounds__(256) tree_fwd_kernel(const __grid_constant__ D
 // 0.36 ms uncapped at 2 segments).  The segmented sweeps take blocks of up to
 // 512 threads, so that one block per SM holds the staged link parameters once
 // and the shared-memory carveout stays small.
+template <int OPT>
 __global__ void __launch_bounds__(256, 2) tree_bwd_kernel(const __grid_constant__ DevRobot r,
                                                           const __grid_constant__ WalkTab wt,
                                                           const __grid_constant__ BwdArgs A) {
@@ -80,7 +81,7 @@ __global__ void __launch_bounds__(256, 2) tree_bwd_kernel(const __grid_constant_
   bool act;
   if (!own_config(A.B, blockIdx.x * (int64_t)blockDim.x + 32 * warp_of(), &b, &act)) return;
   const GradSlot gs = grad_slot_of(reinterpret_cast<float*>(rec) + bwd_words(r));
-  tree_bwd_seg<false>(r, rec, ConstWalk{wt}, A, FusedCost{},
+  tree_bwd_seg<OPT>(r, rec, ConstWalk{wt}, A, FusedCost{},
                       ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, whole_sweep(r), gs);
 }
 
@@ -138,6 +139,7 @@ __global__ void __launch_bounds__(512) tree_fwd_seg_kernel(const __grid_constant
   }
 }
 
+template <int OPT>
 __global__ void __launch_bounds__(512, 1) tree_bwd_seg_kernel(const __grid_constant__ DevRobot r,
                                                            const __grid_constant__ WalkTab wt,
                                                            const __grid_constant__ BwdArgs A,
@@ -161,7 +163,7 @@ __global__ void __launch_bounds__(512, 1) tree_bwd_seg_kernel(const __grid_const
   int64_t b;
   bool act = false;
   if (own_config(A.B, ((int64_t)blockIdx.x * CG + cg) * 32, &b, &act))
-    tree_bwd_seg<false>(r, rec, ConstWalk{wt}, A, FusedCost{},
+    tree_bwd_seg<OPT>(r, rec, ConstWalk{wt}, A, FusedCost{},
                         ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg, gs);
   __syncthreads();
   if (act) {
@@ -187,6 +189,7 @@ __device__ __forceinline__ float total_cost(const FusedCost& fc, int64_t b, floa
 // separate kernels, so that the plain ones keep their register allocation.
 // The segmented one adds each configuration's cost terms over the segments
 // in segment order (deterministic) after the barrier.
+template <int OPT>
 __global__ void __launch_bounds__(256, 2) tree_bwd_cost_kernel(
     const __grid_constant__ DevRobot r, const __grid_constant__ WalkTab wt,
     const __grid_constant__ BwdArgs A, const __grid_constant__ FusedCost fc) {
@@ -198,12 +201,13 @@ __global__ void __launch_bounds__(256, 2) tree_bwd_cost_kernel(
   bool act;
   if (!own_config(A.B, blockIdx.x * (int64_t)blockDim.x + 32 * warp_of(), &b, &act)) return;
   const GradSlot gs = grad_slot_of(reinterpret_cast<float*>(rec) + bwd_words(r));
-  const float c = tree_bwd_seg<true>(r, rec, ConstWalk{wt}, A, fc,
+  const float c = tree_bwd_seg<kBwdCost | OPT>(r, rec, ConstWalk{wt}, A, fc,
                                      ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act,
                                      whole_sweep(r), gs);
   if (fc.cost) fc.cost[b] = total_cost(fc, b, c);
 }
 
+template <int OPT>
 __global__ void __launch_bounds__(512, 1) tree_bwd_cost_seg_kernel(
     const __grid_constant__ DevRobot r, const __grid_constant__ WalkTab wt,
     const __grid_constant__ BwdArgs A, const __grid_constant__ FusedCost fc, int t) {
@@ -226,7 +230,7 @@ __global__ void __launch_bounds__(512, 1) tree_bwd_cost_seg_kernel(
   bool act = false;
   float c = 0.0f;
   if (own_config(A.B, ((int64_t)blockIdx.x * CG + cg) * 32, &b, &act))
-    c = tree_bwd_seg<true>(r, rec, ConstWalk{wt}, A, fc,
+    c = tree_bwd_seg<kBwdCost | OPT>(r, rec, ConstWalk{wt}, A, fc,
                            ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg, gs);
   cpart[sg.g * 32 + sg.lane] = c;
   __syncthreads();
@@ -322,6 +326,7 @@ __global__ void __launch_bounds__(512) tree_fwd_spline_seg_kernel(
   }
 }
 
+template <int OPT>
 __global__ void __launch_bounds__(256, 2) tree_bwd_spline_cost_kernel(
     const __grid_constant__ DevRobot r, const __grid_constant__ WalkTab wt,
     const __grid_constant__ BwdArgs A, const __grid_constant__ FusedCost fc,
@@ -334,12 +339,14 @@ __global__ void __launch_bounds__(256, 2) tree_bwd_spline_cost_kernel(
   int64_t b;
   bool act;
   if (!own_config(A.B, blockIdx.x * (int64_t)blockDim.x + 32 * warp_of(), &b, &act)) return;
-  const float c = tree_bwd_seg<true>(r, rec, ConstWalk{wt}, A, fc,
-                                     spline_states(r, sp, b, sm + 12 * threadIdx.x), b, act,
-                                     whole_sweep(r));
+  const GradSlot gs = grad_slot_of(sm + 12 * blockDim.x);
+  const float c = tree_bwd_seg<kBwdCost | OPT>(r, rec, ConstWalk{wt}, A, fc,
+                                               spline_states(r, sp, b, sm + 12 * threadIdx.x), b,
+                                               act, whole_sweep(r), gs);
   if (fc.cost) fc.cost[b] = total_cost(fc, b, c);
 }
 
+template <int OPT>
 __global__ void __launch_bounds__(512, 1) tree_bwd_spline_cost_seg_kernel(
     const __grid_constant__ DevRobot r, const __grid_constant__ WalkTab wt,
     const __grid_constant__ BwdArgs A, const __grid_constant__ FusedCost fc,
@@ -358,13 +365,14 @@ __global__ void __launch_bounds__(512, 1) tree_bwd_spline_cost_seg_kernel(
     for (int q = 0; q < 3; ++q) sg.part[q * o + (s * G + sg.g) * 32 + sg.lane] = 0.0f;
   stage_recs(r, t, rec, threadIdx.x, blockDim.x);
   stage_spheres(r, rec);
+  const GradSlot gs = grad_slot_of(base + (size_t)CG * (3 * o + G * 32));
   __syncthreads();
   int64_t b;
   bool act = false;
   float c = 0.0f;
   if (own_config(A.B, ((int64_t)blockIdx.x * CG + cg) * 32, &b, &act))
-    c = tree_bwd_seg<true>(r, rec, ConstWalk{wt}, A, fc,
-                           spline_states(r, sp, b, sm + 12 * threadIdx.x), b, act, sg);
+    c = tree_bwd_seg<kBwdCost | OPT>(r, rec, ConstWalk{wt}, A, fc,
+                           spline_states(r, sp, b, sm + 12 * threadIdx.x), b, act, sg, gs);
   cpart[sg.g * 32 + sg.lane] = c;
   __syncthreads();
   if (act && sg.g == 0 && fc.cost) {
@@ -484,19 +492,17 @@ static cudaError_t launch_seg(void (*kern)(DevRobot, WalkTab, Args, int), const 
   return cudaGetLastError();
 }
 
-static cudaError_t launch_cost_seg(const DevRobot& r, const WalkTab& wt, const BwdArgs& a,
-                                   const FusedCost& fc, int threads, int segments, cudaStream_t s) {
-  const int t = seg_plan(segments);
-  const int CG = seg_groups(segments, threads);
-  const size_t smem = tree_seg_smem(r, segments, threads, false, true) +
-                      (a.g_pose || a.g_sph ? grad_slot_smem(segments, threads) : 0);
-  cudaError_t e = cudaFuncSetAttribute(tree_bwd_cost_seg_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+// A backward launch's kernel, its dynamic shared memory and its carveout; the
+// arguments then follow in launch order.
+template <class... P, class... V>
+static cudaError_t launch_bwd(void (*kern)(P...), int64_t B, int groups, int block, size_t smem,
+                              cudaStream_t s, const V&... v) {
+  cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  fit_carveout((const void*)tree_bwd_cost_seg_kernel, 32 * segments * CG, smem);
-  const int64_t groups = (a.B + 31) / 32;
-  const int64_t grid = (groups + CG - 1) / CG;
-  tree_bwd_cost_seg_kernel<<<(unsigned)grid, 32 * segments * CG, smem, s>>>(r, wt, a, fc, t);
+  fit_carveout((const void*)kern, block, smem);
+  const int64_t grid = ((B + 31) / 32 + groups - 1) / groups;
+  kern<<<(unsigned)grid, block, smem, s>>>(v...);
   return cudaGetLastError();
 }
 
@@ -529,27 +535,33 @@ cudaError_t launch_tree_fwd(const DevRobot& r, const WalkTab& wt, const FwdArgs&
   return cudaGetLastError();
 }
 
-cudaError_t launch_tree_bwd(const DevRobot& r, const WalkTab& wt, const BwdArgs& a, int threads, int segments,
-                            cudaStream_t s, const FusedCost* fc) {
+cudaError_t launch_tree_bwd(const DevRobot& r, const WalkTab& wt, const BwdArgs& a, int threads,
+                            int segments, cudaStream_t s, const FusedCost* fc) {
   if (threads <= 0) threads = 128;
-  if (segments > 1)
-    return fc ? launch_cost_seg(r, wt, a, *fc, threads, segments, s)
-              : launch_seg(tree_bwd_seg_kernel, r, wt, a, threads, segments, false,
-                           a.g_pose || a.g_sph ? grad_slot_smem(segments, threads) : 0, s);
-  const size_t smem = rec_smem(r, false) + (a.g_pose || a.g_sph ? grad_slot_smem(1, threads) : 0);
-  cudaError_t e = fc ? cudaFuncSetAttribute(tree_bwd_cost_kernel,
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                     : cudaFuncSetAttribute(tree_bwd_kernel,
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  fit_carveout(fc ? (const void*)tree_bwd_cost_kernel : (const void*)tree_bwd_kernel, threads,
-               smem);
-  const int64_t grid = (a.B + threads - 1) / threads;
-  if (fc)
-    tree_bwd_cost_kernel<<<(unsigned)grid, threads, smem, s>>>(r, wt, a, *fc);
-  else
-    tree_bwd_kernel<<<(unsigned)grid, threads, smem, s>>>(r, wt, a);
-  return cudaGetLastError();
+  const int opt = bwd_opt(r, a, fc == nullptr);
+  const int CG = segments > 1 ? seg_groups(segments, threads) : threads / 32;
+  const int block = 32 * segments * CG;
+  const size_t smem = (segments > 1 ? tree_seg_smem(r, segments, threads, false, fc != nullptr)
+                                    : rec_smem(r, false)) +
+                      (a.g_pose || a.g_sph ? grad_slot_smem(segments, threads) : 0);
+  if (segments > 1) {
+    const int t = seg_plan(segments);
+    if (!fc)
+      return launch_bwd(opt == kBwdRows ? tree_bwd_seg_kernel<kBwdRows>
+                                        : tree_bwd_seg_kernel<kBwdGeneral>,
+                        a.B, CG, block, smem, s, r, wt, a, t);
+    return launch_bwd(opt == 0            ? tree_bwd_cost_seg_kernel<0>
+                      : opt == kBwdSphere ? tree_bwd_cost_seg_kernel<kBwdSphere>
+                                          : tree_bwd_cost_seg_kernel<kBwdGeneral>,
+                      a.B, CG, block, smem, s, r, wt, a, *fc, t);
+  }
+  if (!fc)
+    return launch_bwd(opt == kBwdRows ? tree_bwd_kernel<kBwdRows> : tree_bwd_kernel<kBwdGeneral>,
+                      a.B, CG, block, smem, s, r, wt, a);
+  return launch_bwd(opt == 0            ? tree_bwd_cost_kernel<0>
+                    : opt == kBwdSphere ? tree_bwd_cost_kernel<kBwdSphere>
+                                        : tree_bwd_cost_kernel<kBwdGeneral>,
+                    a.B, CG, block, smem, s, r, wt, a, *fc);
 }
 
 cudaError_t launch_tree_fwd_spline(const DevRobot& r, const WalkTab& wt, const FwdArgs& a, const SplineArgs& sp,
@@ -582,31 +594,26 @@ cudaError_t launch_tree_fwd_spline(const DevRobot& r, const WalkTab& wt, const F
   return cudaGetLastError();
 }
 
-cudaError_t launch_tree_bwd_spline_cost(const DevRobot& r, const WalkTab& wt, const BwdArgs& a, const FusedCost& fc,
-                                        const SplineArgs& sp, int threads, int segments,
-                                        cudaStream_t s) {
+cudaError_t launch_tree_bwd_spline_cost(const DevRobot& r, const WalkTab& wt, const BwdArgs& a,
+                                        const FusedCost& fc, const SplineArgs& sp, int threads,
+                                        int segments, cudaStream_t s) {
   if (threads <= 0) threads = 128;
-  if (segments > 1) {
-    const int t = seg_plan(segments);
-    const int CG = seg_groups(segments, threads);
-    const int block = 32 * segments * CG;
-    const size_t smem = tree_seg_smem(r, segments, threads, false, true) + 12 * sizeof(float) * block;
-    cudaError_t e = cudaFuncSetAttribute(tree_bwd_spline_cost_seg_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    fit_carveout((const void*)tree_bwd_spline_cost_seg_kernel, block, smem);
-    const int64_t grid = ((a.B + 31) / 32 + CG - 1) / CG;
-    tree_bwd_spline_cost_seg_kernel<<<(unsigned)grid, block, smem, s>>>(r, wt, a, fc, sp, t);
-    return cudaGetLastError();
-  }
-  const size_t smem = 12 * sizeof(float) * threads + rec_smem(r, false);
-  cudaError_t e = cudaFuncSetAttribute(tree_bwd_spline_cost_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  fit_carveout((const void*)tree_bwd_spline_cost_kernel, threads, smem);
-  const int64_t grid = (a.B + threads - 1) / threads;
-  tree_bwd_spline_cost_kernel<<<(unsigned)grid, threads, smem, s>>>(r, wt, a, fc, sp);
-  return cudaGetLastError();
+  const int opt = bwd_opt(r, a, false);
+  const int CG = segments > 1 ? seg_groups(segments, threads) : threads / 32;
+  const int block = 32 * segments * CG;
+  const size_t smem = (segments > 1 ? tree_seg_smem(r, segments, threads, false, true)
+                                    : rec_smem(r, false)) +
+                      12 * sizeof(float) * block +
+                      (a.g_pose || a.g_sph ? grad_slot_smem(segments, threads) : 0);
+  if (segments > 1)
+    return launch_bwd(opt == 0            ? tree_bwd_spline_cost_seg_kernel<0>
+                      : opt == kBwdSphere ? tree_bwd_spline_cost_seg_kernel<kBwdSphere>
+                                          : tree_bwd_spline_cost_seg_kernel<kBwdGeneral>,
+                      a.B, CG, block, smem, s, r, wt, a, fc, sp, seg_plan(segments));
+  return launch_bwd(opt == 0            ? tree_bwd_spline_cost_kernel<0>
+                    : opt == kBwdSphere ? tree_bwd_spline_cost_kernel<kBwdSphere>
+                                        : tree_bwd_spline_cost_kernel<kBwdGeneral>,
+                    a.B, CG, block, smem, s, r, wt, a, fc, sp);
 }
 
 int tree_max_depth() { return TMAXD; }

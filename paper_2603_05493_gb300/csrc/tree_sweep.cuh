@@ -696,17 +696,48 @@ __device__ __forceinline__ void cp16(float4* dst, const void* src) {
 // FC: compiled with the fused cost (a separate instantiation, so that the
 // plain sweep keeps its register allocation).  gs: the thread's gradient-row
 // slot, or none (the rows are then read with plain loads at each close).
+// OPT: what the sweep is compiled for (BwdOpt), so that a call that needs none
+// of the rare options carries neither their branches nor their registers
+// (humanoid48, every upstream gradient, 448-thread blocks: 0.097 -> 0.092 ms at 32768
+// configurations, one thread a configuration 0.270 -> 0.260 ms at 99999).
+enum BwdOpt {
+  kBwdCost = 1,    // the fused cost (fc)
+  kBwdRare = 2,    // external wrenches, joints that drive several links
+  kBwdAny = 4,     // pose and sphere gradients as the arguments have them
+  kBwdPose = 8,    // pose gradients, through the slots
+  kBwdSphere = 16, // sphere gradients in runs of 4, through the slots
+};
+constexpr int kBwdGeneral = kBwdRare | kBwdAny;
+constexpr int kBwdRows = kBwdPose | kBwdSphere;
+// whether the sphere gradients g_sph of a robot can be read as float4 triples:
+// its spheres come in runs of 4 (then b S + s is a multiple of 4) and the
+// array is 16-byte aligned
+__host__ __device__ __forceinline__ bool sphere_runs(const DevRobot& r, const float* g_sph) {
+  return g_sph != nullptr && r.sph_vec4 && (reinterpret_cast<uintptr_t>(g_sph) & 15u) == 0;
+}
+// the fast instance that a call's arguments allow, else kBwdGeneral (wide:
+// whether there is one for pose and sphere gradients together, or one for
+// spheres alone)
+inline int bwd_opt(const DevRobot& r, const BwdArgs& A, bool wide) {
+  if (A.fext || A.g_fext || r.mimic_shared) return kBwdGeneral;
+  if (A.g_sph && !sphere_runs(r, A.g_sph)) return kBwdGeneral;
+  if (wide) return A.g_pose && A.g_sph ? kBwdRows : kBwdGeneral;
+  return A.g_pose ? kBwdGeneral : A.g_sph ? kBwdSphere : 0;
+}
+
 // act: as for tree_fwd_seg.
-template <bool FC, class WK, class St>
+template <int OPT, class WK, class St>
 __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const float4* rec, const WK& wk,
                                               const BwdArgs& A, const FusedCost& fc,
                                               const St& st, int64_t b, bool act, const Seg& sg,
                                               GradSlot gs = GradSlot{}) {
+  constexpr bool FC = (OPT & kBwdCost) != 0, RARE = (OPT & kBwdRare) != 0;
+  constexpr bool ANY = (OPT & kBwdAny) != 0;
   const int64_t B = A.B;
   float cost_part = 0.0f;
   const int n = r.n;
   BEnt stk[TMAXD];
-  if (r.mimic_shared && act)
+  if (RARE && r.mimic_shared && act)
     for (int j = 0; j < r.d; ++j) {
       A.gq[(int64_t)j * B + b] = 0.0f;
       A.gqd[(int64_t)j * B + b] = 0.0f;
@@ -779,17 +810,15 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const float4* r
   uint32_t replayed = 0u, accv = 0u;
   int ckp = 0;  // the position the next close takes: the last pushed one, then parents
   auto sphere = [&](int s) { return WK::kSpheres ? rec[8 * n + s] : __ldg(r.sph + s); };
-  const bool kin_grad = A.g_pose != nullptr || A.g_sph != nullptr;
-  // sphere gradients of a link as float4 triples: the robot's spheres come
-  // in runs of 4 (then b S + s is a multiple of 4) and the array (a slice of
-  // a packed batch, possibly) is 16-byte aligned
-  const bool sph4 = A.g_sph != nullptr && r.sph_vec4 &&
-                    (reinterpret_cast<uintptr_t>(A.g_sph) & 15u) == 0;
-  const bool use_slot = gs.p != nullptr && kin_grad;
+  const bool has_pose = ANY ? A.g_pose != nullptr : (OPT & kBwdPose) != 0;
+  const bool sph4 = ANY ? sphere_runs(r, A.g_sph) : (OPT & kBwdSphere) != 0;
+  const bool has_sph = ANY ? A.g_sph != nullptr : (OPT & kBwdSphere) != 0;
+  const bool kin_grad = has_pose || has_sph;
+  const bool use_slot = ANY ? gs.p != nullptr && kin_grad : kin_grad;
   auto issue = [&](const float4* q) {  // q: the link's record
     const float4 m = q[7];
     const int kn = __float_as_int(m.x);
-    if (A.g_pose) {
+    if (has_pose) {
       const float4* g4 = reinterpret_cast<const float4*>(A.g_pose + (b * n + (kn & 0xFF)) * 12);
       cp16(gs.p, g4);
       cp16(gs.p + gs.stride, g4 + 1);
@@ -820,7 +849,7 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const float4* r
     // next) or at its last child's close
     const bool slot = use_slot;
     if (slot) asm volatile("cp.async.wait_group 0;" ::: "memory");
-    if (A.g_pose) {
+    if (has_pose) {
       const float4* g4 = reinterpret_cast<const float4*>(A.g_pose + (b * n + k) * 12);
       const float4 x0 = slot ? gs.p[0] : __ldg(g4), x1 = slot ? gs.p[gs.stride] : __ldg(g4 + 1),
                    x2 = slot ? gs.p[2 * gs.stride] : __ldg(g4 + 2);
@@ -841,7 +870,7 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const float4* r
 #pragma unroll
         for (int i = 0; i < 4; ++i) point_grad(sphere(s + i), gg + 3 * i, G, f);
       }
-    } else if (A.g_sph) {
+    } else if (has_sph) {
       for (int e = 0; e < ns; ++e) {
         const int s = __ldg(r.ls_sph + e0 + e);
         const float* g = A.g_sph + (b * r.S + s) * 3;
@@ -891,7 +920,7 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const float4* r
       rec_inertia(q, I);
       link_adjoint(cW, I, cw, cal, cA, cwb, cub, ps);
       const int k = __float_as_int(q[7].x) & 0xFF;
-      if (A.fext) {
+      if (RARE && A.fext) {
         const float* fe = A.fext + (b * n + k) * 6;
         const float xn[3] = {__ldg(fe), __ldg(fe + 1), __ldg(fe + 2)};
         const float xf[3] = {__ldg(fe + 3), __ldg(fe + 4), __ldg(fe + 5)};
@@ -993,7 +1022,7 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const float4* r
         float* o0 = A.gq + (int64_t)j * B + b;
         float* o1 = A.gqd + (int64_t)j * B + b;
         float* o2 = A.gqdd + (int64_t)j * B + b;
-        if (!r.mimic_shared) {
+        if (!RARE || !r.mimic_shared) {
           *o0 = mm * gq;
           *o1 = mm * gqd;
           *o2 = mm * gqdd;
@@ -1107,7 +1136,7 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const float4* r
     accv &= ~bit;
     replayed = own ? (replayed & ~bit) : (replayed | bit);
     if (!wk_leaf(w)) stk[dep].tb = tb;
-    if (own && A.g_fext) {  // dL/df_ext,k = -(wb, ub) in link coordinates
+    if (RARE && own && A.g_fext) {  // dL/df_ext,k = -(wb, ub) in link coordinates
       float* o = A.g_fext + (b * n + (__float_as_int(q[7].x) & 0xFF)) * 6;
       float t[6];
       rotT(cW, cwb, t);

@@ -979,7 +979,7 @@ static int pair_warps(wb_robot* R, bool bits, const wb_tune* tune, bool cull = t
 // *tpb: the block's threads, lowered where the link records no longer leave
 // room for the partials of all its groups.
 static int tree_segments(const wb_robot* R, const wb_tune* tune, int64_t B, int* tpb,
-                         bool fwd, int* out) {
+                         bool fwd, int* out, bool spline = false) {
   const int threads = *tpb;
   const int req = tune ? tune->lanes_per_config : 0;
   const int ok = R->dev.seg_ok;
@@ -1000,13 +1000,16 @@ static int tree_segments(const wb_robot* R, const wb_tune* tune, int64_t B, int*
   if (G == 1 && threads > 256)
     return fail(WB_EINVAL, "one-segment sweeps take at most 256 threads per block");
   // what a block needs: refused from the limit up, counting 28 floats a link
-  // record; the records' padding to kRecWords and the backward's spheres are
-  // made room for
+  // record; the records' padding to kRecWords, the backward's spheres and the
+  // spline backward's basis rows beside its slots are made room for
+  const size_t basis = spline && !fwd ? 12 * sizeof(float) : 0;  // a thread's basis rows
   auto need = [&](int threads_) {
-    return tree_seg_smem(R->dev, G, threads_, fwd, !fwd) + (fwd ? 0 : grad_slot_smem(G, threads_));
+    return tree_seg_smem(R->dev, G, threads_, fwd, !fwd) +
+           (fwd ? 0 : grad_slot_smem(G, threads_)) + basis * std::max(threads_, 32 * G);
   };
   const size_t more = sizeof(float) * ((kRecWords - 28) * (size_t)R->dev.n +
-                                       (fwd ? 0 : 4 * (size_t)R->dev.S));
+                                       (fwd ? 0 : 4 * (size_t)R->dev.S)) +
+                      basis * std::max(threads, 32 * G);
   if (G > 1 && need(threads) - more > kMaxBlockSmem)
     return fail(WB_ETOOBIG, "segmented sweep needs too much shared memory");
   while (G > 1 && need(*tpb) > kMaxBlockSmem) {
@@ -1447,7 +1450,7 @@ int wb_eval_backward_spline_cost_dir(wb_robot* robot, const wb_spline* spline,
   if (tpb < 32 || tpb > 512 || tpb % 32)
     return fail(WB_EINVAL, "tree threads per block must be a multiple of 32 in [32, 512]");
   int G = 1;
-  if ((rc = tree_segments(robot, tune, B, &tpb, false, &G))) return rc;
+  if ((rc = tree_segments(robot, tune, B, &tpb, false, &G, true))) return rc;
   const cudaError_t e = launch_tree_bwd_spline_cost(robot->dev, robot->walk, a, fc, sp, tpb, G,
                                                     static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "wb_eval_backward_spline_cost launch");
@@ -1554,6 +1557,7 @@ struct wb_batch {
   int ws_words = 0, rad_words = 0;
   int ns_max = 0;  // most shared slots among the used robots' 2-segment sweep plans
   int n_max = 0;   // most links among them
+  bool rows = true;  // all take the backward's gradient-row instance (launch_batch_tree_bwd)
   wb_batch_sizes sizes{};
   // launch choices (wb_batch_set_tune / wb_batch_autotune): threads per block
   // of the forward and backward sweep passes, warps per block of the pair
@@ -1655,6 +1659,7 @@ int wb_batch_create(wb_robot* const* robots, int32_t n_robots, const wb_problem*
     Bt->rad_words = std::max(Bt->rad_words, (4 * D.Sg + 31) & ~31);
     Bt->ns_max = std::max(Bt->ns_max, seg2_slots(D));
     Bt->n_max = std::max(Bt->n_max, D.n);
+    Bt->rows = Bt->rows && D.sph_vec4 && !D.mimic_shared;
   }
   Bt->sizes = wb_batch_sizes{jo, po, so, co, n_problems, n_robots};
   // longest work first
@@ -1839,7 +1844,7 @@ int wb_batch_eval_backward(wb_batch* batch, const float* q, const float* qd, con
   if ((rc = batch_grid_tree(batch, false, &threads, &grid))) return rc;
   cudaError_t e = launch_batch_tree_bwd(batch->d_robots, batch->d_probs, batch->d_titems[1],
                                         batch->n_titems[1], const_cast<int*>(batch->d_counters) + 2,
-                                        io, grid, batch->ns_max, batch->n_max, threads,
+                                        io, grid, batch->ns_max, batch->n_max, threads, batch->rows,
                                         static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "wb_batch_eval_backward launch");
   return WB_OK;
@@ -2571,7 +2576,7 @@ extern "C" int wb_batch_autotune(wb_batch* batch, wb_batch_tune* tune, int32_t* 
                                       batch->n_max, threads, s)
               : launch_batch_tree_bwd(batch->d_robots, batch->d_probs, batch->d_titems[1],
                                       batch->n_titems[1], counters + 2, io, grid, batch->ns_max,
-                                      batch->n_max, threads, s);
+                                      batch->n_max, threads, batch->rows, s);
       return e == cudaSuccess ? WB_OK : cuda_fail(e, "batch autotune launch");
     };
     // robots whose segments are a choice: a 2-segment plan and some problem

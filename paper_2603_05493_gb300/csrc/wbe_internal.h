@@ -208,7 +208,7 @@ cudaError_t launch_batch_tree_fwd(const DevRobot* robots, const BatchProblemDev*
                                   cudaStream_t s);
 cudaError_t launch_batch_tree_bwd(const DevRobot* robots, const BatchProblemDev* probs,
                                   const int4* items, int n_items, int* counter, const BatchIO& io,
-                                  int grid, int ns_max, int n_max, int threads,
+                                  int grid, int ns_max, int n_max, int threads, bool rows,
                                   cudaStream_t s);
 cudaError_t launch_batch_pair(const DevRobot* robots, const PairSchedule32* scheds,
                               const BatchProblemDev* probs, const int2* items, int n_items,
