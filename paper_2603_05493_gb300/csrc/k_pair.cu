@@ -162,6 +162,194 @@ __global__ void __launch_bounds__(kThreadBlock) pair_thread_kernel(DevRobot r, F
   }
 }
 
+// The same small robots when every group of 4 spheres lies on one link
+// (sph_vec4) and no pair bits are wanted: 8 lanes a configuration, 4
+// configurations a warp.  Lane g places group g from its link's pose (48
+// contiguous bytes a lane, the configuration's row contiguous over the 8),
+// keeps the group's constants in registers and writes its centres as float4
+// rows; then the lanes share the 4x4 blocks, 16 distances for six 16-byte
+// shared loads where the thread-per-configuration loop takes six 4-byte loads
+// and a table entry a pair.  The distances use the approximate square root:
+// each lane keeps the least, its pair and the second least, the 8 lanes meet
+// in shuffles, and the winner's distance is computed exactly.  When the second
+// least is within the approximation's margin of the least (or anything is not
+// a number), the configuration's pairs are evaluated exactly in index order,
+// so the result is the exact path's, bit for bit, ties included.  Bound by
+// issue (16 instructions a pair).  7-DoF arm: 0.064 -> @@ ms at 131072
+// configurations, 0.023 -> @@ ms at 3300, 0.026 -> @@ ms at 64, where one
+// thread's 240 serial pairs were the time.
+constexpr int kSmallWarps = 8;
+constexpr int kSmallGroups = kThreadMaxS / 4;
+static bool pair_small_ok(const DevRobot& r, const FwdArgs& a) {
+  return pair_thread_ok(r) && r.sph_vec4 && !a.bits;
+}
+static size_t pair_small_smem(const DevRobot& r) {
+  return sizeof(float4) * kSmallGroups + sizeof(uint2) * (size_t)((r.nblk + 1) & ~1) +
+         sizeof(float4) * kSmallWarps * 4 * 3 * kSmallGroups;
+}
+
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+template <bool FULL>
+__global__ void __launch_bounds__(32 * kSmallWarps) pair_small_kernel(
+    const __grid_constant__ DevRobot r, const __grid_constant__ PairSchedule32 ps,
+    const __grid_constant__ FwdArgs A) {
+  extern __shared__ __align__(16) float4 smf[];
+  constexpr int NG = kSmallGroups;
+  float4* rad = smf;                                    // [NG] radii of each group
+  uint2* blk = reinterpret_cast<uint2*>(smf + NG);      // [nblk] groups i | j << 16, mask
+  const int nblk = r.nblk, Sg = r.Sg, S = r.S, n = r.n;
+  for (int i = threadIdx.x; i < Sg; i += blockDim.x) rad[i] = __ldg(r.grp_rad + i);
+  for (int i = threadIdx.x; i < 32 * ps.rounds; i += blockDim.x) {
+    const uint2 e = __ldg(ps.ent + i);  // byte offsets 16 gi | 16 gj << 16, mask << 16 | block
+    if ((e.y >> 16) != 0u) blk[e.y & 0xFFFF] = make_uint2((e.x >> 4) & 0x0FFF0FFFu, e.y >> 16);
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = lane >> 3, l = lane & 7;
+  // this configuration's centres: [3][NG] float4
+  float4* C = smf + NG + (nblk + 1) / 2 + (warp * 4 + c) * 3 * NG;
+  const float* Cf = reinterpret_cast<const float*>(C);
+  const float* radf = reinterpret_cast<const float*>(rad);
+  const bool has = l < Sg;
+  const int link = has ? __ldg(r.grp_link + l) : 0;
+  float4 sp[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) sp[q] = has ? __ldg(r.sph + 4 * l + q) : make_float4(0, 0, 0, 0);
+  const float inf = __int_as_float(0x7f800000);
+  const bool so4 = (reinterpret_cast<uintptr_t>(A.sph) & 15u) == 0;
+  const int64_t step = (int64_t)gridDim.x * kSmallWarps * 4;
+  for (int64_t b0 = ((int64_t)blockIdx.x * kSmallWarps + warp) * 4; b0 < A.B; b0 += step) {
+    const bool act = b0 + c < A.B;
+    const int64_t b = act ? b0 + c : A.B - 1;
+    if (has) {
+      const float4* P4 = reinterpret_cast<const float4*>(A.pose + (b * n + link) * 12);
+      const float4 t0 = __ldg(P4), t1 = __ldg(P4 + 1), t2 = __ldg(P4 + 2);
+      const float T[12] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w, t2.x, t2.y, t2.z, t2.w};
+      float o[12];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float cl[3] = {sp[q].x, sp[q].y, sp[q].z};
+        rot(T, cl, o + 3 * q);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) o[3 * q + i] += T[9 + i];
+      }
+      C[l] = make_float4(o[0], o[3], o[6], o[9]);
+      C[NG + l] = make_float4(o[1], o[4], o[7], o[10]);
+      C[2 * NG + l] = make_float4(o[2], o[5], o[8], o[11]);
+      if (A.sph && act) {
+        float* so = A.sph + (b * S + 4 * l) * 3;
+        if (so4) {
+          float4* o4 = reinterpret_cast<float4*>(so);
+          o4[0] = make_float4(o[0], o[1], o[2], o[3]);
+          o4[1] = make_float4(o[4], o[5], o[6], o[7]);
+          o4[2] = make_float4(o[8], o[9], o[10], o[11]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 12; ++i) so[i] = o[i];
+        }
+      }
+    }
+    __syncwarp();
+    if (A.dmin) {
+      float m1 = inf, m2 = inf;  // least and second least approximate distance
+      int at = 0;                // the least's slot in blk_pidx
+      for (int k = l; k < nblk; k += 8) {
+        const uint2 e = blk[k];
+        const int gi = e.x & 0xFFFF, gj = e.x >> 16;
+        const float4 xi = C[gi], yi = C[NG + gi], zi = C[2 * NG + gi], ri = rad[gi];
+        const float4 xj = C[gj], yj = C[NG + gj], zj = C[2 * NG + gj], rj = rad[gj];
+        const float ax[4] = {xi.x, xi.y, xi.z, xi.w}, ay[4] = {yi.x, yi.y, yi.z, yi.w},
+                    az[4] = {zi.x, zi.y, zi.z, zi.w}, ar[4] = {ri.x, ri.y, ri.z, ri.w};
+        const float bx[4] = {xj.x, xj.y, xj.z, xj.w}, by[4] = {yj.x, yj.y, yj.z, yj.w},
+                    bz[4] = {zj.x, zj.y, zj.z, zj.w}, br[4] = {rj.x, rj.y, rj.z, rj.w};
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+          const int p = t >> 2, q = t & 3;
+          float d = sqrt_approx(dist2(ax[p], ay[p], az[p], bx[q], by[q], bz[q])) - (ar[p] + br[q]);
+          if (!FULL) d = (e.y >> t) & 1u ? d : inf;
+          m2 = fminf(m2, fmaxf(m1, d));
+          if (d < m1) {
+            m1 = d;
+            at = 16 * k + t;
+          }
+        }
+      }
+#pragma unroll
+      for (int off = 4; off > 0; off >>= 1) {
+        const float o1 = __shfl_xor_sync(0xffffffffu, m1, off);
+        const float o2 = __shfl_xor_sync(0xffffffffu, m2, off);
+        const int oa = __shfl_xor_sync(0xffffffffu, at, off);
+        m2 = fminf(fmaxf(m1, o1), fminf(m2, o2));
+        if (o1 < m1) {
+          m1 = o1;
+          at = oa;
+        }
+      }
+      // exact distance of pair p, as the exact path of every pair kernel
+      auto exact = [&](int2 ij) {
+        return sqrtf(dist2(Cf[ij.x], Cf[4 * NG + ij.x], Cf[8 * NG + ij.x], Cf[ij.y],
+                           Cf[4 * NG + ij.y], Cf[8 * NG + ij.y])) -
+               (radf[ij.x] + radf[ij.y]);
+      };
+      // the approximation is within 3e-7 of the centre distance; the margin
+      // covers it at both distances (a robot's reach, and poses far beyond it)
+      bool close = !(m2 - m1 > fmaf(1e-6f, fabsf(m1), r.margin));
+      float best = inf;
+      int bi = -1;
+      if (!close) {
+        bi = __ldg(r.blk_pidx + at);
+        best = exact(__ldg(r.pairs + bi));
+      }
+      if (__any_sync(0xffffffffu, close)) {
+        float e = inf;
+        int ei = INT_MAX;
+        for (int p = l; p < r.P && close; p += 8) {
+          const float d = exact(__ldg(r.pairs + p));
+          if (d < e) {
+            e = d;
+            ei = p;
+          }
+        }
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) {
+          const float od = __shfl_xor_sync(0xffffffffu, e, off);
+          const int oi = __shfl_xor_sync(0xffffffffu, ei, off);
+          if (od < e || (od == e && oi < ei)) {
+            e = od;
+            ei = oi;
+          }
+        }
+        if (close) {
+          best = e;
+          bi = ei == INT_MAX ? -1 : ei;
+        }
+      }
+      if (l == 0 && act) {
+        A.dmin[b] = best;
+        A.worst[b] = bi;
+        if (A.wdiff) pair_diff(r, A, b, bi, Cf, Cf + 4 * NG, Cf + 8 * NG);
+      }
+    }
+    __syncwarp();  // the centres are the next configurations'
+  }
+}
+
+static cudaError_t launch_pair_small(const DevRobot& r, const PairSchedule32& ps, const FwdArgs& a,
+                                     cudaStream_t s) {
+  const size_t smem = pair_small_smem(r);
+  auto kern = r.all_full ? pair_small_kernel<true> : pair_small_kernel<false>;
+  // blocks of 32 configurations; past 16 a multiprocessor each block takes
+  // several passes, evenly, so that its tables are staged once for them
+  const int64_t need = (a.B + 4 * kSmallWarps - 1) / (4 * kSmallWarps);
+  const int64_t passes = (need + 16 * 152 - 1) / (16 * 152);
+  kern<<<(unsigned)((need + passes - 1) / passes), 32 * kSmallWarps, smem, s>>>(r, ps, a);
+  return cudaGetLastError();
+}
+
 static cudaError_t launch_pair_thread(const DevRobot& r, const FwdArgs& a, cudaStream_t s) {
   const size_t smem = pair_thread_smem(r);
   auto kern = a.bits ? pair_thread_kernel<true> : pair_thread_kernel<false>;
@@ -206,7 +394,8 @@ static cudaError_t pair_dispatch(const DevRobot& r, const PairSchedule32& ps, co
 
 cudaError_t launch_pair(const DevRobot& r, const PairSchedule32& ps, const FwdArgs& a, int grid,
                         int warps, cudaStream_t s, bool cull) {
-  if (cull && pair_thread_ok(r)) return launch_pair_thread(r, a, s);  // small robots
+  if (cull && pair_small_ok(r, a)) return launch_pair_small(r, ps, a, s);  // small robots
+  if (cull && pair_thread_ok(r)) return launch_pair_thread(r, a, s);
   return pair_dispatch(r, ps, a, grid, warps, s, nullptr, cull);
 }
 
