@@ -175,8 +175,8 @@ __global__ void __launch_bounds__(kThreadBlock) pair_thread_kernel(DevRobot r, F
 // least is within the approximation's margin of the least (or anything is not
 // a number), the configuration's pairs are evaluated exactly in index order,
 // so the result is the exact path's, bit for bit, ties included.  Bound by
-// issue (16 instructions a pair).  7-DoF arm: 0.064 -> @@ ms at 131072
-// configurations, 0.023 -> @@ ms at 3300, 0.026 -> @@ ms at 64, where one
+// issue (16 instructions a pair).  7-DoF arm: 0.064 -> 0.039 ms at 131072
+// configurations, 0.023 -> 0.004 ms at 3300, 0.026 -> 0.004 ms at 64, where one
 // thread's 240 serial pairs were the time.
 constexpr int kSmallWarps = 8;
 constexpr int kSmallGroups = kThreadMaxS / 4;
