@@ -293,6 +293,14 @@ int wb_eval_backward_ext(wb_robot* robot, int64_t B, const float* q, const float
                          const float* g_tau, float* gq, float* gqd, float* gqdd, float* g_fext,
                          const wb_tune* tune, void* stream);
 
+/* wb_eval_ext that also writes worst_diff [B][3] as wb_self_collision_dir
+ * does (nullable; needs d_min and the tree kernels): the sweep and the pair
+ * stage in one call. */
+int wb_eval_dir(wb_robot* robot, int64_t B, const float* q, const float* qd, const float* qdd,
+                const float* f_ext, float* link_pose, float* sphere, float* d_min,
+                int32_t* worst_pair, float* worst_diff, float* tau, uint32_t* pair_bits,
+                const wb_tune* tune, void* stream);
+
 /* wb_eval_backward_ext with the worst pair's centre difference worst_diff
  * [B][3] from wb_self_collision_dir on the same poses (nullable: the sweep
  * places the two spheres itself).  The tree kernels use it in place of the

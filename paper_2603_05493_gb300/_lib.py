@@ -151,6 +151,8 @@ SIGNATURES = {
     "wb_eval_backward_dir": (C.c_int, [p, C.c_int64, p, p, p, p, p, p, p, p, p, p, p, p, p, p,
                                        C.POINTER(wb_tune), p]),
     "wb_eval_ext": (C.c_int, [p, C.c_int64, p, p, p, p, p, p, p, p, p, p, C.POINTER(wb_tune), p]),
+    "wb_eval_dir": (C.c_int, [p, C.c_int64, p, p, p, p, p, p, p, p, p, p, p, C.POINTER(wb_tune),
+                              p]),
     "wb_eval_backward_ext": (C.c_int, [p, C.c_int64, p, p, p, p, p, p, p, p, p, p, p, p, p,
                                        C.POINTER(wb_tune), p]),
 }

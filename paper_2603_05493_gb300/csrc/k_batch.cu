@@ -258,8 +258,7 @@ cudaError_t launch_batch_tree_fwd(const DevRobot* robots, const BatchProblemDev*
                                   int n_items, int* counter, const BatchIO& io, int grid,
                                   int ns_max, int n_max, int threads, cudaStream_t s) {
   const size_t smem = batch_tree_smem(true, ns_max, n_max, threads);
-  cudaError_t e = cudaFuncSetAttribute(batch_tree_fwd_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)batch_tree_fwd_kernel, smem);
   if (e != cudaSuccess) return e;
   fit_carveout((const void*)batch_tree_fwd_kernel, threads, smem);
   e = cudaMemsetAsync(counter, 0, sizeof(int), s);
@@ -279,7 +278,7 @@ cudaError_t launch_batch_tree_bwd(const DevRobot* robots, const BatchProblemDev*
                   ? batch_tree_bwd_kernel<kBwdRows>
                   : batch_tree_bwd_kernel<kBwdGeneral>;
   cudaError_t e =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      allow_smem((const void*)kern, smem);
   if (e != cudaSuccess) return e;
   fit_carveout((const void*)kern, threads, smem);
   e = cudaMemsetAsync(counter, 0, sizeof(int), s);
@@ -297,8 +296,7 @@ cudaError_t launch_batch_pair(const DevRobot* robots, const PairSchedule32* sche
                               const BatchIO& io, int grid, int warps, int ws_words,
                               int rad_words, cudaStream_t s) {
   const size_t smem = batch_pair_smem(ws_words, rad_words, warps);
-  cudaError_t e = cudaFuncSetAttribute(batch_pair_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)batch_pair_kernel, smem);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(counter, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
@@ -311,10 +309,9 @@ cudaError_t launch_batch_pair(const DevRobot* robots, const PairSchedule32* sche
 
 cudaError_t batch_pair_max_blocks_per_sm(int warps, int ws_words, int rad_words, int* out) {
   const size_t smem = batch_pair_smem(ws_words, rad_words, warps);
-  cudaError_t e = cudaFuncSetAttribute(batch_pair_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)batch_pair_kernel, smem);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, batch_pair_kernel, warps * 32, smem);
+  return max_blocks((const void*)batch_pair_kernel, warps * 32, smem, out);
 }
 
 cudaError_t batch_tree_max_blocks_per_sm(bool fwd, int ns_max, int n_max, int threads, int* out) {
@@ -325,9 +322,9 @@ cudaError_t batch_tree_max_blocks_per_sm(bool fwd, int ns_max, int n_max, int th
   }
   auto kern = fwd ? batch_tree_fwd_kernel : batch_tree_bwd_kernel<kBwdGeneral>;
   cudaError_t e =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      allow_smem((const void*)kern, smem);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kern, threads, smem);
+  return max_blocks((const void*)kern, threads, smem, out);
 }
 
 int pair_plan_words(const DevRobot& r) { return PairPlan(r.n, r.Sg, r.P, false).total; }

@@ -301,7 +301,7 @@ cudaError_t launch_hinge(const DevRobot& r, const PairSchedule32& ps, const Hing
                          int warps, cudaStream_t s) {
   const size_t smem = hinge_block_smem(r, warps);
   cudaError_t e =
-      cudaFuncSetAttribute(hinge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      allow_smem((const void*)hinge_kernel, smem);
   if (e != cudaSuccess) return e;
   hinge_kernel<<<grid, warps * 32, smem, s>>>(r, ps, a);
   return cudaGetLastError();
@@ -310,9 +310,9 @@ cudaError_t launch_hinge(const DevRobot& r, const PairSchedule32& ps, const Hing
 cudaError_t hinge_max_blocks_per_sm(const DevRobot& r, int warps, int* out) {
   const size_t smem = hinge_block_smem(r, warps);
   cudaError_t e =
-      cudaFuncSetAttribute(hinge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      allow_smem((const void*)hinge_kernel, smem);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, hinge_kernel, warps * 32, smem);
+  return max_blocks((const void*)hinge_kernel, warps * 32, smem, out);
 }
 
 }  // namespace wbe

@@ -164,7 +164,7 @@ size_t kin_smem_per_warp(const DevRobot& r) { return sizeof(float) * kin_words(r
 cudaError_t launch_kin(const DevRobot& r, const KinArgs& a, int grid, int warps, cudaStream_t s) {
   const size_t smem = sizeof(float) * kin_words(r.n) * warps;
   cudaError_t e =
-      cudaFuncSetAttribute(kin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      allow_smem((const void*)kin_kernel, smem);
   if (e != cudaSuccess) return e;
   kin_kernel<<<grid, warps * 32, smem, s>>>(r, a);
   return cudaGetLastError();
@@ -173,9 +173,9 @@ cudaError_t launch_kin(const DevRobot& r, const KinArgs& a, int grid, int warps,
 cudaError_t kin_max_blocks_per_sm(const DevRobot& r, int warps, int* out) {
   const size_t smem = sizeof(float) * kin_words(r.n) * warps;
   cudaError_t e =
-      cudaFuncSetAttribute(kin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      allow_smem((const void*)kin_kernel, smem);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kin_kernel, warps * 32, smem);
+  return max_blocks((const void*)kin_kernel, warps * 32, smem, out);
 }
 
 }  // namespace wbe

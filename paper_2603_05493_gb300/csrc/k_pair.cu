@@ -353,8 +353,7 @@ static cudaError_t launch_pair_small(const DevRobot& r, const PairSchedule32& ps
 static cudaError_t launch_pair_thread(const DevRobot& r, const FwdArgs& a, cudaStream_t s) {
   const size_t smem = pair_thread_smem(r);
   auto kern = a.bits ? pair_thread_kernel<true> : pair_thread_kernel<false>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_smem((const void*)kern, smem);
   if (e != cudaSuccess) return e;
   const int64_t grid = (a.B + kThreadBlock - 1) / kThreadBlock;
   kern<<<(unsigned)grid, kThreadBlock, smem, s>>>(r, a);
@@ -365,10 +364,9 @@ template <bool FULL, bool BITS, bool CULL>
 static cudaError_t pair_launch_t(const DevRobot& r, const PairSchedule32& ps, const FwdArgs& a,
                                  int grid, int warps, size_t smem, cudaStream_t s, int* occ) {
   auto kern = CULL ? pair_kernel<FULL, BITS> : pair_full_kernel<FULL, BITS>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_smem((const void*)kern, smem);
   if (e != cudaSuccess) return e;
-  if (occ) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kern, warps * 32, smem);
+  if (occ) return max_blocks((const void*)kern, warps * 32, smem, occ);
   kern<<<grid, warps * 32, smem, s>>>(r, ps, a);
   return cudaGetLastError();
 }

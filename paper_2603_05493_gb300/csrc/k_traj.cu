@@ -245,8 +245,7 @@ cudaError_t launch_bspline_bwd(int64_t n_traj, int d, int K, int T, float dt, in
                                float* gU, float* gstart, cudaStream_t s) {
   const int hs = has_start ? 1 : 0, es = end_static ? 1 : 0;
   const size_t smem = bspline_bwd_smem(K + 3 * hs + 3 * es, T);
-  cudaError_t e = cudaFuncSetAttribute(bspline_bwd_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)bspline_bwd_kernel, smem);
   if (e != cudaSuccess) return e;
   const int64_t n = n_traj * d * (K + hs);
   bspline_bwd_kernel<<<(unsigned)((n + 255) / 256), 256, smem, s>>>(

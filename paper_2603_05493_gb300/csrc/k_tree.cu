@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <vector>
 
 namespace wbe {
 
@@ -432,6 +433,73 @@ static bool sm_limits(int dev, SmLimits* out) {
   return true;
 }
 
+// The runtime's answers per kernel and device: four of these calls a launch
+// (two attributes set, the kernel's attributes and the occupancy read) were a
+// third of a small call's time in the library.
+namespace {
+struct KernelState {
+  const void* kern;
+  int dev;
+  size_t smem = 0;        // dynamic shared memory it is allowed
+  int carveout = -1;      // the last preference set
+  int regs = -1;          // registers a thread (-1: not read yet)
+  size_t stat = 0;        // static shared memory
+  struct Occ {
+    int threads;
+    size_t smem;
+    int blocks;
+  };
+  std::vector<Occ> occ;   // at most kOcc shapes
+};
+constexpr size_t kOcc = 64;
+std::mutex g_kern_mu;
+std::vector<KernelState> g_kern;
+
+KernelState& kernel_state(const void* kern, int dev) {  // g_kern_mu held
+  for (KernelState& k : g_kern)
+    if (k.kern == kern && k.dev == dev) return k;
+  g_kern.push_back(KernelState{kern, dev});
+  return g_kern.back();
+}
+}  // namespace
+
+void launch_cache_clear(int device) {
+  std::lock_guard<std::mutex> lock(g_kern_mu);
+  g_kern.erase(std::remove_if(g_kern.begin(), g_kern.end(),
+                              [&](const KernelState& k) { return k.dev == device; }),
+               g_kern.end());
+}
+
+cudaError_t allow_smem(const void* kern, size_t smem) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(g_kern_mu);
+  KernelState& k = kernel_state(kern, dev);
+  if (smem <= k.smem) return cudaSuccess;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) k.smem = smem;
+  return e;
+}
+
+cudaError_t max_blocks(const void* kern, int threads, size_t smem, int* out) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(g_kern_mu);
+  KernelState& k = kernel_state(kern, dev);
+  for (const KernelState::Occ& o : k.occ)
+    if (o.threads == threads && o.smem == smem) {
+      *out = o.blocks;
+      return cudaSuccess;
+    }
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kern, threads, smem);
+  if (e != cudaSuccess) return e;
+  if (k.occ.size() >= kOcc) k.occ.clear();
+  k.occ.push_back({threads, smem, *out});
+  return cudaSuccess;
+}
+
 void fit_carveout(const void* kern, int threads, size_t smem) {
   int dev = 0;
   SmLimits L;
@@ -439,17 +507,28 @@ void fit_carveout(const void* kern, int threads, size_t smem) {
     cudaGetLastError();
     return;
   }
-  cudaFuncAttributes fa;
-  if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return;
+  std::lock_guard<std::mutex> lock(g_kern_mu);
+  KernelState& k = kernel_state(kern, dev);
+  if (k.regs < 0) {
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return;
+    k.regs = fa.numRegs;
+    k.stat = fa.sharedSizeBytes;
+  }
   const int warps = (threads + 31) / 32;
-  const int regs_warp = ((fa.numRegs * 32 + 255) / 256) * 256;  // 256-register allocation unit
+  const int regs_warp = ((k.regs * 32 + 255) / 256) * 256;  // 256-register allocation unit
   int nb = std::min(L.threads_sm / (32 * warps), L.blocks_sm);
   if (regs_warp > 0) nb = std::min(nb, (L.regs_sm / regs_warp) / warps);
-  const size_t per = smem + fa.sharedSizeBytes + (size_t)L.reserved;
+  const size_t per = smem + k.stat + (size_t)L.reserved;
   nb = std::min<int>(nb, (int)((size_t)L.smem_sm / per));
   const size_t need = (size_t)std::max(nb, 1) * per;
   const int pct = (int)std::min<size_t>(100, (need * 100 + L.smem_sm - 1) / L.smem_sm);
-  cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+  if (pct == k.carveout) return;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, pct) ==
+      cudaSuccess)
+    k.carveout = pct;
+  else
+    cudaGetLastError();
 }
 
 static size_t rec_smem(const DevRobot& r, bool fwd) {
@@ -483,7 +562,7 @@ static cudaError_t launch_seg(void (*kern)(DevRobot, WalkTab, Args, int), const 
   const int CG = seg_groups(segments, threads);
   const size_t smem = tree_seg_smem(r, segments, threads, fwd, false) + extra;
   cudaError_t e =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      allow_smem((const void*)kern, smem);
   if (e != cudaSuccess) return e;
   fit_carveout((const void*)kern, 32 * segments * CG, smem);
   const int64_t groups = (a.B + 31) / 32;
@@ -498,7 +577,7 @@ template <class... P, class... V>
 static cudaError_t launch_bwd(void (*kern)(P...), int64_t B, int groups, int block, size_t smem,
                               cudaStream_t s, const V&... v) {
   cudaError_t e =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      allow_smem((const void*)kern, smem);
   if (e != cudaSuccess) return e;
   fit_carveout((const void*)kern, block, smem);
   const int64_t grid = ((B + 31) / 32 + groups - 1) / groups;
@@ -527,7 +606,7 @@ cudaError_t launch_tree_fwd(const DevRobot& r, const WalkTab& wt, const FwdArgs&
               : a.tau ? tree_fwd_kernel<kFwdLocal>
                       : tree_fwd_kernel<kFwdPose>;
   cudaError_t e =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      allow_smem((const void*)kern, smem);
   if (e != cudaSuccess) return e;
   fit_carveout((const void*)kern, threads, smem);
   const int64_t grid = (a.B + threads - 1) / threads;
@@ -579,7 +658,7 @@ cudaError_t launch_tree_fwd_spline(const DevRobot& r, const WalkTab& wt, const F
                 : a.tau ? tree_fwd_spline_seg_kernel<kFwdLocal>
                         : tree_fwd_spline_seg_kernel<kFwdPose>;
     cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem((const void*)kern, smem);
     if (e != cudaSuccess) return e;
     fit_carveout((const void*)kern, block, smem);
     const int64_t grid = ((a.B + 31) / 32 + CG - 1) / CG;

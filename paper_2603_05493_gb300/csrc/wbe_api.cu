@@ -687,6 +687,7 @@ int wb_load_robot(const wb_tree* tree, const wb_spheres* sph, const wb_pairs* pa
   R->n = n;
   R->S = H.S;
   DeviceGuard guard(device);
+  launch_cache_clear(device);
   cudaDeviceGetAttribute(&R->num_sms, cudaDevAttrMultiProcessorCount, device);
 
   DevRobot& D = R->dev;
@@ -1035,6 +1036,14 @@ int wb_eval_ext(wb_robot* robot, int64_t B, const float* q, const float* qd, con
                 const float* f_ext, float* link_pose, float* sphere, float* d_min,
                 int32_t* worst_pair, float* tau, uint32_t* pair_bits, const wb_tune* tune,
                 void* stream) {
+  return wb_eval_dir(robot, B, q, qd, qdd, f_ext, link_pose, sphere, d_min, worst_pair, nullptr,
+                     tau, pair_bits, tune, stream);
+}
+
+int wb_eval_dir(wb_robot* robot, int64_t B, const float* q, const float* qd, const float* qdd,
+                const float* f_ext, float* link_pose, float* sphere, float* d_min,
+                int32_t* worst_pair, float* worst_diff, float* tau, uint32_t* pair_bits,
+                const wb_tune* tune, void* stream) {
   g_err.clear();
   if (!robot) return fail(WB_EINVAL, "robot is NULL");
   if (B < 0) return fail(WB_EINVAL, "B < 0");
@@ -1051,16 +1060,21 @@ int wb_eval_ext(wb_robot* robot, int64_t B, const float* q, const float* qd, con
   if ((rc = check_ptr(robot, tau, "tau", false))) return rc;
   if ((rc = check_ptr(robot, pair_bits, "pair_bits", false))) return rc;
   if ((rc = check_ptr(robot, f_ext, "f_ext", false))) return rc;
+  if ((rc = check_ptr(robot, worst_diff, "worst_diff", false))) return rc;
   if (!d_min && worst_pair) return fail(WB_EINVAL, "worst_pair without d_min");
+  if (!d_min && worst_diff) return fail(WB_EINVAL, "worst_diff without d_min");
   DeviceGuard guard(robot->device);
   FwdArgs a{B, q, qd, qdd, link_pose, sphere, d_min, worst_pair, tau, pair_bits};
   a.fext = tau ? f_ext : nullptr;
+  a.wdiff = worst_diff;
   int kernel = tune ? tune->kernel : WB_KERNEL_AUTO;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const bool pairs_wanted = d_min || sphere || pair_bits;
   const bool tree_ok = robot->dev.maxdepth <= tree_max_depth();
   if (kernel == WB_KERNEL_AUTO)
     kernel = (tree_ok && (link_pose || !pairs_wanted)) ? WB_KERNEL_TREE : WB_KERNEL_FUSED;
+  if (worst_diff && kernel != WB_KERNEL_TREE && kernel != WB_KERNEL_TREE_NOCULL)
+    return fail(WB_EINVAL, "worst_diff comes from the tree kernels' pair stage");
   cudaError_t e;
   const bool cull = kernel != WB_KERNEL_TREE_NOCULL;
   if (kernel == WB_KERNEL_TREE_NOCULL) kernel = WB_KERNEL_TREE;

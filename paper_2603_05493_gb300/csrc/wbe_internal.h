@@ -312,6 +312,13 @@ size_t grad_slot_smem(int segments, int threads);
 // shared-memory carveout hint: the smallest that holds every block of `threads`
 // threads and `smem` dynamic bytes one SM can keep, leaving the rest to L1
 void fit_carveout(const void* kern, int threads, size_t smem);
+// What the launchers ask of the runtime, kept per kernel and device (thread
+// safe; a robot load on a device clears its entries, so handles made after a
+// context reset ask again).  allow_smem: the kernel may be launched with smem
+// bytes of dynamic shared memory; max_blocks: blocks an SM can hold.
+cudaError_t allow_smem(const void* kern, size_t smem);
+cudaError_t max_blocks(const void* kern, int threads, size_t smem, int* out);
+void launch_cache_clear(int device);
 int tree_max_depth();
 size_t pair_smem(const DevRobot& r, int warps, bool bits);
 size_t pair_block_smem(const DevRobot& r, int warps, bool bits);  // the same, out of line
