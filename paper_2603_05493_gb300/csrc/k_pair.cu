@@ -188,12 +188,6 @@ static size_t pair_small_smem(const DevRobot& r) {
          sizeof(float4) * kSmallWarps * 4 * 3 * kSmallGroups;
 }
 
-__device__ __forceinline__ float sqrt_approx(float x) {
-  float y;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 template <bool FULL>
 __global__ void __launch_bounds__(32 * kSmallWarps) pair_small_kernel(
     const __grid_constant__ DevRobot r, const __grid_constant__ PairSchedule32 ps,

@@ -60,6 +60,13 @@ inline size_t pair_smem(const DevRobot& r, int warps, bool bits) {
          ((size_t)a32(4 * r.Sg) + (size_t)warps * PairPlan(r.n, r.Sg, r.P, bits).total);
 }
 
+// approximate square root (relative error at most 2^-23)
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 // order-preserving map of a float to a signed int (and back)
 __device__ __forceinline__ int fkey(float f) {
   const int i = __float_as_int(f);
@@ -490,6 +497,9 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
   }
   if (BITS)
     for (int w = lane; w < W; w += 32) bm[w] = 0u;
+  // the far sphere of the schedule's null blocks
+  if (lane == 0)
+    *reinterpret_cast<float4*>(ws + pl.gb + far_words(Sg)) = make_float4(1e15f, 1e15f, 1e15f, 0.0f);
   __syncwarp();
   if (!A.dmin && !BITS) return;  // sphere placement only
   if (rounds == 0) {
@@ -506,42 +516,48 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
   // ---- pass 1: the block of smallest lower bound (approximately: any block
   // gives a valid bound), and the exact minimum of its pairs ----
   // The lower bounds are kept for pass 2 as halves in the (now free) row
-  // region when they fit, rounded down after a widening that covers the
-  // approximate square root, so that pass 2 keeps every block its exact test
-  // would keep (and at most a few more, within the half's rounding).
-  const bool keep_lb = rounds * 32 <= 2 * pl.ra_words();
-  __half* lb16 = reinterpret_cast<__half*>(xr);
-  // the schedule's byte offsets of a block's two groups in the per-warp
-  // sphere arrays (16 bytes a group) are also their offsets in gb
+  // region when they fit, two rounds a word, rounded to nearest: rounding is
+  // monotone, so a bound at most the threshold stays at most the threshold's
+  // half, and pass 2 keeps every block its exact test would keep (and at most
+  // a few more, within the half's rounding).  Two rounds a step with the
+  // blocks' offsets decoded by the host, null blocks against a far sphere in
+  // place of a test, the smallest bound carried with its round in its low 11
+  // bits, and two bounds compared an instruction in pass 2: humanoid48 pair
+  // stage 0.117 -> 0.105 ms at 32768 configurations.
+  const int prs = ps.prs;
+  const bool keep_lb = prs * 32 <= pl.ra_words();
+  __half2* lb2 = reinterpret_cast<__half2*>(xr) + lane;
+  // the blocks' byte offsets in the per-warp sphere arrays (16 bytes a group)
+  // are also their offsets in gb
   const char* cgb = reinterpret_cast<const char*>(gb);
+  auto bound = [&](uint32_t o0, uint32_t o1) {
+    const float4 P4 = lds4(cgb, o0), Q4 = lds4(cgb, o1);
+    // widened for the approximate square root: 4e-6 of the distance here,
+    // 2 x 2e-6 in the group radii
+    return fmaf(sqrt_approx(dist2(P4.x, P4.y, P4.z, Q4.x, Q4.y, Q4.z)), 0.999996f,
+                -(P4.w + Q4.w));
+  };
+  auto keyed = [](float lb, int rr) {  // any block gives a valid bound: 12 bits of it decide
+    return __int_as_float((__float_as_int(lb) & ~0x7FF) | rr);
+  };
   float lbmin = inf;
-  int rbest = 0;  // the round of the lane's smallest bound (its entry is
-                  // reloaded once at the end: 0.1408 -> 0.1375 ms on humanoid48)
-  uint2 en = __ldg(ps.ent + lane);  // one round ahead (the schedule ends with a null round)
-  for (int rr = 0; rr < rounds; ++rr) {
-    const uint2 e = en;
-    en = __ldg(ps.ent + (rr + 1) * 32 + lane);
-    __half low = __float2half(inf);  // null entries are never kept
-    if ((e.y >> 16) != 0u) {  // a real block
-      const float4 P4 = lds4(cgb, e.x & 0xFFFF), Q4 = lds4(cgb, e.x >> 16);
-      const float D2 = fmaxf(dist2(P4.x, P4.y, P4.z, Q4.x, Q4.y, Q4.z), 1e-30f);
-      const float dist = D2 * rsqrtf(D2);  // approximate square root
-      // the lower bound widened for the approximate square root: 4e-6 of
-      // the distance here, 2 x 2e-6 in the group radii
-      const float lb = fmaf(dist, 0.999996f, -(P4.w + Q4.w));
-      if (lb < lbmin) {
-        lbmin = lb;
-        rbest = rr;
-      }
-      low = __float2half_rd(lb);
-    }
-    if (keep_lb) lb16[rr * 32 + lane] = low;
+  const uint4* off = ps.off + lane;
+  uint4 en = __ldg(off);  // one step ahead (the table ends with a null row)
+#pragma unroll 2
+  for (int u = 0; u < prs; ++u) {
+    const uint4 e = en;
+    off += 32;
+    en = __ldg(off);
+    const float b0 = bound(e.x, e.y), b1 = bound(e.z, e.w);
+    if (keep_lb) lb2[u * 32] = __floats2half2_rn(b0, b1);
+    lbmin = fminf(lbmin, fminf(keyed(b0, 2 * u), keyed(b1, 2 * u + 1)));
   }
   float gbest;
   {
     const int kmin = __reduce_min_sync(0xffffffffu, fkey(lbmin));
     const int src = __ffs(__ballot_sync(0xffffffffu, fkey(lbmin) == kmin)) - 1;
-    const uint2 e = __ldg(ps.ent + __shfl_sync(0xffffffffu, rbest, src) * 32 + src);
+    const int rbest = __shfl_sync(0xffffffffu, __float_as_int(lbmin), src) & 0x7FF;
+    const uint2 e = __ldg(ps.ent + rbest * 32 + src);
     float d = inf;
     const int t = lane & 15, a = t >> 2, c = t & 3;
     if (lane < 16 && ((e.y >> 16) >> t) & 1u) {
@@ -564,9 +580,6 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
   // a block survives when its lower bound is within the screen's reach of
   // the current bound (or below zero when every colliding pair is wanted)
   const float reach_tol = 2.0f * margin;
-  // the survival threshold changes only at a drain (hoisted out of the
-  // per-round test: humanoid48 pair stage 0.1517 -> 0.1477 ms)
-  float thr = fminf(best, gbest) + reach_tol;
   auto screen_block = [&](uint2 e) {
     const uint32_t ro = e.x & 0xFFFF, co = e.x >> 16;
     const uint32_t mask = e.y >> 16;
@@ -650,14 +663,14 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
     // order of the screening does not change the result (the exact path keeps
     // the lexicographic (d, index) minimum).  Against a per-round ballot and
     // queue update: humanoid48 pair stage 0.1372 -> 0.1253 ms, same bits.
-    for (int r0 = 0; r0 < rounds; r0 += 32) {
-      const int r1 = min(rounds, r0 + 32);
-      const float th = fminf(best, gbest) + reach_tol;
-      uint32_t km = 0u;
-      for (int rr = r0; rr < r1; ++rr) {  // null entries hold +inf
-        const float lbv = __half2float(lb16[rr * 32 + lane]);
-        km |= (lbv <= th || (BITS && lbv <= reach_tol) ? 1u : 0u) << (rr - r0);
-      }
+    for (int u0 = 0; u0 < prs; u0 += 16) {
+      float th = fminf(best, gbest) + reach_tol;
+      if (BITS) th = fmaxf(th, reach_tol);
+      const __half2 th2 = __float2half2_rn(th);
+      uint32_t km = 0u;  // bit v: round 2 (u0 + v), bit 16 + v: the one after
+#pragma unroll
+      for (int v = 0; v < 16; ++v)
+        if (u0 + v < prs) km |= __hle2_mask(lb2[(u0 + v) * 32], th2) & (0x00010001u << v);
       const int cnt = __popc(km);
       int off = cnt;  // inclusive scan of the counts over the lanes
 #pragma unroll
@@ -669,9 +682,9 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
       int pos = off - cnt;
       for (int w0 = 0; w0 < tot; w0 += 32) {
         while (km && pos < w0 + 32) {
-          const int rr = r0 + __ffs(km) - 1;
+          const int bit = __ffs(km) - 1;
           km &= km - 1u;
-          qu[pos - w0] = (uint32_t)(rr * 32 + lane);
+          qu[pos - w0] = (uint32_t)((2 * (u0 + (bit & 15)) + (bit >> 4)) * 32 + lane);
           ++pos;
         }
         __syncwarp();
@@ -685,10 +698,7 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
       // lb <= bound + tol  <=>  |C_i - C_j| <= t := bound + tol + R_i + R_j,
       // tested on squares (t >= 0); the tolerance covers the float rounding
       bool keep = false;
-      if (keep_lb) {  // null entries hold +inf
-        const float lbv = __half2float(lb16[idx]);
-        keep = lbv <= thr || (BITS && lbv <= reach_tol);
-      } else {
+      {
         const uint2 e = __ldg(ps.ent + idx);
         if ((e.y >> 16) != 0u) {
           const float4 P4 = gb[(e.x & 0xFFFF) >> 4], Q4 = gb[(e.x >> 16) >> 4];
@@ -704,7 +714,6 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
       if (qn >= 32) {
         __syncwarp();
         drain(32);
-        thr = fminf(best, gbest) + reach_tol;
         __syncwarp();
         const uint32_t moved = lane + 32 < qn ? qu[lane + 32] : 0u;  // at most 31 left
         __syncwarp();

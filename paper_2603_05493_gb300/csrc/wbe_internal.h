@@ -104,7 +104,16 @@ struct PairSchedule {
 struct PairSchedule32 {
   int rounds;
   const uint2* ent;          // [rounds + 1][32], the last round all null
+  // for the bounds on whole blocks, two rounds at a time: the two blocks' byte
+  // offsets (16 gi, 16 gj each) in an array of group spheres; a null block is
+  // group 0 against a far sphere that the kernels put far_words(Sg) behind
+  // the array's start (prs = pairs of rounds, rounded up)
+  int prs;
+  const uint4* off;          // [prs + 1][32]
 };
+// where that far sphere sits behind the group spheres of Sg groups: the last 4
+// words of the 64-word queue that follows them
+__host__ __device__ constexpr int far_words(int Sg) { return ((4 * Sg + 31) & ~31) + 60; }
 
 // Kernel-side launch configuration of the fused kernels.
 struct FusedShape {
