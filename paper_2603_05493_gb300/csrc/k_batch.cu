@@ -327,6 +327,6 @@ cudaError_t batch_tree_max_blocks_per_sm(bool fwd, int ns_max, int n_max, int th
   return max_blocks((const void*)kern, threads, smem, out);
 }
 
-int pair_plan_words(const DevRobot& r) { return PairPlan(r.n, r.Sg, r.P, false).total; }
+int pair_plan_words(const DevRobot& r) { return PairPlan(r.n, r.Sg, r.P, false, true).total; }
 
 }  // namespace wbe

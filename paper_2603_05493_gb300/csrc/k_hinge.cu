@@ -40,11 +40,11 @@ struct HingePlan {
     yc = xc + m;
     zc = yc + m;
     gb = zc + m;
-    gx = gb + m;  // m >= 4 x groups
+    q = gb + m;  // m >= 4 x groups; the queue behind the bounds, as the pair stage has it
+    gx = q + 64;
     gy = gx + m;
     gz = gy + m;
-    q = gz + m;
-    total = q + 64;
+    total = gz + m;
   }
   // a block's slot: the 12 gradient floats of its row spheres, then (a second
   // phase) of its column spheres (an odd stride: the lanes' writes hit
@@ -62,6 +62,12 @@ static size_t hinge_block_smem(const DevRobot& r, int warps) {
 
 __device__ __forceinline__ float4 ld4(const char* base, uint32_t off) {
   return *reinterpret_cast<const float4*>(base + off);
+}
+// approximate square root (relative error at most 2^-23)
+__device__ __forceinline__ float approx_sqrt(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 __device__ __forceinline__ float p4(const float4& v, int i) {
   return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w));
@@ -89,7 +95,7 @@ __global__ void __launch_bounds__(256, 3) hinge_kernel(DevRobot r, PairSchedule3
              *czc = reinterpret_cast<const char*>(zc), *crad = reinterpret_cast<const char*>(radw),
              *cgb = reinterpret_cast<const char*>(gb);
   const float eta = A.eta, w = A.w;
-  const int rounds = ps.rounds;
+  const int prs = ps.prs;
   constexpr int SW = HingePlan::kSlotWords;
   for (int64_t b = (int64_t)blockIdx.x * wpb + warp; b < A.B; b += (int64_t)gridDim.x * wpb) {
     {
@@ -103,16 +109,24 @@ __global__ void __launch_bounds__(256, 3) hinge_kernel(DevRobot r, PairSchedule3
       asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     __syncwarp();
-    if (r.sph_vec4) {  // every group of 4 on one link: a lane a group
+    const float4 zero4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (lane == 0)  // the far sphere of the schedule's null blocks
+      *reinterpret_cast<float4*>(ws + pl.gb + far_words(Sg)) = make_float4(1e15f, 1e15f, 1e15f, 0.0f);
+    if (r.sph_vec4) {
+      // every group of 4 on one link: a lane a group places its centres, its
+      // bound and its gradient rows' zeros from one pose
       for (int g = lane; g < Sg; g += 32) {
         const float4* T4 = reinterpret_cast<const float4*>(P) + 3 * __ldg(r.grp_link + g);
         const float4 t0 = T4[0], t1 = T4[1], t2 = T4[2];
         const float T[12] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w, t2.x, t2.y, t2.z, t2.w};
+        const float4 lx = __ldg(r.sph_t + g), ly = __ldg(r.sph_t + Sg + g),
+                     lz = __ldg(r.sph_t + 2 * Sg + g);
+        const float px[4] = {lx.x, lx.y, lx.z, lx.w}, py[4] = {ly.x, ly.y, ly.z, ly.w},
+                    pz[4] = {lz.x, lz.y, lz.z, lz.w};
         float cx[4], cy[4], cz[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const float4 sp = __ldg(r.sph + 4 * g + k);
-          const float cl[3] = {sp.x, sp.y, sp.z};
+          const float cl[3] = {px[k], py[k], pz[k]};
           float c[3];
           rot(T, cl, c);
           cx[k] = c[0] + T[9];
@@ -122,6 +136,17 @@ __global__ void __launch_bounds__(256, 3) hinge_kernel(DevRobot r, PairSchedule3
         reinterpret_cast<float4*>(xc)[g] = make_float4(cx[0], cx[1], cx[2], cx[3]);
         reinterpret_cast<float4*>(yc)[g] = make_float4(cy[0], cy[1], cy[2], cy[3]);
         reinterpret_cast<float4*>(zc)[g] = make_float4(cz[0], cz[1], cz[2], cz[3]);
+        const float4 L = __ldg(r.grp_loc + g);
+        const float cl[3] = {L.x, L.y, L.z};
+        float c[3];
+        rot(T, cl, c);
+        const float scale = fabsf(T[9]) + fabsf(T[10]) + fabsf(T[11]) + fabsf(L.x) +
+                            fabsf(L.y) + fabsf(L.z);
+        gb[g] = make_float4(c[0] + T[9], c[1] + T[10], c[2] + T[11],
+                            fmaf(scale, 1e-6f, fmaf(L.w, 1e-6f, L.w)) + 3e-6f);
+        reinterpret_cast<float4*>(gx)[g] = zero4;
+        reinterpret_cast<float4*>(gy)[g] = zero4;
+        reinterpret_cast<float4*>(gz)[g] = zero4;
       }
     } else {
       for (int s = lane; s < 4 * Sg; s += 32) {
@@ -141,7 +166,7 @@ __global__ void __launch_bounds__(256, 3) hinge_kernel(DevRobot r, PairSchedule3
       }
     }
     __syncwarp();
-    for (int g = lane; g < Sg; g += 32) {  // group bounding spheres (+ the gradient rows' zeros)
+    for (int g = lane; g < Sg && !r.sph_vec4; g += 32) {  // the same for groups over several links
       const int gl = __ldg(r.grp_link + g);
       float4 B4;
       if (gl >= 0) {  // one link: its host-made bound, moved with the link
@@ -173,41 +198,46 @@ __global__ void __launch_bounds__(256, 3) hinge_kernel(DevRobot r, PairSchedule3
         B4 = make_float4(cx, cy, cz, fmaf(R, 1e-6f, R) + 3e-6f);  // widened for rounding
       }
       gb[g] = B4;
-      const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      reinterpret_cast<float4*>(gx)[g] = z;
-      reinterpret_cast<float4*>(gy)[g] = z;
-      reinterpret_cast<float4*>(gz)[g] = z;
+      reinterpret_cast<float4*>(gx)[g] = zero4;
+      reinterpret_cast<float4*>(gy)[g] = zero4;
+      reinterpret_cast<float4*>(gz)[g] = zero4;
     }
     __syncwarp();
     float cost = 0.0f;
-    for (int r0 = 0; r0 < rounds; r0 += 32) {
-      const int r1 = min(rounds, r0 + 32);
+    const uint4* off = ps.off + lane;
+    uint4 en = __ldg(off);  // one step ahead (the table ends with a null row)
+    for (int u0 = 0; u0 < prs; u0 += 16) {
       // blocks whose bound (widened below the true one: 4e-6 of the distance
-      // here, 2 x 2e-6 in the group radii) is under eta can hold an active pair
+      // here, 2 x 2e-6 in the group radii) is under eta can hold an active
+      // pair; bit v: round 2 (u0 + v), bit 16 + v: the one after
       uint32_t km = 0u;
-      for (int rr = r0; rr < r1; ++rr) {
-        const uint2 e = __ldg(ps.ent + rr * 32 + lane);
-        if ((e.y >> 16) != 0u) {
-          const float4 P4 = ld4(cgb, e.x & 0xFFFF), Q4 = ld4(cgb, e.x >> 16);
-          const float D2 = fmaxf(dist2(P4.x, P4.y, P4.z, Q4.x, Q4.y, Q4.z), 1e-30f);
-          const float dist = D2 * rsqrtf(D2);
-          km |= (fmaf(dist, 0.999996f, -(P4.w + Q4.w)) < eta ? 1u : 0u) << (rr - r0);
-        }
+      const int u1 = min(prs - u0, 16);
+#pragma unroll 2
+      for (int v = 0; v < u1; ++v) {
+        const uint4 e = en;
+        off += 32;
+        en = __ldg(off);
+        auto under = [&](uint32_t o0, uint32_t o1) {
+          const float4 P4 = ld4(cgb, o0), Q4 = ld4(cgb, o1);
+          return fmaf(approx_sqrt(dist2(P4.x, P4.y, P4.z, Q4.x, Q4.y, Q4.z)), 0.999996f,
+                      -(P4.w + Q4.w)) < eta;
+        };
+        km |= (under(e.x, e.y) ? 1u << v : 0u) | (under(e.z, e.w) ? 0x10000u << v : 0u);
       }
       const int cnt = __popc(km);
-      int off = cnt;  // inclusive scan of the counts over the lanes
+      int sum = cnt;  // inclusive scan of the counts over the lanes
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, off, o);
-        if (lane >= o) off += v;
+        const int v = __shfl_up_sync(0xffffffffu, sum, o);
+        if (lane >= o) sum += v;
       }
-      const int tot = __shfl_sync(0xffffffffu, off, 31);
-      int pos = off - cnt;
+      const int tot = __shfl_sync(0xffffffffu, sum, 31);
+      int pos = sum - cnt;
       for (int w0 = 0; w0 < tot; w0 += 32) {
         while (km && pos < w0 + 32) {
-          const int rr = r0 + __ffs(km) - 1;
+          const int bit = __ffs(km) - 1;
           km &= km - 1u;
-          qu[pos - w0] = (uint32_t)(rr * 32 + lane);
+          qu[pos - w0] = (uint32_t)((2 * (u0 + (bit & 15)) + (bit >> 4)) * 32 + lane);
           ++pos;
         }
         __syncwarp();

@@ -9,7 +9,7 @@ template <bool FULL, bool BITS, bool CULL>
 __device__ __forceinline__ void pair_warps(const DevRobot& r, const PairSchedule32& ps,
                                            const FwdArgs& A) {
   extern __shared__ __align__(128) float smem[];
-  const PairPlan pl(r.n, r.Sg, r.P, BITS);
+  const PairPlan pl(r.n, r.Sg, r.P, BITS, !CULL);
   float4* radw = reinterpret_cast<float4*>(smem);
   for (int i = threadIdx.x; i < r.Sg; i += blockDim.x) radw[i] = __ldg(r.grp_rad + i);
   __syncthreads();
@@ -369,7 +369,7 @@ template <bool CULL>
 static cudaError_t pair_dispatch_t(const DevRobot& r, const PairSchedule32& ps, const FwdArgs& a,
                                    int grid, int warps, cudaStream_t s, int* occ) {
   const bool bits = a.bits != nullptr;
-  const size_t smem = pair_smem(r, warps, bits);
+  const size_t smem = pair_smem(r, warps, bits, !CULL);
   if (r.all_full) {
     return bits ? pair_launch_t<true, true, CULL>(r, ps, a, grid, warps, smem, s, occ)
                 : pair_launch_t<true, false, CULL>(r, ps, a, grid, warps, smem, s, occ);
@@ -391,7 +391,10 @@ cudaError_t launch_pair(const DevRobot& r, const PairSchedule32& ps, const FwdAr
   return pair_dispatch(r, ps, a, grid, warps, s, nullptr, cull);
 }
 
-size_t pair_block_smem(const DevRobot& r, int warps, bool bits) { return pair_smem(r, warps, bits); }
+// what a launch may need at most (the full map-reduce's)
+size_t pair_block_smem(const DevRobot& r, int warps, bool bits) {
+  return pair_smem(r, warps, bits, true);
+}
 
 cudaError_t pair_max_blocks_per_sm(const DevRobot& r, int warps, bool bits, int* out) {
   FwdArgs a{};

@@ -5,7 +5,7 @@
 // A warp stages its configuration's world link poses (config-major, written by
 // the tree kernel) into shared memory with vector loads, places the spheres
 // (c_s = R_l c_local + p_l, Sec. 6.1.1) as SoA arrays -- column copies x, y,
-// z, N = |c|^2 - r^2 and row copies pre-scaled by -2 -- and writes the
+// z (the full map-reduce also N = |c|^2 - r^2 and row copies pre-scaled by -2) -- and writes the
 // sphere output.  The pair blocks (4x4 sphere groups, dealt by the host so
 // that the 8 lanes of a shared-memory phase read distinct bank groups, rows
 // kept per lane in runs) are then screened with
@@ -38,7 +38,8 @@ __host__ __device__ constexpr int a32(int x) { return (x + 31) & ~31; }
 struct PairPlan {  // per warp, 32-bit words
   int xr, yr, zr, xc, yc, zc, nn, gb, q, bits, total;
   __host__ __device__ int ra_words() const { return xc; }  // the row (and pose) region
-  __host__ __device__ PairPlan(int n, int Sg, int P, bool with_bits) {
+  // full: the full map-reduce, which keeps |c|^2 - r^2 of every sphere
+  __host__ __device__ PairPlan(int n, int Sg, int P, bool with_bits, bool full) {
     const int m = a32(4 * Sg);
     const int ra = 3 * m > a32(12 * n) ? 3 * m : a32(12 * n);  // rows; poses while staging
     xr = 0;
@@ -48,16 +49,16 @@ struct PairPlan {  // per warp, 32-bit words
     yc = ra + m;
     zc = ra + 2 * m;
     nn = ra + 3 * m;
-    gb = ra + 4 * m;  // group bounding spheres (float4 per group), culling only
+    gb = ra + (full ? 4 : 3) * m;  // group bounding spheres (float4 per group), culling only
     q = gb + m;       // queue of surviving schedule entries (64), culling only
     bits = q + 64;
     total = bits + (with_bits ? a32((P + 31) / 32) : 0);
   }
 };
 
-inline size_t pair_smem(const DevRobot& r, int warps, bool bits) {
+inline size_t pair_smem(const DevRobot& r, int warps, bool bits, bool full) {
   return sizeof(float) *
-         ((size_t)a32(4 * r.Sg) + (size_t)warps * PairPlan(r.n, r.Sg, r.P, bits).total);
+         ((size_t)a32(4 * r.Sg) + (size_t)warps * PairPlan(r.n, r.Sg, r.P, bits, full).total);
 }
 
 // approximate square root (relative error at most 2^-23)
@@ -101,7 +102,7 @@ template <bool FULL, bool BITS>
 __device__ __forceinline__ void pair_one(const DevRobot& r, const PairSchedule32& ps,
                                          const FwdArgs& A, int64_t b, float* ws,
                                          const float4* radw, int lane) {
-  const PairPlan pl(r.n, r.Sg, r.P, BITS);
+  const PairPlan pl(r.n, r.Sg, r.P, BITS, true);
   float* xr = ws + pl.xr;
   float* yr = ws + pl.yr;
   float* zr = ws + pl.zr;
@@ -344,19 +345,17 @@ template <bool FULL, bool BITS>
 __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSchedule32& ps,
                                                 const FwdArgs& A, int64_t b, float* ws,
                                                 const float4* radw, int lane) {
-  const PairPlan pl(r.n, r.Sg, r.P, BITS);
+  const PairPlan pl(r.n, r.Sg, r.P, BITS, false);
   float* xr = ws + pl.xr;
   float* xc = ws + pl.xc;
   float* yc = ws + pl.yc;
   float* zc = ws + pl.zc;
-  float* nn = ws + pl.nn;
   float4* gb = reinterpret_cast<float4*>(ws + pl.gb);
   uint32_t* qu = reinterpret_cast<uint32_t*>(ws + pl.q);
   uint32_t* bm = reinterpret_cast<uint32_t*>(ws + pl.bits);
   const char* cxc = reinterpret_cast<const char*>(xc);
   const char* cyc = reinterpret_cast<const char*>(yc);
   const char* czc = reinterpret_cast<const char*>(zc);
-  const char* cnn = reinterpret_cast<const char*>(nn);
   const char* crad = reinterpret_cast<const char*>(radw);
   const int n = r.n, S = r.S, Sg = r.Sg;
   const int W = (r.P + 31) >> 5;
@@ -391,22 +390,25 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
       const float4* T4 = reinterpret_cast<const float4*>(xr) + 3 * gl;  // the staged pose
       const float4 t0 = T4[0], t1 = T4[1], t2 = T4[2];
       const float T[12] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w, t2.x, t2.y, t2.z, t2.w};
-      float cx[4], cy[4], cz[4], nv[4];
+      // the 4 centres by coordinate: the lanes' loads are contiguous (a group's
+      // own 4 float4 are 64 bytes apart, 16 lines a load)
+      const float4 lx = __ldg(r.sph_t + g), ly = __ldg(r.sph_t + Sg + g),
+                   lz = __ldg(r.sph_t + 2 * Sg + g);
+      const float px[4] = {lx.x, lx.y, lx.z, lx.w}, py[4] = {ly.x, ly.y, ly.z, ly.w},
+                  pz[4] = {lz.x, lz.y, lz.z, lz.w};
+      float cx[4], cy[4], cz[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const float4 sp = __ldg(r.sph + 4 * g + q);
-        const float cl[3] = {sp.x, sp.y, sp.z};
+        const float cl[3] = {px[q], py[q], pz[q]};
         float c[3];
         rot(T, cl, c);
         cx[q] = c[0] + T[9];
         cy[q] = c[1] + T[10];
         cz[q] = c[2] + T[11];
-        nv[q] = fmaf(-sp.w, sp.w, fmaf(cz[q], cz[q], fmaf(cy[q], cy[q], cx[q] * cx[q])));
       }
       reinterpret_cast<float4*>(xc)[g] = make_float4(cx[0], cx[1], cx[2], cx[3]);
       reinterpret_cast<float4*>(yc)[g] = make_float4(cy[0], cy[1], cy[2], cy[3]);
       reinterpret_cast<float4*>(zc)[g] = make_float4(cz[0], cz[1], cz[2], cz[3]);
-      reinterpret_cast<float4*>(nn)[g] = make_float4(nv[0], nv[1], nv[2], nv[3]);
       if (so) {
         const float o[12] = {cx[0], cy[0], cz[0], cx[1], cy[1], cz[1],
                              cx[2], cy[2], cz[2], cx[3], cy[3], cz[3]};
@@ -433,7 +435,6 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
   } else {
     for (int s = lane; s < 4 * Sg; s += 32) {
       float c[3] = {0.0f, 0.0f, 0.0f};
-      float rs = 0.0f;
       if (s < S) {
         const float4 sp = __ldg(r.sph + s);
         // the link's staged pose as three vector loads (48-byte rows)
@@ -445,7 +446,6 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
         c[0] += P[9];
         c[1] += P[10];
         c[2] += P[11];
-        rs = sp.w;
         if (A.sph) {
           float* o = A.sph + (b * S + s) * 3;
           o[0] = c[0];
@@ -456,7 +456,6 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
       xc[s] = c[0];
       yc[s] = c[1];
       zc[s] = c[2];
-      nn[s] = fmaf(-rs, rs, fmaf(c[2], c[2], fmaf(c[1], c[1], c[0] * c[0])));  // |c|^2 - r^2
     }
     __syncwarp();
     for (int g = lane; g < Sg; g += 32) {  // group bounding spheres
@@ -523,7 +522,7 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
   // blocks' offsets decoded by the host, null blocks against a far sphere in
   // place of a test, the smallest bound carried with its round in its low 11
   // bits, and two bounds compared an instruction in pass 2: humanoid48 pair
-  // stage 0.117 -> 0.105 ms at 32768 configurations.
+  // stage 0.117 -> 0.105 ms at 32768 configurations (0.097 with the wavefronts saved below).
   const int prs = ps.prs;
   const bool keep_lb = prs * 32 <= pl.ra_words();
   __half2* lb2 = reinterpret_cast<__half2*>(xr) + lane;
@@ -587,17 +586,24 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
     const float4 XR = make_float4(-2.0f * XC.x, -2.0f * XC.y, -2.0f * XC.z, -2.0f * XC.w);
     const float4 YR = make_float4(-2.0f * YC.x, -2.0f * YC.y, -2.0f * YC.z, -2.0f * YC.w);
     const float4 ZR = make_float4(-2.0f * ZC.x, -2.0f * ZC.y, -2.0f * ZC.z, -2.0f * ZC.w);
-    const float4 RR = lds4(crad, ro), NI = lds4(cnn, ro);
-    const float4 CC = make_float4(fmaf(RR.x, RR.x, NI.x), fmaf(RR.y, RR.y, NI.y),
-                                  fmaf(RR.z, RR.z, NI.z), fmaf(RR.w, RR.w, NI.w));  // |c_i|^2
+    const float4 RR = lds4(crad, ro);
+    // |c|^2 formed here, for the blocks that are screened: keeping it for every
+    // sphere cost two more shared loads a block and a store a sphere where
+    // shared-memory wavefronts are what bounds the kernel
+    auto norm2 = [](float x, float y, float z) { return fmaf(z, z, fmaf(y, y, x * x)); };
+    const float4 CC = make_float4(norm2(XC.x, YC.x, ZC.x), norm2(XC.y, YC.y, ZC.y),
+                                  norm2(XC.z, YC.z, ZC.z), norm2(XC.w, YC.w, ZC.w));  // |c_i|^2
     const float bb = fminf(best, gbest) + margin;
     const float T[4] = {fmaxf(bb + RR.x, nrmin), fmaxf(bb + RR.y, nrmin),
                         fmaxf(bb + RR.z, nrmin), fmaxf(bb + RR.w, nrmin)};
     const float C4[4] = {CC.x, CC.y, CC.z, CC.w};
     const float xr4[4] = {XR.x, XR.y, XR.z, XR.w}, yr4[4] = {YR.x, YR.y, YR.z, YR.w},
                 zr4[4] = {ZR.x, ZR.y, ZR.z, ZR.w};
-    const float4 X = lds4(cxc, co), Y = lds4(cyc, co), Z = lds4(czc, co), N = lds4(cnn, co),
-                 Rc = lds4(crad, co);
+    const float4 X = lds4(cxc, co), Y = lds4(cyc, co), Z = lds4(czc, co), Rc = lds4(crad, co);
+    const float4 N = make_float4(fmaf(-Rc.x, Rc.x, norm2(X.x, Y.x, Z.x)),
+                                 fmaf(-Rc.y, Rc.y, norm2(X.y, Y.y, Z.y)),
+                                 fmaf(-Rc.z, Rc.z, norm2(X.z, Y.z, Z.z)),
+                                 fmaf(-Rc.w, Rc.w, norm2(X.w, Y.w, Z.w)));  // |c_j|^2 - r_j^2
     const float xj[4] = {X.x, X.y, X.z, X.w}, yj[4] = {Y.x, Y.y, Y.z, Y.w},
                 zj[4] = {Z.x, Z.y, Z.z, Z.w}, nj[4] = {N.x, N.y, N.z, N.w},
                 rj[4] = {Rc.x, Rc.y, Rc.z, Rc.w};

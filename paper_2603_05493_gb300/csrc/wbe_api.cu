@@ -766,6 +766,14 @@ int wb_load_robot(const wb_tree* tree, const wb_spheres* sph, const wb_pairs* pa
   pk.add_vec(H.ls_sph, &D.ls_sph);
   pk.add_vec(H.sp, &D.sph);
   pk.add_vec(H.sph_link, &D.sph_link);
+  std::vector<float4> sph_t(3 * (size_t)std::max(H.Sg, 1), make_float4(0, 0, 0, 0));
+  for (int s2 = 0; s2 < H.S; ++s2) {
+    const float4 c = H.sp[s2];
+    const float xyz[3] = {c.x, c.y, c.z};
+    for (int k = 0; k < 3; ++k)
+      reinterpret_cast<float*>(&sph_t[(size_t)k * H.Sg + s2 / 4])[s2 % 4] = xyz[k];
+  }
+  pk.add_vec(sph_t, &D.sph_t);
   pk.add_vec(H.pairs_dev, &D.pairs);
   pk.add_vec(H.grp_rad, &D.grp_rad);
   pk.add_vec(H.grp_loc, &D.grp_loc);

@@ -71,6 +71,7 @@ struct DevRobot {
   // spheres and pairs
   const float4* sph;         // [S] centre in link frame (xyz), radius (w)
   const int16_t* sph_link;   // [S]
+  const float4* sph_t;       // [3][Sg] the groups' centres by coordinate (x, y, z of 4 spheres, 0 pad)
   const int2* pairs;         // [P] sorted row-major
   const float4* grp_rad;     // [Sg] radii of the 4 spheres of a group (0 pad)
   const float4* grp_loc;     // [Sg] bounding sphere of a one-link group in its link frame
@@ -329,7 +330,7 @@ cudaError_t allow_smem(const void* kern, size_t smem);
 cudaError_t max_blocks(const void* kern, int threads, size_t smem, int* out);
 void launch_cache_clear(int device);
 int tree_max_depth();
-size_t pair_smem(const DevRobot& r, int warps, bool bits);
+
 size_t pair_block_smem(const DevRobot& r, int warps, bool bits);  // the same, out of line
 cudaError_t launch_pair(const DevRobot& r, const PairSchedule32& ps, const FwdArgs& a, int grid,
                         int warps, cudaStream_t s, bool cull = true);
