@@ -73,10 +73,14 @@ __device__ __forceinline__ float p4(const float4& v, int i) {
   return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w));
 }
 
-// Three 8-warp blocks an SM (24 warps; the slots share the pose region, so
-// three blocks' workspaces fit): 80 registers a thread (humanoid trajopt48
-// hinge 0.337 -> 0.281 ms against two blocks at 122 registers).
-__global__ void __launch_bounds__(256, 3) hinge_kernel(DevRobot r, PairSchedule32 ps, HingeArgs A) {
+// 24 warps an SM (the slots share the pose region, so their workspaces fit):
+// 80 registers a thread (against 16 warps at 122 registers: 0.337 -> 0.281 ms on
+// the humanoid's 32768 configurations).
+// FULL: every block holds all 16 pairs.
+template <bool FULL>
+__global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ DevRobot r,
+                                                       const __grid_constant__ PairSchedule32 ps,
+                                                       const __grid_constant__ HingeArgs A) {
   extern __shared__ __align__(16) float smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
   const int n = r.n, S = r.S, Sg = r.Sg;
@@ -256,7 +260,7 @@ __global__ void __launch_bounds__(256, 3) hinge_kernel(DevRobot r, PairSchedule3
           for (int k = 0; k < 12; ++k) gr[k] = gc[k] = 0.0f;
 #pragma unroll
           for (int t = 0; t < 16; ++t) {
-            if (!((mask >> t) & 1u)) continue;
+            if (!FULL && !((mask >> t) & 1u)) continue;
             const int ia = t >> 2, jc = t & 3;
             const float dx = p4(XR, ia) - p4(XC, jc), dy = p4(YR, ia) - p4(YC, jc),
                         dz = p4(ZR, ia) - p4(ZC, jc);
@@ -283,6 +287,8 @@ __global__ void __launch_bounds__(256, 3) hinge_kernel(DevRobot r, PairSchedule3
         }
         // add the slots into the spheres' gradients: the row groups, then the
         // column groups, each group's slots by their lowest lane in lane order
+        // (shared among the lanes that hold them, a component each, the sums were
+        // slower: 0.091 -> 0.120 ms)
 #pragma unroll
         for (int side = 0; side < 2; ++side) {
           if (side == 1 && lane < count) {
@@ -327,22 +333,27 @@ __global__ void __launch_bounds__(256, 3) hinge_kernel(DevRobot r, PairSchedule3
   }
 }
 
+static const void* hinge_of(const DevRobot& r) {
+  return r.all_full ? (const void*)hinge_kernel<true> : (const void*)hinge_kernel<false>;
+}
+
 cudaError_t launch_hinge(const DevRobot& r, const PairSchedule32& ps, const HingeArgs& a, int grid,
                          int warps, cudaStream_t s) {
   const size_t smem = hinge_block_smem(r, warps);
-  cudaError_t e =
-      allow_smem((const void*)hinge_kernel, smem);
+  const cudaError_t e = allow_smem(hinge_of(r), smem);
   if (e != cudaSuccess) return e;
-  hinge_kernel<<<grid, warps * 32, smem, s>>>(r, ps, a);
+  if (r.all_full)
+    hinge_kernel<true><<<grid, warps * 32, smem, s>>>(r, ps, a);
+  else
+    hinge_kernel<false><<<grid, warps * 32, smem, s>>>(r, ps, a);
   return cudaGetLastError();
 }
 
 cudaError_t hinge_max_blocks_per_sm(const DevRobot& r, int warps, int* out) {
   const size_t smem = hinge_block_smem(r, warps);
-  cudaError_t e =
-      allow_smem((const void*)hinge_kernel, smem);
+  const cudaError_t e = allow_smem(hinge_of(r), smem);
   if (e != cudaSuccess) return e;
-  return max_blocks((const void*)hinge_kernel, warps * 32, smem, out);
+  return max_blocks(hinge_of(r), warps * 32, smem, out);
 }
 
 }  // namespace wbe
