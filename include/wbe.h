@@ -133,11 +133,11 @@ typedef struct {
                                 per configuration, G > 1 = G warps per 32
                                 configurations, each sweeping a contiguous piece
                                 of the depth-first order (not for robots where a
-                                joint drives several links); 0 = the fewest that
-                                give about 12 warps per SM */
+                                joint drives several links); 0 = by the batch's
+                                warps per SM and the segments' lengths */
   int32_t configs_per_block; /* fused: configurations per CTA; tree: threads per block
                                 of the sweep kernels (32..256, up to 512 for
-                                G > 1 segments); 0 = default */
+                                G > 1 segments); 0 = by the batch's share per SM */
   int32_t blocks_per_sm;     /* fused: grid = blocks_per_sm * SMs (0 = occupancy);
                                 tree: warps per block of the pair kernel, 1..8
                                 (0 = of the counts 4..8 whose per-warp

@@ -65,6 +65,7 @@ struct wb_robot {
   int num_sms = 0;
   DevRobot dev{};
   WalkTab walk{};             // the sweeps' walk words (a kernel argument)
+  float seg_cost[4] = {0, 0, 0, 0};  // links a sweep walks in 1, 2, 4, 8 segments
   void* dmem = nullptr;
   size_t dbytes = 0;
   float* d_inert = nullptr;   // device inertia array (inside dmem)
@@ -228,6 +229,7 @@ struct HostPlan {
   std::vector<int16_t> dfs_pos, dfs_end, seg_slot, seg_slot_link;
   int seg_ok = 0;
   int seg_ns[3] = {0, 0, 0};
+  float seg_cost[3] = {0, 0, 0};  // the plan's largest segment, in links
   int16_t seg_pos[3][9] = {};
 };
 
@@ -275,6 +277,7 @@ static void plan_segments(HostPlan& H, int t) {
     }
   }
   H.seg_ns[t] = ns;
+  H.seg_cost[t] = (float)best[at(G, n)];
   H.seg_ok |= 1 << t;
 }
 
@@ -722,6 +725,8 @@ int wb_load_robot(const wb_tree* tree, const wb_spheres* sph, const wb_pairs* pa
   pk.add_vec(H.recs, &D.recs);
   pk.add_vec(H.walk, &D.walk);
   std::copy(H.walk.begin(), H.walk.end(), R->walk.w);
+  R->seg_cost[0] = (float)n;
+  for (int t = 0; t < 3; ++t) R->seg_cost[t + 1] = H.seg_cost[t];
   pk.add_vec(H.chain_start, &D.chain_start);
   pk.add_vec(H.chain, &D.chain);
   D.maxdepth = H.maxdepth;
@@ -996,15 +1001,56 @@ static int pair_warps(wb_robot* R, bool bits, const wb_tune* tune, bool cull = t
 }
 
 // Segments of the sweep kernels (wb_tune.lanes_per_config for TREE): 1, 2, 4
-// or 8; 0 = the fewest of the robot's plans that give about 12 warps per SM --
-// measured on the 48-DoF humanoid at 32768 configurations: both passes best
-// at 2 segments (the register copies of the stack top make each warp
-// faster, so fewer segments suffice), 8 slower than 1.
-// *tpb: the block's threads, lowered where the link records no longer leave
-// room for the partials of all its groups.
+// or 8; 0 = the plan with the least estimated time.  A sweep's time is the
+// links a warp walks times the time of one, which grows with the warps that
+// share the SM: (10 + w) in units of one warp's issue time (humanoid: 1.5 us +
+// 0.16 us a resident warp in the backward, 0.8 + 0.11 in the forward), w at
+// most 16 (the registers of an SM), passes beyond that after one another.
+// Against the fewest segments that give 12 warps an SM, forward / backward ms:
+// humanoid 12000 configurations 0.031 / 0.047 (was 0.042 / 0.062), 20011 0.045 /
+// 0.080 (0.055 / 0.091), 40000 0.084 / 0.131 (0.102 / 0.150), 50000 0.090 / 0.134
+// (0.116 / 0.165); 7-DoF arm 20000 0.011 / 0.017 (0.019 / 0.026); no change at
+// 9150, 32768 and 99999.
+template <class Fits>
+static int auto_segments(const wb_robot* R, int64_t B, Fits&& fits) {
+  const double per_sm = (double)((B + 31) / 32) / std::max(R->num_sms, 1);
+  int best = 1;
+  double least = 0.0;
+  for (int t = 0; t < 4; ++t) {
+    if (t > 0 && (!(R->dev.seg_ok >> (t - 1) & 1) || !fits(1 << t))) continue;
+    const double w = per_sm * (1 << t), full = std::floor(w / 16.0), rest = w - 16.0 * full;
+    const double time =
+        R->seg_cost[t] * (full * 26.0 + (rest > 0.0 ? 10.0 + std::max(rest, 1.0) : 0.0));
+    if (t == 0 || time < least) {
+      least = time;
+      best = 1 << t;
+    }
+  }
+  return best;
+}
+// Threads per block of a sweep when the tune gives none: at 2 and 4 segments
+// one block an SM with an even share of the batch's groups, while it fits
+// (humanoid 32768 configurations: 448 threads, forward 0.062 -> 0.058,
+// backward 0.098 -> 0.093 ms against 128; 20011: 320 threads, 0.080 -> 0.076
+// ms), else 128.
+static int auto_threads(const wb_robot* R, int64_t B, int G, bool fwd, bool spline) {
+  if (G != 2 && G != 4) return 128;
+  const int64_t groups = (B + 31) / 32;
+  const int64_t cg = (groups + R->num_sms - 1) / std::max(R->num_sms, 1);
+  const int64_t threads = 32 * G * cg;
+  if (threads > 512) return 128;
+  const size_t smem = tree_seg_smem(R->dev, G, (int)threads, fwd, !fwd) +
+                      (fwd ? sizeof(float) * 6 * (size_t)R->dev.maxdepth * threads
+                           : grad_slot_smem(G, (int)threads)) +
+                      (spline ? 12 * sizeof(float) * (size_t)threads : 0);
+  return smem <= kMaxBlockSmem ? (int)threads : 128;
+}
+
+// The segments (*out) and threads per block (*tpb, 0 = automatic on entry) of a
+// sweep; the threads are lowered where the link records no longer leave room
+// for the partials of all the block's groups.
 static int tree_segments(const wb_robot* R, const wb_tune* tune, int64_t B, int* tpb,
                          bool fwd, int* out, bool spline = false) {
-  const int threads = *tpb;
   const int req = tune ? tune->lanes_per_config : 0;
   const int ok = R->dev.seg_ok;
   int G = 1;
@@ -1015,28 +1061,32 @@ static int tree_segments(const wb_robot* R, const wb_tune* tune, int64_t B, int*
       return fail(WB_EINVAL, "no %d-segment sweep for this robot (fewer links, or a joint "
                   "driving several links)", req);
     G = req;
-  } else {
+  } else {  // the fewest that give about 12 warps per SM: what a call is held to
     const int64_t warps = (B + 31) / 32;
     const int64_t target = 12LL * R->num_sms;
     for (int t = 0; t < 3 && warps * G < target; ++t)
       if (ok >> t & 1) G = 2 << t;
   }
+  const int threads = *tpb ? *tpb : 128;
   if (G == 1 && threads > 256)
     return fail(WB_EINVAL, "one-segment sweeps take at most 256 threads per block");
   // what a block needs: refused from the limit up, counting 28 floats a link
   // record; the records' padding to kRecWords, the backward's spheres and the
   // spline backward's basis rows beside its slots are made room for
   const size_t basis = spline && !fwd ? 12 * sizeof(float) : 0;  // a thread's basis rows
-  auto need = [&](int threads_) {
-    return tree_seg_smem(R->dev, G, threads_, fwd, !fwd) +
-           (fwd ? 0 : grad_slot_smem(G, threads_)) + basis * std::max(threads_, 32 * G);
+  auto need = [&](int G_, int threads_) {
+    return tree_seg_smem(R->dev, G_, threads_, fwd, !fwd) +
+           (fwd ? 0 : grad_slot_smem(G_, threads_)) + basis * std::max(threads_, 32 * G_);
   };
   const size_t more = sizeof(float) * ((kRecWords - 28) * (size_t)R->dev.n +
                                        (fwd ? 0 : 4 * (size_t)R->dev.S)) +
                       basis * std::max(threads, 32 * G);
-  if (G > 1 && need(threads) - more > kMaxBlockSmem)
+  if (G > 1 && need(G, threads) - more > kMaxBlockSmem)
     return fail(WB_ETOOBIG, "segmented sweep needs too much shared memory");
-  while (G > 1 && need(*tpb) > kMaxBlockSmem) {
+  if (req <= 0 && threads <= 256)
+    G = auto_segments(R, B, [&](int g) { return need(g, threads) <= kMaxBlockSmem; });
+  if (*tpb == 0) *tpb = auto_threads(R, B, G, fwd, spline);
+  while (G > 1 && need(G, *tpb) > kMaxBlockSmem) {
     if (*tpb >= 64 * G)
       *tpb -= 32 * G;
     else
@@ -1109,8 +1159,8 @@ int wb_eval_dir(wb_robot* robot, int64_t B, const float* q, const float* qd, con
     if (!tree_ok) return fail(WB_ETOOBIG, "tree deeper than %d levels", tree_max_depth());
     if (pairs_wanted && !link_pose)
       return fail(WB_EINVAL, "the tree kernel needs link_pose when spheres or pairs are wanted");
-    int tpb = (tune && tune->configs_per_block) ? tune->configs_per_block : 128;
-    if (tpb < 32 || tpb > 512 || tpb % 32)
+    int tpb = tune ? tune->configs_per_block : 0;  // 0 = automatic
+    if (tpb != 0 && (tpb < 32 || tpb > 512 || tpb % 32))
       return fail(WB_EINVAL, "tree threads per block must be a multiple of 32 in [32, 512]");
     const int warps = pair_warps(robot, pair_bits != nullptr, tune, cull);
     if (tune && tune->blocks_per_sm && (warps < 1 || warps > 8))
@@ -1338,8 +1388,8 @@ int wb_eval_backward_dir(wb_robot* robot, int64_t B, const float* q, const float
     e = launch_plain_bwd(robot->dev, a, 128, s);
   } else if (kernel == WB_KERNEL_TREE) {
     if (!tree_ok) return fail(WB_ETOOBIG, "tree deeper than %d levels", tree_max_depth());
-    int tpb = (tune && tune->configs_per_block) ? tune->configs_per_block : 128;
-    if (tpb < 32 || tpb > 512 || tpb % 32)
+    int tpb = tune ? tune->configs_per_block : 0;  // 0 = automatic
+    if (tpb != 0 && (tpb < 32 || tpb > 512 || tpb % 32))
       return fail(WB_EINVAL, "tree threads per block must be a multiple of 32 in [32, 512]");
     int G = 1;
     if ((rc = tree_segments(robot, tune, B, &tpb, false, &G))) return rc;
@@ -1403,11 +1453,11 @@ int wb_eval_spline(wb_robot* robot, const wb_spline* spline, float* link_pose, f
   DeviceGuard guard(robot->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   FwdArgs a{B, nullptr, nullptr, nullptr, link_pose, sphere, d_min, worst_pair, tau, nullptr};
-  int tpb = (tune && tune->configs_per_block) ? tune->configs_per_block : 128;
-  if (tpb < 32 || tpb > 512 || tpb % 32)
+  int tpb = tune ? tune->configs_per_block : 0;  // 0 = automatic
+  if (tpb != 0 && (tpb < 32 || tpb > 512 || tpb % 32))
     return fail(WB_EINVAL, "tree threads per block must be a multiple of 32 in [32, 512]");
   int G = 1;
-  if ((rc = tree_segments(robot, tune, B, &tpb, true, &G))) return rc;
+  if ((rc = tree_segments(robot, tune, B, &tpb, true, &G, true))) return rc;
   cudaError_t e = launch_tree_fwd_spline(robot->dev, robot->walk, a, sp, tpb, G, s);
   if (e == cudaSuccess && pairs_wanted) {
     const int warps = pair_warps(robot, false, tune, kernel != WB_KERNEL_TREE_NOCULL);
@@ -1491,8 +1541,8 @@ int wb_eval_backward_spline_cost_dir(wb_robot* robot, const wb_spline* spline,
   fc.length = W.length;
   fc.e = W.energy * W.dt * W.dt;
   fc.cost = cost;
-  int tpb = (tune && tune->configs_per_block) ? tune->configs_per_block : 128;
-  if (tpb < 32 || tpb > 512 || tpb % 32)
+  int tpb = tune ? tune->configs_per_block : 0;  // 0 = automatic
+  if (tpb != 0 && (tpb < 32 || tpb > 512 || tpb % 32))
     return fail(WB_EINVAL, "tree threads per block must be a multiple of 32 in [32, 512]");
   int G = 1;
   if ((rc = tree_segments(robot, tune, B, &tpb, false, &G, true))) return rc;
@@ -1568,8 +1618,8 @@ int wb_eval_backward_cost_dir(wb_robot* robot, int64_t B, const float* q, const 
   fc.length = W.length;
   fc.e = W.energy * W.dt * W.dt;
   fc.cost = cost;
-  int tpb = (tune && tune->configs_per_block) ? tune->configs_per_block : 128;
-  if (tpb < 32 || tpb > 512 || tpb % 32)
+  int tpb = tune ? tune->configs_per_block : 0;  // 0 = automatic
+  if (tpb != 0 && (tpb < 32 || tpb > 512 || tpb % 32))
     return fail(WB_EINVAL, "tree threads per block must be a multiple of 32 in [32, 512]");
   int G = 1;
   if ((rc = tree_segments(robot, tune, B, &tpb, false, &G))) return rc;
