@@ -15,6 +15,8 @@
 // 1/(T-1) away from the next integer) and alpha = remainder / (T-1).
 #include "spline_basis.cuh"
 
+#include <algorithm>
+
 namespace wbe {
 
 // Boundary conditions (Sec. 4.2).  The spline is evaluated on an extended
@@ -77,51 +79,83 @@ __global__ void __launch_bounds__(256) bspline_fwd_kernel(int64_t n_traj, int d,
 
 // Gradient of extended knot x of one (trajectory, joint): the sum of
 // B(alpha_s)^T g_s over the samples of segments x-3 .. x in sample order.
-struct KnotGrad {
-  const float* tab;  // [T][12] basis rows
-  const int* first;  // [nseg + 1] first sample of each segment
-  int nseg;
-  const float *gq, *gqd, *gqdd, *gqd2, *gqdd2;  // already offset to (joint, trajectory)
-  __device__ __forceinline__ float operator()(int x) const {
-    const int m0 = max(x - 3, 0), m1 = min(x, nseg - 1);
-    float acc = 0.0f;
-    if (m0 <= m1) {
-      int m = m0;
-      for (int s = first[m0]; s < first[m1 + 1]; ++s) {
-        while (s >= first[m + 1]) ++m;  // segment of sample s
-        const int l = x - m;            // this knot's place in the window
-        const float* Bs = tab + s * 12;
-        float c = 0.0f;
-        if (gq) c = fmaf(Bs[l], __ldg(gq + s), c);
-        float gv = gqd ? __ldg(gqd + s) : 0.0f;  // the two qd gradients add
-        if (gqd2) gv += __ldg(gqd2 + s);
-        c = fmaf(Bs[4 + l], gv, c);
-        float ga = gqdd ? __ldg(gqdd + s) : 0.0f;
-        if (gqdd2) ga += __ldg(gqdd2 + s);
-        c = fmaf(Bs[8 + l], ga, c);
-        acc += c;
-      }
+// g.q(s), g.v(s), g.a(s): the row's gradients of q, qd, qdd at sample s.
+template <class G>
+__device__ __forceinline__ float knot_grad(const float* tab, const int* first, int nseg, int T,
+                                           int x, const G& g) {
+  const int m0 = max(x - 3, 0), m1 = min(x, nseg - 1);
+  float acc = 0.0f;
+  int s = m0 <= m1 ? first[m0] : 0;
+  for (int m = m0; m <= m1; ++m) {
+    const int s1 = first[m + 1];
+    const float* Bs = tab + (x - m) * T;  // this knot's place in the window; [3][4][T]
+#pragma unroll 2
+    for (; s < s1; ++s) {
+      float c = fmaf(Bs[s], g.q(s), 0.0f);
+      c = fmaf(Bs[4 * T + s], g.v(s), c);
+      c = fmaf(Bs[8 * T + s], g.a(s), c);
+      acc += c;
     }
-    return acc;
   }
+  return acc;
+}
+struct StagedRow {
+  const float *r0, *r1, *r2;
+  __device__ __forceinline__ float q(int s) const { return r0[s]; }
+  __device__ __forceinline__ float v(int s) const { return r1[s]; }
+  __device__ __forceinline__ float a(int s) const { return r2[s]; }
+};
+struct GlobalRow {  // nullptr: zero
+  const float *gq, *gqd, *gqdd, *gqd2, *gqdd2;
+  __device__ __forceinline__ static float sum(const float* a, const float* b, int64_t at) {
+    float v = a ? __ldg(a + at) : 0.0f;
+    if (b) v += __ldg(b + at);
+    return v;
+  }
+  int64_t at;
+  __device__ __forceinline__ float q(int s) const { return sum(gq, nullptr, at + s); }
+  __device__ __forceinline__ float v(int s) const { return sum(gqd, gqd2, at + s); }
+  __device__ __forceinline__ float a(int s) const { return sum(gqdd, gqdd2, at + s); }
 };
 
 // One thread per control point (trajectory, joint, k), plus with a start
 // state one per (trajectory, joint) for the start-state gradient (no atomics,
-// deterministic).  The basis rows and segment of every sample and the first
-// sample of every segment are tabled in shared memory per block.  With a
-// static goal the last control point also sums the gradients of its three
-// repeats; the start-state gradient is the transpose of the ghost knots'
-// linear map applied to their three gradients.
+// deterministic).  A block takes one joint of R consecutive trajectories; the
+// basis rows and segment of every sample and the first sample of every segment
+// are tabled in shared memory.  With a static goal the last control point also
+// sums the gradients of its three repeats; the start-state gradient is the
+// transpose of the ghost knots' linear map applied to their three gradients.
+// STAGE: the block's R T samples, contiguous in the [d][B] arrays, are read
+// once into shared memory (the two qd and the two qdd gradients added), where
+// each is used by four knots; else (a row too long for that) the threads read
+// them from global memory.  Bound by the latency of a knot's serial sum, which
+// reads shared instead of L2: humanoid 512 x 64 samples, 16 knots 0.020 -> 0.017
+// ms; an arm's 100 x 33 samples with both ends 0.0145 -> 0.0063 ms.
+// *dst (shared) = a[at] (+ b[at]), 0 where there is none: a lone array by an
+// asynchronous copy, so that all of a thread's samples are on their way at once
+__device__ __forceinline__ void stage(float* dst, const float* a, const float* b, int64_t at) {
+  if (a && !b) {
+    const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(a + at));
+  } else {
+    *dst = GlobalRow::sum(a, b, at);
+  }
+}
+
+// the stride of a staged row: rows of a multiple of 32 samples are set 16 banks apart
+__host__ __device__ constexpr int row_stride(int T) { return T % 32 == 0 ? T + 16 : T; }
+
+template <bool STAGE>
 __global__ void __launch_bounds__(256) bspline_bwd_kernel(
-    int64_t n_traj, int d, int K, int T, float dt, int hs, int es, const float* __restrict__ gq,
-    const float* __restrict__ gqd, const float* __restrict__ gqdd,
-    const float* __restrict__ gqd2, const float* __restrict__ gqdd2, float* gU,
-    float* gstart) {
-  extern __shared__ float tab[];  // [T][12] basis rows, then [Kx-2] first samples
+    int64_t n_traj, int d, int K, int T, float dt, int hs, int es, int R,
+    const float* __restrict__ gq, const float* __restrict__ gqd, const float* __restrict__ gqdd,
+    const float* __restrict__ gqd2, const float* __restrict__ gqdd2, float* gU, float* gstart) {
+  extern __shared__ float tab[];  // [12][T] basis rows, then [Kx-2] first samples
   int* first = reinterpret_cast<int*>(tab + (size_t)T * 12);
   const int Kx = K + 3 * hs + 3 * es;
   const int nseg = Kx - 3;
+  const int Tp = row_stride(T);
+  float* rows = tab + (size_t)T * 12 + ((Kx - 2 + 3) & ~3);  // STAGE: [3][nr][Tp]
   for (int s = threadIdx.x; s < T; s += blockDim.x) {
     int k;
     float a;
@@ -131,40 +165,60 @@ __global__ void __launch_bounds__(256) bspline_bwd_kernel(
 #pragma unroll
     for (int r = 0; r < 3; ++r)
 #pragma unroll
-      for (int l = 0; l < 4; ++l) tab[s * 12 + r * 4 + l] = Bm[r][l];
+      for (int l = 0; l < 4; ++l) tab[(r * 4 + l) * T + s] = Bm[r][l];
   }
   // first[m] = first sample of segment m = ceil(m (T-1) / nseg); first[nseg] = T
   for (int m = threadIdx.x; m <= nseg; m += blockDim.x)
     first[m] = m == nseg ? T : (m * (T - 1) + nseg - 1) / nseg;
-  __syncthreads();
   const int64_t B = n_traj * T;
-  const int per = K + hs;  // threads per (trajectory, joint)
-  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (idx >= n_traj * d * per) return;
-  const int64_t tj = idx / per;  // trajectory * d + joint
-  const int t = (int)(idx - tj * per);
-  const int64_t tr = tj / d;
-  const int j = (int)(tj - tr * d);
-  const int64_t base = (int64_t)j * B + tr * T;
-  const KnotGrad kg{tab, first, nseg, gq ? gq + base : nullptr, gqd ? gqd + base : nullptr,
-                    gqdd ? gqdd + base : nullptr, gqd2 ? gqd2 + base : nullptr,
-                    gqdd2 ? gqdd2 + base : nullptr};
-  if (t < hs) {  // the start-state gradient through u_-3, u_-2, u_-1
-    const float g3 = kg(0), g2 = kg(1), g1 = kg(2);
-    if (gstart) {
-      float* o = gstart + tj * 3;
-      o[0] = g3 + g2 + g1;
-      o[1] = dt * fmaf(2.0f, g1, g2);
-      o[2] = dt * dt * fmaf(11.0f / 6.0f, g1, fmaf(1.0f / 3.0f, g2, (-1.0f / 6.0f) * g3));
+  const uint32_t per_joint = (uint32_t)((n_traj + R - 1) / R);  // blocks of a joint
+  const int j = (int)(blockIdx.x / per_joint);
+  const int64_t tr0 = (int64_t)(blockIdx.x - j * per_joint) * R;
+  const int nr = (int)(n_traj - tr0 < R ? n_traj - tr0 : R);
+  const int64_t base = (int64_t)j * B + tr0 * T;
+  if (STAGE) {  // a warp a row
+    const int plane = nr * Tp;
+    for (int row = threadIdx.x >> 5; row < nr; row += blockDim.x >> 5) {
+      float* o = rows + row * Tp;
+      const int64_t at = base + (int64_t)row * T;
+      for (int s = threadIdx.x & 31; s < T; s += 32) {
+        stage(o + s, gq, nullptr, at + s);
+        stage(o + plane + s, gqd, gqd2, at + s);
+        stage(o + 2 * plane + s, gqdd, gqdd2, at + s);
+      }
     }
-    return;
+    asm volatile("cp.async.commit_group;");
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
   }
-  const int k = t - hs;
-  const int x = k + 3 * hs;
-  float acc = kg(x);
-  if (es && k == K - 1)
-    for (int r = 1; r <= 3; ++r) acc += kg(x + r);
-  gU[tj * K + k] = acc;
+  __syncthreads();
+  const int per = K + hs;  // threads per (trajectory, joint)
+  for (int i = threadIdx.x; i < nr * per; i += blockDim.x) {
+    const int row = i / per, t = i - row * per;
+    const int64_t tj = (tr0 + row) * d + j;  // trajectory * d + joint
+    const float* o = rows + row * Tp;
+    auto kg = [&](int x) {
+      if (STAGE)
+        return knot_grad(tab, first, nseg, T, x, StagedRow{o, o + nr * Tp, o + 2 * nr * Tp});
+      return knot_grad(tab, first, nseg, T, x,
+                       GlobalRow{gq, gqd, gqdd, gqd2, gqdd2, base + (int64_t)row * T});
+    };
+    if (t < hs) {  // the start-state gradient through u_-3, u_-2, u_-1
+      const float g3 = kg(0), g2 = kg(1), g1 = kg(2);
+      if (gstart) {
+        float* o = gstart + tj * 3;
+        o[0] = g3 + g2 + g1;
+        o[1] = dt * fmaf(2.0f, g1, g2);
+        o[2] = dt * dt * fmaf(11.0f / 6.0f, g1, fmaf(1.0f / 3.0f, g2, (-1.0f / 6.0f) * g3));
+      }
+      continue;
+    }
+    const int k = t - hs;
+    const int x = k + 3 * hs;
+    float acc = kg(x);
+    if (es && k == K - 1)
+      for (int r = 1; r <= 3; ++r) acc += kg(x + r);
+    gU[tj * K + k] = acc;
+  }
 }
 
 // One thread per configuration.  The motion terms of the loss (smooth |qdd|^2,
@@ -244,12 +298,24 @@ cudaError_t launch_bspline_bwd(int64_t n_traj, int d, int K, int T, float dt, in
                                const float* gqdd, const float* gqd2, const float* gqdd2,
                                float* gU, float* gstart, cudaStream_t s) {
   const int hs = has_start ? 1 : 0, es = end_static ? 1 : 0;
-  const size_t smem = bspline_bwd_smem(K + 3 * hs + 3 * es, T);
-  cudaError_t e = allow_smem((const void*)bspline_bwd_kernel, smem);
+  const int Kx = K + 3 * hs + 3 * es;
+  // trajectories a block: one knot a thread, while their samples fit beside the
+  // tables in 64 KB (rows of which not one does are read from global memory)
+  const size_t limit = 64 * 1024;
+  const size_t tables = sizeof(float) * ((size_t)T * 12 + ((Kx - 2 + 3) & ~3));
+  const size_t row = sizeof(float) * 3 * (size_t)row_stride(T);
+  const int64_t room = tables + row <= limit ? (int64_t)((limit - tables) / row) : 0;
+  const bool stage = room > 0;
+  const int64_t most = std::max(1, 256 / (K + hs));
+  const int R = (int)std::min<int64_t>({most, stage ? room : most, n_traj});
+  const int block = std::min(256, std::max(64, (R * (K + hs) + 31) / 32 * 32));
+  const size_t smem = stage ? tables + row * R : bspline_bwd_smem(Kx, T);
+  auto kern = stage ? bspline_bwd_kernel<true> : bspline_bwd_kernel<false>;
+  cudaError_t e = allow_smem((const void*)kern, smem);
   if (e != cudaSuccess) return e;
-  const int64_t n = n_traj * d * (K + hs);
-  bspline_bwd_kernel<<<(unsigned)((n + 255) / 256), 256, smem, s>>>(
-      n_traj, d, K, T, dt, hs, es, gq, gqd, gqdd, gqd2, gqdd2, gU, gstart);
+  const int64_t grid = (n_traj + R - 1) / R * d;
+  kern<<<(unsigned)grid, block, smem, s>>>(n_traj, d, K, T, dt, hs, es, R, gq, gqd, gqdd, gqd2,
+                                         gqdd2, gU, gstart);
   return cudaGetLastError();
 }
 
