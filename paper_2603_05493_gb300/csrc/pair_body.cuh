@@ -640,19 +640,56 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
       }
     }
     if (BITS && mask) {
+      // Colliding pairs: sqrt(d2) - (r_i + r_j) < 0.  The squares decide all but
+      // those within 2^-20 of touching, which take the square root.
+      uint32_t hit = 0u, near = 0u;
+      const float ri[4] = {RR.x, RR.y, RR.z, RR.w};
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+      for (int t = 0; t < 16; ++t) {
+        const int a = t >> 2, c = t & 3;
+        const float d2 = dist2(-0.5f * xr4[a], -0.5f * yr4[a], -0.5f * zr4[a], xj[c], yj[c], zj[c]);
+        const float rs = ri[a] + rj[c], r2 = rs * rs;
+        hit |= (d2 < r2 ? 1u : 0u) << t;
+        near |= (fabsf(d2 - r2) <= 9.6e-7f * r2 ? 1u : 0u) << t;
+      }
+      near &= mask;
+      while (near) {
+        const int t = __ffs(near) - 1;
+        near &= near - 1u;
+        const int a = t >> 2, c = t & 3;
+        const float d2 = dist2(reinterpret_cast<const float*>(cxc + ro)[a],
+                               reinterpret_cast<const float*>(cyc + ro)[a],
+                               reinterpret_cast<const float*>(czc + ro)[a],
+                               reinterpret_cast<const float*>(cxc + co)[c],
+                               reinterpret_cast<const float*>(cyc + co)[c],
+                               reinterpret_cast<const float*>(czc + co)[c]);
+        const float d = sqrtf(d2) - (reinterpret_cast<const float*>(crad + ro)[a] +
+                                     reinterpret_cast<const float*>(crad + co)[c]);
+        hit = (hit & ~(1u << t)) | ((d < 0.0f ? 1u : 0u) << t);
+      }
+      hit &= mask;
+      const int32_t* pix = r.blk_pidx + 16 * (e.y & 0xFFFF);
+      if (FULL) {
+        // the four pairs of a row sphere have consecutive indices: their bits
+        // are one shift, over at most two words
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          if ((mask >> (4 * a + c)) & 1u) {
-            const float d2 = dist2(-0.5f * xr4[a], -0.5f * yr4[a], -0.5f * zr4[a], xj[c], yj[c],
-                                   zj[c]);
-            if (sqrtf(d2) - (pick(RR, a) + rj[c]) < 0.0f) {
-              const int pidx = __ldg(r.blk_pidx + 16 * (e.y & 0xFFFF) + 4 * a + c);
-              atomicOr(bm + (pidx >> 5), 1u << (pidx & 31));
-            }
+        for (int a = 0; a < 4; ++a) {
+          const uint32_t h = (hit >> (4 * a)) & 15u;
+          if (h) {
+            const int p = __ldg(pix + 4 * a);
+            const uint64_t w = (uint64_t)h << (p & 31);
+            atomicOr(bm + (p >> 5), (uint32_t)w);
+            if (w >> 32) atomicOr(bm + (p >> 5) + 1, (uint32_t)(w >> 32));
           }
         }
+      } else {
+        while (hit) {
+          const int t = __ffs(hit) - 1;
+          hit &= hit - 1u;
+          const int p = __ldg(pix + t);
+          atomicOr(bm + (p >> 5), 1u << (p & 31));
+        }
+      }
     }
   };
   auto drain = [&](int count) {  // screen queue entries [0, count), one per lane
