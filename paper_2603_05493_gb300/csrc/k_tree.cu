@@ -21,6 +21,13 @@ __host__ __device__ __forceinline__ size_t bwd_words(const DevRobot& r) {
   return kRecWords * (size_t)r.n + 4 * (size_t)r.S;
 }
 
+// levels of the forward's force stack (one less would hold: the deepest level never
+// stores; but the fifth 128-thread block that then fits an SM takes its room from
+// L1: humanoid, 99999 configurations in one segment, 0.190 -> 0.206 ms)
+__host__ __device__ __forceinline__ size_t fs_levels(const DevRobot& r) {
+  return (size_t)r.maxdepth;
+}
+
 // this thread's warp, known to be the same for its whole warp
 __device__ __forceinline__ int warp_of() { return __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0); }
 
@@ -49,7 +56,7 @@ __global__ void __launch_bounds__(256) tree_fwd_kernel(const __grid_constant__ D
                                                        const __grid_constant__ FwdArgs A) {
   extern __shared__ float4 rec[];
   float* sm = reinterpret_cast<float*>(rec) + kRecWords * (size_t)r.n;
-  if (MODE == kFwdShared && !smem_holds(kRecWords * (size_t)r.n + 6 * (size_t)r.maxdepth * blockDim.x)) return;
+  if (MODE == kFwdShared && !smem_holds(kRecWords * (size_t)r.n + 6 * fs_levels(r) * blockDim.x)) return;
   stage_recs(r, -1, rec, threadIdx.x, blockDim.x);
   __syncthreads();
   int64_t b;
@@ -96,7 +103,7 @@ __device__ __forceinline__ Seg seg_of(const DevRobot& r, int t, int g, float* pa
              (int)(threadIdx.x & 31)};
 }
 
-// MODE kFwdShared: the force stack in shared memory, [maxdepth][3][threads] float2 behind
+// MODE kFwdShared: the force stack in shared memory, [fs_levels][3][threads] float2 behind
 // the partials (a link's F is stored when its first child is pushed
 // and read back at that child's close; in local memory these round trips
 // missed L1 61 % of the time)
@@ -115,7 +122,7 @@ __global__ void __launch_bounds__(512) tree_fwd_seg_kernel(const __grid_constant
   // finds less shared memory than that does nothing (its outputs stay
   // unwritten) instead of indexing past it
   if (MODE == kFwdShared && !smem_holds((size_t)CG * ns * G * 32 + kRecWords * (size_t)r.n +
-                        6 * (size_t)r.maxdepth * blockDim.x))
+                        6 * fs_levels(r) * blockDim.x))
     return;
   Seg sg = seg_of(r, t, wid % G, part + (size_t)cg * ns * G * 32);
   for (int s = 0; s < ns; ++s) sg.part[(s * G + sg.g) * 32 + sg.lane] = 0.0f;
@@ -301,7 +308,7 @@ __global__ void __launch_bounds__(512) tree_fwd_spline_seg_kernel(
   const int wid = warp_of(), cg = wid / G;
   const int ns = r.seg_ns[t];
   if (MODE == kFwdShared && !smem_holds(12 * (size_t)blockDim.x + (size_t)CG * ns * G * 32 +
-                        kRecWords * (size_t)r.n + 6 * (size_t)r.maxdepth * blockDim.x))
+                        kRecWords * (size_t)r.n + 6 * fs_levels(r) * blockDim.x))
     return;
   Seg sg = seg_of(r, t, wid % G, part + (size_t)cg * ns * G * 32);
   for (int s = 0; s < ns; ++s) sg.part[(s * G + sg.g) * 32 + sg.lane] = 0.0f;
@@ -593,13 +600,13 @@ cudaError_t launch_tree_fwd(const DevRobot& r, const WalkTab& wt, const FwdArgs&
     // humanoid's 13 levels x 448 threads: 140 KB; forward 0.0835 ->
     // 0.0809 ms), else in local memory
     const size_t bt = (size_t)32 * segments * seg_groups(segments, threads);
-    const size_t fs = sizeof(float) * 6 * (size_t)r.maxdepth * bt;
+    const size_t fs = sizeof(float) * 6 * fs_levels(r) * bt;
     if (a.tau && tree_seg_smem(r, segments, threads, true, false) + fs <= kSegSmemMax)
       return launch_seg(tree_fwd_seg_kernel<kFwdShared>, r, wt, a, threads, segments, true, fs, s);
     return launch_seg(a.tau ? tree_fwd_seg_kernel<kFwdLocal> : tree_fwd_seg_kernel<kFwdPose>, r, wt,
                       a, threads, segments, true, 0, s);
   }
-  const size_t fs = sizeof(float) * 6 * (size_t)r.maxdepth * threads;  // the force stack
+  const size_t fs = sizeof(float) * 6 * fs_levels(r) * threads;  // the force stack
   const bool use_fs = a.tau && rec_smem(r, true) + fs <= kSegSmemMax;
   const size_t smem = rec_smem(r, true) + (use_fs ? fs : 0);
   auto kern = use_fs ? tree_fwd_kernel<kFwdShared>
@@ -651,7 +658,7 @@ cudaError_t launch_tree_fwd_spline(const DevRobot& r, const WalkTab& wt, const F
     const int CG = seg_groups(segments, threads);
     const int block = 32 * segments * CG;
     const size_t base = tree_seg_smem(r, segments, threads, true, false) + 12 * sizeof(float) * block;
-    const size_t fs = sizeof(float) * 6 * (size_t)r.maxdepth * block;  // the force stack
+    const size_t fs = sizeof(float) * 6 * fs_levels(r) * block;  // the force stack
     const bool use_fs = a.tau && base + fs <= kSegSmemMax;
     const size_t smem = use_fs ? base + fs : base;
     auto kern = use_fs ? tree_fwd_spline_seg_kernel<kFwdShared>
