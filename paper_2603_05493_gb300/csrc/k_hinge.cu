@@ -63,12 +63,6 @@ static size_t hinge_block_smem(const DevRobot& r, int warps) {
 __device__ __forceinline__ float4 ld4(const char* base, uint32_t off) {
   return *reinterpret_cast<const float4*>(base + off);
 }
-// approximate square root (relative error at most 2^-23)
-__device__ __forceinline__ float approx_sqrt(float x) {
-  float y;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 __device__ __forceinline__ float p4(const float4& v, int i) {
   return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w));
 }
@@ -91,7 +85,7 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
   float* ws = smem + ((4 * Sg + 31) & ~31) + (size_t)warp * pl.total;
   float* P = ws;
   float *xc = ws + pl.xc, *yc = ws + pl.yc, *zc = ws + pl.zc;
-  float4* gb = reinterpret_cast<float4*>(ws + pl.gb);
+  uint2* gb = reinterpret_cast<uint2*>(ws + pl.gb);
   float *gx = ws + pl.gx, *gy = ws + pl.gy, *gz = ws + pl.gz;
   float* slot = ws;  // over the poses, once the spheres are placed
   uint32_t* qu = reinterpret_cast<uint32_t*>(ws + pl.q);
@@ -113,9 +107,12 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
       asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     __syncwarp();
+    // bounds relative to the first link, as in the pair stage
+    const float ox = P[9], oy = P[10], oz = P[11];
+    const float ow = fmaf(fabsf(ox) + fabsf(oy) + fabsf(oz), 1e-6f, 3e-6f);
     const float4 zero4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (lane == 0)  // the far sphere of the schedule's null blocks
-      *reinterpret_cast<float4*>(ws + pl.gb + far_words(Sg)) = make_float4(1e15f, 1e15f, 1e15f, 0.0f);
+      *reinterpret_cast<uint2*>(ws + pl.gb + far_words(Sg)) = half_bound(6e4f, 6e4f, 6e4f, 0.0f);
     if (r.sph_vec4) {
       // every group of 4 on one link: a lane a group places its centres, its
       // bound and its gradient rows' zeros from one pose
@@ -146,8 +143,8 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
         rot(T, cl, c);
         const float scale = fabsf(T[9]) + fabsf(T[10]) + fabsf(T[11]) + fabsf(L.x) +
                             fabsf(L.y) + fabsf(L.z);
-        gb[g] = make_float4(c[0] + T[9], c[1] + T[10], c[2] + T[11],
-                            fmaf(scale, 1e-6f, fmaf(L.w, 1e-6f, L.w)) + 3e-6f);
+        gb[g] = half_bound(c[0] + T[9] - ox, c[1] + T[10] - oy, c[2] + T[11] - oz,
+                           fmaf(scale, 1e-6f, fmaf(L.w, 1e-6f, L.w)) + ow);
         reinterpret_cast<float4*>(gx)[g] = zero4;
         reinterpret_cast<float4*>(gy)[g] = zero4;
         reinterpret_cast<float4*>(gz)[g] = zero4;
@@ -181,8 +178,8 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
         rot(T, cl, c);
         const float scale = fabsf(T[9]) + fabsf(T[10]) + fabsf(T[11]) + fabsf(L.x) +
                             fabsf(L.y) + fabsf(L.z);
-        B4 = make_float4(c[0] + T[9], c[1] + T[10], c[2] + T[11],
-                         fmaf(scale, 1e-6f, fmaf(L.w, 1e-6f, L.w)) + 3e-6f);
+        B4 = make_float4(c[0] + T[9] - ox, c[1] + T[10] - oy, c[2] + T[11] - oz,
+                         fmaf(scale, 1e-6f, fmaf(L.w, 1e-6f, L.w)) + ow);
       } else {
         const int s1 = min(S, 4 * g + 4);
         float cx = 0.0f, cy = 0.0f, cz = 0.0f;
@@ -199,9 +196,11 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
         float R = 0.0f;
         for (int s = 4 * g; s < s1; ++s)
           R = fmaxf(R, sqrtf(dist2(cx, cy, cz, xc[s], yc[s], zc[s])) + p4(rad, s - 4 * g));
-        B4 = make_float4(cx, cy, cz, fmaf(R, 1e-6f, R) + 3e-6f);  // widened for rounding
+        const float dx = cx - ox, dy = cy - oy, dz = cz - oz;
+        const float e = fmaf(fabsf(dx) + fabsf(dy) + fabsf(dz), 1e-6f, ow);  // for rounding
+        B4 = make_float4(dx, dy, dz, fmaf(R, 1e-6f, R) + e);
       }
-      gb[g] = B4;
+      gb[g] = half_bound(B4.x, B4.y, B4.z, B4.w);
       reinterpret_cast<float4*>(gx)[g] = zero4;
       reinterpret_cast<float4*>(gy)[g] = zero4;
       reinterpret_cast<float4*>(gz)[g] = zero4;
@@ -211,9 +210,8 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
     const uint4* off = ps.off + lane;
     uint4 en = __ldg(off);  // one step ahead (the table ends with a null row)
     for (int u0 = 0; u0 < prs; u0 += 16) {
-      // blocks whose bound (widened below the true one: 4e-6 of the distance
-      // here, 2 x 2e-6 in the group radii) is under eta can hold an active
-      // pair; bit v: round 2 (u0 + v), bit 16 + v: the one after
+      // blocks whose bound is under eta can hold an active pair; bit v: round
+      // 2 (u0 + v), bit 16 + v: the one after
       uint32_t km = 0u;
       const int u1 = min(prs - u0, 16);
 #pragma unroll 2
@@ -221,10 +219,9 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
         const uint4 e = en;
         off += 32;
         en = __ldg(off);
-        auto under = [&](uint32_t o0, uint32_t o1) {
-          const float4 P4 = ld4(cgb, o0), Q4 = ld4(cgb, o1);
-          return fmaf(approx_sqrt(dist2(P4.x, P4.y, P4.z, Q4.x, Q4.y, Q4.z)), 0.999996f,
-                      -(P4.w + Q4.w)) < eta;
+        auto under = [&](uint32_t o0, uint32_t o1) {  // also where the bound is no number
+          return !(half_gap(*reinterpret_cast<const uint2*>(cgb + o0),
+                            *reinterpret_cast<const uint2*>(cgb + o1)) >= eta);
         };
         km |= (under(e.x, e.y) ? 1u << v : 0u) | (under(e.z, e.w) ? 0x10000u << v : 0u);
       }

@@ -27,8 +27,6 @@
 
 #include "spatial.cuh"
 
-#include <cuda_fp16.h>
-
 #include <climits>
 
 namespace wbe {
@@ -49,7 +47,7 @@ struct PairPlan {  // per warp, 32-bit words
     yc = ra + m;
     zc = ra + 2 * m;
     nn = ra + 3 * m;
-    gb = ra + (full ? 4 : 3) * m;  // group bounding spheres (float4 per group), culling only
+    gb = ra + (full ? 4 : 3) * m;  // group bounding spheres (half_bound), culling only
     q = gb + m;       // queue of surviving schedule entries (64), culling only
     bits = q + 64;
     total = bits + (with_bits ? a32((P + 31) / 32) : 0);
@@ -59,13 +57,6 @@ struct PairPlan {  // per warp, 32-bit words
 inline size_t pair_smem(const DevRobot& r, int warps, bool bits, bool full) {
   return sizeof(float) *
          ((size_t)a32(4 * r.Sg) + (size_t)warps * PairPlan(r.n, r.Sg, r.P, bits, full).total);
-}
-
-// approximate square root (relative error at most 2^-23)
-__device__ __forceinline__ float sqrt_approx(float x) {
-  float y;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
 }
 
 // order-preserving map of a float to a signed int (and back)
@@ -350,7 +341,7 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
   float* xc = ws + pl.xc;
   float* yc = ws + pl.yc;
   float* zc = ws + pl.zc;
-  float4* gb = reinterpret_cast<float4*>(ws + pl.gb);
+  uint2* gb = reinterpret_cast<uint2*>(ws + pl.gb);
   uint32_t* qu = reinterpret_cast<uint32_t*>(ws + pl.q);
   uint32_t* bm = reinterpret_cast<uint32_t*>(ws + pl.bits);
   const char* cxc = reinterpret_cast<const char*>(xc);
@@ -376,6 +367,10 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
     asm volatile("cp.async.wait_group 0;" ::: "memory");
   }
   __syncwarp();
+  // The bounds are taken relative to the first link, so that their halves stay as
+  // fine for a robot far from the origin; ow: the rounding that this adds.
+  const float ox = xr[9], oy = xr[10], oz = xr[11];
+  const float ow = fmaf(fabsf(ox) + fabsf(oy) + fabsf(oz), 1e-6f, 3e-6f);
   if (r.sph_vec4) {
     // Every group of 4 spheres lies on one link: one lane a group reads the
     // link's pose once, places the 4 centres (the same arithmetic as the
@@ -429,8 +424,8 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
       rot(T, cl, c);
       const float scale = fabsf(T[9]) + fabsf(T[10]) + fabsf(T[11]) + fabsf(L.x) + fabsf(L.y) +
                           fabsf(L.z);
-      gb[g] = make_float4(c[0] + T[9], c[1] + T[10], c[2] + T[11],
-                          fmaf(scale, 1e-6f, fmaf(L.w, 1e-6f, L.w)) + 3e-6f);
+      gb[g] = half_bound(c[0] + T[9] - ox, c[1] + T[10] - oy, c[2] + T[11] - oz,
+                         fmaf(scale, 1e-6f, fmaf(L.w, 1e-6f, L.w)) + ow);
     }
   } else {
     for (int s = lane; s < 4 * Sg; s += 32) {
@@ -472,8 +467,8 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
         // placement (a few ulp of the coordinates' size each)
         const float scale = fabsf(T[9]) + fabsf(T[10]) + fabsf(T[11]) + fabsf(L.x) + fabsf(L.y) +
                             fabsf(L.z);
-        gb[g] = make_float4(c[0] + T[9], c[1] + T[10], c[2] + T[11],
-                            fmaf(scale, 1e-6f, fmaf(L.w, 1e-6f, L.w)) + 3e-6f);
+        gb[g] = half_bound(c[0] + T[9] - ox, c[1] + T[10] - oy, c[2] + T[11] - oz,
+                           fmaf(scale, 1e-6f, fmaf(L.w, 1e-6f, L.w)) + ow);
         continue;
       }
       const int s0 = 4 * g, s1 = min(S, s0 + 4);
@@ -491,14 +486,16 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
       float R = 0.0f;
       for (int s = s0; s < s1; ++s)
         R = fmaxf(R, sqrtf(dist2(cx, cy, cz, xc[s], yc[s], zc[s])) + pick(rad, s - s0));
-      gb[g] = make_float4(cx, cy, cz, fmaf(R, 1e-6f, R) + 3e-6f);  // widened for rounding
+      const float dx = cx - ox, dy = cy - oy, dz = cz - oz;
+      const float e = fmaf(fabsf(dx) + fabsf(dy) + fabsf(dz), 1e-6f, ow);  // widened for rounding
+      gb[g] = half_bound(dx, dy, dz, fmaf(R, 1e-6f, R) + e);
     }
   }
   if (BITS)
     for (int w = lane; w < W; w += 32) bm[w] = 0u;
   // the far sphere of the schedule's null blocks
   if (lane == 0)
-    *reinterpret_cast<float4*>(ws + pl.gb + far_words(Sg)) = make_float4(1e15f, 1e15f, 1e15f, 0.0f);
+    *reinterpret_cast<uint2*>(ws + pl.gb + far_words(Sg)) = half_bound(6e4f, 6e4f, 6e4f, 0.0f);
   __syncwarp();
   if (!A.dmin && !BITS) return;  // sphere placement only
   if (rounds == 0) {
@@ -522,19 +519,15 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
   // blocks' offsets decoded by the host, null blocks against a far sphere in
   // place of a test, the smallest bound carried with its round in its low 11
   // bits, and two bounds compared an instruction in pass 2: humanoid48 pair
-  // stage 0.117 -> 0.105 ms at 32768 configurations (0.097 with the wavefronts saved below).
+  // stage 0.117 -> 0.105 ms at 32768 configurations (0.097 with the wavefronts
+  // saved below, 0.092 with the bounds in halves).
   const int prs = ps.prs;
   const bool keep_lb = prs * 32 <= pl.ra_words();
   __half2* lb2 = reinterpret_cast<__half2*>(xr) + lane;
-  // the blocks' byte offsets in the per-warp sphere arrays (16 bytes a group)
-  // are also their offsets in gb
   const char* cgb = reinterpret_cast<const char*>(gb);
   auto bound = [&](uint32_t o0, uint32_t o1) {
-    const float4 P4 = lds4(cgb, o0), Q4 = lds4(cgb, o1);
-    // widened for the approximate square root: 4e-6 of the distance here,
-    // 2 x 2e-6 in the group radii
-    return fmaf(sqrt_approx(dist2(P4.x, P4.y, P4.z, Q4.x, Q4.y, Q4.z)), 0.999996f,
-                -(P4.w + Q4.w));
+    return half_gap(*reinterpret_cast<const uint2*>(cgb + o0),
+                    *reinterpret_cast<const uint2*>(cgb + o1));
   };
   auto keyed = [](float lb, int rr) {  // any block gives a valid bound: 12 bits of it decide
     return __int_as_float((__float_as_int(lb) & ~0x7FF) | rr);
@@ -713,7 +706,7 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
       uint32_t km = 0u;  // bit v: round 2 (u0 + v), bit 16 + v: the one after
 #pragma unroll
       for (int v = 0; v < 16; ++v)
-        if (u0 + v < prs) km |= __hle2_mask(lb2[(u0 + v) * 32], th2) & (0x00010001u << v);
+        if (u0 + v < prs) km |= __hleu2_mask(lb2[(u0 + v) * 32], th2) & (0x00010001u << v);
       const int cnt = __popc(km);
       int off = cnt;  // inclusive scan of the counts over the lanes
 #pragma unroll
@@ -738,17 +731,12 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
   } else {
     for (int rr = 0; rr < rounds; ++rr) {
       const int idx = rr * 32 + lane;
-      // lb <= bound + tol  <=>  |C_i - C_j| <= t := bound + tol + R_i + R_j,
-      // tested on squares (t >= 0); the tolerance covers the float rounding
       bool keep = false;
       {
         const uint2 e = __ldg(ps.ent + idx);
         if ((e.y >> 16) != 0u) {
-          const float4 P4 = gb[(e.x & 0xFFFF) >> 4], Q4 = gb[(e.x >> 16) >> 4];
-          const float D2 = dist2(P4.x, P4.y, P4.z, Q4.x, Q4.y, Q4.z);
-          const float RR2 = P4.w + Q4.w + reach_tol;
-          const float t = fminf(best, gbest) + RR2;
-          keep = (t >= 0.0f && D2 <= t * t) || (BITS && RR2 >= 0.0f && D2 <= RR2 * RR2);
+          const float lb = bound((e.x & 0xFFFF) >> 1, (e.x >> 16) >> 1);
+          keep = !(lb > fminf(best, gbest) + reach_tol) || (BITS && !(lb > reach_tol));
         }
       }
       const uint32_t ball = __ballot_sync(0xffffffffu, keep);

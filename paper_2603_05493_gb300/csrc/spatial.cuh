@@ -13,6 +13,8 @@
 
 #include "wbe_internal.h"
 
+#include <cuda_fp16.h>
+
 namespace wbe {
 
 __device__ __forceinline__ void cross3(const float* a, const float* b, float* c) {
@@ -287,6 +289,38 @@ __device__ __forceinline__ float dist2(float xi, float yi, float zi, float xj, f
                                        float zj) {
   const float dx = xi - xj, dy = yi - yj, dz = zi - zj;
   return fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+}
+
+// approximate square root (relative error at most 2^-23)
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// A bounding sphere of a group of collision spheres as four halves (x, y and
+// z, radius): the centre rounded, the radius grown by what that moved it and by
+// 5e-4 (the rounding of a sum of two radii), rounded up -- still a bound.  The
+// pair stage reads two of them for every block of every configuration, and the
+// shared memory's wavefronts, half as many for 8 bytes, are what it runs out of.
+__device__ __forceinline__ uint2 half_bound(float x, float y, float z, float R) {
+  const __half2 xy = __floats2half2_rn(x, y);
+  const __half hz = __float2half_rn(z);
+  const float2 f = __half22float2(xy);
+  const float e = fabsf(x - f.x) + fabsf(y - f.y) + fabsf(z - __half2float(hz));
+  const __half2 zr = __halves2half2(hz, __float2half_ru((R + e) * 1.0005f));
+  return make_uint2(*reinterpret_cast<const uint32_t*>(&xy), *reinterpret_cast<const uint32_t*>(&zr));
+}
+// Lower bound of the distance between the surfaces of two such spheres (and so
+// of any spheres within them): differences in half are off by at most 2^-11 of
+// themselves, which 6e-4 of the distance covers with the square root's error;
+// not a number where they overflow, which a caller has to keep.
+__device__ __forceinline__ float half_gap(uint2 a, uint2 b) {
+  const __half2 axy = *reinterpret_cast<const __half2*>(&a.x), azr = *reinterpret_cast<const __half2*>(&a.y);
+  const __half2 bxy = *reinterpret_cast<const __half2*>(&b.x), bzr = *reinterpret_cast<const __half2*>(&b.y);
+  const float2 d = __half22float2(__hsub2(axy, bxy));
+  const float2 zr = __half22float2(__hfma2(bzr, __floats2half2_rn(-1.0f, 1.0f), azr));
+  return fmaf(sqrt_approx(fmaf(zr.x, zr.x, fmaf(d.y, d.y, d.x * d.x))), 0.9994f, -zr.y);
 }
 
 }  // namespace wbe

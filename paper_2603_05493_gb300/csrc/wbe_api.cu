@@ -809,8 +809,8 @@ int wb_load_robot(const wb_tree* tree, const wb_spheres* sph, const wb_pairs* pa
       const size_t at = (2 * u + h) * 32 + l;
       const uint2 e = at < ent32.size() ? ent32[at] : uint2{0u, 0u};
       const bool block = (e.y >> 16) != 0u;
-      o[2 * h] = block ? e.x & 0xFFFF : 0u;
-      o[2 * h + 1] = block ? e.x >> 16 : 4u * (uint32_t)far_words(H.Sg);
+      o[2 * h] = block ? (e.x & 0xFFFF) / 2 : 0u;
+      o[2 * h + 1] = block ? (e.x >> 16) / 2 : 4u * (uint32_t)far_words(H.Sg);
     }
     off32[i] = make_uint4(o[0], o[1], o[2], o[3]);
   }

@@ -106,7 +106,7 @@ struct PairSchedule32 {
   int rounds;
   const uint2* ent;          // [rounds + 1][32], the last round all null
   // for the bounds on whole blocks, two rounds at a time: the two blocks' byte
-  // offsets (16 gi, 16 gj each) in an array of group spheres; a null block is
+  // offsets (8 gi, 8 gj each) in an array of group bounds; a null block is
   // group 0 against a far sphere that the kernels put far_words(Sg) behind
   // the array's start (prs = pairs of rounds, rounded up)
   int prs;
