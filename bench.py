@@ -967,10 +967,10 @@ def run_kinematics(args, rank=0, world=1, local_rank=0):
                    "targets": targets, "l2": "flushed between timed steps"},
         "kernels": {"tree_fwd": {"kernel": "tree_fwd_seg_kernel or tree_fwd_kernel (poses only)",
                                  "ms": fk_ms},
-                    "kinematics": {"kernel": "kin_kernel", "ms": kin_ms, "bound": "hbm",
+                    "kinematics": {"kernel": "kin_single_kernel", "ms": kin_ms, "bound": "hbm",
                                    "bytes_per_eval": kin_bytes, "achieved": ach,
                                    "peak": hbm_peak, "unit": "GB/s", "frac": ach / hbm_peak}},
-        "roofline": {"kernel": "kin_kernel", "bound": "hbm", "achieved": ach, "peak": hbm_peak,
+        "roofline": {"kernel": "kin_single_kernel", "bound": "hbm", "achieved": ach, "peak": hbm_peak,
                      "unit": "GB/s", "frac": ach / hbm_peak, "traffic": None},
         "gpu_launches": 2 * args.steps * world, "clocks": clocks.summary()}), flush=True)
 

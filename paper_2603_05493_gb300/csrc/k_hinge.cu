@@ -11,8 +11,8 @@
 // 6.1.1) as SoA rows and bounds every group of 4 with a sphere (C_g, R_g)
 // (for a group on one link, the host-made sphere in its link frame moved
 // with the link), as the pair stage does.  It then walks the pair stage's
-// 4x4 block schedule: a block whose bound |C_i - C_j| - R_i - R_j (widened
-// for the approximate square root) is at least eta holds no active pair.
+// 4x4 block schedule: a block whose bound |C_i - C_j| - R_i - R_j (in halves,
+// widened for their rounding) is at least eta holds no active pair.
 // Each lane marks its surviving blocks of 32 rounds in a bit mask, the
 // survivors are queued from a warp scan of the counts and worked 32 at a
 // time, one block a lane, every masked pair exactly (sqrt distance).  A
@@ -28,7 +28,7 @@ namespace wbe {
 
 // per warp, 32-bit words: link poses while the spheres are placed, then the
 // 32 block slots in the same region; the sphere SoA rows x, y, z, the group
-// bounds (float4), the gradient SoA rows gx, gy, gz and the queue of
+// bounds (half_bound), the gradient SoA rows gx, gy, gz and the queue of
 // surviving schedule entries
 struct HingePlan {
   int xc, yc, zc, gb, gx, gy, gz, q, total;

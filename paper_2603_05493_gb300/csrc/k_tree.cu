@@ -71,10 +71,9 @@ __global__ void __launch_bounds__(256) tree_fwd_kernel(const __grid_constant__ D
 }
 
 // The backward sweeps are capped at 128 registers (two 256-thread blocks per
-// SM, or one 512-thread block of a segmented sweep): with the register copies
-// of the stack top they would take ~165, and the occupancy lost costs more
-// than the few spills (measured on the 48-DoF humanoid: 0.29 ms capped vs
-// 0.36 ms uncapped at 2 segments).  The segmented sweeps take blocks of up to
+// SM, or one 512-thread block of a segmented sweep): more a thread cost the
+// occupancy that hides each link's chain, fewer (104) spilled and were 2 %
+// slower at the same number of resident warps.  The segmented sweeps take blocks of up to
 // 512 threads, so that one block per SM holds the staged link parameters once
 // and the shared-memory carveout stays small.
 template <int OPT>
