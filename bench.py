@@ -1062,9 +1062,9 @@ def run_arm7(args, rank=0, world=1, local_rank=0):
                          kernel="tree_fwd_seg_kernel" if seg > 1 else "tree_fwd_kernel",
                          bytes_per_eval=w["tree_fwd"]["bytes"]),
         # robots of at most 32 spheres and 1024 pairs take the library's
-        # one-thread-per-configuration pair kernel
+        # eight-lanes-a-configuration pair kernel
         "pair": dict(hbm(w["pair"]["bytes"], pair_ms), ms=pair_ms,
-                     kernel="pair_thread_kernel" if desc.S <= 32 and desc.P <= 1024
+                     kernel="pair_small_kernel" if desc.S <= 32 and desc.P <= 1024
                      else "pair_kernel", bytes_per_eval=w["pair"]["bytes"]),
     }
     dom = max(kernels, key=lambda k: kernels[k]["ms"])

@@ -254,14 +254,17 @@ size_t batch_tree_smem(bool fwd, int ns_max, int n_max, int threads) {
          (fwd ? 0 : 16 + (size_t)kGradSlotBytes * threads);
 }
 
+// clears: the work counters to clear, this pass's alone or also the next's (the
+// pair pass of the same call): one clear and its gap less on the stream, uneven
+// batch of 768 problems 0.251 -> 0.248 ms
 cudaError_t launch_batch_tree_fwd(const DevRobot* robots, const BatchProblemDev* probs, const int4* items,
-                                  int n_items, int* counter, const BatchIO& io, int grid,
+                                  int n_items, int* counter, int clears, const BatchIO& io, int grid,
                                   int ns_max, int n_max, int threads, cudaStream_t s) {
   const size_t smem = batch_tree_smem(true, ns_max, n_max, threads);
   cudaError_t e = allow_smem((const void*)batch_tree_fwd_kernel, smem);
   if (e != cudaSuccess) return e;
   fit_carveout((const void*)batch_tree_fwd_kernel, threads, smem);
-  e = cudaMemsetAsync(counter, 0, sizeof(int), s);
+  e = cudaMemsetAsync(counter, 0, clears * sizeof(int), s);
   if (e != cudaSuccess) return e;
   batch_tree_fwd_kernel<<<grid, threads, smem, s>>>(robots, probs, items, n_items, counter, io,
                                                     ns_max, n_max);
@@ -293,12 +296,12 @@ size_t batch_pair_smem(int ws_words, int rad_words, int warps) {
 
 cudaError_t launch_batch_pair(const DevRobot* robots, const PairSchedule32* scheds,
                               const BatchProblemDev* probs, const int2* items, int n_items, int* counter,
-                              const BatchIO& io, int grid, int warps, int ws_words,
+                              bool cleared, const BatchIO& io, int grid, int warps, int ws_words,
                               int rad_words, cudaStream_t s) {
   const size_t smem = batch_pair_smem(ws_words, rad_words, warps);
   cudaError_t e = allow_smem((const void*)batch_pair_kernel, smem);
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(counter, 0, sizeof(int), s);
+  if (!cleared) e = cudaMemsetAsync(counter, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   batch_pair_kernel<<<grid, warps * 32, smem, s>>>(robots, scheds,
                                                   probs,

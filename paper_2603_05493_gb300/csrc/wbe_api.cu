@@ -1887,15 +1887,16 @@ int wb_batch_eval(wb_batch* batch, const float* q, const float* qd, const float*
              nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   int* counters = const_cast<int*>(batch->d_counters);
   cudaError_t e = cudaSuccess;
-  if (link_pose || tau) {
+  const bool tree_pass = link_pose || tau, pair_pass = pairs && batch->n_pitems > 0;
+  if (tree_pass) {
     int threads = 0, grid = 1;
     if ((rc = batch_grid_tree(batch, true, &threads, &grid))) return rc;
     e = launch_batch_tree_fwd(batch->d_robots, batch->d_probs, batch->d_titems[0],
-                              batch->n_titems[0], counters, io, grid, batch->ns_max,
+                              batch->n_titems[0], counters, pair_pass ? 2 : 1, io, grid, batch->ns_max,
                               batch->n_max, threads, s);
     if (e != cudaSuccess) return cuda_fail(e, "wb_batch_eval launch");
   }
-  if (pairs && batch->n_pitems > 0) {
+  if (pair_pass) {
     const int warps = batch_pair_warps(batch);
     if (warps == 0) return fail(WB_ETOOBIG, "batch pair kernel does not fit on an SM");
     int bps = 0;
@@ -1905,8 +1906,8 @@ int wb_batch_eval(wb_batch* batch, const float* q, const float* qd, const float*
     const int need = (batch->n_pitems + warps - 1) / warps;
     const int grid = std::min(need, bps * batch->num_sms);
     e = launch_batch_pair(batch->d_robots, batch->d_scheds, batch->d_probs, batch->d_pitems,
-                          batch->n_pitems, counters + 1, io, grid, warps, batch->ws_words,
-                          batch->rad_words, s);
+                          batch->n_pitems, counters + 1, tree_pass, io, grid, warps,
+                          batch->ws_words, batch->rad_words, s);
     if (e != cudaSuccess) return cuda_fail(e, "wb_batch_eval launch");
   }
   return WB_OK;
@@ -2257,8 +2258,8 @@ int wb_batch_eval_noalloc(wb_robot* const* robots, int32_t n_robots, const wb_pr
     int threads = 128, grid = 1;
     const int rc2 = batch_sweep_shape(true, ns_max, n_max, n_titems, R0->num_sms, &threads, &grid);
     if (rc2) return rc2;
-    e = launch_batch_tree_fwd(T.robots, T.probs, T.titems, n_titems, T.counters, io, grid, ns_max,
-                              n_max, threads, s);
+    e = launch_batch_tree_fwd(T.robots, T.probs, T.titems, n_titems, T.counters, pairs ? 2 : 1, io,
+                              grid, ns_max, n_max, threads, s);
     if (e != cudaSuccess) return cuda_fail(e, "wb_batch_eval_noalloc launch");
   }
   if (pairs) {
@@ -2269,8 +2270,8 @@ int wb_batch_eval_noalloc(wb_robot* const* robots, int32_t n_robots, const wb_pr
     if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
     if (bps < 1) return fail(WB_ETOOBIG, "batch pair kernel does not fit on an SM");
     const int grid = std::min((n_pitems + warps - 1) / warps, bps * R0->num_sms);
-    e = launch_batch_pair(T.robots, T.scheds, T.probs, T.pitems, n_pitems, T.counters + 1, io, grid,
-                          warps, ws_words, rad_words, s);
+    e = launch_batch_pair(T.robots, T.scheds, T.probs, T.pitems, n_pitems, T.counters + 1,
+                          link_pose || tau, io, grid, warps, ws_words, rad_words, s);
     if (e != cudaSuccess) return cuda_fail(e, "wb_batch_eval_noalloc launch");
   }
   return WB_OK;
@@ -2667,7 +2668,7 @@ extern "C" int wb_batch_autotune(wb_batch* batch, wb_batch_tune* tune, int32_t* 
       cudaError_t e =
           pass == 0
               ? launch_batch_tree_fwd(batch->d_robots, batch->d_probs, batch->d_titems[0],
-                                      batch->n_titems[0], counters, io, grid, batch->ns_max,
+                                      batch->n_titems[0], counters, 1, io, grid, batch->ns_max,
                                       batch->n_max, threads, s)
               : launch_batch_tree_bwd(batch->d_robots, batch->d_probs, batch->d_titems[1],
                                       batch->n_titems[1], counters + 2, io, grid, batch->ns_max,
@@ -2744,7 +2745,7 @@ extern "C" int wb_batch_autotune(wb_batch* batch, wb_batch_tune* tune, int32_t* 
         const int grid = std::min((batch->n_pitems + w - 1) / w, bps * batch->num_sms);
         auto run = [&]() {
           return launch_batch_pair(batch->d_robots, batch->d_scheds, batch->d_probs,
-                                   batch->d_pitems, batch->n_pitems, counters + 1, io, grid, w,
+                                   batch->d_pitems, batch->n_pitems, counters + 1, false, io, grid, w,
                                    batch->ws_words, batch->rad_words, s);
         };
         if (run() != cudaSuccess) {

@@ -213,7 +213,7 @@ struct BatchIO {
 // slots among the robots' 2-segment plans; threads: 64, 128 or 256 (pairs of
 // warps per block).
 cudaError_t launch_batch_tree_fwd(const DevRobot* robots, const BatchProblemDev* probs,
-                                  const int4* items, int n_items, int* counter, const BatchIO& io,
+                                  const int4* items, int n_items, int* counter, int clears, const BatchIO& io,
                                   int grid, int ns_max, int n_max, int threads,
                                   cudaStream_t s);
 cudaError_t launch_batch_tree_bwd(const DevRobot* robots, const BatchProblemDev* probs,
@@ -222,7 +222,7 @@ cudaError_t launch_batch_tree_bwd(const DevRobot* robots, const BatchProblemDev*
                                   cudaStream_t s);
 cudaError_t launch_batch_pair(const DevRobot* robots, const PairSchedule32* scheds,
                               const BatchProblemDev* probs, const int2* items, int n_items,
-                              int* counter, const BatchIO& io, int grid, int warps, int ws_words,
+                              int* counter, bool cleared, const BatchIO& io, int grid, int warps, int ws_words,
                               int rad_words, cudaStream_t s);
 cudaError_t batch_pair_max_blocks_per_sm(int warps, int ws_words, int rad_words, int* out);
 size_t batch_pair_smem(int ws_words, int rad_words, int warps);
