@@ -305,9 +305,15 @@ __device__ __forceinline__ uint2 half_bound(float x, float y, float z, float R) 
 __device__ __forceinline__ float half_gap(uint2 a, uint2 b) {
   const __half2 axy = *reinterpret_cast<const __half2*>(&a.x), azr = *reinterpret_cast<const __half2*>(&a.y);
   const __half2 bxy = *reinterpret_cast<const __half2*>(&b.x), bzr = *reinterpret_cast<const __half2*>(&b.y);
-  const float2 d = __half22float2(__hsub2(axy, bxy));
-  const float2 zr = __half22float2(__hfma2(bzr, __floats2half2_rn(-1.0f, 1.0f), azr));
-  return fmaf(sqrt_approx(fmaf(zr.x, zr.x, fmaf(d.y, d.y, d.x * d.x))), 0.9994f, -zr.y);
+  const __half2 d = __hsub2(axy, bxy), zr = __hfma2(bzr, __floats2half2_rn(-1.0f, 1.0f), azr);
+  float d2;  // squares of halves added in fp32
+  asm("{\n\t.reg .f16 x, y, z, r;\n\t.reg .f32 s;\n\t"
+      "mov.b32 {x, y}, %1;\n\tmov.b32 {z, r}, %2;\n\t"
+      "fma.rn.f32.f16 s, x, x, 0f00000000;\n\tfma.rn.f32.f16 s, y, y, s;\n\t"
+      "fma.rn.f32.f16 %0, z, z, s;\n\t}"
+      : "=f"(d2)
+      : "r"(*reinterpret_cast<const uint32_t*>(&d)), "r"(*reinterpret_cast<const uint32_t*>(&zr)));
+  return fmaf(sqrt_approx(d2), 0.9994f, -__high2float(zr));
 }
 
 }  // namespace wbe
