@@ -51,23 +51,41 @@ __device__ __forceinline__ bool own_config(int64_t B, int64_t b0, int64_t* b, bo
 // MODE kFwdShared: the force stack in shared memory behind the link records,
 // as in the segmented forward below
 template <int MODE>
-__global__ void __launch_bounds__(256) tree_fwd_kernel(const __grid_constant__ DevRobot r,
-                                                       const __grid_constant__ WalkTab wt,
-                                                       const __grid_constant__ FwdArgs A) {
-  extern __shared__ float4 rec[];
+__device__ __forceinline__ void fwd_block(const DevRobot& r, const WalkTab& wt, const FwdArgs& A,
+                                          float4* rec) {
+  constexpr bool FS = MODE == kFwdShared;
   float* sm = reinterpret_cast<float*>(rec) + kRecWords * (size_t)r.n;
-  if (MODE == kFwdShared && !smem_holds(kRecWords * (size_t)r.n + 6 * fs_levels(r) * blockDim.x)) return;
+  if (FS && !smem_holds(kRecWords * (size_t)r.n + 6 * fs_levels(r) * blockDim.x)) return;
   stage_recs(r, -1, rec, threadIdx.x, blockDim.x);
   __syncthreads();
   int64_t b;
   bool act;
   if (!own_config(A.B, blockIdx.x * (int64_t)blockDim.x + 32 * warp_of(), &b, &act)) return;
   Seg sg = whole_sweep(r);
-  if (MODE == kFwdShared) {
+  if (FS) {
     sg.fst = reinterpret_cast<float2*>(sm) + threadIdx.x;
     sg.fstr = blockDim.x;
   }
   tree_fwd_seg<MODE>(r, rec, ConstWalk{wt}, A, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg);
+}
+template <int MODE>
+__global__ void __launch_bounds__(256) tree_fwd_kernel(const __grid_constant__ DevRobot r,
+                                                       const __grid_constant__ WalkTab wt,
+                                                       const __grid_constant__ FwdArgs A) {
+  extern __shared__ float4 rec[];
+  fwd_block<MODE>(r, wt, A, rec);
+}
+// The same for robots without branches, capped at 72 registers: 28 warps an SM
+// where 78 allow 24.  The sweep is latency-bound, a chain never touches the branch
+// stack, and its force stack leaves the shared memory for them (21 KB a 128-thread
+// block for 7 links; the humanoid's 46 KB stop at 4 blocks, and there the cap only
+// spills: 0.190 -> 0.228 ms).  7-DoF arm, 131072 configurations: 0.0280 -> 0.0249
+// ms (64 registers: 0.0293; the branch code compiled out besides: 0.0263).
+__global__ void __maxnreg__(72) tree_fwd_chain_kernel(const __grid_constant__ DevRobot r,
+                                                      const __grid_constant__ WalkTab wt,
+                                                      const __grid_constant__ FwdArgs A) {
+  extern __shared__ float4 rec[];
+  fwd_block<kFwdShared>(r, wt, A, rec);
 }
 
 // The backward sweeps are capped at 128 registers (two 256-thread blocks per
@@ -608,7 +626,8 @@ cudaError_t launch_tree_fwd(const DevRobot& r, const WalkTab& wt, const FwdArgs&
   const size_t fs = sizeof(float) * 6 * fs_levels(r) * threads;  // the force stack
   const bool use_fs = a.tau && rec_smem(r, true) + fs <= kSegSmemMax;
   const size_t smem = rec_smem(r, true) + (use_fs ? fs : 0);
-  auto kern = use_fs ? tree_fwd_kernel<kFwdShared>
+  auto kern = use_fs ? (r.maxdepth == r.n ? tree_fwd_chain_kernel  // a link a level: no branches
+                                          : tree_fwd_kernel<kFwdShared>)
               : a.tau ? tree_fwd_kernel<kFwdLocal>
                       : tree_fwd_kernel<kFwdPose>;
   cudaError_t e =
