@@ -78,16 +78,16 @@ PAIR_SRC = ["paper_2603_05493_gb300/csrc/k_pair.cu", "paper_2603_05493_gb300/csr
             "paper_2603_05493_gb300/csrc/spatial.cuh"] + API_SRC
 SPLINE_SRC = ["paper_2603_05493_gb300/csrc/k_traj.cu",
               "paper_2603_05493_gb300/csrc/spline_basis.cuh"] + API_SRC
-TREE_SHA = "34d82c5e7fcbd5bbf26fefaa10ba98d7438ad699d80e19b7310edf1022f0fe0d"
-PAIR_SHA = "22f28c936d6573ba8f9fe8846b1d102cd8a666a308fde619b2cf38e9043abcea"
+TREE_SHA = "64cc9fda4690329b746f0f04e4a372709be5fedcd36b57d47725e0573bfc8aba"
+PAIR_SHA = "2fab9d8345554adbafa0ec6520f79625942c3ce3a6dd3bb06b04b48f7b16b928"
 SPLINE_SHA = "472e279cf6f19c37f18a16f2f0fb68bcd07d7dd7673b35533c279f420e26b5fa"
 MEASURED_TRAFFIC = {  # kernel[@workload]: (sources, their hash, bytes / evaluation)
-    "tree_fwd_seg_kernel": (TREE_SRC, TREE_SHA, (24.14e6 + 51.59e6) / 32768),
-    "pair_kernel": (PAIR_SRC, PAIR_SHA, (77.30e6 + 32.25e6) / 32768),
-    "tree_bwd_seg_kernel": (TREE_SRC, TREE_SHA, (233.05e6 + 30.19e6) / 32768),
-    "tree_fwd_spline_seg_kernel": (TREE_SRC, TREE_SHA, (5.50e6 + 51.47e6) / 32768),
-    "pair_kernel@trajopt48": (PAIR_SRC, PAIR_SHA, (77.27e6 + 0.84e6) / 32768),
-    "tree_bwd_spline_cost_seg_kernel": (TREE_SRC, TREE_SHA, (8.66e6 + 0.31e6) / 32768),
+    "tree_fwd_seg_kernel": (TREE_SRC, TREE_SHA, (24.17e6 + 51.58e6) / 32768),
+    "pair_kernel": (PAIR_SRC, PAIR_SHA, (77.30e6 + 32.16e6) / 32768),
+    "tree_bwd_seg_kernel": (TREE_SRC, TREE_SHA, (233.20e6 + 30.19e6) / 32768),
+    "tree_fwd_spline_seg_kernel": (TREE_SRC, TREE_SHA, (5.48e6 + 51.73e6) / 32768),
+    "pair_kernel@trajopt48": (PAIR_SRC, PAIR_SHA, (77.26e6 + 0.69e6) / 32768),
+    "tree_bwd_spline_cost_seg_kernel": (TREE_SRC, TREE_SHA, (8.66e6 + 0.34e6) / 32768),
     "bspline_bwd_kernel": (SPLINE_SRC, SPLINE_SHA, (18.91e6 + 0.00e6) / 32768),
 }
 
