@@ -243,11 +243,13 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
         }
         __syncwarp();
         const int count = min(32, tot - w0);
-        // one block a lane: every masked pair exactly, in pair order
+        // one block a lane: every masked pair exactly, in pair order.  A null entry
+        // is here where its bound was under eta or no number: no block
+        const uint2 e = lane < count ? __ldg(ps.ent + qu[lane]) : make_uint2(0u, 0u);
+        const bool block = (e.y >> 16) != 0u;
         uint32_t key = 0xFFFFFFFFu;  // no block
         float gr[12];  // the lane's block: its row spheres' gradients, then its columns'
-        if (lane < count) {
-          const uint2 e = __ldg(ps.ent + qu[lane]);
+        if (block) {
           const uint32_t ro = e.x & 0xFFFF, co = e.x >> 16, mask = e.y >> 16;
           key = e.x;
           const float4 XR = ld4(cxc, ro), YR = ld4(cyc, ro), ZR = ld4(czc, ro), RR = ld4(crad, ro);
@@ -288,15 +290,15 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
         // slower: 0.091 -> 0.120 ms)
 #pragma unroll
         for (int side = 0; side < 2; ++side) {
-          if (side == 1 && lane < count) {
+          if (side == 1 && block) {
             float* sl = slot + lane * SW;
 #pragma unroll
             for (int k = 0; k < 12; ++k) sl[k] = gr[k];
           }
           __syncwarp();
           const uint32_t grp = side == 0 ? (key & 0xFFFFu) : (key >> 16);  // byte offset
-          const uint32_t same = __match_any_sync(0xffffffffu, lane < count ? grp : 0xFFFFFFFFu);
-          if (lane < count && (__ffs(same) - 1) == lane) {
+          const uint32_t same = __match_any_sync(0xffffffffu, block ? grp : 0xFFFFFFFFu);
+          if (block && (__ffs(same) - 1) == lane) {
             float4* X4 = reinterpret_cast<float4*>(reinterpret_cast<char*>(gx) + grp);
             float4* Y4 = reinterpret_cast<float4*>(reinterpret_cast<char*>(gy) + grp);
             float4* Z4 = reinterpret_cast<float4*>(reinterpret_cast<char*>(gz) + grp);
