@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
     const float ow = fmaf(fabsf(ox) + fabsf(oy) + fabsf(oz), 1e-6f, 3e-6f);
     const float4 zero4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (lane == 0)  // the far sphere of the schedule's null blocks
-      *reinterpret_cast<uint2*>(ws + pl.gb + far_words(Sg)) = half_bound(6e4f, 6e4f, 6e4f, 0.0f);
+      *reinterpret_cast<uint2*>(ws + pl.gb + far_words(Sg)) = far_bound();
     if (r.sph_vec4) {
       // every group of 4 on one link: a lane a group places its centres, its
       // bound and its gradient rows' zeros from one pose

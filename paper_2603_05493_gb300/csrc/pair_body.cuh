@@ -495,7 +495,7 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
     for (int w = lane; w < W; w += 32) bm[w] = 0u;
   // the far sphere of the schedule's null blocks
   if (lane == 0)
-    *reinterpret_cast<uint2*>(ws + pl.gb + far_words(Sg)) = half_bound(6e4f, 6e4f, 6e4f, 0.0f);
+    *reinterpret_cast<uint2*>(ws + pl.gb + far_words(Sg)) = far_bound();
   __syncwarp();
   if (!A.dmin && !BITS) return;  // sphere placement only
   if (rounds == 0) {

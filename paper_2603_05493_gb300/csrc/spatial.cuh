@@ -290,18 +290,29 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 // 5e-4 (the rounding of a sum of two radii), rounded up -- still a bound.  The
 // pair stage reads two of them for every block of every configuration, and the
 // shared memory's wavefronts, half as many for 8 bytes, are what it runs out of.
+// A coordinate beyond 32752 makes the radius infinite: two such could differ by
+// more than a half holds, and their gap would come out as infinite.
 __device__ __forceinline__ uint2 half_bound(float x, float y, float z, float R) {
   const __half2 xy = __floats2half2_rn(x, y);
   const __half hz = __float2half_rn(z);
   const float2 f = __half22float2(xy);
   const float e = fabsf(x - f.x) + fabsf(y - f.y) + fabsf(z - __half2float(hz));
-  const __half2 zr = __halves2half2(hz, __float2half_ru((R + e) * 1.0005f));
+  const bool fits = fmaxf(fabsf(x), fmaxf(fabsf(y), fabsf(z))) <= 32752.0f;
+  const float grown = fits ? (R + e) * 1.0005f : __int_as_float(0x7f800000);
+  const __half2 zr = __halves2half2(hz, __float2half_ru(grown));
+  return make_uint2(*reinterpret_cast<const uint32_t*>(&xy), *reinterpret_cast<const uint32_t*>(&zr));
+}
+// The sphere that stands for the groups of a null block: far from every finite
+// bound, so that a null block is rarely kept (and then has no pair to work).
+__device__ __forceinline__ uint2 far_bound() {
+  const __half2 xy = __floats2half2_rn(6e4f, 6e4f), zr = __floats2half2_rn(6e4f, 0.0f);
   return make_uint2(*reinterpret_cast<const uint32_t*>(&xy), *reinterpret_cast<const uint32_t*>(&zr));
 }
 // Lower bound of the distance between the surfaces of two such spheres (and so
 // of any spheres within them): differences in half are off by at most 2^-11 of
-// themselves, which 6e-4 of the distance covers with the square root's error;
-// not a number where they overflow, which a caller has to keep.
+// themselves, which 6e-4 of the distance covers with the square root's error.
+// Finite bounds' coordinates never overflow; where a radius or the sum of two
+// does, the gap is minus infinity or not a number: a caller has to keep both.
 __device__ __forceinline__ float half_gap(uint2 a, uint2 b) {
   const __half2 axy = *reinterpret_cast<const __half2*>(&a.x), azr = *reinterpret_cast<const __half2*>(&a.y);
   const __half2 bxy = *reinterpret_cast<const __half2*>(&b.x), bzr = *reinterpret_cast<const __half2*>(&b.y);
