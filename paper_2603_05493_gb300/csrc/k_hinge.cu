@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
       float4* dst = reinterpret_cast<float4*>(P);
       for (int i = lane; i < 3 * n; i += 32) {  // asynchronous copies into shared memory
         const unsigned a = static_cast<unsigned>(__cvta_generic_to_shared(dst + i));
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src + i));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src + i) : "memory");
       }
       asm volatile("cp.async.commit_group;");
       asm volatile("cp.async.wait_group 0;" ::: "memory");

@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(256) kin_single_kernel(const __grid_constant__
       const float4* src = reinterpret_cast<const float4*>(A.pose + b * (int64_t)n * 12);
       for (int i = lane; i < 3 * n; i += 32) {
         const unsigned to = static_cast<unsigned>(__cvta_generic_to_shared(dst + i));
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to), "l"(src + i));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to), "l"(src + i) : "memory");
       }
     }
     asm volatile("cp.async.commit_group;");

@@ -136,7 +136,7 @@ struct GlobalRow {  // nullptr: zero
 __device__ __forceinline__ void stage(float* dst, const float* a, const float* b, int64_t at) {
   if (a && !b) {
     const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(a + at));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(a + at) : "memory");
   } else {
     *dst = GlobalRow::sum(a, b, at);
   }

@@ -361,7 +361,7 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
     float4* dst = reinterpret_cast<float4*>(xr);
     for (int i = lane; i < 3 * n; i += 32) {
       const unsigned a = static_cast<unsigned>(__cvta_generic_to_shared(dst + i));
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src + i));
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src + i) : "memory");
     }
     asm volatile("cp.async.commit_group;");
     asm volatile("cp.async.wait_group 0;" ::: "memory");

@@ -684,7 +684,7 @@ __device__ __forceinline__ GradSlot grad_slot_of(float* after) {
 }
 __device__ __forceinline__ void cp16(float4* dst, const void* src) {
   const unsigned a = static_cast<unsigned>(__cvta_generic_to_shared(dst));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src));
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src) : "memory");
 }
 
 // With a fused cost (FC, fc) the sweep computes g_tau = [tau > hi] -
