@@ -137,7 +137,11 @@ typedef struct {
                                 warps per SM and the segments' lengths */
   int32_t configs_per_block; /* fused: configurations per CTA; tree: threads per block
                                 of the sweep kernels (32..256, up to 512 for
-                                G > 1 segments); 0 = by the batch's share per SM */
+                                G > 1 segments); 0 = by the batch's share per SM.
+                                A segmented sweep takes fewer threads than asked
+                                for, and if one group of warps does not fit fewer
+                                segments, where its block would pass the shared
+                                memory (robots near 255 links) */
   int32_t blocks_per_sm;     /* fused: grid = blocks_per_sm * SMs (0 = occupancy);
                                 tree: warps per block of the pair kernel, 1..8
                                 (0 = of the counts 4..8 whose per-warp

@@ -1072,8 +1072,8 @@ static int tree_segments(const wb_robot* R, const wb_tune* tune, int64_t B, int*
     return fail(WB_EINVAL, "one-segment sweeps take at most 256 threads per block");
   // what a block needs: refused from the limit up, counting 28 floats a link
   // record; the records' padding to kRecWords, the backward's spheres and the
-  // spline backward's basis rows beside its slots are made room for
-  const size_t basis = spline && !fwd ? 12 * sizeof(float) : 0;  // a thread's basis rows
+  // basis rows of states from control points are made room for
+  const size_t basis = spline ? 12 * sizeof(float) : 0;  // a thread's basis rows
   auto need = [&](int G_, int threads_) {
     return tree_seg_smem(R->dev, G_, threads_, fwd, !fwd) +
            (fwd ? 0 : grad_slot_smem(G_, threads_)) + basis * std::max(threads_, 32 * G_);
