@@ -662,25 +662,25 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
       }
       hit &= mask;
       const int32_t* pix = r.blk_pidx + 16 * (e.y & 0xFFFF);
-      if (FULL) {
-        // the four pairs of a row sphere have consecutive indices: their bits
-        // are one shift, over at most two words
+      // the pairs of a row sphere in a block have consecutive indices: their bits
+      // are one shift, over at most two words
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          const uint32_t h = (hit >> (4 * a)) & 15u;
-          if (h) {
-            const int p = __ldg(pix + 4 * a);
-            const uint64_t w = (uint64_t)h << (p & 31);
-            atomicOr(bm + (p >> 5), (uint32_t)w);
-            if (w >> 32) atomicOr(bm + (p >> 5) + 1, (uint32_t)(w >> 32));
+      for (int a = 0; a < 4; ++a) {
+        uint32_t h = (hit >> (4 * a)) & 15u;
+        if (h) {
+          int first = 4 * a;
+          if (!FULL) {  // squeeze out the pairs that are not masked in
+            const uint32_t m = (mask >> (4 * a)) & 15u;
+            first += __ffs(m) - 1;
+            uint32_t c = h & 1u;
+            c |= ((h >> 1) & 1u) << (m & 1u);
+            c |= ((h >> 2) & 1u) << __popc(m & 3u);
+            h = c | ((h >> 3) & 1u) << __popc(m & 7u);
           }
-        }
-      } else {
-        while (hit) {
-          const int t = __ffs(hit) - 1;
-          hit &= hit - 1u;
-          const int p = __ldg(pix + t);
-          atomicOr(bm + (p >> 5), 1u << (p & 31));
+          const int p = __ldg(pix + first);
+          const uint64_t w = (uint64_t)h << (p & 31);
+          atomicOr(bm + (p >> 5), (uint32_t)w);
+          if (w >> 32) atomicOr(bm + (p >> 5) + 1, (uint32_t)(w >> 32));
         }
       }
     }
