@@ -236,16 +236,18 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
       int pos = sum - cnt;
       for (int w0 = 0; w0 < tot; w0 += 32) {
         while (km && pos < w0 + 32) {
-          const int bit = __ffs(km) - 1;
+          qu[pos - w0] = (uint32_t)(32 * (__ffs(km) - 1) + lane);  // bit and lane
           km &= km - 1u;
-          qu[pos - w0] = (uint32_t)((2 * (u0 + (bit & 15)) + (bit >> 4)) * 32 + lane);
           ++pos;
         }
         __syncwarp();
         const int count = min(32, tot - w0);
         // one block a lane: every masked pair exactly, in pair order.  A null entry
         // is here where its bound was under eta or no number: no block
-        const uint2 e = lane < count ? __ldg(ps.ent + qu[lane]) : make_uint2(0u, 0u);
+        // (the entries' rounds are decoded here: the queue is filled by few lanes)
+        const uint32_t c = qu[lane], bit = c >> 5;
+        const uint32_t at = (2 * (u0 + (bit & 15)) + (bit >> 4)) * 32 + (c & 31);
+        const uint2 e = lane < count ? __ldg(ps.ent + at) : make_uint2(0u, 0u);
         const bool block = (e.y >> 16) != 0u;
         uint32_t key = 0xFFFFFFFFu;  // no block
         float gr[12];  // the lane's block: its row spheres' gradients, then its columns'

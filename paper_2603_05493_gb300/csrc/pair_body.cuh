@@ -685,8 +685,9 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
       }
     }
   };
-  auto drain = [&](int count) {  // screen queue entries [0, count), one per lane
-    const uint2 e = lane < count ? __ldg(ps.ent + qu[lane]) : make_uint2(0u, 0u);
+  // screen queue entries [0, count), one per lane; at: an entry's place in ps.ent
+  auto drain = [&](int count, auto&& at) {
+    const uint2 e = lane < count ? __ldg(ps.ent + at(qu[lane])) : make_uint2(0u, 0u);
     __syncwarp();
     if ((e.y >> 16) != 0u) screen_block(e);
     gbest = fminf(gbest, fkey_inv(__reduce_min_sync(0xffffffffu, fkey(best))));
@@ -718,17 +719,22 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
       int pos = off - cnt;
       for (int w0 = 0; w0 < tot; w0 += 32) {
         while (km && pos < w0 + 32) {
-          const int bit = __ffs(km) - 1;
+          qu[pos - w0] = (uint32_t)(32 * (__ffs(km) - 1) + lane);  // bit and lane
           km &= km - 1u;
-          qu[pos - w0] = (uint32_t)((2 * (u0 + (bit & 15)) + (bit >> 4)) * 32 + lane);
           ++pos;
         }
         __syncwarp();
-        drain(min(32, tot - w0));
+        // the queue is filled by few lanes one after the other: the entries'
+        // rounds are decoded here, a lane each
+        drain(min(32, tot - w0), [&](uint32_t c) {
+          const uint32_t bit = c >> 5;
+          return (2 * (u0 + (bit & 15)) + (bit >> 4)) * 32 + (c & 31);
+        });
         __syncwarp();
       }
     }
   } else {
+    auto itself = [](uint32_t c) { return c; };
     for (int rr = 0; rr < rounds; ++rr) {
       const int idx = rr * 32 + lane;
       bool keep = false;
@@ -744,7 +750,7 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
       qn += __popc(ball);
       if (qn >= 32) {
         __syncwarp();
-        drain(32);
+        drain(32, itself);
         __syncwarp();
         const uint32_t moved = lane + 32 < qn ? qu[lane + 32] : 0u;  // at most 31 left
         __syncwarp();
@@ -754,7 +760,7 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
       }
     }
     __syncwarp();
-    if (qn > 0) drain(qn);
+    if (qn > 0) drain(qn, itself);
   }
   bidx = bidx == INT_MAX ? INT_MAX : __ldg(r.blk_pidx + bidx);  // slot -> pair index
 #pragma unroll
