@@ -169,7 +169,6 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
     __syncwarp();
     for (int g = lane; g < Sg && !r.sph_vec4; g += 32) {  // the same for groups over several links
       const int gl = __ldg(r.grp_link + g);
-      float4 B4;
       if (gl >= 0) {  // one link: its host-made bound, moved with the link
         const float4 L = __ldg(r.grp_loc + g);
         const float* T = P + 12 * gl;
@@ -178,29 +177,12 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
         rot(T, cl, c);
         const float scale = fabsf(T[9]) + fabsf(T[10]) + fabsf(T[11]) + fabsf(L.x) +
                             fabsf(L.y) + fabsf(L.z);
-        B4 = make_float4(c[0] + T[9] - ox, c[1] + T[10] - oy, c[2] + T[11] - oz,
-                         fmaf(scale, 1e-6f, fmaf(L.w, 1e-6f, L.w)) + ow);
+        gb[g] = half_bound(c[0] + T[9] - ox, c[1] + T[10] - oy, c[2] + T[11] - oz,
+                           fmaf(scale, 1e-6f, fmaf(L.w, 1e-6f, L.w)) + ow);
       } else {
-        const int s1 = min(S, 4 * g + 4);
-        float cx = 0.0f, cy = 0.0f, cz = 0.0f;
-        for (int s = 4 * g; s < s1; ++s) {
-          cx += xc[s];
-          cy += yc[s];
-          cz += zc[s];
-        }
-        const float inv = 1.0f / (float)max(s1 - 4 * g, 1);
-        cx *= inv;
-        cy *= inv;
-        cz *= inv;
-        const float4 rad = radw[g];
-        float R = 0.0f;
-        for (int s = 4 * g; s < s1; ++s)
-          R = fmaxf(R, sqrtf(dist2(cx, cy, cz, xc[s], yc[s], zc[s])) + p4(rad, s - 4 * g));
-        const float dx = cx - ox, dy = cy - oy, dz = cz - oz;
-        const float e = fmaf(fabsf(dx) + fabsf(dy) + fabsf(dz), 1e-6f, ow);  // for rounding
-        B4 = make_float4(dx, dy, dz, fmaf(R, 1e-6f, R) + e);
+        gb[g] = mixed_bound(reinterpret_cast<const float4*>(xc)[g], reinterpret_cast<const float4*>(yc)[g],
+                            reinterpret_cast<const float4*>(zc)[g], radw[g], S - 4 * g, ox, oy, oz, ow);
       }
-      gb[g] = half_bound(B4.x, B4.y, B4.z, B4.w);
       reinterpret_cast<float4*>(gx)[g] = zero4;
       reinterpret_cast<float4*>(gy)[g] = zero4;
       reinterpret_cast<float4*>(gz)[g] = zero4;

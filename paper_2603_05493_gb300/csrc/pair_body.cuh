@@ -471,24 +471,8 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
                            fmaf(scale, 1e-6f, fmaf(L.w, 1e-6f, L.w)) + ow);
         continue;
       }
-      const int s0 = 4 * g, s1 = min(S, s0 + 4);
-      float cx = 0.0f, cy = 0.0f, cz = 0.0f;
-      for (int s = s0; s < s1; ++s) {
-        cx += xc[s];
-        cy += yc[s];
-        cz += zc[s];
-      }
-      const float inv = 1.0f / (float)max(s1 - s0, 1);
-      cx *= inv;
-      cy *= inv;
-      cz *= inv;
-      const float4 rad = radw[g];
-      float R = 0.0f;
-      for (int s = s0; s < s1; ++s)
-        R = fmaxf(R, sqrtf(dist2(cx, cy, cz, xc[s], yc[s], zc[s])) + pick(rad, s - s0));
-      const float dx = cx - ox, dy = cy - oy, dz = cz - oz;
-      const float e = fmaf(fabsf(dx) + fabsf(dy) + fabsf(dz), 1e-6f, ow);  // widened for rounding
-      gb[g] = half_bound(dx, dy, dz, fmaf(R, 1e-6f, R) + e);
+      gb[g] = mixed_bound(reinterpret_cast<const float4*>(xc)[g], reinterpret_cast<const float4*>(yc)[g],
+                          reinterpret_cast<const float4*>(zc)[g], radw[g], S - 4 * g, ox, oy, oz, ow);
     }
   }
   if (BITS)

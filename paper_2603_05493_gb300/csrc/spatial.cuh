@@ -302,6 +302,27 @@ __device__ __forceinline__ uint2 half_bound(float x, float y, float z, float R) 
   const __half2 zr = __halves2half2(hz, __float2half_ru(grown));
   return make_uint2(*reinterpret_cast<const uint32_t*>(&xy), *reinterpret_cast<const uint32_t*>(&zr));
 }
+// The bound of a group over several links: the mean of its m centres, and the
+// farthest sphere's reach from it, widened by 1e-6 of itself (the approximate
+// square root's error is 2^-23 of it) and of the centre's place, and by ow.
+// X, Y, Z: the 4 centres (0 past the m-th), rad: their radii; ox, oy, oz: the
+// origin the bound is relative to.
+__device__ __forceinline__ uint2 mixed_bound(float4 X, float4 Y, float4 Z, float4 rad, int m,
+                                             float ox, float oy, float oz, float ow) {
+  const float inv = m >= 4 ? 0.25f : m == 3 ? 1.0f / 3.0f : m == 2 ? 0.5f : 1.0f;
+  const float cx = (X.x + X.y + X.z + X.w) * inv, cy = (Y.x + Y.y + Y.z + Y.w) * inv,
+              cz = (Z.x + Z.y + Z.z + Z.w) * inv;
+  auto reach = [&](float x, float y, float z, float r) {
+    return sqrt_approx(dist2(cx, cy, cz, x, y, z)) + r;
+  };
+  float R = m > 0 ? reach(X.x, Y.x, Z.x, rad.x) : 0.0f;
+  if (m > 1) R = fmaxf(R, reach(X.y, Y.y, Z.y, rad.y));
+  if (m > 2) R = fmaxf(R, reach(X.z, Y.z, Z.z, rad.z));
+  if (m > 3) R = fmaxf(R, reach(X.w, Y.w, Z.w, rad.w));
+  const float dx = cx - ox, dy = cy - oy, dz = cz - oz;
+  const float e = fmaf(fabsf(dx) + fabsf(dy) + fabsf(dz), 1e-6f, ow);
+  return half_bound(dx, dy, dz, fmaf(R, 1e-6f, R) + e);
+}
 // The sphere that stands for the groups of a null block: far from every finite
 // bound, so that a null block is rarely kept (and then has no pair to work).
 __device__ __forceinline__ uint2 far_bound() {
