@@ -189,8 +189,8 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
     }
     __syncwarp();
     float cost = 0.0f;
-    const uint4* off = ps.off + lane;
-    uint4 en = __ldg(off);  // one step ahead (the table ends with a null row)
+    const uint2* off = ps.off + lane;
+    uint2 en = __ldg(off);  // one step ahead (the table ends with a null row)
     for (int u0 = 0; u0 < prs; u0 += 16) {
       // blocks whose bound is under eta can hold an active pair; bit v: round
       // 2 (u0 + v), bit 16 + v: the one after
@@ -198,14 +198,14 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
       const int u1 = min(prs - u0, 16);
 #pragma unroll 2
       for (int v = 0; v < u1; ++v) {
-        const uint4 e = en;
+        const uint2 e = en;
         off += 32;
         en = __ldg(off);
-        auto under = [&](uint32_t o0, uint32_t o1) {  // also where the bound is no number
-          return !(half_gap(*reinterpret_cast<const uint2*>(cgb + o0),
-                            *reinterpret_cast<const uint2*>(cgb + o1)) >= eta);
+        auto under = [&](uint32_t o) {  // also where the bound is no number
+          return !(half_gap(*reinterpret_cast<const uint2*>(cgb + (o & 0xFFFF)),
+                            *reinterpret_cast<const uint2*>(cgb + (o >> 16))) >= eta);
         };
-        km |= (under(e.x, e.y) ? 1u << v : 0u) | (under(e.z, e.w) ? 0x10000u << v : 0u);
+        km |= (under(e.x) ? 1u << v : 0u) | (under(e.y) ? 0x10000u << v : 0u);
       }
       const int cnt = __popc(km);
       int sum = cnt;  // inclusive scan of the counts over the lanes
@@ -228,8 +228,8 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
         // is here where its bound was under eta or no number: no block
         // (the entries' rounds are decoded here: the queue is filled by few lanes)
         const uint32_t c = qu[lane], bit = c >> 5;
-        const uint32_t at = (2 * (u0 + (bit & 15)) + (bit >> 4)) * 32 + (c & 31);
-        const uint2 e = lane < count ? __ldg(ps.ent + at) : make_uint2(0u, 0u);
+        const uint32_t at = 2 * ((u0 + (bit & 15)) * 32 + (c & 31)) + (bit >> 4);
+        const uint2 e = lane < count ? ps.at(at) : make_uint2(0u, 0u);
         const bool block = (e.y >> 16) != 0u;
         uint32_t key = 0xFFFFFFFFu;  // no block
         float gr[12];  // the lane's block: its row spheres' gradients, then its columns'

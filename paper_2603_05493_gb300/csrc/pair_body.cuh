@@ -509,22 +509,22 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
   const bool keep_lb = prs * 32 <= pl.ra_words();
   __half2* lb2 = reinterpret_cast<__half2*>(xr) + lane;
   const char* cgb = reinterpret_cast<const char*>(gb);
-  auto bound = [&](uint32_t o0, uint32_t o1) {
-    return half_gap(*reinterpret_cast<const uint2*>(cgb + o0),
-                    *reinterpret_cast<const uint2*>(cgb + o1));
+  auto bound = [&](uint32_t o) {  // the two groups' offsets
+    return half_gap(*reinterpret_cast<const uint2*>(cgb + (o & 0xFFFF)),
+                    *reinterpret_cast<const uint2*>(cgb + (o >> 16)));
   };
   auto keyed = [](float lb, int rr) {  // any block gives a valid bound: 12 bits of it decide
     return __int_as_float((__float_as_int(lb) & ~0x7FF) | rr);
   };
   float lbmin = inf;
-  const uint4* off = ps.off + lane;
-  uint4 en = __ldg(off);  // one step ahead (the table ends with a null row)
+  const uint2* off = ps.off + lane;
+  uint2 en = __ldg(off);  // one step ahead (the table ends with a null row)
 #pragma unroll 2
   for (int u = 0; u < prs; ++u) {
-    const uint4 e = en;
+    const uint2 e = en;
     off += 32;
     en = __ldg(off);
-    const float b0 = bound(e.x, e.y), b1 = bound(e.z, e.w);
+    const float b0 = bound(e.x), b1 = bound(e.y);
     if (keep_lb) lb2[u * 32] = __floats2half2_rn(b0, b1);
     lbmin = fminf(lbmin, fminf(keyed(b0, 2 * u), keyed(b1, 2 * u + 1)));
   }
@@ -533,7 +533,7 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
     const int kmin = __reduce_min_sync(0xffffffffu, fkey(lbmin));
     const int src = __ffs(__ballot_sync(0xffffffffu, fkey(lbmin) == kmin)) - 1;
     const int rbest = __shfl_sync(0xffffffffu, __float_as_int(lbmin), src) & 0x7FF;
-    const uint2 e = __ldg(ps.ent + rbest * 32 + src);
+    const uint2 e = ps.at(round_entry(rbest, src));
     float d = inf;
     const int t = lane & 15, a = t >> 2, c = t & 3;
     if (lane < 16 && ((e.y >> 16) >> t) & 1u) {
@@ -669,9 +669,9 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
       }
     }
   };
-  // screen queue entries [0, count), one per lane; at: an entry's place in ps.ent
+  // screen queue entries [0, count), one per lane; at: an entry's place in the schedule
   auto drain = [&](int count, auto&& at) {
-    const uint2 e = lane < count ? __ldg(ps.ent + at(qu[lane])) : make_uint2(0u, 0u);
+    const uint2 e = lane < count ? ps.at(at(qu[lane])) : make_uint2(0u, 0u);
     __syncwarp();
     if ((e.y >> 16) != 0u) screen_block(e);
     gbest = fminf(gbest, fkey_inv(__reduce_min_sync(0xffffffffu, fkey(best))));
@@ -712,35 +712,35 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
         // rounds are decoded here, a lane each
         drain(min(32, tot - w0), [&](uint32_t c) {
           const uint32_t bit = c >> 5;
-          return (2 * (u0 + (bit & 15)) + (bit >> 4)) * 32 + (c & 31);
+          return 2 * ((u0 + (bit & 15)) * 32 + (c & 31)) + (bit >> 4);
         });
         __syncwarp();
       }
     }
   } else {
     auto itself = [](uint32_t c) { return c; };
-    for (int rr = 0; rr < rounds; ++rr) {
-      const int idx = rr * 32 + lane;
-      bool keep = false;
-      {
-        const uint2 e = __ldg(ps.ent + idx);
-        if ((e.y >> 16) != 0u) {
-          const float lb = bound((e.x & 0xFFFF) >> 1, (e.x >> 16) >> 1);
+    for (int u = 0; u < prs; ++u) {
+      const uint2 o = __ldg(ps.off + u * 32 + lane), y = __ldg(ps.blk + u * 32 + lane);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        bool keep = false;
+        if (((h ? y.y : y.x) >> 16) != 0u) {
+          const float lb = bound(h ? o.y : o.x);
           keep = !(lb > fminf(best, gbest) + reach_tol) || (BITS && !(lb > reach_tol));
         }
-      }
-      const uint32_t ball = __ballot_sync(0xffffffffu, keep);
-      if (keep) qu[qn + __popc(ball & ((1u << lane) - 1u))] = (uint32_t)idx;
-      qn += __popc(ball);
-      if (qn >= 32) {
-        __syncwarp();
-        drain(32, itself);
-        __syncwarp();
-        const uint32_t moved = lane + 32 < qn ? qu[lane + 32] : 0u;  // at most 31 left
-        __syncwarp();
-        if (lane + 32 < qn) qu[lane] = moved;
-        qn -= 32;
-        __syncwarp();
+        const uint32_t ball = __ballot_sync(0xffffffffu, keep);
+        if (keep) qu[qn + __popc(ball & ((1u << lane) - 1u))] = (uint32_t)(64 * u + 2 * lane + h);
+        qn += __popc(ball);
+        if (qn >= 32) {
+          __syncwarp();
+          drain(32, itself);
+          __syncwarp();
+          const uint32_t moved = lane + 32 < qn ? qu[lane + 32] : 0u;  // at most 31 left
+          __syncwarp();
+          if (lane + 32 < qn) qu[lane] = moved;
+          qn -= 32;
+          __syncwarp();
+        }
       }
     }
     __syncwarp();

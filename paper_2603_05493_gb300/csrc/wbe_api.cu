@@ -801,20 +801,23 @@ int wb_load_robot(const wb_tree* tree, const wb_spheres* sph, const wb_pairs* pa
   R->sched32.rounds = R->sched[3].rounds;
   pk.add_vec(ent32, &R->sched32.ent);
   R->sched32.prs = (R->sched32.rounds + 1) / 2;
-  std::vector<uint4> off32((size_t)(R->sched32.prs + 1) * 32);
+  std::vector<uint2> off32((size_t)(R->sched32.prs + 1) * 32), blk32(off32.size());
   for (size_t i = 0; i < off32.size(); ++i) {
     const size_t u = i / 32, l = i % 32;
-    uint32_t o[4];
+    uint32_t o[4], y[2];
     for (int h = 0; h < 2; ++h) {
       const size_t at = (2 * u + h) * 32 + l;
       const uint2 e = at < ent32.size() ? ent32[at] : uint2{0u, 0u};
       const bool block = (e.y >> 16) != 0u;
+      y[h] = block ? e.y : 0u;
       o[2 * h] = block ? (e.x & 0xFFFF) / 2 : 0u;
       o[2 * h + 1] = block ? (e.x >> 16) / 2 : 4u * (uint32_t)far_words(H.Sg);
     }
-    off32[i] = make_uint4(o[0], o[1], o[2], o[3]);
+    off32[i] = make_uint2(o[0] | o[1] << 16, o[2] | o[3] << 16);
+    blk32[i] = make_uint2(y[0], y[1]);
   }
   pk.add_vec(off32, &R->sched32.off);
+  pk.add_vec(blk32, &R->sched32.blk);
   cudaError_t e = cudaMalloc(&R->dmem, pk.host.size());
   if (e != cudaSuccess) {
     delete R;

@@ -105,13 +105,25 @@ struct PairSchedule {
 struct PairSchedule32 {
   int rounds;
   const uint2* ent;          // [rounds + 1][32], the last round all null
-  // for the bounds on whole blocks, two rounds at a time: the two blocks' byte
-  // offsets (8 gi, 8 gj each) in an array of group bounds; a null block is
-  // group 0 against a far sphere that the kernels put far_words(Sg) behind
-  // the array's start (prs = pairs of rounds, rounded up)
+  // The same for the kernels that bound whole blocks, two rounds at a time: the two
+  // blocks' byte offsets 8 gi | (8 gj) << 16 in an array of group bounds, and (in
+  // an array of its own, read for the kept blocks only) their mask << 16 | id; a
+  // null block is group 0 against a far sphere that the kernels put far_words(Sg)
+  // behind the array's start (prs = pairs of rounds, rounded up).  8 bytes a block
+  // in all: with 16 the tables of two robots of a batch no longer fit the L1 that
+  // the workspaces of a third, of 255 links, leave (23- and 48-DoF beside one:
+  // 0.42 ms, 0.37 with 12 bytes)
   int prs;
-  const uint4* off;          // [prs + 1][32]
+  const uint2* off;          // [prs + 1][32]
+  const uint2* blk;          // [prs + 1][32]
+  // entry i of those arrays, as `ent` has it
+  __device__ __forceinline__ uint2 at(int i) const {
+    return make_uint2(__ldg(reinterpret_cast<const uint32_t*>(off) + i) << 1,
+                      __ldg(reinterpret_cast<const uint32_t*>(blk) + i));
+  }
 };
+// where lane l's entry of round rr is in them
+__host__ __device__ constexpr int round_entry(int rr, int l) { return ((rr & ~1) << 5) + 2 * l + (rr & 1); }
 // where that far sphere sits behind the group spheres of Sg groups: the last 4
 // words of the 64-word queue that follows them
 __host__ __device__ constexpr int far_words(int Sg) { return ((4 * Sg + 31) & ~31) + 60; }
