@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(128, 6) hinge_kernel(const __grid_constant__ D
         // (the entries' rounds are decoded here: the queue is filled by few lanes)
         const uint32_t c = qu[lane], bit = c >> 5;
         const uint32_t at = 2 * ((u0 + (bit & 15)) * 32 + (c & 31)) + (bit >> 4);
-        const uint2 e = lane < count ? ps.at(at) : make_uint2(0u, 0u);
+        const uint2 e = lane < count ? sched_at(ps, at) : make_uint2(0u, 0u);
         const bool block = (e.y >> 16) != 0u;
         uint32_t key = 0xFFFFFFFFu;  // no block
         float gr[12];  // the lane's block: its row spheres' gradients, then its columns'

@@ -533,7 +533,7 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
     const int kmin = __reduce_min_sync(0xffffffffu, fkey(lbmin));
     const int src = __ffs(__ballot_sync(0xffffffffu, fkey(lbmin) == kmin)) - 1;
     const int rbest = __shfl_sync(0xffffffffu, __float_as_int(lbmin), src) & 0x7FF;
-    const uint2 e = ps.at(round_entry(rbest, src));
+    const uint2 e = sched_at(ps, round_entry(rbest, src));
     float d = inf;
     const int t = lane & 15, a = t >> 2, c = t & 3;
     if (lane < 16 && ((e.y >> 16) >> t) & 1u) {
@@ -671,7 +671,7 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
   };
   // screen queue entries [0, count), one per lane; at: an entry's place in the schedule
   auto drain = [&](int count, auto&& at) {
-    const uint2 e = lane < count ? ps.at(at(qu[lane])) : make_uint2(0u, 0u);
+    const uint2 e = lane < count ? sched_at(ps, at(qu[lane])) : make_uint2(0u, 0u);
     __syncwarp();
     if ((e.y >> 16) != 0u) screen_block(e);
     gbest = fminf(gbest, fkey_inv(__reduce_min_sync(0xffffffffu, fkey(best))));

@@ -278,6 +278,12 @@ __device__ __forceinline__ float dist2(float xi, float yi, float zi, float xj, f
   return fmaf(dz, dz, fmaf(dy, dy, dx * dx));
 }
 
+// entry i of the schedule's arrays for the bounds (round_entry), as `ent` has it
+__device__ __forceinline__ uint2 sched_at(const PairSchedule32& ps, int i) {
+  return make_uint2(__ldg(reinterpret_cast<const uint32_t*>(ps.off) + i) << 1,
+                    __ldg(reinterpret_cast<const uint32_t*>(ps.blk) + i));
+}
+
 // approximate square root (relative error at most 2^-23)
 __device__ __forceinline__ float sqrt_approx(float x) {
   float y;

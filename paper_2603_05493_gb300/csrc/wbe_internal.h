@@ -116,11 +116,6 @@ struct PairSchedule32 {
   int prs;
   const uint2* off;          // [prs + 1][32]
   const uint2* blk;          // [prs + 1][32]
-  // entry i of those arrays, as `ent` has it
-  __device__ __forceinline__ uint2 at(int i) const {
-    return make_uint2(__ldg(reinterpret_cast<const uint32_t*>(off) + i) << 1,
-                      __ldg(reinterpret_cast<const uint32_t*>(blk) + i));
-  }
 };
 // where lane l's entry of round rr is in them
 __host__ __device__ constexpr int round_entry(int rr, int l) { return ((rr & ~1) << 5) + 2 * l + (rr & 1); }
