@@ -54,13 +54,78 @@ int main() {
 """
 
 
+OCCUPANCY = r"""
+#include "wbe_internal.h"
+#include <cstdio>
+static int g_pct = -1, g_asked = 0;
+extern "C" {
+cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
+  *v = a == cudaDevAttrMaxRegistersPerMultiprocessor ? 65536
+     : a == cudaDevAttrMaxThreadsPerMultiProcessor ? 2048
+     : a == cudaDevAttrMaxBlocksPerMultiprocessor ? 32
+     : a == cudaDevAttrReservedSharedMemoryPerBlock ? 1024 : 228 * 1024;
+  return cudaSuccess;
+}
+cudaError_t cudaFuncGetAttributes(cudaFuncAttributes* f, const void*) {
+  f->numRegs = 128;
+  f->sharedSizeBytes = 0;
+  return cudaSuccess;
+}
+cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute a, int v) {
+  if (a == cudaFuncAttributePreferredSharedMemoryCarveout) g_pct = v;
+  return cudaSuccess;
+}
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* n, const void*, int, size_t smem) {
+  ++g_asked;
+  *n = (int)((g_pct < 0 ? 100 : g_pct) * 228 * 1024 / 100 / (smem + 1024));
+  return cudaSuccess;
+}
+}
+int bad = 0;
+#define EXPECT(x) if (!(x)) { std::printf("line %d: %s (carveout %d)\n", __LINE__, #x, g_pct); ++bad; }
+int main() {
+  const int k = 0, other = 0;
+  using namespace wbe;
+  int first = 0, n = 0;
+  EXPECT(max_blocks(&other, 128, 18 * 1024, &first) == cudaSuccess && first == 12);
+  EXPECT(g_pct == -1);  // a kernel without a preference keeps none
+  fit_carveout(&k, 128, 3 * 1024);
+  const int small = g_pct;
+  EXPECT(small > 0 && small < 10);
+  EXPECT(max_blocks(&k, 128, 18 * 1024, &n) == cudaSuccess && n == first);
+  EXPECT(g_pct == small);
+  fit_carveout(&k, 128, 18 * 1024);
+  EXPECT(g_pct > small);
+  launch_cache_clear(0);
+  EXPECT(max_blocks(&k, 128, 18 * 1024, &n) == cudaSuccess && n == first);
+  fit_carveout(&k, 128, 3 * 1024);
+  EXPECT(g_pct == small);
+  const int asked = g_asked;
+  EXPECT(max_blocks(&k, 128, 18 * 1024, &n) == cudaSuccess && n == first && g_asked == asked);
+  return bad;
+}
+"""
+
+
+def test_occupancy_does_not_depend_on_earlier_launches(tmp_path):
+    """The blocks an SM holds, asked after a launch of another shape has left its
+    carveout: the same, and the carveout is put back."""
+    run(tmp_path, OCCUPANCY)
+
+
 def test_limit_is_only_raised(tmp_path):
+    run(tmp_path, HARNESS)
+
+
+def run(tmp_path, source):
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
     cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
     if shutil.which("g++") is None or not os.path.exists(os.path.join(cuda, "cuda_runtime.h")):
         pytest.skip("needs g++ and the CUDA headers")
     main = tmp_path / "main.cpp"
-    main.write_text(HARNESS)
+    main.write_text(source)
     exe = str(tmp_path / "cache")
     subprocess.run(["g++", "-std=c++17", "-I" + CSRC, "-I" + cuda, str(main), "-x", "c++",
                     os.path.join(CSRC, "launch_cache.cu"), "-o", exe], check=True)
