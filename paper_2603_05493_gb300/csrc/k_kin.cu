@@ -356,36 +356,41 @@ static int kin_single_warps(const DevRobot& r, int warps) {
 
 size_t kin_smem_per_warp(const DevRobot& r) { return sizeof(float) * kin_words(r.n); }
 
-// a block of the general kernel has `warps` warps; the single-link one at most
-// as many
-cudaError_t launch_kin(const DevRobot& r, const KinArgs& a, int grid, int warps, cudaStream_t s) {
-  if (kin_single_ok(r)) {
-    const int w = kin_single_warps(r, warps);
-    const size_t smem = KinPlan(r.n, r.d).bytes(w);
-    const cudaError_t e = allow_smem((const void*)kin_single_kernel, smem);
-    if (e != cudaSuccess) return e;
-    kin_single_kernel<<<grid, w * 32, smem, s>>>(r, a);
-    return cudaGetLastError();
-  }
+// Which kernel a call takes and how many of its blocks an SM holds.  A block of the
+// general kernel has `warps` warps; the single-link one's at most as many.  The
+// tables cost a block about half a microsecond, which one or two outputs (targets,
+// the centre of mass) of robots with a joint a lane repay only when a warp takes
+// more than one or two configurations: 23-DoF, one target, 3000 configurations 3.5
+// us by the general kernel and 4.0 by the other, 32768 12.5 and 11.8; two targets
+// 4.2 and 4.4, 17.2 and 14.4; four targets 5.4 and 5.1 (48-DoF, one target: 4.8 and
+// 4.8, 25.4 and 24.4).
+cudaError_t kin_shape(const DevRobot& r, const KinArgs& a, int warps, int num_sms, bool* single,
+                      int* bps) {
   const size_t smem = sizeof(float) * kin_words(r.n) * warps;
-  const cudaError_t e = allow_smem((const void*)kin_kernel, smem);
+  cudaError_t e = allow_smem((const void*)kin_kernel, smem);
+  if (e == cudaSuccess) e = max_blocks((const void*)kin_kernel, warps * 32, smem, bps);
   if (e != cudaSuccess) return e;
-  kin_kernel<<<grid, warps * 32, smem, s>>>(r, a);
-  return cudaGetLastError();
+  const int outputs = (a.jac ? a.nt : 0) + (a.com || a.jac_com ? 1 : 0);
+  const int64_t resident = (int64_t)*bps * warps * num_sms;
+  const int64_t few = r.d > 32 || outputs > 2 ? 0 : outputs == 2 ? resident : 2 * resident;
+  *single = kin_single_ok(r) && a.B > few;
+  if (!*single) return cudaSuccess;
+  const int w = kin_single_warps(r, warps);
+  const size_t smem1 = KinPlan(r.n, r.d).bytes(w);
+  e = allow_smem((const void*)kin_single_kernel, smem1);
+  if (e != cudaSuccess) return e;
+  return max_blocks((const void*)kin_single_kernel, w * 32, smem1, bps);
 }
 
-cudaError_t kin_max_blocks_per_sm(const DevRobot& r, int warps, int* out) {
-  if (kin_single_ok(r)) {
+cudaError_t launch_kin(const DevRobot& r, const KinArgs& a, bool single, int grid, int warps,
+                       cudaStream_t s) {
+  if (single) {
     const int w = kin_single_warps(r, warps);
-    const size_t smem = KinPlan(r.n, r.d).bytes(w);
-    const cudaError_t e = allow_smem((const void*)kin_single_kernel, smem);
-    if (e != cudaSuccess) return e;
-    return max_blocks((const void*)kin_single_kernel, w * 32, smem, out);
+    kin_single_kernel<<<grid, w * 32, KinPlan(r.n, r.d).bytes(w), s>>>(r, a);
+  } else {
+    kin_kernel<<<grid, warps * 32, sizeof(float) * kin_words(r.n) * warps, s>>>(r, a);
   }
-  const size_t smem = sizeof(float) * kin_words(r.n) * warps;
-  const cudaError_t e = allow_smem((const void*)kin_kernel, smem);
-  if (e != cudaSuccess) return e;
-  return max_blocks((const void*)kin_kernel, warps * 32, smem, out);
+  return cudaGetLastError();
 }
 
 }  // namespace wbe

@@ -1275,19 +1275,20 @@ int wb_kinematics(wb_robot* robot, int64_t B, const float* link_pose, int32_t n_
   DeviceGuard guard(robot->device);
   const int warps = warps_that_fit(0, kin_smem_per_warp(robot->dev));
   if (warps == 0) return fail(WB_ETOOBIG, "kinematics kernel does not fit on an SM");
-  int bps = 0;
-  cudaError_t e = kin_max_blocks_per_sm(robot->dev, warps, &bps);
-  if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
-  if (bps < 1) return fail(WB_ETOOBIG, "kinematics kernel does not fit on an SM");
-  const int64_t need = (B + warps - 1) / warps;
-  const int grid = (int)std::min<int64_t>(need, (int64_t)bps * robot->num_sms);
   a.B = B;
   a.pose = link_pose;
   a.nt = n_targets;
   a.jac = jac;
   a.com = com;
   a.jac_com = jac_com;
-  e = launch_kin(robot->dev, a, grid, warps, static_cast<cudaStream_t>(stream));
+  bool single = false;
+  int bps = 0;
+  cudaError_t e = kin_shape(robot->dev, a, warps, robot->num_sms, &single, &bps);
+  if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
+  if (bps < 1) return fail(WB_ETOOBIG, "kinematics kernel does not fit on an SM");
+  const int64_t need = (B + warps - 1) / warps;
+  const int grid = (int)std::min<int64_t>(need, (int64_t)bps * robot->num_sms);
+  e = launch_kin(robot->dev, a, single, grid, warps, static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "wb_kinematics launch");
   return WB_OK;
 }

@@ -275,8 +275,10 @@ struct KinArgs {
   float* com;         // [B][3] or nullptr
   float* jac_com;     // [B][3][d] or nullptr
 };
-cudaError_t launch_kin(const DevRobot& r, const KinArgs& a, int grid, int warps, cudaStream_t s);
-cudaError_t kin_max_blocks_per_sm(const DevRobot& r, int warps, int* out);
+cudaError_t kin_shape(const DevRobot& r, const KinArgs& a, int warps, int num_sms, bool* single,
+                      int* bps);
+cudaError_t launch_kin(const DevRobot& r, const KinArgs& a, bool single, int grid, int warps,
+                       cudaStream_t s);
 size_t kin_smem_per_warp(const DevRobot& r);
 
 // all-pairs summed collision hinge (k_hinge.cu)
