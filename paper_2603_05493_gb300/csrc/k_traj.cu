@@ -99,6 +99,25 @@ __device__ __forceinline__ float knot_grad(const float* tab, const int* first, i
   }
   return acc;
 }
+// The same sum walking the samples instead of the segments, most of which are empty
+// where the knots outnumber the samples.
+template <class G>
+__device__ __forceinline__ float knot_grad_sparse(const float* tab, const int* first, int nseg,
+                                                  int T, int x, const G& g) {
+  const int m0 = max(x - 3, 0), m1 = min(x, nseg - 1);
+  float acc = 0.0f;
+  if (m0 > m1) return acc;
+  int m = m0;
+  for (int s = first[m0]; s < first[m1 + 1]; ++s) {
+    while (s >= first[m + 1]) ++m;  // the sample's segment
+    const float* Bs = tab + (x - m) * T + s;
+    float c = fmaf(Bs[0], g.q(s), 0.0f);
+    c = fmaf(Bs[4 * T], g.v(s), c);
+    c = fmaf(Bs[8 * T], g.a(s), c);
+    acc += c;
+  }
+  return acc;
+}
 struct StagedRow {
   const float *r0, *r1, *r2;
   __device__ __forceinline__ float q(int s) const { return r0[s]; }
@@ -118,19 +137,6 @@ struct GlobalRow {  // nullptr: zero
   __device__ __forceinline__ float a(int s) const { return sum(gqdd, gqdd2, at + s); }
 };
 
-// One thread per control point (trajectory, joint, k), plus with a start
-// state one per (trajectory, joint) for the start-state gradient (no atomics,
-// deterministic).  A block takes one joint of R consecutive trajectories; the
-// basis rows and segment of every sample and the first sample of every segment
-// are tabled in shared memory.  With a static goal the last control point also
-// sums the gradients of its three repeats; the start-state gradient is the
-// transpose of the ghost knots' linear map applied to their three gradients.
-// STAGE: the block's R T samples, contiguous in the [d][B] arrays, are read
-// once into shared memory (the two qd and the two qdd gradients added), where
-// each is used by four knots; else (a row too long for that) the threads read
-// them from global memory.  Bound by the latency of a knot's serial sum, which
-// reads shared instead of L2: humanoid 512 x 64 samples, 16 knots 0.020 -> 0.017
-// ms; an arm's 100 x 33 samples with both ends 0.0145 -> 0.0063 ms.
 // *dst (shared) = a[at] (+ b[at]), 0 where there is none: a lone array by an
 // asynchronous copy, so that all of a thread's samples are on their way at once
 __device__ __forceinline__ void stage(float* dst, const float* a, const float* b, int64_t at) {
@@ -145,7 +151,22 @@ __device__ __forceinline__ void stage(float* dst, const float* a, const float* b
 // the stride of a staged row: rows of a multiple of 32 samples are set 16 banks apart
 __host__ __device__ constexpr int row_stride(int T) { return T % 32 == 0 ? T + 16 : T; }
 
-template <bool STAGE>
+// One thread per control point (trajectory, joint, k), plus with a start
+// state one per (trajectory, joint) for the start-state gradient (no atomics,
+// deterministic).  The basis rows of every sample and the first sample of every
+// segment are tabled in shared memory.  With a static goal the last control point
+// also sums the gradients of its three repeats; the start-state gradient is the
+// transpose of the ghost knots' linear map applied to their three gradients.
+// kKnotStaged: a block takes one joint of R consecutive trajectories and reads their
+// R T samples, contiguous in the [d][B] arrays, once into shared memory (the two qd
+// and the two qdd gradients added), where each is used by four knots.  kKnotRows:
+// the same with rows too long for that, read from global memory.  kKnotFlat: a block
+// takes 256 consecutive control points of any rows (see launch_bspline_bwd).  Bound
+// by the latency of a knot's serial sum, which reads shared instead of L2: humanoid
+// 512 x 64 samples, 16 knots 0.020 -> 0.016 ms; an arm's 100 x 33 samples with both
+// ends 0.0145 -> 0.0056 ms.
+enum KnotMode { kKnotStaged, kKnotRows, kKnotFlat };
+template <int MODE>
 __global__ void __launch_bounds__(256) bspline_bwd_kernel(
     int64_t n_traj, int d, int K, int T, float dt, int hs, int es, int R,
     const float* __restrict__ gq, const float* __restrict__ gqd, const float* __restrict__ gqdd,
@@ -155,7 +176,7 @@ __global__ void __launch_bounds__(256) bspline_bwd_kernel(
   const int Kx = K + 3 * hs + 3 * es;
   const int nseg = Kx - 3;
   const int Tp = row_stride(T);
-  float* rows = tab + (size_t)T * 12 + ((Kx - 2 + 3) & ~3);  // STAGE: [3][nr][Tp]
+  float* rows = tab + (size_t)T * 12 + ((Kx - 2 + 3) & ~3);  // kKnotStaged: [3][nr][Tp]
   for (int s = threadIdx.x; s < T; s += blockDim.x) {
     int k;
     float a;
@@ -171,12 +192,42 @@ __global__ void __launch_bounds__(256) bspline_bwd_kernel(
   for (int m = threadIdx.x; m <= nseg; m += blockDim.x)
     first[m] = m == nseg ? T : (m * (T - 1) + nseg - 1) / nseg;
   const int64_t B = n_traj * T;
+  const int per = K + hs;  // threads per (trajectory, joint)
+  // item t of trajectory and joint tj = trajectory * d + joint; kg: its row's knots
+  auto item = [&](int t, int64_t tj, auto&& kg) {
+    if (t < hs) {  // the start-state gradient through u_-3, u_-2, u_-1
+      const float g3 = kg(0), g2 = kg(1), g1 = kg(2);
+      if (gstart) {
+        float* o = gstart + tj * 3;
+        o[0] = g3 + g2 + g1;
+        o[1] = dt * fmaf(2.0f, g1, g2);
+        o[2] = dt * dt * fmaf(11.0f / 6.0f, g1, fmaf(1.0f / 3.0f, g2, (-1.0f / 6.0f) * g3));
+      }
+      return;
+    }
+    const int k = t - hs;
+    const int x = k + 3 * hs;
+    float acc = kg(x);
+    if (es && k == K - 1)
+      for (int r = 1; r <= 3; ++r) acc += kg(x + r);
+    gU[tj * K + k] = acc;
+  };
+  if (MODE == kKnotFlat) {
+    __syncthreads();
+    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (idx >= n_traj * d * per) return;
+    const int64_t tj = idx / per, tr = tj / d;
+    const GlobalRow g{gq, gqd, gqdd, gqd2, gqdd2, (tj - tr * d) * B + tr * T};
+    item((int)(idx - tj * per), tj,
+         [&](int x) { return knot_grad_sparse(tab, first, nseg, T, x, g); });
+    return;
+  }
   const uint32_t per_joint = (uint32_t)((n_traj + R - 1) / R);  // blocks of a joint
   const int j = (int)(blockIdx.x / per_joint);
   const int64_t tr0 = (int64_t)(blockIdx.x - j * per_joint) * R;
   const int nr = (int)(n_traj - tr0 < R ? n_traj - tr0 : R);
   const int64_t base = (int64_t)j * B + tr0 * T;
-  if (STAGE) {  // a warp a row
+  if (MODE == kKnotStaged) {  // a warp a row
     const int plane = nr * Tp;
     for (int row = threadIdx.x >> 5; row < nr; row += blockDim.x >> 5) {
       float* o = rows + row * Tp;
@@ -191,33 +242,15 @@ __global__ void __launch_bounds__(256) bspline_bwd_kernel(
     asm volatile("cp.async.wait_group 0;" ::: "memory");
   }
   __syncthreads();
-  const int per = K + hs;  // threads per (trajectory, joint)
   for (int i = threadIdx.x; i < nr * per; i += blockDim.x) {
-    const int row = i / per, t = i - row * per;
-    const int64_t tj = (tr0 + row) * d + j;  // trajectory * d + joint
+    const int row = i / per;
     const float* o = rows + row * Tp;
-    auto kg = [&](int x) {
-      if (STAGE)
+    item(i - row * per, (tr0 + row) * d + j, [&](int x) {
+      if (MODE == kKnotStaged)
         return knot_grad(tab, first, nseg, T, x, StagedRow{o, o + nr * Tp, o + 2 * nr * Tp});
       return knot_grad(tab, first, nseg, T, x,
                        GlobalRow{gq, gqd, gqdd, gqd2, gqdd2, base + (int64_t)row * T});
-    };
-    if (t < hs) {  // the start-state gradient through u_-3, u_-2, u_-1
-      const float g3 = kg(0), g2 = kg(1), g1 = kg(2);
-      if (gstart) {
-        float* o = gstart + tj * 3;
-        o[0] = g3 + g2 + g1;
-        o[1] = dt * fmaf(2.0f, g1, g2);
-        o[2] = dt * dt * fmaf(11.0f / 6.0f, g1, fmaf(1.0f / 3.0f, g2, (-1.0f / 6.0f) * g3));
-      }
-      continue;
-    }
-    const int k = t - hs;
-    const int x = k + 3 * hs;
-    float acc = kg(x);
-    if (es && k == K - 1)
-      for (int r = 1; r <= 3; ++r) acc += kg(x + r);
-    gU[tj * K + k] = acc;
+    });
   }
 }
 
@@ -305,15 +338,29 @@ cudaError_t launch_bspline_bwd(int64_t n_traj, int d, int K, int T, float dt, in
   const size_t tables = sizeof(float) * ((size_t)T * 12 + ((Kx - 2 + 3) & ~3));
   const size_t row = sizeof(float) * 3 * (size_t)row_stride(T);
   const int64_t room = tables + row <= limit ? (int64_t)((limit - tables) / row) : 0;
-  const bool stage = room > 0;
-  const int64_t most = std::max(1, 256 / (K + hs));
-  const int R = (int)std::min<int64_t>({most, stage ? room : most, n_traj});
-  const int block = std::min(256, std::max(64, (R * (K + hs) + 31) / 32 * 32));
+  const int per = K + hs;
+  const int64_t joints = n_traj * d;
+  // Where the knots outnumber the samples a row is little work, and rows of up to 256
+  // knots fill a block badly: the flat deal is the better one (8178 x 1, 139 knots of
+  // 32 samples 14.3 us against 21.9 by rows; 3755 x 48, 19 of 12 49 and 66).  So it is
+  // for longer rows as long as its blocks, each with tables of its own, are all
+  // resident (one arm's 4096 knots of 4096 samples 8.2 and 24.3 us, 1024 of 2048 6.1
+  // and 10.4; but 86 x 7, 1730 of 87: 20.7 and 13.6; 48 joints' 4096 of 4096: 41.8 and
+  // 24.3).
+  const int64_t deal = (joints * per + 255) / 256;
+  const int64_t resident = sm_count() * std::min<int64_t>(8, 227 * 1024 / (bspline_bwd_smem(Kx, T) + 1024));
+  const bool flat = per <= 256 ? 2 * per >= 3 * T : 2 * per >= T && deal <= resident;
+  const int most = std::max(1, 256 / per);
+  const int R = (int)std::min<int64_t>({(int64_t)most, room > 0 ? room : most, n_traj});
+  const bool stage = room > 0 && !flat;
+  const int block = flat ? 256 : std::min(256, std::max(64, (R * per + 31) / 32 * 32));
   const size_t smem = stage ? tables + row * R : bspline_bwd_smem(Kx, T);
-  auto kern = stage ? bspline_bwd_kernel<true> : bspline_bwd_kernel<false>;
+  auto kern = flat    ? bspline_bwd_kernel<kKnotFlat>
+              : stage ? bspline_bwd_kernel<kKnotStaged>
+                      : bspline_bwd_kernel<kKnotRows>;
   cudaError_t e = allow_smem((const void*)kern, smem);
   if (e != cudaSuccess) return e;
-  const int64_t grid = (n_traj + R - 1) / R * d;
+  const int64_t grid = flat ? deal : (n_traj + R - 1) / R * d;
   kern<<<(unsigned)grid, block, smem, s>>>(n_traj, d, K, T, dt, hs, es, R, gq, gqd, gqdd, gqd2,
                                          gqdd2, gU, gstart);
   return cudaGetLastError();

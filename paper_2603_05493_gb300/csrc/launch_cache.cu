@@ -97,7 +97,7 @@ cudaError_t max_blocks(const void* kern, int threads, size_t smem, int* out) {
 // the SM limits fit_carveout needs, queried once per device (host threads may
 // launch on several devices at once)
 struct SmLimits {
-  int smem_sm, regs_sm, threads_sm, blocks_sm, reserved;
+  int smem_sm, regs_sm, threads_sm, blocks_sm, reserved, sms;
 };
 static bool sm_limits(int dev, SmLimits* out) {
   constexpr int kDevices = 64;
@@ -111,6 +111,7 @@ static bool sm_limits(int dev, SmLimits* out) {
                cudaSuccess &&
            cudaDeviceGetAttribute(&l->blocks_sm, cudaDevAttrMaxBlocksPerMultiprocessor, d) ==
                cudaSuccess &&
+           cudaDeviceGetAttribute(&l->sms, cudaDevAttrMultiProcessorCount, d) == cudaSuccess &&
            cudaDeviceGetAttribute(&l->reserved, cudaDevAttrReservedSharedMemoryPerBlock, d) ==
                cudaSuccess &&
            cudaDeviceGetAttribute(&l->smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, d) ==
@@ -124,6 +125,14 @@ static bool sm_limits(int dev, SmLimits* out) {
   }
   *out = cache[dev];
   return true;
+}
+
+int sm_count() {
+  int dev = 0;
+  SmLimits L;
+  if (cudaGetDevice(&dev) == cudaSuccess && sm_limits(dev, &L) && L.sms > 0) return L.sms;
+  cudaGetLastError();
+  return 152;
 }
 
 // Shared memory and L1 are one array per SM.  Without a preference the

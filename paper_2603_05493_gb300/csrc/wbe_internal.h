@@ -338,6 +338,7 @@ void fit_carveout(const void* kern, int threads, size_t smem);
 cudaError_t allow_smem(const void* kern, size_t smem);
 cudaError_t max_blocks(const void* kern, int threads, size_t smem, int* out);
 void launch_cache_clear(int device);
+int sm_count();  // of the current device
 int tree_max_depth();
 
 size_t pair_block_smem(const DevRobot& r, int warps, bool bits);  // the same, out of line
