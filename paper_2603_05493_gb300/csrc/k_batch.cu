@@ -42,10 +42,14 @@ __device__ __forceinline__ void pair_bar(int id) {
 }
 
 // shared memory: one item slot per pair (32 words, up to 32 pairs), then per
-// pair its robot's link records and walk words (n_max links), staged when the
-// pair's robot changes, and the partials [nout][ns_max][2][32]
+// pair its robot's link records and walk words (n_max links) and the second
+// segment's ancestors, staged when the pair's robot changes, and the partials
+// [nout][ns_max][2][32]
+__host__ __device__ inline size_t batch_walk_words(int n_max) {
+  return (size_t)kRecWords * n_max + ((n_max + 31) & ~31) + kRepDepth;
+}
 __host__ __device__ inline size_t batch_pair_words(int nout, int ns_max, int n_max) {
-  return (size_t)kRecWords * n_max + ((n_max + 31) & ~31) + (size_t)nout * ns_max * 64;
+  return batch_walk_words(n_max) + (size_t)nout * ns_max * 64;
 }
 __host__ __device__ inline size_t batch_tree_words(int nout, int ns_max, int n_max, int pairs) {
   return 32 + (size_t)pairs * batch_pair_words(nout, ns_max, n_max);
@@ -67,9 +71,11 @@ __device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, 
 
 // the pair's robot changed: its records (with plan 0's slots, read only by a
 // segmented sweep) and walk words
-__device__ __forceinline__ void stage_robot(const DevRobot& r, float4* rec, uint32_t* wk, int i0) {
+__device__ __forceinline__ void stage_robot(const DevRobot& r, float4* rec, uint32_t* wk,
+                                            uint32_t* rep, int i0) {
   stage_recs(r, 0, rec, i0, 64);
   for (int i = i0; i < r.n; i += 64) wk[i] = __ldg(r.walk + i);
+  if (i0 < kRepDepth) rep[i0] = __ldg(r.walk_rep + 3 * kRepDepth + i0);
 }
 
 __global__ void __launch_bounds__(256) batch_tree_fwd_kernel(const DevRobot* robots,
@@ -84,7 +90,8 @@ __global__ void __launch_bounds__(256) batch_tree_fwd_kernel(const DevRobot* rob
   float* base = sm + 32 + (size_t)pi * batch_pair_words(1, ns_max, n_max);
   float4* rec = reinterpret_cast<float4*>(base);
   uint32_t* wk = reinterpret_cast<uint32_t*>(base + (size_t)kRecWords * n_max);
-  float* part = base + (size_t)kRecWords * n_max + ((n_max + 31) & ~31);
+  float* part = base + batch_walk_words(n_max);
+  uint32_t* rep = reinterpret_cast<uint32_t*>(part) - kRepDepth;
   int cur = -1;
   for (;;) {
     if (g == 0 && lane == 0) *slot = atomicAdd(counter, 1);
@@ -96,7 +103,7 @@ __global__ void __launch_bounds__(256) batch_tree_fwd_kernel(const DevRobot* rob
     const DevRobot& r = robots[pb.robot];
     const int robot = uniform(pb.robot);
     if (robot != cur) {
-      stage_robot(r, rec, wk, 32 * g + lane);
+      stage_robot(r, rec, wk, rep, 32 * g + lane);
       cur = robot;
       pair_bar(bar);
     }
@@ -122,7 +129,7 @@ __global__ void __launch_bounds__(256) batch_tree_fwd_kernel(const DevRobot* rob
     sg.p1 = uniform(sg.p1);
     for (int q = 0; q < ns; ++q) part[(q * 2 + g) * 32 + lane] = 0.0f;
     if (some)
-      tree_fwd_seg<kFwdLocal>(r, rec, SharedWalk{wk}, A, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b,
+      tree_fwd_seg<kFwdLocal>(r, rec, SharedWalk{wk, rep}, A, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b,
                           act, sg);
     pair_bar(bar);
     if (lane < w.z && A.tau)
@@ -148,7 +155,8 @@ __global__ void __launch_bounds__(256, 2) batch_tree_bwd_kernel(const DevRobot* 
   float* base = sm + 32 + (size_t)pi * batch_pair_words(3, ns_max, n_max);
   float4* rec = reinterpret_cast<float4*>(base);
   uint32_t* wk = reinterpret_cast<uint32_t*>(base + (size_t)kRecWords * n_max);
-  float* part = base + (size_t)kRecWords * n_max + ((n_max + 31) & ~31);
+  float* part = base + batch_walk_words(n_max);
+  uint32_t* rep = reinterpret_cast<uint32_t*>(part) - kRepDepth;
   // the gradient-row slots behind every pair's partials
   const GradSlot gs = grad_slot_of(sm + batch_tree_words(3, ns_max, n_max, blockDim.x / 64));
   int cur = -1;
@@ -162,7 +170,7 @@ __global__ void __launch_bounds__(256, 2) batch_tree_bwd_kernel(const DevRobot* 
     const DevRobot& r = robots[pb.robot];
     const int robot = uniform(pb.robot);
     if (robot != cur) {
-      stage_robot(r, rec, wk, 32 * g + lane);
+      stage_robot(r, rec, wk, rep, 32 * g + lane);
       cur = robot;
       pair_bar(bar);
     }
@@ -191,7 +199,7 @@ __global__ void __launch_bounds__(256, 2) batch_tree_bwd_kernel(const DevRobot* 
     for (int q = 0; q < ns; ++q)
       for (int k = 0; k < 3; ++k) part[k * o + (q * 2 + g) * 32 + lane] = 0.0f;
     if (some)
-      tree_bwd_seg<OPT>(r, rec, SharedWalk{wk}, A, FusedCost{},
+      tree_bwd_seg<OPT>(r, rec, SharedWalk{wk, rep}, A, FusedCost{},
                           ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg, gs);
     pair_bar(bar);
     if (lane < w.z)

@@ -64,7 +64,7 @@ __device__ __forceinline__ void fwd_block(const DevRobot& r, const WalkTab& wt, 
     sg.fst = reinterpret_cast<float2*>(sm) + threadIdx.x;
     sg.fstr = blockDim.x;
   }
-  tree_fwd_seg<MODE>(r, rec, ConstWalk{wt}, A, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg);
+  tree_fwd_seg<MODE>(r, rec, ConstWalk<true>{wt}, A, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg);
 }
 template <int MODE>
 __global__ void __launch_bounds__(256) tree_fwd_kernel(const __grid_constant__ DevRobot r,
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(256, 2) tree_bwd_kernel(const __grid_constant_
   bool act;
   if (!own_config(A.B, blockIdx.x * (int64_t)blockDim.x + 32 * warp_of(), &b, &act)) return;
   const GradSlot gs = grad_slot_of(reinterpret_cast<float*>(rec) + bwd_words(r));
-  tree_bwd_seg<OPT>(r, rec, ConstWalk{wt}, A, FusedCost{},
+  tree_bwd_seg<OPT>(r, rec, ConstWalk<false>{wt}, A, FusedCost{},
                       ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, whole_sweep(r), gs);
 }
 
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(512) tree_fwd_seg_kernel(const __grid_constant
   int64_t b;
   bool act = false;
   if (own_config(A.B, ((int64_t)blockIdx.x * CG + cg) * 32, &b, &act))
-    tree_fwd_seg<MODE>(r, rec, ConstWalk{wt}, A, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg);
+    tree_fwd_seg<MODE>(r, rec, ConstWalk<true>{wt}, A, ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg);
   __syncthreads();
   if (act && A.tau) {
     for (int s = sg.g; s < ns; s += G) {
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(512, 1) tree_bwd_seg_kernel(const __grid_const
   int64_t b;
   bool act = false;
   if (own_config(A.B, ((int64_t)blockIdx.x * CG + cg) * 32, &b, &act))
-    tree_bwd_seg<OPT>(r, rec, ConstWalk{wt}, A, FusedCost{},
+    tree_bwd_seg<OPT>(r, rec, ConstWalk<false>{wt}, A, FusedCost{},
                         ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg, gs);
   __syncthreads();
   if (act) {
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(256, 2) tree_bwd_cost_kernel(
   bool act;
   if (!own_config(A.B, blockIdx.x * (int64_t)blockDim.x + 32 * warp_of(), &b, &act)) return;
   const GradSlot gs = grad_slot_of(reinterpret_cast<float*>(rec) + bwd_words(r));
-  const float c = tree_bwd_seg<kBwdCost | OPT>(r, rec, ConstWalk{wt}, A, fc,
+  const float c = tree_bwd_seg<kBwdCost | OPT>(r, rec, ConstWalk<false>{wt}, A, fc,
                                      ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act,
                                      whole_sweep(r), gs);
   if (fc.cost) fc.cost[b] = total_cost(fc, b, c);
@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(512, 1) tree_bwd_cost_seg_kernel(
   bool act = false;
   float c = 0.0f;
   if (own_config(A.B, ((int64_t)blockIdx.x * CG + cg) * 32, &b, &act))
-    c = tree_bwd_seg<kBwdCost | OPT>(r, rec, ConstWalk{wt}, A, fc,
+    c = tree_bwd_seg<kBwdCost | OPT>(r, rec, ConstWalk<false>{wt}, A, fc,
                            ArrayStates{A.q, A.qd, A.qdd, A.B, b}, b, act, sg, gs);
   cpart[sg.g * 32 + sg.lane] = c;
   __syncthreads();
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(256) tree_fwd_spline_kernel(
   bool act;
   if (!own_config(A.B, blockIdx.x * (int64_t)blockDim.x + 32 * warp_of(), &b, &act)) return;
   const SplineStates st = spline_states(r, sp, b, sm + 12 * threadIdx.x);
-  tree_fwd_seg<MODE>(r, rec, ConstWalk{wt}, A, st, b, act, whole_sweep(r));
+  tree_fwd_seg<MODE>(r, rec, ConstWalk<true>{wt}, A, st, b, act, whole_sweep(r));
 }
 
 // MODE as for tree_fwd_seg_kernel; the force stack follows the partials
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(512) tree_fwd_spline_seg_kernel(
   int64_t b;
   bool act = false;
   if (own_config(A.B, ((int64_t)blockIdx.x * CG + cg) * 32, &b, &act))
-    tree_fwd_seg<MODE>(r, rec, ConstWalk{wt}, A, spline_states(r, sp, b, sm + 12 * threadIdx.x), b,
+    tree_fwd_seg<MODE>(r, rec, ConstWalk<true>{wt}, A, spline_states(r, sp, b, sm + 12 * threadIdx.x), b,
                      act, sg);
   __syncthreads();
   if (act && A.tau) {
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(256, 2) tree_bwd_spline_cost_kernel(
   bool act;
   if (!own_config(A.B, blockIdx.x * (int64_t)blockDim.x + 32 * warp_of(), &b, &act)) return;
   const GradSlot gs = grad_slot_of(sm + 12 * blockDim.x);
-  const float c = tree_bwd_seg<kBwdCost | OPT>(r, rec, ConstWalk{wt}, A, fc,
+  const float c = tree_bwd_seg<kBwdCost | OPT>(r, rec, ConstWalk<false>{wt}, A, fc,
                                                spline_states(r, sp, b, sm + 12 * threadIdx.x), b,
                                                act, whole_sweep(r), gs);
   if (fc.cost) fc.cost[b] = total_cost(fc, b, c);
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(512, 1) tree_bwd_spline_cost_seg_kernel(
   bool act = false;
   float c = 0.0f;
   if (own_config(A.B, ((int64_t)blockIdx.x * CG + cg) * 32, &b, &act))
-    c = tree_bwd_seg<kBwdCost | OPT>(r, rec, ConstWalk{wt}, A, fc,
+    c = tree_bwd_seg<kBwdCost | OPT>(r, rec, ConstWalk<false>{wt}, A, fc,
                            spline_states(r, sp, b, sm + 12 * threadIdx.x), b, act, sg, gs);
   cpart[sg.g * 32 + sg.lane] = c;
   __syncthreads();

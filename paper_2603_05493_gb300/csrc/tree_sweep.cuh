@@ -78,18 +78,6 @@ constexpr int TMAXD = 32;  // deepest tree the sweep kernels accept
 // come from the constant bank into uniform registers, so the sweep's branches
 // need no reconvergence (with the words in global memory a fifth of the
 // forward's instructions were branches, barriers and moves around them).
-struct ConstWalk {
-  static constexpr bool kSpheres = true;  // the spheres are staged behind the records
-  const WalkTab& t;
-  __device__ __forceinline__ uint32_t operator()(int pos) const { return t.w[pos]; }
-};
-struct SharedWalk {  // the batch's: staged with the link records, made uniform by a shuffle
-  static constexpr bool kSpheres = false;
-  const uint32_t* w;
-  __device__ __forceinline__ uint32_t operator()(int pos) const {
-    return __shfl_sync(0xffffffffu, w[pos], 0);
-  }
-};
 __device__ __forceinline__ int wk_dep(uint32_t w) { return w & 31; }
 __device__ __forceinline__ bool wk_branch(uint32_t w) { return (w >> 5) & 1; }  // >= 2 children
 __device__ __forceinline__ int wk_jt(uint32_t w) { return (w >> 6) & 3; }
@@ -97,6 +85,34 @@ __device__ __forceinline__ bool wk_ident(uint32_t w) { return (w >> 8) & 1; }
 __device__ __forceinline__ bool wk_leaf(uint32_t w) { return (w >> 9) & 1; }
 __device__ __forceinline__ int wk_j(uint32_t w) { return (w >> 10) & 255; }
 __device__ __forceinline__ int wk_par(uint32_t w) { return (w >> 18) & 255; }
+
+// TABLE: the ancestors that a segment replays come from a table.  The backward climbs
+// to each of them from the segment's first link instead: with the table's address
+// beside its state it spilled (128 registers).
+template <bool TABLE>
+struct ConstWalk {
+  static constexpr bool kSpheres = true;  // the spheres are staged behind the records
+  const WalkTab& t;
+  __device__ __forceinline__ uint32_t operator()(int pos) const { return t.w[pos]; }
+  // the position of the ancestor at depth c of p0, the first link of segment g of G
+  __device__ __forceinline__ int ancestor(int p0, int G, int g, int c) const {
+    if (TABLE) return t.rep[G + g][c];
+    int pos = p0;
+    for (uint32_t w = t.w[pos]; wk_dep(w) > c; w = t.w[pos]) pos = wk_par(w);
+    return pos;
+  }
+};
+struct SharedWalk {  // the batch's: staged with the link records, made uniform by a shuffle
+  static constexpr bool kSpheres = false;
+  const uint32_t* w;    // the walk words
+  const uint32_t* rep;  // [kRepDepth] the ancestors of the second of two segments' first link
+  __device__ __forceinline__ uint32_t operator()(int pos) const {
+    return __shfl_sync(0xffffffffu, w[pos], 0);
+  }
+  __device__ __forceinline__ int ancestor(int, int, int g, int c) const {
+    return g == 0 ? 0 : (int)__shfl_sync(0xffffffffu, rep[c], 0);
+  }
+};
 
 // One segment of a segmented sweep (see above).  part == nullptr: the whole
 // DFS order, outputs written directly.
@@ -115,17 +131,6 @@ struct Seg {
 
 __device__ __forceinline__ Seg whole_sweep(const DevRobot& r) {
   return Seg{0, r.n, 0, 1, nullptr, 0, 0};
-}
-
-// the position of the ancestor at depth c of position pos
-template <class WK>
-__device__ __forceinline__ int ancestor_at(const WK& wk, int pos, int c) {
-  uint32_t w = wk(pos);
-  while (wk_dep(w) > c) {
-    pos = wk_par(w);
-    w = wk(pos);
-  }
-  return pos;
 }
 
 // the robot's spheres, behind its staged records (the backward reads a link's
@@ -513,7 +518,7 @@ __device__ __forceinline__ void tree_fwd_seg(const DevRobot& r, const float4* re
   // current link's closes and push.
   const int nrep = wk_dep(wk(sg.p0)), total = nrep + sg.p1 - sg.p0;
   int sp = 0;
-  int npos = ancestor_at(wk, sg.p0, 0);
+  int npos = wk.ancestor(sg.p0, sg.G, sg.g, 0);
   uint32_t nw = wk(npos);
   float nq = 0.0f, nqd = 0.0f, nqdd = 0.0f;
   auto ahead = [&]() {
@@ -535,7 +540,7 @@ __device__ __forceinline__ void tree_fwd_seg(const DevRobot& r, const float4* re
     const int dep = end ? 0 : wk_dep(w);
     const float cq = nq, cqd = nqd, cqdd = nqdd;
     if (i + 1 < total) {
-      npos = i + 1 < nrep ? ancestor_at(wk, sg.p0, i + 1) : sg.p0 + i + 1 - nrep;
+      npos = i + 1 < nrep ? wk.ancestor(sg.p0, sg.G, sg.g, i + 1) : sg.p0 + i + 1 - nrep;
       nw = wk(npos);
       ahead();
     }
@@ -1150,7 +1155,7 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const float4* r
   // forward
   const int nrep = wk_dep(wk(sg.p0)), total = nrep + sg.p1 - sg.p0;
   int sp = 0;
-  int npos = ancestor_at(wk, sg.p0, 0);
+  int npos = wk.ancestor(sg.p0, sg.G, sg.g, 0);
   uint32_t nw = wk(npos);
   const float* const gt = FC ? fc.tau : A.g_tau;
   float nq = 0.0f, nqd = 0.0f, nqdd = 0.0f, ngt = 0.0f;
@@ -1175,7 +1180,7 @@ __device__ __forceinline__ float tree_bwd_seg(const DevRobot& r, const float4* r
     // 0.314 ms at 99999)
     if (!end) fetch(w);
     if (i + 1 < total) {
-      npos = i + 1 < nrep ? ancestor_at(wk, sg.p0, i + 1) : sg.p0 + i + 1 - nrep;
+      npos = i + 1 < nrep ? wk.ancestor(sg.p0, sg.G, sg.g, i + 1) : sg.p0 + i + 1 - nrep;
       nw = wk(npos);
       if (wk_jt(nw)) {
         st.prefetch(wk_j(nw), true);

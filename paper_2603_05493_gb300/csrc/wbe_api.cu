@@ -725,6 +725,13 @@ int wb_load_robot(const wb_tree* tree, const wb_spheres* sph, const wb_pairs* pa
   pk.add_vec(H.recs, &D.recs);
   pk.add_vec(H.walk, &D.walk);
   std::copy(H.walk.begin(), H.walk.end(), R->walk.w);
+  for (int t = 0; t < 3; ++t)
+    for (int g = 0; g < 2 << t && (H.seg_ok >> t & 1); ++g)
+      for (int p = H.seg_pos[t][g], k = H.dfs[p].x; k >= 0; k = H.parent[k])
+        if (H.dfs[H.dfs_pos[k]].y < kRepDepth)
+          R->walk.rep[(2 << t) + g][H.dfs[H.dfs_pos[k]].y] = (uint8_t)H.dfs_pos[k];
+  const uint8_t* rep0 = &R->walk.rep[0][0];
+  pk.add_vec(std::vector<uint8_t>(rep0, rep0 + sizeof(R->walk.rep)), &D.walk_rep);
   R->seg_cost[0] = (float)n;
   for (int t = 0; t < 3; ++t) R->seg_cost[t + 1] = H.seg_cost[t];
   pk.add_vec(H.chain_start, &D.chain_start);
