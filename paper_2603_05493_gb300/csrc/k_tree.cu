@@ -74,11 +74,10 @@ __global__ void __launch_bounds__(256) tree_fwd_kernel(const __grid_constant__ D
   fwd_block<MODE>(r, wt, A, rec);
 }
 // The same for robots without branches, capped at 72 registers: 28 warps an SM
-// where 78 allow 24.  The sweep is latency-bound, a chain never touches the branch
-// stack, and its force stack leaves the shared memory for them (21 KB a 128-thread
-// block for 7 links; the humanoid's 46 KB stop at 4 blocks, and there the cap only
-// spills: 0.190 -> 0.228 ms).  7-DoF arm, 131072 configurations: 0.0280 -> 0.0249
-// ms (64 registers: 0.0293; the branch code compiled out besides: 0.0263).
+// where 78 allow 24, at the price of spills (fwd_chain: when it is taken).  The
+// sweep is latency-bound and a chain never touches the branch stack.  7-DoF arm,
+// 131072 configurations: 0.0280 -> 0.0249 ms (64 registers: 0.0293; the branch code
+// compiled out besides: 0.0263).
 __global__ void __maxnreg__(72) tree_fwd_chain_kernel(const __grid_constant__ DevRobot r,
                                                       const __grid_constant__ WalkTab wt,
                                                       const __grid_constant__ FwdArgs A) {
@@ -471,6 +470,27 @@ static cudaError_t launch_bwd(void (*kern)(P...), int64_t B, int groups, int blo
   return cudaGetLastError();
 }
 
+// Whether the chain kernel is the better one: where the batch has more warps an SM
+// than the general kernel's registers hold and the force stacks of its blocks leave
+// the shared memory for more (21 KB a 128-thread block for 7 links do; 37 KB for 12
+// do not, nor do the humanoid's 46).  Elsewhere the spills are all it brings: 12, 20
+// and 32 links, 131072 configurations 0.058, 0.124, 0.291 ms against 0.040, 0.101,
+// 0.193; the arm's 99999 configurations 0.0209 and 0.0182.
+static cudaError_t fwd_chain(const DevRobot& r, int64_t B, int threads, size_t smem, bool* out) {
+  *out = false;
+  if (r.maxdepth != r.n) return cudaSuccess;  // a link a level: no branches
+  const void* kerns[2] = {(const void*)tree_fwd_kernel<kFwdShared>,
+                          (const void*)tree_fwd_chain_kernel};
+  int blocks[2] = {0, 0};
+  for (int i = 0; i < 2; ++i) {
+    cudaError_t e = allow_smem(kerns[i], smem);
+    if (e == cudaSuccess) e = max_blocks(kerns[i], threads, smem, &blocks[i]);
+    if (e != cudaSuccess) return e;
+  }
+  *out = blocks[1] > blocks[0] && B > (int64_t)blocks[0] * threads * sm_count();
+  return cudaSuccess;
+}
+
 cudaError_t launch_tree_fwd(const DevRobot& r, const WalkTab& wt, const FwdArgs& a, int threads, int segments,
                             cudaStream_t s) {
   if (threads <= 0) threads = 128;
@@ -488,12 +508,14 @@ cudaError_t launch_tree_fwd(const DevRobot& r, const WalkTab& wt, const FwdArgs&
   const size_t fs = sizeof(float) * 6 * fs_levels(r) * threads;  // the force stack
   const bool use_fs = a.tau && rec_smem(r, true) + fs <= kSegSmemMax;
   const size_t smem = rec_smem(r, true) + (use_fs ? fs : 0);
-  auto kern = use_fs ? (r.maxdepth == r.n ? tree_fwd_chain_kernel  // a link a level: no branches
-                                          : tree_fwd_kernel<kFwdShared>)
-              : a.tau ? tree_fwd_kernel<kFwdLocal>
-                      : tree_fwd_kernel<kFwdPose>;
-  cudaError_t e =
-      allow_smem((const void*)kern, smem);
+  bool chain = false;
+  cudaError_t e = use_fs ? fwd_chain(r, a.B, threads, smem, &chain) : cudaSuccess;
+  if (e != cudaSuccess) return e;
+  auto kern = chain    ? tree_fwd_chain_kernel
+              : use_fs ? tree_fwd_kernel<kFwdShared>
+              : a.tau  ? tree_fwd_kernel<kFwdLocal>
+                       : tree_fwd_kernel<kFwdPose>;
+  e = allow_smem((const void*)kern, smem);
   if (e != cudaSuccess) return e;
   fit_carveout((const void*)kern, threads, smem);
   const int64_t grid = (a.B + threads - 1) / threads;
