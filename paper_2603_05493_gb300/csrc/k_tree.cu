@@ -470,6 +470,24 @@ static cudaError_t launch_bwd(void (*kern)(P...), int64_t B, int groups, int blo
   return cudaGetLastError();
 }
 
+// Dynamic shared memory of a block of G segments that writes poses only.  Its 46 or 48
+// registers a thread allow 40 warps an SM, whose lanes each write 48 bytes at a time
+// into rows of their own (G places of a row at once); when the poses no longer fit
+// the L2 (129 MB) it evicts lines that are not yet full.  So batches of more than 20
+// warps an SM then have at most 16 at a time: humanoid, 131072 configurations (308
+// MB) 0.239 -> 0.195 ms (12 warps the same, 20 0.201), 23-DoF (150 MB) 0.118 -> 0.093;
+// 99999 configurations 0.171 -> 0.155 and, at 110 MB in two segments, 0.081 -> 0.064.
+// Smaller poses are better off without (20 links, 110 MB: 0.041 ms), and so are up to
+// 20 warps (32 links, 80000 configurations 0.068 and 0.073).
+static size_t pose_smem(const DevRobot& r, int64_t B, int G, int threads, size_t smem) {
+  const int64_t warps = (B + 31) / 32 * G;
+  if (B * r.n * 48 <= (int64_t)(G > 1 ? 100 : 112) << 20 || warps <= 20LL * sm_count())
+    return smem;
+  const size_t blocks = std::max(1, 16 * 32 / threads);
+  const size_t share = 228 * 1024 / blocks - 1024;  // 228 KB an SM, 1 KB of it each block's own
+  return std::max(smem, std::min(kSegSmemMax, share));
+}
+
 // Whether the chain kernel is the better one: where the batch has more warps an SM
 // than the general kernel's registers hold and the force stacks of its blocks leave
 // the shared memory for more (21 KB a 128-thread block for 7 links do; 37 KB for 12
@@ -502,12 +520,15 @@ cudaError_t launch_tree_fwd(const DevRobot& r, const WalkTab& wt, const FwdArgs&
     const size_t fs = sizeof(float) * 6 * fs_levels(r) * bt;
     if (a.tau && tree_seg_smem(r, segments, threads, true, false) + fs <= kSegSmemMax)
       return launch_seg(tree_fwd_seg_kernel<kFwdShared>, r, wt, a, threads, segments, true, fs, s);
+    const size_t base = tree_seg_smem(r, segments, threads, true, false);
     return launch_seg(a.tau ? tree_fwd_seg_kernel<kFwdLocal> : tree_fwd_seg_kernel<kFwdPose>, r, wt,
-                      a, threads, segments, true, 0, s);
+                      a, threads, segments, true,
+                      a.tau ? 0 : pose_smem(r, a.B, segments, (int)bt, base) - base, s);
   }
   const size_t fs = sizeof(float) * 6 * fs_levels(r) * threads;  // the force stack
   const bool use_fs = a.tau && rec_smem(r, true) + fs <= kSegSmemMax;
-  const size_t smem = rec_smem(r, true) + (use_fs ? fs : 0);
+  size_t smem = rec_smem(r, true) + (use_fs ? fs : 0);
+  if (!a.tau) smem = pose_smem(r, a.B, 1, threads, smem);
   bool chain = false;
   cudaError_t e = use_fs ? fwd_chain(r, a.B, threads, smem, &chain) : cudaSuccess;
   if (e != cudaSuccess) return e;
@@ -562,7 +583,7 @@ cudaError_t launch_tree_fwd_spline(const DevRobot& r, const WalkTab& wt, const F
     const size_t base = tree_seg_smem(r, segments, threads, true, false) + 12 * sizeof(float) * block;
     const size_t fs = sizeof(float) * 6 * fs_levels(r) * block;  // the force stack
     const bool use_fs = a.tau && base + fs <= kSegSmemMax;
-    const size_t smem = use_fs ? base + fs : base;
+    const size_t smem = use_fs ? base + fs : a.tau ? base : pose_smem(r, a.B, segments, block, base);
     auto kern = use_fs ? tree_fwd_spline_seg_kernel<kFwdShared>
                 : a.tau ? tree_fwd_spline_seg_kernel<kFwdLocal>
                         : tree_fwd_spline_seg_kernel<kFwdPose>;
@@ -574,8 +595,11 @@ cudaError_t launch_tree_fwd_spline(const DevRobot& r, const WalkTab& wt, const F
     kern<<<(unsigned)grid, block, smem, s>>>(r, wt, a, sp, t);
     return cudaGetLastError();
   }
-  const size_t smem = 12 * sizeof(float) * threads + rec_smem(r, true);
+  size_t smem = 12 * sizeof(float) * threads + rec_smem(r, true);
+  if (!a.tau) smem = pose_smem(r, a.B, 1, threads, smem);
   auto kern = a.tau ? tree_fwd_spline_kernel<kFwdLocal> : tree_fwd_spline_kernel<kFwdPose>;
+  const cudaError_t e = allow_smem((const void*)kern, smem);
+  if (e != cudaSuccess) return e;
   fit_carveout((const void*)kern, threads, smem);
   const int64_t grid = (a.B + threads - 1) / threads;
   kern<<<(unsigned)grid, threads, smem, s>>>(r, wt, a, sp);
