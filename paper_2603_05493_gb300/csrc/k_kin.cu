@@ -363,9 +363,11 @@ size_t kin_smem_per_warp(const DevRobot& r) { return sizeof(float) * kin_words(r
 // more than one or two configurations: 23-DoF, one target, 3000 configurations 3.5
 // us by the general kernel and 4.0 by the other, 32768 12.5 and 11.8; two targets
 // 4.2 and 4.4, 17.2 and 14.4; four targets 5.4 and 5.1 (48-DoF, one target: 4.8 and
-// 4.8, 25.4 and 24.4).
-cudaError_t kin_shape(const DevRobot& r, const KinArgs& a, int warps, int num_sms, bool* single,
-                      int* bps) {
+// 4.8, 25.4 and 24.4).  A lone target that few joints move is little work but for the
+// tables, which a joint that does not move it needs all the same: the base of the
+// 23-DoF tree, 32768 configurations 10.6 and 11.6.
+cudaError_t kin_shape(const DevRobot& r, const KinArgs& a, int warps, int num_sms, int movers,
+                      bool* single, int* bps) {
   const size_t smem = sizeof(float) * kin_words(r.n) * warps;
   cudaError_t e = allow_smem((const void*)kin_kernel, smem);
   if (e == cudaSuccess) e = max_blocks((const void*)kin_kernel, warps * 32, smem, bps);
@@ -373,7 +375,8 @@ cudaError_t kin_shape(const DevRobot& r, const KinArgs& a, int warps, int num_sm
   const int outputs = (a.jac ? a.nt : 0) + (a.com || a.jac_com ? 1 : 0);
   const int64_t resident = (int64_t)*bps * warps * num_sms;
   const int64_t few = r.d > 32 || outputs > 2 ? 0 : outputs == 2 ? resident : 2 * resident;
-  *single = kin_single_ok(r) && a.B > few;
+  const bool still = outputs == 1 && a.jac && 8 * movers <= r.d;
+  *single = kin_single_ok(r) && !still && a.B > few;
   if (!*single) return cudaSuccess;
   const int w = kin_single_warps(r, warps);
   const size_t smem1 = KinPlan(r.n, r.d).bytes(w);

@@ -72,6 +72,7 @@ struct wb_robot {
   PairSchedule sched[4]{};    // G = 4, 8, 16, 32
   PairSchedule32 sched32{};   // the pair kernel's (byte-offset encoding)
   wb_robot_info info{};
+  std::vector<int16_t> movers;  // joints that move each link
   // host copies needed by set_inertials
   int n = 0, S = 0;
   float* h_stage = nullptr;   // pinned staging buffer for inertia uploads
@@ -730,6 +731,9 @@ int wb_load_robot(const wb_tree* tree, const wb_spheres* sph, const wb_pairs* pa
       for (int p = H.seg_pos[t][g], k = H.dfs[p].x; k >= 0; k = H.parent[k])
         if (H.dfs[H.dfs_pos[k]].y < kRepDepth)
           R->walk.rep[(2 << t) + g][H.dfs[H.dfs_pos[k]].y] = (uint8_t)H.dfs_pos[k];
+  R->movers.assign(n, 0);
+  for (int k = 0; k < n; ++k)
+    R->movers[k] = (int16_t)((H.parent[k] < 0 ? 0 : R->movers[H.parent[k]]) + (H.jidx[k] >= 0));
   const uint8_t* rep0 = &R->walk.rep[0][0];
   pk.add_vec(std::vector<uint8_t>(rep0, rep0 + sizeof(R->walk.rep)), &D.walk_rep);
   R->seg_cost[0] = (float)n;
@@ -1288,9 +1292,10 @@ int wb_kinematics(wb_robot* robot, int64_t B, const float* link_pose, int32_t n_
   a.jac = jac;
   a.com = com;
   a.jac_com = jac_com;
+  const int movers = n_targets == 1 ? robot->movers[targets[0]] : robot->dev.d;
   bool single = false;
   int bps = 0;
-  cudaError_t e = kin_shape(robot->dev, a, warps, robot->num_sms, &single, &bps);
+  cudaError_t e = kin_shape(robot->dev, a, warps, robot->num_sms, movers, &single, &bps);
   if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
   if (bps < 1) return fail(WB_ETOOBIG, "kinematics kernel does not fit on an SM");
   const int64_t need = (B + warps - 1) / warps;

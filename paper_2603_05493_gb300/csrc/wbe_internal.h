@@ -281,8 +281,9 @@ struct KinArgs {
   float* com;         // [B][3] or nullptr
   float* jac_com;     // [B][3][d] or nullptr
 };
-cudaError_t kin_shape(const DevRobot& r, const KinArgs& a, int warps, int num_sms, bool* single,
-                      int* bps);
+// movers: the joints that move a lone target
+cudaError_t kin_shape(const DevRobot& r, const KinArgs& a, int warps, int num_sms, int movers,
+                      bool* single, int* bps);
 cudaError_t launch_kin(const DevRobot& r, const KinArgs& a, bool single, int grid, int warps,
                        cudaStream_t s);
 size_t kin_smem_per_warp(const DevRobot& r);

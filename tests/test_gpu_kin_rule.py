@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("com", [False, True])
-@pytest.mark.parametrize("targets", [[], [4], [6, 2], [1, 3, 6]])
+@pytest.mark.parametrize("targets", [[], [4], [0], [6, 2], [1, 3, 6]])
 @pytest.mark.parametrize("name", ["R7", "R23"])
 def test_batches_agree(name, targets, com):
     from paper_2603_05493_gb300 import build, wbe
