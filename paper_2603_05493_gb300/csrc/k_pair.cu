@@ -3,6 +3,8 @@
 // or the full map-reduce pair_one (pair_body.cuh).
 #include "pair_body.cuh"
 
+#include <algorithm>
+
 namespace wbe {
 
 template <bool FULL, bool BITS, bool CULL>
@@ -332,6 +334,34 @@ __global__ void __launch_bounds__(32 * kSmallWarps) pair_small_kernel(
   }
 }
 
+// Whether the thread-per-configuration kernel is the faster one: estimates in us from
+// both kernels at 9150 to 300000 configurations of 8 to 32 spheres and 1 to 336 pairs
+// (within 20 %).  A warp of the eight-lane kernel takes 4 configurations, a fixed
+// price and one more for every 8 blocks beyond the first 8; a thread of the other its
+// spheres and pairs one after the other, for which its blocks, 128 configurations'
+// centres each, have to be resident.  So the latter is the better one for a few pairs
+// and a batch that fills the chip: two links, 16 pairs, 131072 configurations 11.9 us
+// and 21.3; the arm with 16 pairs, 50000 12.3 and 16.9; with all 240 30.1 and 22.6.
+static cudaError_t thread_better(const DevRobot& r, int64_t B, bool* out) {
+  *out = false;
+  if (B < 24576) return cudaSuccess;  // too few to fill the chip with threads
+  const size_t smem = pair_thread_smem(r);
+  int blocks = 0;
+  cudaError_t e = allow_smem((const void*)pair_thread_kernel<false>, smem);
+  if (e == cudaSuccess)
+    e = max_blocks((const void*)pair_thread_kernel<false>, kThreadBlock, smem, &blocks);
+  if (e != cudaSuccess || blocks < 1) return e;
+  const float k = 1e-3f * (float)B, S = (float)r.S, P = (float)r.P;
+  const int more = (r.nblk > 8 ? (r.nblk + 7) / 8 : 1) - 1;
+  const float lanes = 4.5f + k * (0.125f + 0.0016f * S + 0.073f * (float)more);
+  const int64_t wave = (int64_t)blocks * kThreadBlock * sm_count();
+  const float waves = (float)((B + wave - 1) / wave);
+  const float one = 5.0f + 0.11f * S + 0.075f * P;  // a wave's latency
+  const float rate = 3.0f + k * (0.006f * S + 0.0012f * P);
+  *out = std::max(waves * one, rate) * (0.85f + 0.15f * waves) < lanes;
+  return cudaSuccess;
+}
+
 static cudaError_t launch_pair_small(const DevRobot& r, const PairSchedule32& ps, const FwdArgs& a,
                                      cudaStream_t s) {
   const size_t smem = pair_small_smem(r);
@@ -339,7 +369,7 @@ static cudaError_t launch_pair_small(const DevRobot& r, const PairSchedule32& ps
   // blocks of 32 configurations; past 16 a multiprocessor each block takes
   // several passes, evenly, so that its tables are staged once for them
   const int64_t need = (a.B + 4 * kSmallWarps - 1) / (4 * kSmallWarps);
-  const int64_t passes = (need + 16 * 152 - 1) / (16 * 152);
+  const int64_t most = 16 * (int64_t)sm_count(), passes = (need + most - 1) / most;
   kern<<<(unsigned)((need + passes - 1) / passes), 32 * kSmallWarps, smem, s>>>(r, ps, a);
   return cudaGetLastError();
 }
@@ -386,7 +416,12 @@ static cudaError_t pair_dispatch(const DevRobot& r, const PairSchedule32& ps, co
 
 cudaError_t launch_pair(const DevRobot& r, const PairSchedule32& ps, const FwdArgs& a, int grid,
                         int warps, cudaStream_t s, bool cull) {
-  if (cull && pair_small_ok(r, a)) return launch_pair_small(r, ps, a, s);  // small robots
+  if (cull && pair_small_ok(r, a)) {  // small robots
+    bool thread = false;
+    const cudaError_t e = thread_better(r, a.B, &thread);
+    if (e != cudaSuccess) return e;
+    return thread ? launch_pair_thread(r, a, s) : launch_pair_small(r, ps, a, s);
+  }
   if (cull && pair_thread_ok(r)) return launch_pair_thread(r, a, s);
   return pair_dispatch(r, ps, a, grid, warps, s, nullptr, cull);
 }
