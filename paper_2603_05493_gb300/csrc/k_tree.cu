@@ -479,10 +479,12 @@ static cudaError_t launch_bwd(void (*kern)(P...), int64_t B, int groups, int blo
 // 99999 configurations 0.171 -> 0.155 and, at 110 MB in two segments, 0.081 -> 0.064.
 // Smaller poses are better off without (20 links, 110 MB: 0.041 ms), and so are up to
 // 20 warps (32 links, 80000 configurations 0.068 and 0.073).
+bool poses_beyond_l2(const DevRobot& r, int64_t B, int G) {
+  return B * r.n * 48 > (int64_t)(G > 1 ? 100 : 112) << 20;
+}
 static size_t pose_smem(const DevRobot& r, int64_t B, int G, int threads, size_t smem) {
   const int64_t warps = (B + 31) / 32 * G;
-  if (B * r.n * 48 <= (int64_t)(G > 1 ? 100 : 112) << 20 || warps <= 20LL * sm_count())
-    return smem;
+  if (!poses_beyond_l2(r, B, G) || warps <= 20LL * sm_count()) return smem;
   const size_t blocks = std::max(1, 16 * 32 / threads);
   const size_t share = 228 * 1024 / blocks - 1024;  // 228 KB an SM, 1 KB of it each block's own
   return std::max(smem, std::min(kSegSmemMax, share));
@@ -509,6 +511,51 @@ static cudaError_t fwd_chain(const DevRobot& r, int64_t B, int threads, size_t s
   return cudaSuccess;
 }
 
+// The one-segment forward sweep's kernel and dynamic shared memory.
+struct WholeKernel {
+  void (*kern)(DevRobot, WalkTab, FwdArgs);
+  size_t smem;
+};
+static cudaError_t fwd_whole(const DevRobot& r, int64_t B, int threads, bool tau, WholeKernel* out) {
+  const size_t fs = sizeof(float) * 6 * fs_levels(r) * threads;  // the force stack
+  const bool use_fs = tau && rec_smem(r, true) + fs <= kSegSmemMax;
+  size_t smem = rec_smem(r, true) + (use_fs ? fs : 0);
+  if (!tau) smem = pose_smem(r, B, 1, threads, smem);
+  bool chain = false;
+  const cudaError_t e = use_fs ? fwd_chain(r, B, threads, smem, &chain) : cudaSuccess;
+  out->kern = chain    ? tree_fwd_chain_kernel
+              : use_fs ? tree_fwd_kernel<kFwdShared>
+              : tau    ? tree_fwd_kernel<kFwdLocal>
+                       : tree_fwd_kernel<kFwdPose>;
+  out->smem = smem;
+  return e;
+}
+static size_t fwd_spline_smem(const DevRobot& r, int64_t B, int threads, bool tau) {
+  const size_t smem = 12 * sizeof(float) * threads + rec_smem(r, true);
+  return tau ? smem : pose_smem(r, B, 1, threads, smem);
+}
+
+// the blocks of `threads` threads that an SM holds of it (spline: with states from
+// control points)
+cudaError_t fwd_whole_blocks(const DevRobot& r, int64_t B, int threads, bool tau, bool spline,
+                             int* out) {
+  const void* kern;
+  size_t smem;
+  if (spline) {
+    kern = tau ? (const void*)tree_fwd_spline_kernel<kFwdLocal>
+               : (const void*)tree_fwd_spline_kernel<kFwdPose>;
+    smem = fwd_spline_smem(r, B, threads, tau);
+  } else {
+    WholeKernel w;
+    const cudaError_t e = fwd_whole(r, B, threads, tau, &w);
+    if (e != cudaSuccess) return e;
+    kern = (const void*)w.kern;
+    smem = w.smem;
+  }
+  const cudaError_t e = allow_smem(kern, smem);
+  return e != cudaSuccess ? e : max_blocks(kern, threads, smem, out);
+}
+
 cudaError_t launch_tree_fwd(const DevRobot& r, const WalkTab& wt, const FwdArgs& a, int threads, int segments,
                             cudaStream_t s) {
   if (threads <= 0) threads = 128;
@@ -525,22 +572,13 @@ cudaError_t launch_tree_fwd(const DevRobot& r, const WalkTab& wt, const FwdArgs&
                       a, threads, segments, true,
                       a.tau ? 0 : pose_smem(r, a.B, segments, (int)bt, base) - base, s);
   }
-  const size_t fs = sizeof(float) * 6 * fs_levels(r) * threads;  // the force stack
-  const bool use_fs = a.tau && rec_smem(r, true) + fs <= kSegSmemMax;
-  size_t smem = rec_smem(r, true) + (use_fs ? fs : 0);
-  if (!a.tau) smem = pose_smem(r, a.B, 1, threads, smem);
-  bool chain = false;
-  cudaError_t e = use_fs ? fwd_chain(r, a.B, threads, smem, &chain) : cudaSuccess;
+  WholeKernel w;
+  cudaError_t e = fwd_whole(r, a.B, threads, a.tau != nullptr, &w);
+  if (e == cudaSuccess) e = allow_smem((const void*)w.kern, w.smem);
   if (e != cudaSuccess) return e;
-  auto kern = chain    ? tree_fwd_chain_kernel
-              : use_fs ? tree_fwd_kernel<kFwdShared>
-              : a.tau  ? tree_fwd_kernel<kFwdLocal>
-                       : tree_fwd_kernel<kFwdPose>;
-  e = allow_smem((const void*)kern, smem);
-  if (e != cudaSuccess) return e;
-  fit_carveout((const void*)kern, threads, smem);
+  fit_carveout((const void*)w.kern, threads, w.smem);
   const int64_t grid = (a.B + threads - 1) / threads;
-  kern<<<(unsigned)grid, threads, smem, s>>>(r, wt, a);
+  w.kern<<<(unsigned)grid, threads, w.smem, s>>>(r, wt, a);
   return cudaGetLastError();
 }
 
@@ -595,8 +633,7 @@ cudaError_t launch_tree_fwd_spline(const DevRobot& r, const WalkTab& wt, const F
     kern<<<(unsigned)grid, block, smem, s>>>(r, wt, a, sp, t);
     return cudaGetLastError();
   }
-  size_t smem = 12 * sizeof(float) * threads + rec_smem(r, true);
-  if (!a.tau) smem = pose_smem(r, a.B, 1, threads, smem);
+  const size_t smem = fwd_spline_smem(r, a.B, threads, a.tau != nullptr);
   auto kern = a.tau ? tree_fwd_spline_kernel<kFwdLocal> : tree_fwd_spline_kernel<kFwdPose>;
   const cudaError_t e = allow_smem((const void*)kern, smem);
   if (e != cudaSuccess) return e;

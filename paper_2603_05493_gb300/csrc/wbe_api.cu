@@ -1014,27 +1014,71 @@ static int pair_warps(wb_robot* R, bool bits, const wb_tune* tune, bool cull = t
   return best;
 }
 
+// What a sweep call needs, as far as its shape goes.
+struct SweepKind {
+  bool fwd, spline, tau;
+};
+
+// Threads per block of a one-segment sweep and the warps an SM then holds of it: 128,
+// or for a forward sweep of more warps than that holds the first of these counts that
+// takes the fewest passes.  The force stacks decide: the humanoid's allow 4 blocks of
+// 128 threads but 4 of 160 and 3 of 224 too (16, 20, 21 warps), 80000 configurations
+// (16.4 warps an SM) 0.173, 0.132, 0.136 ms, 99999 (20.6) 0.196, 0.203, 0.165.
+// price: of a link in one segment against one in several.  Poses alone beyond the L2:
+// 16 warps are let in, and two segments' more even writes are the better ones (60000
+// configurations of the humanoid, 141 MB, 0.089 and 0.080 ms; 80000 0.132 and 0.121).
+struct WholeShape {
+  int threads, warps;
+  double price;
+};
+static WholeShape whole_shape(const wb_robot* R, int64_t B, SweepKind k) {
+  const int64_t sms = std::max(R->num_sms, 1);
+  if (k.fwd && !k.tau && (B + 31) / 32 > 12 * sms && poses_beyond_l2(R->dev, B, 2))
+    return {128, 16, 1.2};
+  if (!k.fwd || (B + 31) / 32 <= 16 * sms) return {128, 16, 1.0};
+  WholeShape best{128, 16, 1.0};
+  int64_t least = 0;
+  for (int threads : {128, 160, 224, 192, 256, 96}) {
+    int blocks = 0;
+    if (fwd_whole_blocks(R->dev, B, threads, k.tau, k.spline, &blocks) != cudaSuccess ||
+        blocks < 1) {
+      cudaGetLastError();
+      continue;
+    }
+    const int64_t share = ((B + threads - 1) / threads + sms - 1) / sms;
+    const int64_t passes = (share + blocks - 1) / blocks;
+    if (least == 0 || passes < least) {
+      least = passes;
+      best = {threads, blocks * threads / 32, 1.0};
+    }
+  }
+  return best;
+}
+
 // Segments of the sweep kernels (wb_tune.lanes_per_config for TREE): 1, 2, 4
 // or 8; 0 = the plan with the least estimated time.  A sweep's time is the
 // links a warp walks times the time of one, which grows with the warps that
 // share the SM: (10 + w) in units of one warp's issue time (humanoid: 1.5 us +
 // 0.16 us a resident warp in the backward, 0.8 + 0.11 in the forward), w at
-// most 16 (the registers of an SM), passes beyond that after one another.
+// most what an SM holds (16 of the backward's warps and of the segmented
+// forward's, which keep 128 and 100 registers a thread; `whole` of a
+// one-segment forward's), passes beyond that after one another.
 // Against the fewest segments that give 12 warps an SM, forward / backward ms:
-// humanoid 12000 configurations 0.031 / 0.047 (was 0.042 / 0.062), 20011 0.045 /
-// 0.080 (0.055 / 0.091), 40000 0.084 / 0.131 (0.102 / 0.150), 50000 0.090 / 0.134
-// (0.116 / 0.165); 7-DoF arm 20000 0.011 / 0.017 (0.019 / 0.026); no change at
+// humanoid 12000 configurations 0.028 / 0.047 (was 0.042 / 0.062), 20011 0.041 /
+// 0.080 (0.055 / 0.091), 40000 0.083 / 0.131 (0.102 / 0.150), 50000 0.088 / 0.134
+// (0.116 / 0.165); 7-DoF arm 20000 0.009 / 0.017 (0.019 / 0.026); no change at
 // 9150, 32768 and 99999.
 template <class Fits>
-static int auto_segments(const wb_robot* R, int64_t B, Fits&& fits) {
+static int auto_segments(const wb_robot* R, int64_t B, const WholeShape& whole, Fits&& fits) {
   const double per_sm = (double)((B + 31) / 32) / std::max(R->num_sms, 1);
   int best = 1;
   double least = 0.0;
   for (int t = 0; t < 4; ++t) {
     if (t > 0 && (!(R->dev.seg_ok >> (t - 1) & 1) || !fits(1 << t))) continue;
-    const double w = per_sm * (1 << t), full = std::floor(w / 16.0), rest = w - 16.0 * full;
-    const double time =
-        R->seg_cost[t] * (full * 26.0 + (rest > 0.0 ? 10.0 + std::max(rest, 1.0) : 0.0));
+    const double most = t == 0 ? std::max(whole.warps, 1) : 16.0;
+    const double w = per_sm * (1 << t), full = std::floor(w / most), rest = w - most * full;
+    const double pass = full * (10.0 + most) + (rest > 0.0 ? 10.0 + std::max(rest, 1.0) : 0.0);
+    const double time = R->seg_cost[t] * (t == 0 ? whole.price : 1.0) * pass;
     if (t == 0 || time < least) {
       least = time;
       best = 1 << t;
@@ -1046,8 +1090,10 @@ static int auto_segments(const wb_robot* R, int64_t B, Fits&& fits) {
 // one block an SM with an even share of the batch's groups, while it fits
 // (humanoid 32768 configurations: 448 threads, forward 0.062 -> 0.058,
 // backward 0.098 -> 0.093 ms against 128; 20011: 320 threads, 0.080 -> 0.076
-// ms), else 128.
-static int auto_threads(const wb_robot* R, int64_t B, int G, bool fwd, bool spline) {
+// ms), else 128; at one segment whole_shape's.
+static int auto_threads(const wb_robot* R, int64_t B, int G, bool fwd, bool spline,
+                        const WholeShape& whole) {
+  if (G == 1) return whole.threads;
   if (G != 2 && G != 4) return 128;
   const int64_t groups = (B + 31) / 32;
   const int64_t cg = (groups + R->num_sms - 1) / std::max(R->num_sms, 1);
@@ -1064,7 +1110,8 @@ static int auto_threads(const wb_robot* R, int64_t B, int G, bool fwd, bool spli
 // sweep; the threads are lowered where the link records no longer leave room
 // for the partials of all the block's groups.
 static int tree_segments(const wb_robot* R, const wb_tune* tune, int64_t B, int* tpb,
-                         bool fwd, int* out, bool spline = false) {
+                         const SweepKind& kind, int* out) {
+  const bool fwd = kind.fwd, spline = kind.spline;
   const int req = tune ? tune->lanes_per_config : 0;
   const int ok = R->dev.seg_ok;
   int G = 1;
@@ -1075,7 +1122,10 @@ static int tree_segments(const wb_robot* R, const wb_tune* tune, int64_t B, int*
       return fail(WB_EINVAL, "no %d-segment sweep for this robot (fewer links, or a joint "
                   "driving several links)", req);
     G = req;
-  } else {  // the fewest that give about 12 warps per SM: what a call is held to
+  } else {
+    // The fewest that give about 12 warps per SM.  A call without a tune is refused for
+    // what this shape does not fit, whatever shape it takes below, so that the robots
+    // and batches that are accepted do not change with the estimates.
     const int64_t warps = (B + 31) / 32;
     const int64_t target = 12LL * R->num_sms;
     for (int t = 0; t < 3 && warps * G < target; ++t)
@@ -1097,9 +1147,11 @@ static int tree_segments(const wb_robot* R, const wb_tune* tune, int64_t B, int*
                       basis * std::max(threads, 32 * G);
   if (G > 1 && need(G, threads) - more > kMaxBlockSmem)
     return fail(WB_ETOOBIG, "segmented sweep needs too much shared memory");
+  const WholeShape whole = req <= 1 ? whole_shape(R, B, kind) : WholeShape{128, 16, 1.0};
   if (req <= 0 && threads <= 256)
-    G = auto_segments(R, B, [&](int g) { return need(g, threads) <= kMaxBlockSmem; });
-  if (*tpb == 0) *tpb = auto_threads(R, B, G, fwd, spline);
+    G = auto_segments(R, B, whole,
+                      [&](int g) { return need(g, threads) <= kMaxBlockSmem; });
+  if (*tpb == 0) *tpb = auto_threads(R, B, G, fwd, spline, whole);
   while (G > 1 && need(G, *tpb) > kMaxBlockSmem) {
     if (*tpb >= 64 * G)
       *tpb -= 32 * G;
@@ -1183,7 +1235,7 @@ int wb_eval_dir(wb_robot* robot, int64_t B, const float* q, const float* qd, con
     if (pairs_wanted && pair_block_smem(robot->dev, warps, pair_bits != nullptr) > kMaxBlockSmem)
       return fail(WB_ETOOBIG, "%d pair warps per block need too much shared memory", warps);
     int G = 1;
-    if ((rc = tree_segments(robot, tune, B, &tpb, true, &G))) return rc;
+    if ((rc = tree_segments(robot, tune, B, &tpb, {true, false, tau != nullptr}, &G))) return rc;
     e = launch_tree_fwd(robot->dev, robot->walk, a, tpb, G, s);
     if (e == cudaSuccess && pairs_wanted) {
       int bps = 0;
@@ -1408,7 +1460,7 @@ int wb_eval_backward_dir(wb_robot* robot, int64_t B, const float* q, const float
     if (tpb != 0 && (tpb < 32 || tpb > 512 || tpb % 32))
       return fail(WB_EINVAL, "tree threads per block must be a multiple of 32 in [32, 512]");
     int G = 1;
-    if ((rc = tree_segments(robot, tune, B, &tpb, false, &G))) return rc;
+    if ((rc = tree_segments(robot, tune, B, &tpb, {false, false, true}, &G))) return rc;
     e = launch_tree_bwd(robot->dev, robot->walk, a, tpb, G, s);
   } else if (kernel == WB_KERNEL_FUSED) {
     if (a.fext || a.g_fext) return fail(WB_EINVAL, "the fused kernels take no external forces");
@@ -1473,7 +1525,7 @@ int wb_eval_spline(wb_robot* robot, const wb_spline* spline, float* link_pose, f
   if (tpb != 0 && (tpb < 32 || tpb > 512 || tpb % 32))
     return fail(WB_EINVAL, "tree threads per block must be a multiple of 32 in [32, 512]");
   int G = 1;
-  if ((rc = tree_segments(robot, tune, B, &tpb, true, &G, true))) return rc;
+  if ((rc = tree_segments(robot, tune, B, &tpb, {true, true, tau != nullptr}, &G))) return rc;
   cudaError_t e = launch_tree_fwd_spline(robot->dev, robot->walk, a, sp, tpb, G, s);
   if (e == cudaSuccess && pairs_wanted) {
     const int warps = pair_warps(robot, false, tune, kernel != WB_KERNEL_TREE_NOCULL);
@@ -1561,7 +1613,7 @@ int wb_eval_backward_spline_cost_dir(wb_robot* robot, const wb_spline* spline,
   if (tpb != 0 && (tpb < 32 || tpb > 512 || tpb % 32))
     return fail(WB_EINVAL, "tree threads per block must be a multiple of 32 in [32, 512]");
   int G = 1;
-  if ((rc = tree_segments(robot, tune, B, &tpb, false, &G, true))) return rc;
+  if ((rc = tree_segments(robot, tune, B, &tpb, {false, true, true}, &G))) return rc;
   const cudaError_t e = launch_tree_bwd_spline_cost(robot->dev, robot->walk, a, fc, sp, tpb, G,
                                                     static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "wb_eval_backward_spline_cost launch");
@@ -1638,7 +1690,7 @@ int wb_eval_backward_cost_dir(wb_robot* robot, int64_t B, const float* q, const 
   if (tpb != 0 && (tpb < 32 || tpb > 512 || tpb % 32))
     return fail(WB_EINVAL, "tree threads per block must be a multiple of 32 in [32, 512]");
   int G = 1;
-  if ((rc = tree_segments(robot, tune, B, &tpb, false, &G))) return rc;
+  if ((rc = tree_segments(robot, tune, B, &tpb, {false, false, true}, &G))) return rc;
   const cudaError_t e =
       launch_tree_bwd(robot->dev, robot->walk, a, tpb, G, static_cast<cudaStream_t>(stream), &fc);
   if (e != cudaSuccess) return cuda_fail(e, "wb_eval_backward_cost launch");

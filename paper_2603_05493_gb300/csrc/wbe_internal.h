@@ -322,6 +322,11 @@ cudaError_t launch_trajopt_cost(int64_t B, int d, const float* tau, const float*
 // threads: threads per block, a multiple of 32, at most 256 for one segment
 // and 512 for a segmented sweep (its launch bounds); every sweep block also
 // stages the robot's link parameters in shared memory
+// whether poses written by G segments a configuration outgrow the L2 (k_tree.cu)
+bool poses_beyond_l2(const DevRobot& r, int64_t B, int G);
+// blocks of `threads` threads an SM holds of the one-segment forward sweep
+cudaError_t fwd_whole_blocks(const DevRobot& r, int64_t B, int threads, bool tau, bool spline,
+                             int* out);
 cudaError_t launch_tree_fwd(const DevRobot& r, const WalkTab& wt, const FwdArgs& a, int threads, int segments,
                             cudaStream_t s);
 cudaError_t launch_tree_bwd(const DevRobot& r, const WalkTab& wt, const BwdArgs& a, int threads, int segments,
