@@ -92,6 +92,15 @@ MEASURED_TRAFFIC = {  # kernel[@workload]: (sources, their hash, bytes / evaluat
 }
 
 
+def arm_sweep_kernel(seg, B, num_sms):
+    """The forward sweep that the library runs for the 7-DoF arm with torques: its
+    one-segment batches of more than 24 warps a multiprocessor go to the kernel of
+    robots without branches."""
+    if seg > 1:
+        return "tree_fwd_seg_kernel"
+    return "tree_fwd_chain_kernel" if B > 24 * 32 * num_sms else "tree_fwd_kernel"
+
+
 def source_hash(files):
     import hashlib
     h = hashlib.sha256()
@@ -1059,7 +1068,8 @@ def run_arm7(args, rank=0, world=1, local_rank=0):
     pair_ms = ms - sweep_ms
     kernels = {
         "tree_fwd": dict(hbm(w["tree_fwd"]["bytes"], sweep_ms), ms=sweep_ms,
-                         kernel="tree_fwd_seg_kernel" if seg > 1 else "tree_fwd_kernel",
+                         kernel=arm_sweep_kernel(
+                             seg, B, torch.cuda.get_device_properties(dev).multi_processor_count),
                          bytes_per_eval=w["tree_fwd"]["bytes"]),
         # robots of at most 32 spheres and 1024 pairs take the library's
         # eight-lanes-a-configuration pair kernel
