@@ -316,22 +316,23 @@ __device__ __forceinline__ void pair_one(const DevRobot& r, const PairSchedule32
 // Every 4-sphere group gets a bounding sphere (C_g, R_g): for a group on one
 // link, a host-made sphere in that link's frame moved with the link;
 // otherwise the mean of its centres and the largest |c - C_g| + r; both
-// widened for float rounding.  For any
-// pair (a in group i, b in group j), d_ab >= |C_i - C_j| - R_i - R_j =: lb, so
-// a block whose lb exceeds an upper bound on d_min holds no candidate for the
-// minimum (nor, with lb >= 0, a colliding pair).  Pass 1 finds the block of
-// smallest lb and the exact minimum of its pairs, a real pair distance and
-// so an upper bound on d_min, and keeps every block's lb as a half, rounded
-// down below a margin for the approximate square root; pass 2 walks the
-// schedule again, keeps the blocks whose stored lb is within the margin of
-// the current bound (or below 0 when the pair bits are wanted) -- a superset
-// of the blocks an exact test would keep -- queues them warp-wide (ballot +
-// prefix count) and screens 32 queued blocks at a time with the usual screen
-// and exact path.  The culled path forms the row copies of a block's spheres
-// (-2 c) when it screens the block, and keeps the bounds where the full
-// map-reduce keeps those copies.  The result -- d_min, the worst pair with its tie rule, the bits --
-// is that of the full map-reduce; only blocks that cannot affect it are
-// skipped.
+// widened for rounding and held as halves relative to the first link
+// (half_bound, mixed_bound).  For any pair (a in group i, b in group j), d_ab >=
+// |C_i - C_j| - R_i - R_j >= lb (half_gap), so a block whose lb exceeds an upper
+// bound on d_min holds no candidate for the minimum (nor, with lb >= 0, a
+// colliding pair); a lb that is no number keeps its block.  Pass 1 finds the block
+// of smallest lb and the exact minimum of its pairs, a real pair distance and so
+// an upper bound on d_min, and keeps every block's lb as a half, rounded to
+// nearest.  Pass 2 keeps the blocks whose stored lb is at most the current bound
+// (or 0 when the pair bits are wanted) and a margin, rounded the same way: rounding
+// is monotone, so these are a superset of the blocks an exact test would keep.  It
+// queues them from a warp scan of the lanes' counts and screens 32 at a time with
+// the usual screen and exact path.  Where the lbs do not fit the row region they
+// are formed again and queued by ballots.  The culled path forms the row copies of
+// a block's spheres (-2 c) when it screens the block, and keeps the lbs where the
+// full map-reduce keeps those copies.  The result -- d_min, the worst pair with its
+// tie rule, the bits -- is that of the full map-reduce; only blocks that cannot
+// affect it are skipped.
 template <bool FULL, bool BITS>
 __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSchedule32& ps,
                                                 const FwdArgs& A, int64_t b, float* ws,
@@ -499,12 +500,12 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
   // region when they fit, two rounds a word, rounded to nearest: rounding is
   // monotone, so a bound at most the threshold stays at most the threshold's
   // half, and pass 2 keeps every block its exact test would keep (and at most
-  // a few more, within the half's rounding).  Two rounds a step with the
-  // blocks' offsets decoded by the host, null blocks against a far sphere in
-  // place of a test, the smallest bound carried with its round in its low 11
-  // bits, and two bounds compared an instruction in pass 2: humanoid48 pair
-  // stage 0.117 -> 0.105 ms at 32768 configurations (0.097 with the wavefronts
-  // saved below, 0.092 with the bounds in halves).
+  // a few more, within the half's rounding).  Two rounds a step, two offsets a
+  // word, null blocks against a far sphere in place of a test, the smallest bound
+  // carried with its round in its low 11 bits, and two bounds compared an
+  // instruction in pass 2: humanoid48 pair stage 0.117 -> 0.105 ms at 32768
+  // configurations (0.097 with the wavefronts saved below, 0.092 with the bounds in
+  // halves, 0.087 with two offsets a word and the queue decoded by its takers).
   const int prs = ps.prs;
   const bool keep_lb = prs * 32 <= pl.ra_words();
   __half2* lb2 = reinterpret_cast<__half2*>(xr) + lane;
@@ -678,7 +679,7 @@ __device__ __forceinline__ void pair_one_culled(const DevRobot& r, const PairSch
   };
   if (keep_lb) {
     // Per chunk of 32 rounds, each lane first marks its surviving blocks in a
-    // bit mask (one half load and one compare a round), then the survivors are
+    // bit mask (one load and one compare two rounds), then the survivors are
     // queued in lane order, positions from a warp scan of the lanes' counts,
     // and screened 32 at a time.  The threshold is refreshed per chunk; the
     // order of the screening does not change the result (the exact path keeps
