@@ -78,16 +78,16 @@ PAIR_SRC = ["paper_2603_05493_gb300/csrc/k_pair.cu", "paper_2603_05493_gb300/csr
             "paper_2603_05493_gb300/csrc/spatial.cuh"] + API_SRC
 SPLINE_SRC = ["paper_2603_05493_gb300/csrc/k_traj.cu",
               "paper_2603_05493_gb300/csrc/spline_basis.cuh"] + API_SRC
-TREE_SHA = "64cc9fda4690329b746f0f04e4a372709be5fedcd36b57d47725e0573bfc8aba"
-PAIR_SHA = "2fab9d8345554adbafa0ec6520f79625942c3ce3a6dd3bb06b04b48f7b16b928"
-SPLINE_SHA = "472e279cf6f19c37f18a16f2f0fb68bcd07d7dd7673b35533c279f420e26b5fa"
+TREE_SHA = "66c700c960645caa350abda4f32d5f48069d17171c67a181d94609d900a6faa8"
+PAIR_SHA = "f448dc92d424d8996d8add12a859ce1485eeba43f42dd39613d0ad9e36c2d2b5"
+SPLINE_SHA = "f95c26d8998c45e69466c086987a060c937ca80053e26e4f9f2f1151674c5815"
 MEASURED_TRAFFIC = {  # kernel[@workload]: (sources, their hash, bytes / evaluation)
-    "tree_fwd_seg_kernel": (TREE_SRC, TREE_SHA, (24.17e6 + 51.58e6) / 32768),
-    "pair_kernel": (PAIR_SRC, PAIR_SHA, (77.30e6 + 32.16e6) / 32768),
-    "tree_bwd_seg_kernel": (TREE_SRC, TREE_SHA, (233.20e6 + 30.19e6) / 32768),
-    "tree_fwd_spline_seg_kernel": (TREE_SRC, TREE_SHA, (5.48e6 + 51.73e6) / 32768),
-    "pair_kernel@trajopt48": (PAIR_SRC, PAIR_SHA, (77.26e6 + 0.69e6) / 32768),
-    "tree_bwd_spline_cost_seg_kernel": (TREE_SRC, TREE_SHA, (8.66e6 + 0.34e6) / 32768),
+    "tree_fwd_seg_kernel": (TREE_SRC, TREE_SHA, (24.26e6 + 51.66e6) / 32768),
+    "pair_kernel": (PAIR_SRC, PAIR_SHA, (77.29e6 + 33.54e6) / 32768),
+    "tree_bwd_seg_kernel": (TREE_SRC, TREE_SHA, (233.03e6 + 30.12e6) / 32768),
+    "tree_fwd_spline_seg_kernel": (TREE_SRC, TREE_SHA, (5.58e6 + 51.89e6) / 32768),
+    "pair_kernel@trajopt48": (PAIR_SRC, PAIR_SHA, (77.26e6 + 0.61e6) / 32768),
+    "tree_bwd_spline_cost_seg_kernel": (TREE_SRC, TREE_SHA, (8.66e6 + 0.32e6) / 32768),
     "bspline_bwd_kernel": (SPLINE_SRC, SPLINE_SHA, (18.91e6 + 0.00e6) / 32768),
 }
 
