@@ -6,7 +6,7 @@
 // u = (c_i - c_j) / |c_i - c_j|).  Feeding that gradient to the backward
 // sweep as the sphere upstream gradient gives dcost/dq.
 //
-// One warp per configuration (persistent grid).  The warp stages the
+// One warp per configuration (a persistent grid beyond 4 passes).  The warp stages the
 // configuration's link poses into shared memory, places its spheres (Sec.
 // 6.1.1) as SoA rows and bounds every group of 4 with a sphere (C_g, R_g)
 // (for a group on one link, the host-made sphere in its link frame moved
