@@ -78,9 +78,9 @@ PAIR_SRC = ["paper_2603_05493_gb300/csrc/k_pair.cu", "paper_2603_05493_gb300/csr
             "paper_2603_05493_gb300/csrc/spatial.cuh"] + API_SRC
 SPLINE_SRC = ["paper_2603_05493_gb300/csrc/k_traj.cu",
               "paper_2603_05493_gb300/csrc/spline_basis.cuh"] + API_SRC
-TREE_SHA = "66c700c960645caa350abda4f32d5f48069d17171c67a181d94609d900a6faa8"
-PAIR_SHA = "f448dc92d424d8996d8add12a859ce1485eeba43f42dd39613d0ad9e36c2d2b5"
-SPLINE_SHA = "f95c26d8998c45e69466c086987a060c937ca80053e26e4f9f2f1151674c5815"
+TREE_SHA = "30743b721b42c5778969816afd187b5c348d606f7cf039d1275b840634c686bb"
+PAIR_SHA = "3cb64f1ebed4ad76f729af8d33591d0ae12c8b072c5a21363c43137dbac1c2b0"
+SPLINE_SHA = "418a5b53dbef80e671b13ab7d4583693282fbf9f6d8ab6a3927818966cbcf963"
 MEASURED_TRAFFIC = {  # kernel[@workload]: (sources, their hash, bytes / evaluation)
     "tree_fwd_seg_kernel": (TREE_SRC, TREE_SHA, (24.26e6 + 51.66e6) / 32768),
     "pair_kernel": (PAIR_SRC, PAIR_SHA, (77.29e6 + 33.54e6) / 32768),

@@ -1148,9 +1148,14 @@ static int tree_segments(const wb_robot* R, const wb_tune* tune, int64_t B, int*
   if (G > 1 && need(G, threads) - more > kMaxBlockSmem)
     return fail(WB_ETOOBIG, "segmented sweep needs too much shared memory");
   const WholeShape whole = req <= 1 ? whole_shape(R, B, kind) : WholeShape{128, 16, 1.0};
-  if (req <= 0 && threads <= 256)
-    G = auto_segments(R, B, whole,
-                      [&](int g) { return need(g, threads) <= kMaxBlockSmem; });
+  if (req <= 0 && threads <= 256) {
+    // By the sweep of joint states also where they come from control points: with the
+    // same segments both give the same torques to the bit.  That has its price where
+    // the two are apart (humanoid, 99968 configurations: one segment 0.165 ms from
+    // joint states, but 0.248 from control points, and two would take 0.179).
+    const WholeShape by = spline ? whole_shape(R, B, {fwd, false, kind.tau}) : whole;
+    G = auto_segments(R, B, by, [&](int g) { return need(g, threads) <= kMaxBlockSmem; });
+  }
   if (*tpb == 0) *tpb = auto_threads(R, B, G, fwd, spline, whole);
   while (G > 1 && need(G, *tpb) > kMaxBlockSmem) {
     if (*tpb >= 64 * G)
